@@ -76,7 +76,14 @@ enum {
                                     solves replay it and one graph for the remainder), captured
                                     on first use and kept while the launch configuration holds;
                                     0: direct launches */
-    FUSE_OPT_LATENT_IMPL = 3,    /* latent pass: 1 (default) bulk-copy ring, 0 register-staged loads */
+    FUSE_OPT_LATENT_IMPL = 3,    /* latent pass: 1 (default) or 0: keep the state entry by entry, with
+                                    register-staged loads.  By default (3 x 3 and 5 x 5 patches, state
+                                    in the iterate type, S <= 15) solves keep the entries of a (tau,
+                                    pixel, band) as a few levels and update those; the same results
+                                    bit for bit.  Where the levels do not apply (other patches, the
+                                    16-bit state, a state or weights set while a solve is continued,
+                                    no memory for them) the entries stream through a bulk-copy ring,
+                                    which the next three options shape. */
     FUSE_OPT_LATENT_THREADS = 4, /* consumer threads per latent block, 32..256 (default 128;
                                     256 in batches) */
     FUSE_OPT_LATENT_STAGES = 5,  /* ring slots of the bulk-copy latent pass, 2..32 (default 6) */
@@ -147,7 +154,10 @@ enum {
 };
 
 /* Bytes of device memory fuse_init would allocate for this problem (state in the default
- * half-window mode, weights, FFT buffers and constants).  No device work.  Errors: FUSE_EINVAL, FUSE_EUNSUPPORTED. */
+ * half-window mode, weights, FFT buffers and constants).  The first solve (fuse_batch_create for a
+ * batch) also allocates the records of the compact state where that applies: 16 bytes (FP64: 32) per
+ * kept offset, band and pixel, 8 more with 5 x 5 patches, and one value per kept offset, patch entry
+ * and pixel; without the memory for them solves run on the entries alone.  No device work.  Errors: FUSE_EINVAL, FUSE_EUNSUPPORTED. */
 fuse_status fuse_workspace_bytes(const fuse_geometry* g, int K, int S, int ratio,
                                  fuse_dtype dtype, fuse_dtype wdtype, size_t* bytes);
 

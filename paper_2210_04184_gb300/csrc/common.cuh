@@ -203,6 +203,21 @@ struct TauMap {
     }
 };
 
+// Kept offset q (the state's offset index) -> (tau1, tau2): inverse of TauMap::s_index.
+__device__ __forceinline__ void tau_of_state_index(int q, int S, int half, int* t1, int* t2) {
+    const int side = 2 * S + 1;
+    if (half) {
+        if (q < S) { *t1 = 0; *t2 = q + 1; return; }
+        const int r = q - S;
+        *t1 = r / side + 1;
+        *t2 = r % side - S;
+        return;
+    }
+    const int cell = q >= (side * side) / 2 ? q + 1 : q;
+    *t1 = cell / side - S;
+    *t2 = cell % side - S;
+}
+
 // A batched launch is a 1D grid whose blocks are split into segments; segment s covers the
 // blocks [start, start + gx*gy*gz) of problem `prob`, laid out x fastest, with block row z
 // starting at z0.  Segments are sorted by start.

@@ -59,7 +59,7 @@ constexpr int kGraphIters = 256;
 // remainder of a long solve), the least recently used one is replaced.
 struct LoopGraph {
     cudaGraphExec_t exec = nullptr;
-    int len = 0, cold = 0;
+    int len = 0, cold = 0, form = 0;        // form: that of the latent state (fuse_ctx::form)
     long long launches = 0;
     unsigned long long used = 0;
 };
@@ -67,9 +67,9 @@ struct LoopGraph {
 struct LoopCache {
     LoopGraph g[2];
     unsigned long long tick = 0;
-    LoopGraph* find(int len, int cold) {
+    LoopGraph* find(int len, int cold, int form) {
         for (LoopGraph& x : g)
-            if (x.exec && x.len == len && x.cold == cold) { x.used = ++tick; return &x; }
+            if (x.exec && x.len == len && x.cold == cold && x.form == form) { x.used = ++tick; return &x; }
         return nullptr;
     }
     LoopGraph* victim() { return g[0].used <= g[1].used ? &g[0] : &g[1]; }
@@ -166,6 +166,18 @@ struct fuse_ctx {
     int half = 1;
     // latent state storage: 0 = the iterate type, 1 = 16-bit fixed point relative to mu
     int sfmt = 0;
+    // Compact latent state (k_levels.cuh; patch half-sizes 1 and 2, state in the iterate type):
+    // records and level masks in hdr, level values in Sig, sorted thresholds of the current weights in
+    // tab (formed by the first solve that needs them), X with its code sums in pt.  form: what the state is kept as, 0 = entries in Sig, 1 = levels.
+    // grid [3]: the state's grid, that for omega_was, and that for weights up to 1 (fuse_weights).
+    // entries_ok: the entries are known to be those of a run on the current weights, so they convert to
+    // levels.  was: the weights changed since the levels were formed; omega_was holds the old ones.
+    // reg_chosen: the caller selected the register-staged pass.
+    void *hdr = nullptr, *tab = nullptr, *pt = nullptr, *grid = nullptr, *omega_was = nullptr;
+    int form = 0;
+    bool entries_ok = false, was = false, grid_set = false, reg_chosen = false, tab_ok = false, lv_refused = false;
+    int lv_Ty = 1, lv_threads = 0, lv_nb = 1;
+    size_t lv_smem = 0;
     // sampling mask [H][W] (uint8, ratio 1) replacing the regular lattice; NULL = lattice.
     // The buffer (mask_buf) is kept once allocated, so launch arguments taken earlier (a batch)
     // never point to freed memory.
@@ -443,6 +455,12 @@ struct Sizes {
     size_t img, cimg, sig, planes, omega, d9a;
 };
 
+// Bytes of the compact state's records (and, for 5 x 5 patches, level masks) of nk kept offsets; no
+// compact state for other patches.
+size_t header_bytes(int K, size_t nk, int Ls, size_t n, size_t esz) {
+    return latent_grid_k(K) ? nk * Ls * n * (4 * esz + (K == 1 ? 0 : sizeof(uint2))) : 0;
+}
+
 Sizes sizes_of(const fuse_geometry* g, int K, int S, int ratio, size_t esz, size_t wsz, int half = 1) {
     Sizes z;
     const size_t n = (size_t)g->H * g->W;
@@ -480,6 +498,91 @@ bool latent_tma_shape(fuse_ctx* c) {
     return true;
 }
 
+void levels_free(fuse_ctx* c) {
+    for (void** p : {&c->hdr, &c->tab, &c->pt, &c->omega_was}) {
+        if (*p) cudaFree(*p);
+        *p = nullptr;
+    }
+}
+
+// Launch shape of the latent pass on the compact state: `threads` per block, rows for about as many
+// pixels, and as many bands as the event lists and `room` bytes of shared memory allow.
+struct LevelShape {
+    int Ty = 1, nb = 0;         // nb 0: the pass does not fit
+    size_t smem = 0;
+};
+LevelShape level_shape(const fuse_ctx* c, int threads, size_t room) {
+    LevelShape z;
+    const int nt2 = 2 * c->S + 1;
+    z.Ty = std::max(1, std::min(threads / c->W, c->H));
+    const int tile = z.Ty * c->W;
+    if (!latent_grid_k(c->K) || nt2 > kLevelSteps || tile > kLevelTile) return z;
+    auto smem = [&](int b) { return c->esz == 8 ? levels_smem<double>(b * nt2, tile) : levels_smem<float>(b * nt2, tile); };
+    z.nb = std::min(c->Ls, kLevelSteps / nt2);
+    while (z.nb > 1 && smem(z.nb) > room) --z.nb;
+    z.smem = smem(z.nb);
+    if (z.smem > (size_t)kMaxSmem) z.nb = 0;
+    return z;
+}
+// Threads an SM holds at the kernel's registers (64 in FP32, 80 in FP64) and the shared memory that
+// lets it hold them in blocks of kLevelThreads.  Measured at HS+MS 256 x 256 (iteration 64): 262 us with
+// 128 threads and 28 KB a block, 272 us with 256 threads and 56 KB, 319 us with 128 threads and 20 KB;
+// 24 tiles of 96 to 384: 2.5 ms with 128 threads and 20 KB, 2.7 ms with 32 KB.
+constexpr int kLevelThreads = 128;
+int level_sm_threads(size_t esz) { return esz == 8 ? 768 : 1024; }
+size_t level_room(size_t esz) { return (size_t)227 * 1024 / (level_sm_threads(esz) / kLevelThreads) - 1024; }
+
+// A problem alone: fewer bands per block until the pass has about three blocks per SM; blocks of half
+// the threads where those all fit the device at once and the larger ones do not (FP64 pansharpening
+// at 128 x 128: 35 us against 45).
+void levels_shape(fuse_ctx* c) {
+    const LevelShape z = level_shape(c, kLevelThreads, level_room(c->esz));
+    c->lv_threads = 0;
+    if (z.nb == 0) return;
+    const long long rows = (long long)((c->H + z.Ty - 1) / z.Ty) * (c->half ? c->S + 1 : 2 * c->S + 1);
+    auto blocks = [&](int b) { return rows * ((c->Ls + b - 1) / b); };
+    c->lv_Ty = z.Ty;
+    c->lv_nb = z.nb;
+    while (c->lv_nb > 1 && blocks(c->lv_nb) < 6ll * c->nsm) --c->lv_nb;
+    c->lv_smem = z.smem / z.nb * c->lv_nb;
+    c->lv_threads = kLevelThreads;
+    const long long slots = (long long)c->nsm * level_sm_threads(c->esz) / kLevelThreads;
+    if (blocks(c->lv_nb) > slots && blocks(c->lv_nb) <= 2 * slots) c->lv_threads = kLevelThreads / 2;
+}
+
+// The latent state lives on the grid (latent_grid.cuh), whichever form and kernel a solve uses.
+bool on_grid(const fuse_ctx* c) { return c->lv_threads > 0 && c->sfmt == 0; }
+
+// The buffers of the compact state, allocated by the first solve that would use them (not while its
+// stream is captured) and kept.  Without the memory for them solves keep the state as entries, with the
+// same results.
+bool levels_alloc(fuse_ctx* c) {
+    if (c->hdr) return true;
+    if (c->lv_refused || c->fault_alloc >= 0) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    const size_t nk = c->half ? c->nW / 2 : c->nW;
+    const size_t img = c->n * c->Ls * c->esz;
+    void** p[] = {&c->hdr, &c->tab, &c->pt, &c->omega_was};
+    const size_t bytes[] = {header_bytes(c->K, nk, c->Ls, c->n, c->esz), nk * c->nP * c->n * c->esz, 4 * img,
+                            (size_t)c->nW * c->n * c->wsz};
+    bool ok = true;
+    for (int i = 0; i < 4 && ok; ++i) ok = *p[i] || cudaMalloc(p[i], bytes[i]) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(c->pt, 0, 4 * img, c->stream) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        levels_free(c);
+        c->lv_refused = true;
+    }
+    return ok;
+}
+
+// Solves keep the latent state as levels.
+bool uses_levels(fuse_ctx* c) { return on_grid(c) && !c->reg_chosen && levels_alloc(c); }
+
 // Dynamic shared-memory cap of the monitoring latent kernels of this context's types.
 bool set_monitor_smem(fuse_ctx* c) {
     cudaError_t e;
@@ -514,10 +617,23 @@ struct Impl {
     }
     template <typename WT>
     static LatentArgs<T, WT> lat_args(fuse_ctx* c, int Ty, int ncons, int D, int bpb, int zero_in = 0) {
-        return LatentArgs<T, WT>{(const T*)c->X, (const WT*)c->omega, (const T*)lat_src(c), (T*)lat_dst(c),
-                                 (T*)c->planes, c->H, c->W,
-                                 c->Ls, c->S, Ty, ncons, D, (T)(c->lam2 / c->rho), c->d_err, c->wait_limit,
-                                 c->half, bpb, zero_in};
+        LatentArgs<T, WT> a{(const T*)c->X, (const WT*)c->omega, (const T*)lat_src(c), (T*)lat_dst(c),
+                            (T*)c->planes, c->H, c->W,
+                            c->Ls, c->S, Ty, ncons, D, (T)(c->lam2 / c->rho), c->d_err, c->wait_limit,
+                            c->half, bpb, zero_in};
+        a.grid = (const LatentGrid<T>*)c->grid;
+        return a;
+    }
+    // old: the weights (and their bound) from before the last change
+    template <typename WT>
+    static LevelArgs<T, WT> lv_args(fuse_ctx* c, bool old = false) {
+        using C = ucode_t<T>;
+        const size_t nk = c->half ? c->nW / 2 : c->nW;
+        LevelRecord<C>* rec = (LevelRecord<C>*)c->hdr;
+        return LevelArgs<T, WT>{(const T*)c->X, (const WT*)(old ? c->omega_was : c->omega), rec,
+                                (uint2*)(rec + nk * c->Ls * c->n), (C*)c->Sig,
+                                (const code_t<T>*)c->tab, (const LevelPoint<T>*)c->pt, (T*)c->planes, c->H, c->W, c->Ls, c->S, c->lv_Ty, c->lv_nb,
+                                (T)(c->lam2 / c->rho), (const LatentGrid<T>*)c->grid + (old ? 1 : 0), c->half};
     }
 
     static fuse_status set_attrs(fuse_ctx* c) {
@@ -539,6 +655,7 @@ struct Impl {
         const auto A = cudaFuncAttributeMaxDynamicSharedMemorySize;
         CK(c, cudaFuncSetAttribute(weights_kernel<T, WT>, A, kMaxSmem));
         CK(c, (latent_set_smem<T, WT>(c->K, kMaxSmem)));
+        if (latent_grid_k(c->K)) CK(c, (levels_set_smem<T, WT>(c->K, kMaxSmem)));
         return FUSE_OK;
     }
 
@@ -594,17 +711,47 @@ struct Impl {
     template <typename WT>
     static void latent(fuse_ctx* c, cudaStream_t s, bool zero_in) {
         const unsigned rowsW = (unsigned)(c->half ? c->S + 1 : 2 * c->S + 1);
+        const bool taped = c->lat_in || c->lat_out;
+        if (c->form == 1 && !taped) {
+            dim3 grid((unsigned)((c->H + c->lv_Ty - 1) / c->lv_Ty), (unsigned)((c->Ls + c->lv_nb - 1) / c->lv_nb), rowsW);
+            points_launch<T>((const T*)c->X, (LevelPoint<T>*)c->pt, c->n * c->Ls, (const LatentGrid<T>*)c->grid, zero_in,
+                             s);
+            const LevelArgs<T, WT> a = lv_args<WT>(c);
+            if (zero_in) levels_init_launch<T, WT>(a, c->K, c->half ? c->nW / 2 : c->nW, s);
+            // X of a cold first iteration is zero with the paper's splitting, and so are the planes
+            if (!zero_in || c->xmode == 1)
+                levels_launch<T, WT>(a, c->K, grid, (unsigned)c->lv_threads, c->lv_smem, s);
+            return;
+        }
         if (c->lat_impl == 1) {
             dim3 grid((unsigned)((c->H + c->lt_Ty - 1) / c->lt_Ty), (unsigned)((c->Ls + c->lat_bpb - 1) / c->lat_bpb),
                       rowsW);
             const LatentArgs<T, WT> a = lat_args<WT>(c, c->lt_Ty, c->lt_ncons, c->lat_stages, c->lat_bpb, zero_in);
-            latent_tma_launch<T, WT>(a, c->K, c->sfmt == 1, grid, (unsigned)(c->lt_ncons + 32), c->lt_smem, s);
+            latent_tma_launch<T, WT>(a, c->K, c->sfmt == 1, on_grid(c) && !taped, grid, (unsigned)(c->lt_ncons + 32), c->lt_smem, s);
             return;
         }
         dim3 grid((unsigned)((c->H + c->lat_Ty - 1) / c->lat_Ty), (unsigned)c->Ls, rowsW);
         latent_reg_launch<T, WT>((const T*)c->X, (const WT*)c->omega, (const T*)lat_src(c), (T*)lat_dst(c),
                                  (T*)c->planes, c->H, c->W, c->Ls, c->S, c->lat_Ty, (T)(c->lam2 / c->rho), c->half,
-                                 c->K, grid, (unsigned)c->lat_threads, c->lat_smem, s);
+                                 (const LatentGrid<T>*)c->grid, c->K, on_grid(c) && !taped, grid, (unsigned)c->lat_threads, c->lat_smem, s);
+    }
+
+    // The state between its two forms, in place (see levels_convert_launch).
+    template <typename WT>
+    static void convert(fuse_ctx* c, bool to_levels, bool check, int* bad) {
+        const int kept = c->half ? c->nW / 2 : c->nW;
+        levels_convert_launch<T, WT>(lv_args<WT>(c, !to_levels && c->was), c->K, kept, to_levels, check, bad, c->stream);
+    }
+    static void convert_any(fuse_ctx* c, bool to_levels, bool check, int* bad);
+    template <typename WT>
+    static void table(fuse_ctx* c) {
+        level_table_launch<T, WT>((const WT*)c->omega, (code_t<T>*)c->tab, c->H, c->W, c->K, c->S, c->half,
+                                  c->half ? c->nW / 2 : c->nW, (T)(c->lam2 / c->rho), (const LatentGrid<T>*)c->grid, c->stream);
+    }
+    static void table_any(fuse_ctx* c);
+    template <typename WT>
+    static void weights_bound(fuse_ctx* c) {
+        wmax_launch<T, WT>((const WT*)c->omega, (size_t)c->nW * c->n, (LatentGrid<T>*)c->grid, (T)(c->lam2 / c->rho), c->stream);
     }
 
     static void latent_any(fuse_ctx* c, cudaStream_t s, bool zero_in);
@@ -621,7 +768,7 @@ struct Impl {
         a.mpart = c->mon_part;
         c->mon_lat = (size_t)grid.x * grid.y * grid.z;
         const size_t smem = c->lt_smem + 2 * (size_t)c->lt_Ty * c->W * sizeof(T);     // two more tiles
-        latent_monitor_launch<T, WT>(a, c->K, grid, (unsigned)(c->lt_ncons + 32), smem, s);
+        latent_monitor_launch<T, WT>(a, c->K, on_grid(c), grid, (unsigned)(c->lt_ncons + 32), smem, s);
     }
 
     static fuse_status monitor_sums(fuse_ctx* c, cudaStream_t s) {
@@ -765,6 +912,26 @@ void Impl<T>::latent_any(fuse_ctx* c, cudaStream_t s, bool zero_in) {
 }
 
 template <typename T>
+void Impl<T>::convert_any(fuse_ctx* c, bool to_levels, bool check, int* bad) {
+    if constexpr (sizeof(T) == 8) {
+        convert<double>(c, to_levels, check, bad);
+    } else {
+        if (c->wdtype == FUSE_BF16) convert<__nv_bfloat16>(c, to_levels, check, bad);
+        else convert<float>(c, to_levels, check, bad);
+    }
+}
+
+template <typename T>
+void Impl<T>::table_any(fuse_ctx* c) {
+    if constexpr (sizeof(T) == 8) {
+        table<double>(c);
+    } else {
+        if (c->wdtype == FUSE_BF16) table<__nv_bfloat16>(c);
+        else table<float>(c);
+    }
+}
+
+template <typename T>
 fuse_status Impl<T>::objective(fuse_ctx* c, const void* Yl, const void* Yh, double out[4]) {
     const size_t n = c->n;
     stencil<0>(c, c->stream, c->X, c->BX, c->tapsB);
@@ -811,6 +978,58 @@ fuse_status guard(fuse_ctx* c) {
     return FUSE_OK;
 }
 
+fuse_status convert_state(fuse_ctx* c, bool to_levels, bool check = false, int* bad = nullptr) {
+    if (c->dtype == FUSE_F64) Impl<double>::convert_any(c, to_levels, check, bad);
+    else Impl<float>::convert_any(c, to_levels, check, bad);
+    c->launches_all++;
+    CKL(c, "latent state conversion");
+    return FUSE_OK;
+}
+
+// The state as entries.  Levels formed with weights that have changed since give entries that need
+// not be those of a run on the current ones.
+fuse_status need_entries(fuse_ctx* c) {
+    if (c->form == 0) return FUSE_OK;
+    const fuse_status st = convert_state(c, false);
+    if (st != FUSE_OK) return st;
+    c->form = 0;
+    c->entries_ok = !c->was;
+    c->was = false;
+    return FUSE_OK;
+}
+
+// The sorted thresholds of the current weights, which the iterations on levels read.
+fuse_status need_table(fuse_ctx* c) {
+    if (c->form != 1 || c->tab_ok) return FUSE_OK;
+    if (c->dtype == FUSE_F64) Impl<double>::table_any(c);
+    else Impl<float>::table_any(c);
+    c->launches_all++;
+    CKL(c, "level_table_kernel");
+    c->tab_ok = true;
+    return FUSE_OK;
+}
+
+// The form in which the iterations of a warm solve continue: levels where the state allows it.
+fuse_status warm_form(fuse_ctx* c) {
+    if (c->form == 1 && (c->was || !uses_levels(c))) return need_entries(c);
+    if (c->form == 0 && c->entries_ok && uses_levels(c)) {
+        const fuse_status st = convert_state(c, true);
+        if (st != FUSE_OK) return st;
+        c->form = 1;
+    }
+    return FUSE_OK;
+}
+
+// Before the weights change: levels stay readable through the weights they were formed with.
+fuse_status weights_change(fuse_ctx* c) {
+    c->entries_ok = c->tab_ok = false;
+    if (c->form != 1 || !c->have_state || c->was) return FUSE_OK;
+    CK(c, cudaMemcpyAsync(c->omega_was, c->omega, (size_t)c->nW * c->n * c->wsz, cudaMemcpyDeviceToDevice, c->stream));
+    CK(c, cudaMemcpyAsync((char*)c->grid + 3 * c->esz, c->grid, 3 * c->esz, cudaMemcpyDeviceToDevice, c->stream));
+    c->was = true;
+    return FUSE_OK;
+}
+
 // Zero ADMM state.  clear_sigma = false leaves the latent state as it is: the caller's next
 // iteration then runs a latent pass that reads none of it (zero_in) and overwrites all of it.
 fuse_status zero_state(fuse_ctx* c, cudaStream_t s, bool clear_sigma = true) {
@@ -826,12 +1045,12 @@ fuse_status zero_state(fuse_ctx* c, cudaStream_t s, bool clear_sigma = true) {
 }
 
 // kernels launched by one iteration (Impl::iterate)
-int iteration_launches(const fuse_ctx* c) { return c->xmode == 1 ? 6 : 7; }
+int iteration_launches(const fuse_ctx* c) { return (c->xmode == 1 ? 6 : 7) + (c->form == 1 ? 1 : 0); }
 
 // Replays `len` iterations from one captured graph (captured on first use; `cold`: the first
 // iteration's latent pass reads no state).
 fuse_status launch_loop(fuse_ctx* c, int len, bool cold) {
-    LoopGraph* lg = c->loops.find(len, cold);
+    LoopGraph* lg = c->loops.find(len, cold, c->form);
     if (!lg) {
         const bool f64 = c->dtype == FUSE_F64;
         CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -855,6 +1074,7 @@ fuse_status launch_loop(fuse_ctx* c, int len, bool cold) {
         if (e != cudaSuccess) { lg->exec = nullptr; return fail_cuda(c, "cudaGraphInstantiate", e); }
         lg->len = len;
         lg->cold = cold;
+        lg->form = c->form;
         lg->launches = (long long)len * iteration_launches(c);
         lg->used = ++c->loops.tick;
     }
@@ -878,6 +1098,10 @@ fuse_status monitored_iteration(fuse_ctx* c, bool zero_in) {
                                           "iterate type and the paper's splitting");
     if (c->lt_smem + 2 * (size_t)c->lt_Ty * c->W * c->esz > (size_t)kMaxSmem)
         return fail(c, FUSE_EUNSUPPORTED, "the monitoring latent pass does not fit shared memory");
+    fuse_status st = FUSE_OK;
+    if (zero_in) c->form = 0;                  // the pass reads no state and writes entries
+    else if ((st = need_entries(c)) != FUSE_OK) return st;
+    c->entries_ok = true;
     const size_t img = c->n * c->Ls * c->esz;
     cudaStream_t s = c->stream;
     CK(c, cudaMemcpyAsync(c->mL1, c->Lam1, img, cudaMemcpyDeviceToDevice, s));
@@ -885,8 +1109,8 @@ fuse_status monitored_iteration(fuse_ctx* c, bool zero_in) {
     CK(c, cudaMemcpyAsync(c->mL2, c->Lam2, img, cudaMemcpyDeviceToDevice, s));
     CK(c, cudaMemcpyAsync(c->mU2, c->U2, img, cudaMemcpyDeviceToDevice, s));
     CK(c, cudaMemcpyAsync(c->mPo, c->planes, c->plane_bytes, cudaMemcpyDeviceToDevice, s));
-    fuse_status st = c->dtype == FUSE_F64 ? Impl<double>::iterate(c, s, false, zero_in, true)
-                                          : Impl<float>::iterate(c, s, false, zero_in, true);
+    st = c->dtype == FUSE_F64 ? Impl<double>::iterate(c, s, false, zero_in, true)
+                              : Impl<float>::iterate(c, s, false, zero_in, true);
     if (st != FUSE_OK) return st;
     c->launches_all += iteration_launches(c);
     c->launches_latent += 1;
@@ -937,11 +1161,17 @@ fuse_status solve_impl(fuse_ctx* c, const void* Yl, const void* Yh, int iters, i
     // latent pass of the bulk-copy kernel takes it as zero and overwrites every entry.
     bool cold = false;
     if (!warm || !c->have_state) {
-        cold = iters > 0 && c->lat_impl == 1;
+        cold = iters > 0 && (c->lat_impl == 1 || uses_levels(c));
         st = zero_state(c, c->stream, !cold);
         if (st != FUSE_OK) return st;
         c->have_state = true;
+        c->form = cold && uses_levels(c) ? 1 : 0;
+        c->entries_ok = true;                  // zeros are the entries of a run on any weights
+        c->was = false;
+    } else if ((st = warm_form(c)) != FUSE_OK) {
+        return st;
     }
+    if ((st = need_table(c)) != FUSE_OK) return st;
     if (c->xmode == 1) {
         // the fixed data term of the variant: U1 = G = B^T S^T Y_l E^T / rho (B X as scratch)
         st = f64 ? Impl<double>::sb_data_term(c, c->stream) : Impl<float>::sb_data_term(c, c->stream);
@@ -964,6 +1194,11 @@ fuse_status solve_impl(fuse_ctx* c, const void* Yl, const void* Yh, int iters, i
 fuse_status weights_impl(fuse_ctx* c, const void* G) {
     fuse_status st;
     ++c->epoch;
+    if ((st = weights_change(c)) != FUSE_OK) return st;
+    if (c->grid_set) {
+        CK(c, cudaMemcpyAsync(c->grid, (char*)c->grid + 6 * c->esz, 3 * c->esz, cudaMemcpyDeviceToDevice, c->stream));
+        c->grid_set = false;
+    }
     if (c->dtype == FUSE_F64) st = Impl<double>::weights<double>(c, G);
     else if (c->wdtype == FUSE_BF16) st = Impl<float>::weights<__nv_bfloat16>(c, G);
     else st = Impl<float>::weights<float>(c, G);
@@ -981,12 +1216,17 @@ fuse_status realloc_state(fuse_ctx* c, int h, int f) {
     for (auto& p : c->allocs)
         if (p == c->Sig) { CK(c, cudaStreamSynchronize(c->stream)); cudaFree(p); p = nullptr; }
     c->Sig = nullptr;
+    levels_free(c);
+    c->lv_refused = false;
     fuse_status s2 = dalloc(c, &c->Sig, bytes);
     if (s2 != FUSE_OK) return s2;
     c->sig_bytes = bytes;
     c->half = h;
     c->sfmt = f;
+    c->form = 0;
+    c->entries_ok = c->was = c->tab_ok = false;
     latent_tma_shape(c);
+    levels_shape(c);
     ++c->epoch;
     c->have_state = false;
     c->have_x = false;
@@ -999,6 +1239,7 @@ void release(fuse_ctx* c) {
     c->gw = nullptr;
     drop_graphs(c);
     for (auto& e : c->ev) { cudaEventDestroy(e.a); cudaEventDestroy(e.b); }
+    levels_free(c);
     for (void* p : c->allocs)
         if (p) cudaFree(p);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -1110,6 +1351,12 @@ struct fuse_batch {
     int fr_rpb = 4, fc_cw = 8;
     // device tables: [args of every problem] and segments per kernel
     void* d_lat = nullptr; Segment* d_lat_seg = nullptr; int lat_nseg = 0, lat_blocks = 0;
+    // latent pass on the compact state (levels: every problem allows it): its arguments, blocks of the
+    // pass and of the points
+    bool levels = false;
+    void* d_lv = nullptr; Segment* d_lv_seg = nullptr; Segment* d_pt_seg = nullptr;
+    int lv_nseg = 0, lv_blocks = 0, pt_nseg = 0, pt_blocks = 0;
+    size_t lv_smem = 0;
     void* d_st1 = nullptr; void* d_st0 = nullptr; Segment* d_st_seg = nullptr; int st_nseg = 0, st_blocks = 0;
     // separable B X: blocks of stencil_sep_bands bands (band groups in z)
     Segment* d_sep0_seg = nullptr; int sep0_nseg = 0, sep0_blocks = 0;
@@ -1210,6 +1457,38 @@ struct BatchImpl {
         fuse_status st;
         if ((st = bupload(b, &b->d_lat, la)) != FUSE_OK) return st;
         if ((st = bupload(b, (void**)&b->d_lat_seg, seg)) != FUSE_OK) return st;
+
+        b->levels = true;
+        for (fuse_ctx* c : b->ctx) b->levels = b->levels && on_grid(c) && levels_alloc(c);
+        if (b->levels) {
+            std::vector<LevelArgs<T, WT>> lv(n);
+            std::vector<Segment> sp;
+            int np = 0;
+            seg.clear();
+            next = 0;
+            b->lv_smem = 0;
+            for (int i = 0; i < n; ++i) {
+                fuse_ctx* c = b->ctx[i];
+                // the launch fills the device whatever one problem's size: as many bands per block as fit
+                lv[i] = Impl<T>::template lv_args<WT>(c);
+                const LevelShape z = level_shape(c, kLevelThreads, level_room(esz));
+                lv[i].Ty = z.Ty;
+                lv[i].nb = z.nb;
+                b->lv_smem = std::max(b->lv_smem, z.smem);
+                add_segment(sp, i, (int)((c->n * c->Ls + 1023) / 1024), 1, 1, 0, &np);
+            }
+            for (int heavy = 1; heavy >= 0; --heavy)       // tau1 != 0 rows of every problem first
+                for (int i = 0; i < n; ++i)
+                    add_segment(seg, i, (b->ctx[i]->H + lv[i].Ty - 1) / lv[i].Ty, (b->Ls + lv[i].nb - 1) / lv[i].nb,
+                                heavy ? rows - 1 : 1, heavy ? 0 : rows - 1, &next);
+            b->lv_nseg = (int)seg.size();
+            b->lv_blocks = next;
+            b->pt_nseg = (int)sp.size();
+            b->pt_blocks = np;
+            if ((st = bupload(b, &b->d_lv, lv)) != FUSE_OK) return st;
+            if ((st = bupload(b, (void**)&b->d_lv_seg, seg)) != FUSE_OK) return st;
+            if ((st = bupload(b, (void**)&b->d_pt_seg, sp)) != FUSE_OK) return st;
+        }
 
         // stencils (same blur for all problems)
         std::vector<StencilArgs<T>> s1(n), s0(n);
@@ -1340,8 +1619,19 @@ struct BatchImpl {
             b->ev_used++;
             BCK(b, cudaEventRecord(e0, s));
         }
+        if (b->levels) {
+            const LevelArgs<T, WT>* lv = (const LevelArgs<T, WT>*)b->d_lv;
+            points_batch_launch<T, WT>(lv, b->d_pt_seg, b->pt_nseg, zero_in ? 1 : 0, (unsigned)b->pt_blocks, s);
+            if (zero_in) {              // X of a cold first iteration is zero, and so are the planes
+                for (fuse_ctx* c : b->ctx)
+                    levels_init_launch<T, WT>(Impl<T>::template lv_args<WT>(c), c->K, c->half ? c->nW / 2 : c->nW, s);
+            } else {
+                levels_batch_launch<T, WT>(lv, b->d_lv_seg, b->lv_nseg, b->K, (unsigned)b->lv_blocks, kLevelThreads,
+                                           b->lv_smem, s);
+            }
+        } else
         latent_tma_batch_launch<T, WT>((const LatentArgs<T, WT>*)b->d_lat, b->d_lat_seg, b->lat_nseg, zero_in ? 1 : 0,
-                                       b->K, b->sfmt != 0, (unsigned)b->lat_blocks, (unsigned)(b->lat_ncons + 32),
+                                       b->K, b->sfmt != 0, on_grid(b->ctx[0]), (unsigned)b->lat_blocks, (unsigned)(b->lat_ncons + 32),
                                        b->lat_smem, s);
         if (timed) BCK(b, cudaEventRecord(e1, s));
         BCK(b, cudaGetLastError());
@@ -1392,7 +1682,7 @@ fuse_status batch_set_shape(fuse_batch* b, int threads, int stages, int bands) {
 
 // Batched counterpart of launch_loop: `len` batched iterations replayed from one graph.
 fuse_status batch_launch_loop(fuse_batch* b, int len, bool cold) {
-    LoopGraph* lg = b->loops.find(len, cold);
+    LoopGraph* lg = b->loops.find(len, cold, 0);
     if (!lg) {
         BCK(b, cudaStreamBeginCapture(b->cap_stream, cudaStreamCaptureModeThreadLocal));
         fuse_status st = FUSE_OK;
@@ -1414,7 +1704,7 @@ fuse_status batch_launch_loop(fuse_batch* b, int len, bool cold) {
         if (e != cudaSuccess) { lg->exec = nullptr; BCK(b, e); }
         lg->len = len;
         lg->cold = cold;
-        lg->launches = 7LL * len;
+        lg->launches = (b->levels ? 8LL : 7LL) * len;
         lg->used = ++b->loops.tick;
     }
     BCK(b, cudaGraphLaunch(lg->exec, b->stream));
@@ -1431,7 +1721,7 @@ fuse_status batch_run(fuse_batch* b, int iters, bool cold = false) {
         for (int t = 0; t < iters; ++t) {
             fuse_status st = batch_iterate(b, b->stream, b->profile, cold && t == 0);
             if (st != FUSE_OK) return st;
-            b->launches_all += 7;
+            b->launches_all += b->levels ? 8 : 7;
             b->launches_latent += 1;
         }
         return FUSE_OK;
@@ -1675,6 +1965,19 @@ fuse_status fuse_init(fuse_ctx** out, const fuse_geometry* g, const double* blur
     if ((st = dalloc(c, &c->planes, z.planes)) != FUSE_OK) return bail(st);
     if ((st = dalloc(c, &c->omega, z.omega)) != FUSE_OK) return bail(st);
     if ((st = dalloc(c, &c->D9a, z.d9a)) != FUSE_OK) return bail(st);
+    {
+        std::vector<double> gv;
+        for (int i = 0; i < 3; ++i) {
+            if (c->dtype == FUSE_F64) {
+                const LatentGrid<double> g1 = latent_grid(lambda2 / rho, 1.0);
+                gv.insert(gv.end(), {g1.g, g1.ig, g1.wmax});
+            } else {
+                const LatentGrid<float> g1 = latent_grid((float)(lambda2 / rho), 1.0f);
+                gv.insert(gv.end(), {(double)g1.g, (double)g1.ig, (double)g1.wmax});
+            }
+        }
+        if ((st = upload_any(c, &c->grid, gv)) != FUSE_OK) return bail(st);
+    }
     if ((st = upload_any(c, &c->tapsT, tT)) != FUSE_OK) return bail(st);
     if ((st = upload_any(c, &c->tapsB, tB)) != FUSE_OK) return bail(st);
     if ((st = upload_any(c, &c->fpf, fh)) != FUSE_OK) return bail(st);
@@ -1710,6 +2013,7 @@ fuse_status fuse_init(fuse_ctx** out, const fuse_geometry* g, const double* blur
         c->lat_stages = 4;
         if (!latent_tma_shape(c)) c->lat_impl = 0;
     }
+    levels_shape(c);
     const size_t nb = (c->n + 255) / 256;
     c->npartial = nb * 3 + nb * (size_t)c->nW;
     if ((st = dalloc(c, (void**)&c->partial, c->npartial * sizeof(double))) != FUSE_OK) return bail(st);
@@ -1754,7 +2058,18 @@ fuse_status fuse_set_weights(fuse_ctx* c, const void* w) {
     fuse_status st = guard(c);
     if (st != FUSE_OK) return st;
     if (!w) return fail(c, FUSE_EINVAL, "weights pointer is NULL");
+    if ((st = weights_change(c)) != FUSE_OK) return st;
     CK(c, cudaMemcpyAsync(c->omega, w, (size_t)c->nW * c->n * c->wsz, cudaMemcpyDefault, c->stream));
+    if (latent_grid_k(c->K)) {
+        // the grid of the latent state is set by the largest weight
+        CK(c, cudaMemsetAsync(c->grid, 0, 3 * c->esz, c->stream));
+        if (c->dtype == FUSE_F64) Impl<double>::weights_bound<double>(c);
+        else if (c->wdtype == FUSE_BF16) Impl<float>::weights_bound<__nv_bfloat16>(c);
+        else Impl<float>::weights_bound<float>(c);
+        c->launches_all += 2;
+        c->grid_set = true;
+        CKL(c, "wmax_kernel");
+    }
     c->have_weights = true;
     ++c->epoch;
     return FUSE_OK;
@@ -1852,6 +2167,7 @@ fuse_status fuse_get_state(fuse_ctx* c, void* dst) {
     if (st != FUSE_OK) return st;
     if (!dst) return fail(c, FUSE_EINVAL, "NULL state buffer");
     if (!c->have_state) return FUSE_ESTATE;
+    if ((st = need_entries(c)) != FUSE_OK) return st;
     const size_t img = c->n * c->Ls * c->esz;
     char* p = (char*)dst;
     void* bufs[] = {c->Lam1, c->U1, c->Lam2, c->U2, c->X};
@@ -1874,6 +2190,18 @@ fuse_status fuse_set_state(fuse_ctx* c, const void* src) {
     CK(c, cudaMemcpyAsync(c->Sig, p, c->sig_bytes, cudaMemcpyDefault, c->stream));
     p += c->sig_bytes;
     CK(c, cudaMemcpyAsync(c->planes, p, c->plane_bytes, cudaMemcpyDefault, c->stream));
+    c->form = 0;
+    c->entries_ok = c->was = false;
+    if (c->have_weights && uses_levels(c)) {
+        // a state saved from a run on these weights continues as levels, any other as entries
+        int* bad = (int*)c->partial;
+        int flag = 0;
+        CK(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
+        if ((st = convert_state(c, true, true, bad)) != FUSE_OK) return st;
+        CK(c, cudaMemcpyAsync(&flag, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        CK(c, cudaStreamSynchronize(c->stream));
+        c->entries_ok = flag == 0;
+    }
     CK(c, cudaStreamSynchronize(c->stream));
     c->have_state = true;
     c->have_x = true;
@@ -1912,6 +2240,7 @@ fuse_status fuse_set_option(fuse_ctx* c, int option, long long value) {
                 latent_tma_shape(c);
                 return fail(c, FUSE_EINVAL, "latent launch option out of range");
             }
+            if (option == FUSE_OPT_LATENT_IMPL) c->reg_chosen = !value;
             drop_graphs(c);
             return FUSE_OK;
         }
@@ -2079,9 +2408,10 @@ fuse_status fuse_autotune(fuse_ctx* c, const void* Yl, const void* Yh, int iters
     // inputs and a zero state (the timed iterations run on it; the next solve starts over)
     st = solve_impl(c, Yl, Yh, 0, 0, nullptr, nullptr);
     if (st != FUSE_OK) return st;
+    if ((st = warm_form(c)) != FUSE_OK || (st = need_table(c)) != FUSE_OK) return st;
     double best = 1e30, t = 0;
-    // 1. latent pass: ring shape and bands per block
-    if (c->lat_impl == 1) {
+    // 1. latent pass: ring shape and bands per block (the pass on the compact state has one shape)
+    if (c->lat_impl == 1 && c->form == 0) {
         const int bt = c->lat_target, bs = c->lat_stages, bb = c->lat_bpb;
         int best_t = bt, best_s = bs, best_b = bb;
         const int threads[] = {128, 192, 256}, stages[] = {4, 6, 8, 12, 16, 24}, bands[] = {1, 2};
@@ -2255,6 +2585,10 @@ fuse_status fuse_batch_solve(fuse_batch* b, const void* const* Yl, const void* c
         if (st == FUSE_OK) st = zero_state(c, b->stream, iters == 0);
         if (st != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
         c->have_state = true;
+        c->form = b->levels && iters > 0 ? 1 : 0;
+        c->entries_ok = iters == 0;
+        c->was = false;
+        if ((st = need_table(c)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
     }
     fuse_status st = batch_run(b, iters, iters > 0);
     if (st != FUSE_OK) return st;
@@ -2351,6 +2685,7 @@ fuse_status fuse_batch_get_option(fuse_batch* b, int option, long long* value) {
 fuse_status fuse_batch_autotune(fuse_batch* b, const void* const* Yl, const void* const* Yh, int iters) {
     if (!b || !Yl || !Yh || iters < 1) return FUSE_EINVAL;
     if (b->sticky != FUSE_OK) return FUSE_ESTATE;
+    if (b->levels) return fuse_batch_solve(b, Yl, Yh, 0, nullptr, nullptr);   // the pass has one shape
     const bool g = b->use_graph, pr = b->profile;
     b->use_graph = false;
     b->profile = false;

@@ -471,6 +471,7 @@ fuse_status grad_forward_impl(fuse_ctx* c, const void* Yl, const void* Yh, int i
             return FUSE_OK;
         });
         if (st != FUSE_OK) return st;
+        c->entries_ok = false;                  // entries rounded to the iterate type, not on the grid
     }
     c->have_x = true;
     const size_t img = c->n * c->Ls * c->esz;

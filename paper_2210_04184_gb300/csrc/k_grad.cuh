@@ -505,21 +505,6 @@ __global__ void __launch_bounds__(256) axpy_kernel(T* __restrict__ y, const T* _
         y[i] += x[i];
 }
 
-// Kept offset q (the state's offset index) -> (tau1, tau2): inverse of TauMap::s_index.
-__device__ __forceinline__ void tau_of_state_index(int q, int S, int half, int* t1, int* t2) {
-    const int side = 2 * S + 1;
-    if (half) {
-        if (q < S) { *t1 = 0; *t2 = q + 1; return; }
-        const int r = q - S;
-        *t1 = r / side + 1;
-        *t2 = r % side - S;
-        return;
-    }
-    const int cell = q >= (side * side) / 2 ? q + 1 : q;
-    *t1 = cell / side - S;
-    *t2 = cell % side - S;
-}
-
 // dL/domega of one reverse iteration, run before the latent reverse pass overwrites the state
 // adjoint.  mu = coef omega with coef = lambda2/rho, so for the output pixel i and offset tau
 //   omega_bar_tau(i) += scale sum_{k, c} mubar_{tau k c}(i),  scale = coef (x2 in half-window mode:

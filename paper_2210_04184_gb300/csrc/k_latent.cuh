@@ -29,15 +29,34 @@
 //
 // Layouts: X [L_s][H][W]; omega [|W|][H][W]; Sig' [|W| or |W|/2][|P|][L_s][H][W];
 // planes [L_s][2(2S+1)][H][W].  Threads: (W/VEC) x Ty, each owning VEC consecutive pixels.
+//
+// GRID (K = 1, 2, every pass but the taped forward's): the update on the grid of latent_grid.cuh,
+// where each entry and the sums over k are exact, so these kernels and the pass on the compact state
+// (k_levels.cuh) give the same bits; without it the entries are rounded to the iterate type.
 #pragma once
 #include "common.cuh"
+#include "latent_grid.cuh"
 
 namespace fuse {
 
-template <typename T, typename WT, int K, int VEC>
+// The threshold of one weight column: in the iterate type, or as a code on the grid.
+template <typename T, bool GRID>
+struct latent_bound {
+    SymBound<T> b;
+    __device__ __forceinline__ static latent_bound of(T mu, T) { return {SymBound<T>::of(mu)}; }
+    __device__ __forceinline__ T clamp(T u) const { return b.clamp(u); }
+};
+template <typename T>
+struct latent_bound<T, true> {
+    code_t<T> m;
+    __device__ __forceinline__ static latent_bound of(T mu, T ig) { return {mu_code(mu, ig)}; }
+    __device__ __forceinline__ code_t<T> clamp(code_t<T> u) const { return u > m ? m : (u < -m ? -m : u); }
+};
+
+template <typename T, typename WT, int K, int VEC, bool GRID>
 __global__ void __launch_bounds__(256)
 latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Sig, T* Sout,
-              T* __restrict__ planes, int H, int W, int Ls, int S, int Ty, T coef, int half) {
+              T* __restrict__ planes, int H, int W, int Ls, int S, int Ty, T coef, int half, const LatentGrid<T>* grid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* Hs = reinterpret_cast<T*>(smem_raw);           // [(2S+1)][Ty][W]
     constexpr int PS = 2 * K + 1;
@@ -56,6 +75,8 @@ latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Si
     const int side = 2 * S + 1;
     const T* Xc = X + (size_t)c * n;
     const size_t kstride = (size_t)Ls * n;
+    LatentGrid<T> gr{T(1), T(1), T(1)};
+    if constexpr (GRID) gr = *grid;
 
     T Xm[VEC];
     T A[VEC];
@@ -70,8 +91,13 @@ latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Si
         if (active) {
             const int ys = wrap1(y - t1, H);
             T delta[VEC];
+            code_t<T> dc[GRID ? VEC : 1], acc[GRID ? VEC : 1];
 #pragma unroll
-            for (int j = 0; j < VEC; ++j) delta[j] = Xm[j] - Xc[(size_t)ys * W + wrap1(x0 + j - t2, W)];
+            for (int j = 0; j < VEC; ++j) {
+                const T xs = Xc[(size_t)ys * W + wrap1(x0 + j - t2, W)];
+                delta[j] = Xm[j] - xs;
+                if constexpr (GRID) { dc[j] = delta_code<T>(Xm[j], xs, gr.ig); acc[j] = 0; }
+            }
             const WT* om = omega + (size_t)tm.w_index(t1, t2) * n;
             const size_t soff = ((size_t)tm.s_index(t1, t2) * NP * Ls + c) * n + (size_t)y * W + x0;
             const vecT<T, VEC>* sp = reinterpret_cast<const vecT<T, VEC>*>(Sig + soff);
@@ -81,10 +107,10 @@ latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Si
             for (int k1 = -K; k1 <= K; ++k1) {
                 // mu for the output pixels i = m + k, k2 in [-K, K]: columns x0-K .. x0+VEC-1+K
                 const int yw = wrap1(y + k1, H);
-                SymBound<T> mu[VEC + 2 * K];
+                latent_bound<T, GRID> mu[VEC + 2 * K];
 #pragma unroll
                 for (int j = 0; j < VEC + 2 * K; ++j)
-                    mu[j] = SymBound<T>::of(coef * (T)wload(om + (size_t)yw * W + wrap1(x0 - K + j, W)));
+                    mu[j] = latent_bound<T, GRID>::of(coef * (T)wload(om + (size_t)yw * W + wrap1(x0 - K + j, W)), gr.ig);
                 // issue the 2K+1 loads of this patch row before any store
                 vecT<T, VEC> s[PS];
 #pragma unroll
@@ -93,15 +119,25 @@ latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Si
                 for (int k2 = 0; k2 < PS; ++k2) {
 #pragma unroll
                     for (int j = 0; j < VEC; ++j) {
-                        const T u = s[k2].v[j] - delta[j];         // -v
-                        const T s2 = mu[j + k2].clamp(u);          // Sigma' = -clamp(v)
-                        Hacc[j] += T(2) * s2 - u;                  // G = v + 2 Sigma'
-                        s[k2].v[j] = s2;
+                        if constexpr (GRID) {
+                            const code_t<T> sc = to_code(s[k2].v[j] * gr.ig), s2 = mu[j + k2].clamp(sc - dc[j]);
+                            acc[j] += 2 * s2 - sc;
+                            s[k2].v[j] = (T)s2 * gr.g;
+                        } else {
+                            const T u = s[k2].v[j] - delta[j];     // -v
+                            const T s2 = mu[j + k2].clamp(u);      // Sigma' = -clamp(v)
+                            Hacc[j] += T(2) * s2 - u;              // G = v + 2 Sigma'
+                            s[k2].v[j] = s2;
+                        }
                     }
                     st_stream(so + (size_t)k2 * vstride, s[k2]);
                 }
                 sp += (size_t)PS * vstride;
                 so += (size_t)PS * vstride;
+            }
+            if constexpr (GRID) {
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) Hacc[j] = latent_h<NP>(delta[j], acc[j], gr.g);
             }
         }
 #pragma unroll
@@ -176,6 +212,7 @@ struct LatentArgs {
     // layout as `planes`) and one FP64 sum of (Sigma' - Sigma)^2 per block
     T* mplanes;
     double* mpart;
+    const LatentGrid<T>* grid;  // GRID only
 };
 
 __device__ __forceinline__ void consumer_barrier(int ncons) {
@@ -221,7 +258,7 @@ struct WRow {
 // the adjoint sums of Q' + Sigma = v + Sigma' + Sigma (into args.mplanes) and the block's sum of
 // (Sigma' - Sigma)^2 (into args.mpart): the latent parts of the ADMM dual and primal residuals
 // (Sec. IV, eq. dualvar3_main: D X - Q' = Sigma - Sigma').
-template <typename T, typename WT, int K, int VEC, typename ST, bool MON = false>
+template <typename T, typename WT, int K, int VEC, typename ST, bool GRID, bool MON = false>
 __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, int bx, int g, int row,
                                                 unsigned char* smem_tma) {
     const T* __restrict__ X = args.X;
@@ -319,6 +356,8 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
     unsigned par = 0;
     unsigned lim = limit;                                // 64 polls once a wait has timed out
     int hb = 0;                                          // H tile written next
+    LatentGrid<T> gr{T(1), T(1), T(1)};
+    if constexpr (GRID) gr = *args.grid;
     double dsq = 0.0;                                    // MON only: sum of (Sigma' - Sigma)^2
     for (int item = 0; item < nb; ++item) {
         const int c = c0 + item;
@@ -350,12 +389,19 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
             const int t2 = tm.t2_of(t1, jt);
             T Hacc[VEC], delta[VEC];
             T Macc[MON ? VEC : 1];
+            code_t<T> dc[GRID ? VEC : 1], acc[GRID ? VEC : 1], accm[GRID && MON ? VEC : 1];
             if (active) vload<T, VEC>(xo, delta);
 #pragma unroll
             for (int j = 0; j < VEC; ++j) {
                 Hacc[j] = T(0);
                 if constexpr (MON) Macc[j] = T(0);
-                delta[j] = active ? delta[j] - Xs[(size_t)r * W + ishift<VEC>(tcol, j - t2, tpr)] : T(0);
+                const T xm = delta[j], xs = active ? Xs[(size_t)r * W + ishift<VEC>(tcol, j - t2, tpr)] : T(0);
+                delta[j] = active ? xm - xs : T(0);
+                if constexpr (GRID) {
+                    dc[j] = active ? delta_code<T>(xm, xs, gr.ig) : code_t<T>(0);
+                    acc[j] = 0;
+                    if constexpr (MON) accm[j] = 0;
+                }
             }
             const WT* om = omega + (size_t)tm.w_index(t1, t2) * n;
             const WT* om_next = jt + 1 < nt2 ? omega + (size_t)tm.w_index(t1, tm.t2_of(t1, jt + 1)) * n : om;
@@ -363,9 +409,10 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
 #pragma unroll
             for (int k1 = 0; k1 < PS; ++k1) {
                 if constexpr (std::is_same<ST, T>::value) {
-                    SymBound<T> mu[VEC + 2 * K];
+                    latent_bound<T, GRID> mu[VEC + 2 * K];
 #pragma unroll
-                    for (int j = 0; j < VEC + 2 * K; ++j) mu[j] = SymBound<T>::of(active ? coef * (T)wr.get(j) : T(0));
+                    for (int j = 0; j < VEC + 2 * K; ++j)
+                        mu[j] = latent_bound<T, GRID>::of(active ? coef * (T)wr.get(j) : T(0), gr.ig);
                     // the next weight row: row k1 + 1, or the first row of the next tau2
                     if (active) {
                         if (k1 + 1 < PS) wr.load(om + (size_t)wrap1(y + k1 + 1 - K, H) * W, x0, W);
@@ -387,15 +434,26 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
                             }
 #pragma unroll
                             for (int j = 0; j < VEC; ++j) {
-                                const T u = sv[j] - delta[j];
-                                const T s2 = mu[j + k2].clamp(u);
-                                Hacc[j] += T(2) * s2 - u;
-                                if constexpr (MON) {
-                                    Macc[j] += s2 + sv[j] - u;              // Q' + Sigma
-                                    const double dd = (double)(s2 - sv[j]);
-                                    dsq += dd * dd;
+                                if constexpr (GRID) {
+                                    const code_t<T> sc = to_code(sv[j] * gr.ig), s2 = mu[j + k2].clamp(sc - dc[j]);
+                                    acc[j] += 2 * s2 - sc;
+                                    if constexpr (MON) {
+                                        accm[j] += s2;                      // Q' + Sigma = delta + Sigma'
+                                        const double dd = (double)(s2 - sc) * (double)gr.g;
+                                        dsq += dd * dd;
+                                    }
+                                    sv[j] = (T)s2 * gr.g;
+                                } else {
+                                    const T u = sv[j] - delta[j];
+                                    const T s2 = mu[j + k2].clamp(u);
+                                    Hacc[j] += T(2) * s2 - u;
+                                    if constexpr (MON) {
+                                        Macc[j] += s2 + sv[j] - u;              // Q' + Sigma
+                                        const double dd = (double)(s2 - sv[j]);
+                                        dsq += dd * dd;
+                                    }
+                                    sv[j] = s2;
                                 }
-                                sv[j] = s2;
                             }
                             vstore_stream<T, VEC>(gp, sv);
                         }
@@ -463,6 +521,13 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
                     }
                 }
             }
+            if constexpr (GRID) {
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) {
+                    Hacc[j] = active ? latent_h<NP>(delta[j], acc[j], gr.g) : T(0);
+                    if constexpr (MON) Macc[j] = active ? latent_h<NP>(delta[j], accm[j], gr.g) : T(0);
+                }
+            }
             // A += H_tau; publish H_tau so the row can form V(m) += H_tau(m + (0, tau2))
             T* ht = Hb + (size_t)hb * tile + (size_t)r * W;
             T* mt = Mb + (size_t)hb * tile + (size_t)r * W;
@@ -527,24 +592,24 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
 template <typename ST>
 constexpr int latent_max_regs() { return sizeof(ST) == 2 ? 96 : 112; }
 
-template <typename T, typename WT, int K, int VEC, typename ST = T>
+template <typename T, typename WT, int K, int VEC, typename ST = T, bool GRID = false>
 __global__ void __maxnreg__(latent_max_regs<ST>()) latent_tma_kernel(LatentArgs<T, WT> args) {
     extern __shared__ __align__(128) unsigned char smem_tma[];
-    latent_tma_body<T, WT, K, VEC, ST>(args, blockIdx.x, blockIdx.y, blockIdx.z, smem_tma);
+    latent_tma_body<T, WT, K, VEC, ST, GRID>(args, blockIdx.x, blockIdx.y, blockIdx.z, smem_tma);
 }
 
 // The monitoring instance (state in the iterate type): the same update, plus the latent parts of
 // the ADMM residuals (see latent_tma_body); needs (2S+1) Ty W more elements of shared memory.
-template <typename T, typename WT, int K, int VEC>
+template <typename T, typename WT, int K, int VEC, bool GRID>
 __global__ void __launch_bounds__(288, 1) latent_tma_monitor_kernel(LatentArgs<T, WT> args) {
     extern __shared__ __align__(128) unsigned char smem_tma[];
-    latent_tma_body<T, WT, K, VEC, T, true>(args, blockIdx.x, blockIdx.y, blockIdx.z, smem_tma);
+    latent_tma_body<T, WT, K, VEC, T, GRID, true>(args, blockIdx.x, blockIdx.y, blockIdx.z, smem_tma);
 }
 
 // One launch over many problems (batched uneven sizes): blocks are mapped to (problem, block)
 // by the segment table; every problem's launch shape fits the common block size and shared
 // memory size of the launch.  zero_in applies to every problem (see LatentArgs).
-template <typename T, typename WT, int K, int VEC, typename ST = T>
+template <typename T, typename WT, int K, int VEC, typename ST = T, bool GRID = false>
 __global__ void __maxnreg__(latent_max_regs<ST>())
 latent_tma_batch_kernel(const LatentArgs<T, WT>* __restrict__ args, const Segment* __restrict__ seg, int nseg,
                         int zero_in) {
@@ -553,7 +618,7 @@ latent_tma_batch_kernel(const LatentArgs<T, WT>* __restrict__ args, const Segmen
     segment_of_block(seg, nseg, blockIdx.x, &prob, &bx, &by, &bz);
     LatentArgs<T, WT> a = args[prob];
     a.zero_in = zero_in;
-    latent_tma_body<T, WT, K, VEC, ST>(a, bx, by, bz, smem_tma);
+    latent_tma_body<T, WT, K, VEC, ST, GRID>(a, bx, by, bz, smem_tma);
 }
 
 }  // namespace fuse

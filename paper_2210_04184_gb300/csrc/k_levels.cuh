@@ -1,0 +1,623 @@
+// Latent pass on the compact state (latent_grid.cuh): the update of eqs. Qj_main and dualvar3_main
+// and the adjoint sums A, V of k_latent.cuh (same planes, same order of summation over tau2), with the
+// NP entries of a (tau, c, m) kept as levels.  Layouts: records [|W|][L_s][H][W] (|W| the kept
+// offsets) and, for 25 entries, the level masks in the same order; level values [|W|][NP][L_s][H][W]
+// (plane p of a (tau, c, m) in use for its level of height p); prefix sums of the sorted threshold
+// codes of every patch window [|W|][H][W][NP], formed once per weights; points [L_s][H][W]: X with the
+// running sum of its codes after this X update and before it, so w = sum(m - tau) - sum(m).
+//
+// One block owns rows [y0, y0 + Ty) of one tau1 row and nb bands.  Per band and tau2 (a step) a thread
+// reads its pixel's record and the shifted point; with its own point these give delta, w and the
+// previous w, and where the linear stretch holds H_tau(m) follows from them.  The (pixel, step) pairs
+// with an event are collected in a list of the block; its threads then take the pairs in turn and try
+// the frequent event (level_grow), collecting the others in a second list that is processed last: the
+// rare paths run with full warps, evenly spread.  Every H_tau of the block is kept in shared memory, and
+// A(m) = sum H_tau(m), V(m) = sum H_tau(m + (0, tau2)) are formed at the end in the order of tau2,
+// whatever the order of the lists.
+#pragma once
+#include <type_traits>
+
+#include "latent_grid.cuh"
+
+namespace fuse {
+
+// X and the running sum of its codes, after the current X update and before it.
+template <typename T>
+struct alignas(4 * sizeof(T)) LevelPoint {
+    T x;
+    ucode_t<T> after, before;
+};
+
+template <typename T, typename WT>
+struct LevelArgs {
+    const T* X;
+    const WT* omega;
+    LevelRecord<ucode_t<T>>* rec;
+    uint2* masks;
+    ucode_t<T>* e;
+    const code_t<T>* tab;
+    const LevelPoint<T>* pt;
+    T* planes;
+    int H, W, Ls, S, Ty, nb;
+    T coef;
+    const LatentGrid<T>* grid;  // device
+    int half;
+};
+
+template <typename C>
+__device__ __forceinline__ LevelRecord<C> load_record(const LevelRecord<C>* p) {
+    LevelRecord<C> r;
+    if constexpr (sizeof(C) == 4) {
+        const int4 v = *reinterpret_cast<const int4*>(p);
+        r.alpha = (C)v.x;
+        r.trig = (C)v.y;
+        r.half = (C)v.z;
+        r.meta = (uint32_t)v.w;
+    } else {
+        const longlong2 a = reinterpret_cast<const longlong2*>(p)[0], b = reinterpret_cast<const longlong2*>(p)[1];
+        r.alpha = (C)a.x;
+        r.trig = (C)a.y;
+        r.half = (C)b.x;
+        r.meta = (uint32_t)b.y;
+    }
+    return r;
+}
+template <typename C>
+__device__ __forceinline__ void store_record(LevelRecord<C>* p, const LevelRecord<C>& r) {
+    if constexpr (sizeof(C) == 4) {
+        *reinterpret_cast<int4*>(p) = make_int4((int)r.alpha, (int)r.trig, (int)r.half, (int)r.meta);
+    } else {
+        longlong2 a, b;
+        a.x = (long long)r.alpha;
+        a.y = (long long)r.trig;
+        b.x = (long long)r.half;
+        b.y = (long long)r.meta;
+        reinterpret_cast<longlong2*>(p)[0] = a;
+        reinterpret_cast<longlong2*>(p)[1] = b;
+    }
+}
+
+template <typename T>
+__device__ __forceinline__ LevelPoint<T> load_point(const LevelPoint<T>* p) {
+    LevelPoint<T> r;
+    if constexpr (sizeof(T) == 4) {
+        const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+        r.x = __int_as_float(v.x);
+        r.after = (uint32_t)v.y;
+        r.before = (uint32_t)v.z;
+    } else {
+        const longlong2 a = __ldg(reinterpret_cast<const longlong2*>(p));
+        r.x = __longlong_as_double(a.x);
+        r.after = (uint64_t)a.y;
+        r.before = (uint64_t)__ldg(reinterpret_cast<const long long*>(p) + 2);
+    }
+    return r;
+}
+template <typename T>
+__device__ __forceinline__ void store_point(LevelPoint<T>* p, T x, ucode_t<T> after, ucode_t<T> before) {
+    if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<int4*>(p) = make_int4(__float_as_int(x), (int)after, (int)before, 0);
+    } else {
+        longlong2 a, b;
+        a.x = __double_as_longlong(x);
+        a.y = (long long)after;
+        b.x = (long long)before;
+        b.y = 0;
+        reinterpret_cast<longlong2*>(p)[0] = a;
+        reinterpret_cast<longlong2*>(p)[1] = b;
+    }
+}
+
+// The points of the current X; first: the sums start at zero.  Elements i0, i0 + step, ... below n.
+template <typename T>
+__device__ __forceinline__ void points_body(const T* __restrict__ X, LevelPoint<T>* __restrict__ pt, size_t n,
+                                            const LatentGrid<T>* grid, int first, size_t i0, size_t step) {
+    using U = ucode_t<T>;
+    const LatentGrid<T> gr = *grid;
+    for (size_t i = i0; i < n; i += step) {
+        const T x = X[i];
+        const U was = first ? U(0) : pt[i].after;
+        store_point<T>(pt + i, x, was + (U)x_code(x, gr.ig), was);
+    }
+}
+template <typename T>
+__global__ void __launch_bounds__(256)
+points_kernel(const T* __restrict__ X, LevelPoint<T>* __restrict__ pt, size_t n, const LatentGrid<T>* grid, int first) {
+    points_body<T>(X, pt, n, grid, first, (size_t)blockIdx.x * 256 + threadIdx.x, (size_t)gridDim.x * 256);
+}
+
+template <typename C>
+__device__ __forceinline__ void order2(C& a, C& b) {
+    const C lo = a < b ? a : b, hi = a < b ? b : a;
+    a = lo;
+    b = hi;
+}
+
+// Batcher's merge exchange (Knuth, TAOCP 5.2.2 M) on N registers; every index is a compile-time
+// constant after unrolling.
+template <int N, typename C>
+__device__ __forceinline__ void sort_network(C (&v)[N]) {
+    constexpr int T = N <= 16 ? 4 : 5;
+    static_assert(N > 8 && N <= 32, "9 to 32 values");
+#pragma unroll
+    for (int lp = T - 1; lp >= 0; --lp) {
+#pragma unroll
+        for (int step = 0; step <= T - 1 - lp; ++step) {
+            const int p = 1 << lp;
+            const int d = step == 0 ? p : ((1 << (T - 1)) >> (step - 1)) - p;
+            const int r = step == 0 ? 0 : p;
+#pragma unroll
+            for (int i = 0; i < N; ++i)
+                if (i + d < N && (i & p) == r) order2(v[i], v[i + d]);
+        }
+    }
+}
+
+// Threshold codes of the patch window of (y, x): code of coef omega_tau(m + k), k in row-major order.
+template <typename T, typename WT, int K>
+__device__ __forceinline__ void window_codes(const WT* __restrict__ om, int y, int x, int H, int W, T coef, T ig,
+                                             code_t<T> (&v)[(2 * K + 1) * (2 * K + 1)]) {
+    constexpr int PS = 2 * K + 1;
+    int col[PS];
+#pragma unroll
+    for (int j = 0; j < PS; ++j) col[j] = wrap1(x + j - K, W);
+#pragma unroll
+    for (int i = 0; i < PS; ++i) {
+        const WT* row = om + (size_t)wrap1(y + i - K, H) * W;
+#pragma unroll
+        for (int j = 0; j < PS; ++j) v[i * PS + j] = mu_code(coef * (T)wload(row + col[j]), ig);
+    }
+}
+
+// Prefix sums of the sorted threshold codes of every window; grid (ceil(n / 128), kept offsets).
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128)
+level_table_kernel(const WT* __restrict__ omega, code_t<T>* __restrict__ tab, int H, int W, int S, int half, T coef,
+                   const LatentGrid<T>* grid) {
+    using C = code_t<T>;
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    __shared__ C sm[128 * NP];                        // NP is odd: conflict-free
+    const size_t n = (size_t)H * W;
+    const size_t p0 = (size_t)blockIdx.x * 128, p = p0 + threadIdx.x;
+    const int si = blockIdx.y;
+    const TauMap tm{S, half};
+    int t1, t2;
+    tau_of_state_index(si, S, half, &t1, &t2);
+    if (p < n) {
+        const LatentGrid<T> gr = *grid;
+        C v[NP];
+        window_codes<T, WT, K>(omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / W), (int)(p % W), H, W, coef, gr.ig, v);
+        sort_network<NP>(v);
+        C sum = 0;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            sum += v[q];
+            sm[threadIdx.x * NP + q] = sum;
+        }
+    }
+    __syncthreads();
+    const int cnt = (int)(n - p0 < 128 ? n - p0 : 128) * NP;
+    C* out = tab + ((size_t)si * n + p0) * NP;
+    for (int i = threadIdx.x; i < cnt; i += 128) out[i] = sm[i];
+}
+
+// Steps (bands x offsets) of a block: one bit each in a thread's event mask, five in a list entry.
+constexpr int kLevelSteps = 32;
+constexpr int kLevelTile = 2048;                      // pixels of a block: eleven bits in a list entry
+
+// The zero state: no rank has reached its threshold, e = 0, and the first event is |w| reaching the
+// smallest threshold.  Grid (ceil(n / 128), kept offsets).
+template <typename T, int K>
+__global__ void __launch_bounds__(128)
+levels_init_kernel(LevelRecord<ucode_t<T>>* __restrict__ rec, uint2* __restrict__ masks, ucode_t<T>* __restrict__ e,
+                   const code_t<T>* __restrict__ tab, size_t n, int Ls) {
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    using U = ucode_t<T>;
+    const size_t p = (size_t)blockIdx.x * 128 + threadIdx.x;
+    if (p >= n) return;
+    const size_t si = blockIdx.y, kst = (size_t)Ls * n;
+    const LevelRecord<U> q{0, 0, (U)tab[(si * n + p) * NP], levels_meta<NP>(Levels{1u << (NP - 1), 0u, 0, true, true})};
+    for (int c = 0; c < Ls; ++c) {
+        const size_t o = si * kst + (size_t)c * n + p;
+        store_record(rec + o, q);
+        if constexpr (NP != 9) masks[o] = make_uint2(1u << (NP - 1), 0u);
+        e[si * NP * kst + (size_t)c * n + p] = 0;
+    }
+}
+
+// Shared memory: H [steps][tile], the first event list [steps tile] and the second [steps tile / 4].
+template <typename T>
+__host__ __device__ constexpr size_t levels_smem(int steps, int tile) {
+    return (size_t)steps * tile * sizeof(T) + ((size_t)steps * tile + (size_t)steps * tile / 4) * sizeof(uint16_t);
+}
+
+template <typename T, typename WT, int K>
+__device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, int bx, int gz, int row,
+                                                   unsigned char* smem_raw) {
+    using U = ucode_t<T>;
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    const int H = a.H, W = a.W, Ls = a.Ls, S = a.S;
+    const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31;
+    const TauMap tm{S, a.half};
+    const int t1 = tm.t1_of_block(row);
+    const int nt2 = tm.nt2(t1);
+    const int c0 = gz * a.nb;
+    const int nb = min(a.nb, Ls - c0);
+    const int tile = a.Ty * W, cap = nb * nt2 * tile;
+    T* Hs = reinterpret_cast<T*>(smem_raw);                           // [nb][nt2][tile]
+    uint16_t* list1 = reinterpret_cast<uint16_t*>(Hs + cap);
+    uint16_t* list2 = list1 + cap;
+    __shared__ int cnt[2];
+    const int y0 = bx * a.Ty;
+    const int npix = min(a.Ty, H - y0) * W;
+    const uint32_t n = (uint32_t)H * W;
+    const int side = 2 * S + 1;
+    const LatentGrid<T> gr = *a.grid;
+    const LevelPoint<T>* pt = a.pt + (size_t)c0 * n;
+    const size_t kst = (size_t)Ls * n;                                // records of one offset
+    const size_t s0i = (size_t)tm.s_index(t1, tm.t2_of(t1, 0));       // kept offsets of a row are consecutive
+    LevelRecord<U>* rec = a.rec + s0i * kst + (size_t)c0 * n;
+    if (tid < 2) cnt[tid] = 0;
+    __syncthreads();
+    // every step: the linear stretches; events to list1
+    const int t2first = tm.t2_of(t1, 0);
+    const int gap = !a.half && t1 == 0 ? S : nt2;                     // the offsets skip tau2 = 0 there
+    for (int base = 0; base < npix; base += nt) {
+        const int p = base + tid;
+        uint32_t ev = 0;                                              // steps with an event
+        if (p < npix) {
+            const int r = a.Ty == 1 ? 0 : p / W, x = p - r * W, y = y0 + r;
+            const uint32_t pix = (uint32_t)y * W + x, prow = (uint32_t)wrap1(y - t1, H) * W;
+            T* Hp = Hs + p;
+            uint32_t bit = 1u;
+            for (int b = 0; b < nb; ++b) {
+                const LevelPoint<T> u = load_point(pt + (size_t)b * n + pix);
+                const LevelPoint<T>* ptb = pt + (size_t)b * n;
+                for (int part = 0; part < nt2; part += gap) {         // one part but for that skip
+                    const int end = part + gap < nt2 ? part + gap : nt2;
+                    uint32_t xs = prow + wrap1(x - t2first - part - (part ? 1 : 0), W);
+                    const LevelRecord<U>* rb = rec + (size_t)part * kst + (size_t)b * n;
+                    // D steps whose records are loaded together
+                    auto batch = [&](auto dd) {
+                        constexpr int D = decltype(dd)::value;
+                        LevelRecord<U> q[D];
+                        LevelPoint<T> v[D];
+#pragma unroll
+                        for (int i = 0; i < D; ++i) {
+                            q[i] = load_record(rb + pix);
+                            rb += kst;
+                        }
+#pragma unroll
+                        for (int i = 0; i < D; ++i) {
+                            v[i] = load_point(ptb + xs);
+                            xs = xs == prow ? xs + (W - 1) : xs - 1;
+                        }
+#pragma unroll
+                        for (int i = 0; i < D; ++i) {
+                            const T delta = u.x - v[i].x;
+                            const U w1 = v[i].after - u.after, w0 = v[i].before - u.before;
+                            const bool due = level_due<U>(q[i], w1, delta < T(0), delta > T(0),
+                                                          big_move<T>(delta, gr.ig));
+                            const U t = q[i].alpha + (q[i].meta & 31u) * (2 * w1 - w0);
+                            *Hp = latent_h<NP>(delta, signed_of(t), gr.g);
+                            if (due) ev |= bit;
+                            Hp += tile;
+                            bit <<= 1;
+                        }
+                    };
+                    int left = end - part;
+                    for (; left >= 4; left -= 4) batch(std::integral_constant<int, 4>{});
+                    if (left == 3) batch(std::integral_constant<int, 3>{});
+                    else if (left == 2) batch(std::integral_constant<int, 2>{});
+                    else if (left == 1) batch(std::integral_constant<int, 1>{});
+                }
+            }
+        }
+        if (!__any_sync(0xffffffffu, ev != 0)) continue;
+        int pos = __popc(ev);                                         // inclusive scan over the warp
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int up = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += up;
+        }
+        int first = 0;
+        if (lane == 31) first = atomicAdd(&cnt[0], pos);
+        pos += __shfl_sync(0xffffffffu, first, 31) - __popc(ev);
+        for (uint32_t m = ev; m; m &= m - 1) list1[pos++] = (uint16_t)(p | (lowest_bit(m) - 1) << 11);
+    }
+    __syncthreads();
+    int todo = cnt[0];
+    if (todo > 0) {
+        const uint16_t* src = list1;
+        // one (pixel, step) pair: the event, then its H_tau
+        auto pair = [&](int item, bool grow) {
+            const int p = item & (kLevelTile - 1), step = item >> 11, b = step / nt2, jt = step - b * nt2;
+            const int r = a.Ty == 1 ? 0 : p / W, x = p - r * W, y = y0 + r;
+            const uint32_t pix = (uint32_t)y * W + x;
+            const uint32_t pxs = (uint32_t)wrap1(y - t1, H) * W + wrap1(x - tm.t2_of(t1, jt), W);
+            const size_t o = (size_t)b * n + pix;
+            uint2* mp = NP == 9 ? nullptr : a.masks + (s0i + jt) * kst + (size_t)c0 * n + o;
+            LevelRecord<U>* rp = rec + jt * kst + o;
+            LevelRecord<U> q = load_record(rp);
+            const uint2 mk = NP == 9 ? make_uint2(0u, 0u) : *mp;
+            const LevelPoint<T> u = load_point(pt + o), v = load_point(pt + ((size_t)b * n + pxs));
+            const T delta = u.x - v.x;
+            const U w1 = v.after - u.after, w0 = v.before - u.before;
+            const U s0 = q.alpha + (q.meta & 31u) * w0;
+            Levels l = levels_of<NP>(q.meta, mk);
+            const bool big = big_move<T>(delta, gr.ig);
+            const code_t<T>* Pc = a.tab + ((s0i + jt) * n + pix) * NP - 1;
+            auto P = [&](int k) { return k == 0 ? U(0) : (U)__ldg(Pc + k); };
+            if (grow) {
+                if (!level_grow<NP, U>(l, q, w0, w1, big, P)) return false;
+            } else {
+                U* ep = a.e + (s0i + jt) * NP * kst + (size_t)c0 * n + o;
+                level_event<NP, U>(
+                    l, q, w0, w1, delta < T(0), big, P, [&](int pl) { return ep[(size_t)pl * kst]; },
+                    [&](int pl, U e) { ep[(size_t)pl * kst] = e; });
+            }
+            store_record(rp, q);
+            if constexpr (NP != 9) *mp = make_uint2(l.E, l.G);
+            const U s1 = q.alpha + (q.meta & 31u) * w1;
+            Hs[step * tile + p] = latent_h<NP>(delta, signed_of(2 * s1 - s0), gr.g);
+            return true;
+        };
+        if (todo <= cap / 4) {
+            for (int i0 = tid - lane; i0 < todo; i0 += nt) {
+                const bool has = i0 + lane < todo;
+                const int item = has ? src[i0 + lane] : 0;
+                const bool left = has && !pair(item, true);
+                const uint32_t m = __ballot_sync(0xffffffffu, left);
+                if (m == 0) continue;
+                int first = 0;
+                if (lane == 0) first = atomicAdd(&cnt[1], __popc(m));
+                first = __shfl_sync(0xffffffffu, first, 0);
+                if (left) list2[first + __popc(m & ((1u << lane) - 1u))] = (uint16_t)item;
+            }
+            __syncthreads();
+            todo = cnt[1];
+            src = list2;
+        }
+        for (int i = tid; i < todo; i += nt) pair(src[i], false);
+        __syncthreads();
+    }
+    for (int p = tid; p < npix; p += nt) {
+        const int r = a.Ty == 1 ? 0 : p / W, x = p - r * W;
+        for (int b = 0; b < nb; ++b) {
+            const T* hp = Hs + (size_t)b * nt2 * tile + r * W;
+            T A = T(0), V = T(0);
+            int xv = wrap1(x + t2first, W);
+            for (int jt = 0; jt < nt2; ++jt) {
+                if (jt == gap) xv = xv + 1 == W ? 0 : xv + 1;
+                A += hp[x];
+                V += hp[xv];
+                hp += tile;
+                xv = xv + 1 == W ? 0 : xv + 1;
+            }
+            const size_t o = (size_t)(c0 + b) * 2 * side * n + (size_t)y0 * W + p;
+            a.planes[o + (size_t)(t1 + S) * n] = A;
+            a.planes[o + (size_t)(side + t1 + S) * n] = V;
+        }
+    }
+}
+
+// ---- the two forms of the state ---------------------------------------------------------------
+// Both conversions are exact and in place: the thread of a (tau, pixel) reads every word of one
+// (tau, c, m) before it writes any, and no other thread touches those words.
+
+// Threshold codes of a window, ascending, each with its patch index in the low 5 bits.
+template <typename T, typename WT, int K>
+__device__ __forceinline__ void window_keys(const WT* __restrict__ om, int y, int x, int H, int W, T coef, T ig,
+                                            typename grid_code<T>::utype (&key)[(2 * K + 1) * (2 * K + 1)]) {
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    using U = typename grid_code<T>::utype;
+    code_t<T> v[NP];
+    window_codes<T, WT, K>(om, y, x, H, W, coef, ig, v);
+#pragma unroll
+    for (int k = 0; k < NP; ++k) key[k] = ((U)v[k] << 5) | (U)k;
+    sort_network<NP>(key);
+}
+
+// Levels -> entries s_k (in the iterate type).
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT> a) {
+    using C = code_t<T>;
+    using U = typename grid_code<T>::utype;
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    const size_t n = (size_t)a.H * a.W;
+    const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const int si = blockIdx.y;
+    const TauMap tm{a.S, a.half};
+    int t1, t2;
+    tau_of_state_index(si, a.S, a.half, &t1, &t2);
+    const LatentGrid<T> gr = *a.grid;
+    U key[NP];
+    window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
+                          gr.ig, key);
+    const size_t kst = (size_t)a.Ls * n;
+    const size_t ps = (size_t)wrap1((int)(p / a.W) - t1, a.H) * a.W + wrap1((int)(p % a.W) - t2, a.W);
+    for (int c = 0; c < a.Ls; ++c) {
+        const size_t o = ((size_t)si * a.Ls + c) * n + p;
+        const Levels l = levels_of<NP>(load_record(a.rec + o).meta, NP == 9 ? make_uint2(0u, 0u) : a.masks[o]);
+        U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
+        const U w = a.pt[(size_t)c * n + ps].after - a.pt[(size_t)c * n + p].after;
+        C s[NP];
+        int height = bits_set(l.E);
+        C d = 0, sg = 0;
+#pragma unroll
+        for (int r = 0; r < NP; ++r) {
+            if (r == 0 || ((l.E >> (r == 0 ? 0 : r - 1)) & 1u)) {
+                --height;
+                const int end = r + lowest_bit(l.E >> r) - 1;
+                sg = l.free && height == 0 ? 0 : (((l.G >> end) & 1u) ? 1 : -1);
+                d = r == 0 && l.q > 0 ? C(0) : (C)(w - ob[(size_t)height * kst]);
+            }
+            s[r] = sg * (C)(key[r] >> 5) + d;
+        }
+        T* eb = reinterpret_cast<T*>(ob);
+#pragma unroll
+        for (int r = 0; r < NP; ++r) eb[(size_t)(key[r] & 31u) * kst] = (T)s[r] * gr.g;
+    }
+}
+
+// Entries -> levels.  check: nothing is written; *bad is set when some entry is off the grid or
+// the entries of some (tau, c, m) are not the state of a stop operator (|s| <= mu, 1-Lipschitz in
+// mu), which the level update needs.
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128) entries_to_levels_kernel(LevelArgs<T, WT> a, int check, int* bad) {
+    using C = code_t<T>;
+    using U = typename grid_code<T>::utype;
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    const size_t n = (size_t)a.H * a.W;
+    const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= n) return;
+    const int si = blockIdx.y;
+    const TauMap tm{a.S, a.half};
+    int t1, t2;
+    tau_of_state_index(si, a.S, a.half, &t1, &t2);
+    const LatentGrid<T> gr = *a.grid;
+    U key[NP];
+    window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
+                          gr.ig, key);
+    const size_t kst = (size_t)a.Ls * n;
+    const size_t ps = (size_t)wrap1((int)(p / a.W) - t1, a.H) * a.W + wrap1((int)(p % a.W) - t2, a.W);
+    for (int c = 0; c < a.Ls; ++c) {
+        U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
+        const T* eb = reinterpret_cast<const T*>(ob);
+        C s[NP];
+        bool ok = true;
+#pragma unroll
+        for (int r = 0; r < NP; ++r) {
+            const T v = eb[(size_t)(key[r] & 31u) * kst] * gr.ig;
+            const T lim = (T)(key[r] >> 5);
+            ok = ok && v >= -lim && v <= lim && v == trunc(v);
+            s[r] = to_code(v);
+        }
+        if (check) {
+#pragma unroll
+            for (int r = 1; r < NP; ++r) {
+                const C dm = (C)(key[r] >> 5) - (C)(key[r - 1] >> 5), ds = s[r] - s[r - 1];
+                ok = ok && ds <= dm && -ds <= dm;
+            }
+            if (!ok) atomicOr(bad, 1);
+            continue;
+        }
+        // From the largest threshold down: a level is extended while one of its forms s = d,
+        // s = mu + d, s = -mu + d still fits (d = w - e).  alpha accumulates the closed levels.
+        const U w = a.pt[(size_t)c * n + ps].after - a.pt[(size_t)c * n + p].after;
+        Levels l = {0u, 0u, 0, false, false};
+        bool f0 = true, fp = true, fm = true;
+        C d0 = 0, dp = 0, dm = 0;
+        int height = 0, end = NP - 1;
+        U alpha = 0, trig = 0, half = 0;
+        U run = 0;                                    // sum of the open level's thresholds
+        U le = 0, lmu = 0;                            // last closed level: e, its smallest threshold
+        bool lplus = false, lfree = false;
+        auto close = [&](C mu_low) {
+            lfree = f0;
+            lplus = !f0 && fp;
+            le = w - (U)(f0 ? d0 : (fp ? dp : dm));
+            lmu = (U)mu_low;
+            ob[(size_t)height * kst] = le;
+            ++height;
+        };
+#pragma unroll
+        for (int r = NP - 1; r >= 0; --r) {
+            const C mu = (C)(key[r] >> 5);
+            if (r < NP - 1) {
+                const bool k0 = f0 && s[r] == d0, kp = fp && s[r] - mu == dp, km = fm && s[r] + mu == dm;
+                if (k0 || kp || km) {
+                    f0 = k0;
+                    fp = kp;
+                    fm = km;
+                    run += (U)mu;
+                    continue;
+                }
+                close((C)(key[r + 1] >> 5));
+                l.E |= 1u << end;
+                if (lfree) l.free = true;
+                if (lplus) l.G |= 1u << end;
+                alpha += (lfree ? U(0) : (lplus ? run : U(0) - run)) - (U)(end - r) * le;
+                end = r;
+            }
+            run = (U)mu;
+            f0 = r == NP - 1;                         // sigma = 0: the highest level only
+            fp = fm = true;
+            d0 = s[r];
+            dp = s[r] - mu;
+            dm = s[r] + mu;
+        }
+        l.E |= 1u << end;
+        if ((fp && dp == 0) || (fm && dm == 0)) {     // saturated
+            l.up = fp && dp == 0;
+            l.q = end + 1;
+            if (l.up) l.G |= 1u << end;
+            alpha += l.up ? run : U(0) - run;
+            const U a2 = lfree ? lmu : (lplus == l.up ? U(0) : 2 * lmu);
+            if (l.q < NP) trig = l.up ? le + a2 : le - a2 + 1;
+        } else {
+            close((C)(key[0] >> 5));
+            if (lfree) l.free = true;
+            if (lplus) l.G |= 1u << end;
+            alpha += (lfree ? U(0) : (lplus ? run : U(0) - run)) - (U)(end + 1) * le;
+            half = lmu;
+            trig = lfree ? le : (lplus ? le - lmu : le + lmu);
+        }
+        const LevelRecord<U> q{alpha, trig, half, levels_meta<NP>(l)};
+        const size_t o = ((size_t)si * a.Ls + c) * n + p;
+        store_record(a.rec + o, q);
+        if constexpr (NP != 9) a.masks[o] = make_uint2(l.E, l.G);
+    }
+}
+
+// grid->wmax = the largest finite |w| of n weights (zeroed before; the order of non-negative
+// floating-point values is that of their bit patterns); then the grid from it.
+template <typename T, typename WT>
+__global__ void __launch_bounds__(256) wmax_kernel(const WT* __restrict__ w, size_t n, LatentGrid<T>* grid) {
+    T m = T(0);
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const T v = (T)wload(w + i);
+        const T av = v < T(0) ? -v : v;
+        if (av > m && av <= (sizeof(T) == 4 ? (T)3.0e38 : (T)1.0e308)) m = av;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = tmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) {
+        if constexpr (sizeof(T) == 4) atomicMax(reinterpret_cast<int*>(&grid->wmax), __float_as_int(m));
+        else atomicMax(reinterpret_cast<long long*>(&grid->wmax), __double_as_longlong(m));
+    }
+}
+template <typename T>
+__global__ void grid_kernel(LatentGrid<T>* grid, T coef) { *grid = latent_grid(coef, grid->wmax); }
+
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 6) latent_levels_kernel(LevelArgs<T, WT> a) {
+    extern __shared__ __align__(16) unsigned char smem_levels[];
+    latent_levels_body<T, WT, K>(a, blockIdx.x, blockIdx.y, blockIdx.z, smem_levels);
+}
+
+// Batched forms over the segment table (see latent_tma_batch_kernel): the points (blocks of 1024
+// elements of one problem) and the latent pass.
+template <typename T, typename WT>
+__global__ void __launch_bounds__(256)
+points_batch_kernel(const LevelArgs<T, WT>* __restrict__ args, const Segment* __restrict__ seg, int nseg, int first) {
+    int prob, bx, by, bz;
+    segment_of_block(seg, nseg, blockIdx.x, &prob, &bx, &by, &bz);
+    const LevelArgs<T, WT>& a = args[prob];
+    const size_t n = (size_t)a.H * a.W * a.Ls, end = (size_t)(bx + 1) * 1024;
+    points_body<T>(a.X, const_cast<LevelPoint<T>*>(a.pt), n < end ? n : end, a.grid, first,
+                   (size_t)bx * 1024 + threadIdx.x, 256);
+}
+
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 6)
+latent_levels_batch_kernel(const LevelArgs<T, WT>* __restrict__ args, const Segment* __restrict__ seg, int nseg) {
+    extern __shared__ __align__(16) unsigned char smem_levels[];
+    int prob, bx, by, bz;
+    segment_of_block(seg, nseg, blockIdx.x, &prob, &bx, &by, &bz);
+    const LevelArgs<T, WT> a = args[prob];
+    latent_levels_body<T, WT, K>(a, bx, by, bz, smem_levels);
+}
+
+}  // namespace fuse

@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "k_grad.cuh"
 #include "k_latent.cuh"
+#include "k_levels.cuh"
 #include "k_pixel.cuh"
 #include "k_stencil.cuh"
 #include "k_wfft.cuh"
@@ -19,27 +20,59 @@ namespace fuse {
 
 // ---- latent pass (k_latent.cuh) ----
 // Bulk-copy latent pass of one problem; K = patch half-size; int16_state: 16-bit fixed-point
-// state (T = float only).
+// state (T = float only); on_grid: the arithmetic of latent_grid.cuh (K = 1, 2; ignored otherwise).
 template <typename T, typename WT>
-void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, dim3 grid, unsigned threads,
-                       size_t smem, cudaStream_t s);
+void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, bool on_grid, dim3 grid,
+                       unsigned threads, size_t smem, cudaStream_t s);
 // Batched bulk-copy latent pass over the segment table.
 template <typename T, typename WT>
 void latent_tma_batch_launch(const LatentArgs<T, WT>* args, const Segment* seg, int nseg, int zero_in, int K,
-                             bool int16_state, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s);
+                             bool int16_state, bool on_grid, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s);
 // Register-staged latent pass.
 template <typename T, typename WT>
 void latent_reg_launch(const T* X, const WT* omega, const T* Sig, T* Sout, T* planes, int H, int W, int Ls, int S,
-                       int Ty, T coef, int half, int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s);
+                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, int K, bool on_grid, dim3 grid, unsigned threads,
+                       size_t smem, cudaStream_t s);
 // Monitoring latent pass (state in the iterate type): also the latent parts of the residuals.
 template <typename T, typename WT>
-void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, dim3 grid, unsigned threads, size_t smem,
+void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, bool on_grid, dim3 grid, unsigned threads, size_t smem,
                            cudaStream_t s);
 // Dynamic shared-memory cap of the single-problem and batched latent kernels for patch size K.
 template <typename T, typename WT>
 cudaError_t latent_set_smem(int K, int bytes);
 template <typename T, typename WT>
 cudaError_t latent_batch_set_smem(int K, int bytes);
+
+// ---- latent pass on the compact state (k_levels.cuh; K = 1, 2) ----
+template <typename T, typename WT>
+void levels_launch(const LevelArgs<T, WT>& a, int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s);
+// The zero state of `kept` offsets (in place of the pass of an iteration whose X is zero).
+template <typename T, typename WT>
+void levels_init_launch(const LevelArgs<T, WT>& a, int K, int kept, cudaStream_t s);
+// Batched forms over segment tables.
+template <typename T, typename WT>
+void levels_batch_launch(const LevelArgs<T, WT>* args, const Segment* seg, int nseg, int K, unsigned blocks,
+                         unsigned threads, size_t smem, cudaStream_t s);
+template <typename T, typename WT>
+void points_batch_launch(const LevelArgs<T, WT>* args, const Segment* seg, int nseg, int first, unsigned blocks,
+                         cudaStream_t s);
+// The points of the current X (one launch per iteration, before the latent pass).
+template <typename T>
+void points_launch(const T* X, LevelPoint<T>* pt, size_t n, const LatentGrid<T>* grid, int first, cudaStream_t s);
+// The sorted threshold codes of the current weights, as prefix sums.
+template <typename T, typename WT>
+void level_table_launch(const WT* omega, code_t<T>* tab, int H, int W, int K, int S, int half, int kept, T coef,
+                        const LatentGrid<T>* grid, cudaStream_t s);
+// In-place conversion of the state of `kept` offsets (to_levels: entries to levels, check only
+// validates and sets *bad; else levels to entries).
+template <typename T, typename WT>
+void levels_convert_launch(const LevelArgs<T, WT>& a, int K, int kept, int to_levels, int check, int* bad,
+                           cudaStream_t s);
+// The grid of n weights from the largest finite one (grid zeroed by the caller); two launches.
+template <typename T, typename WT>
+void wmax_launch(const WT* w, size_t n, LatentGrid<T>* grid, T coef, cudaStream_t s);
+template <typename T, typename WT>
+cudaError_t levels_set_smem(int K, int bytes);
 
 // ---- pixel updates and blur stencils (k_pixel.cuh, k_stencil.cuh) ----
 // Pixel closed forms of one problem (register kernel for L_s <= 32, else the wide kernel).
@@ -100,14 +133,27 @@ template <typename T, typename WT>
 cudaError_t latent_bwd_set_smem(int K, int bytes);
 
 #define FUSE_LAUNCH_EXTERN_T_WT(T, WT)                                                                      \
-    extern template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned, size_t,   \
-                                                  cudaStream_t);                                               \
-    extern template void latent_tma_batch_launch<T, WT>(const LatentArgs<T, WT>*, const Segment*, int, int, int, \
-                                                        bool, unsigned, unsigned, size_t, cudaStream_t);       \
-    extern template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, \
-                                                  T, int, int, dim3, unsigned, size_t, cudaStream_t);          \
-    extern template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, dim3, unsigned, size_t,    \
+    extern template void levels_launch<T, WT>(const LevelArgs<T, WT>&, int, dim3, unsigned, size_t, cudaStream_t); \
+    extern template void levels_init_launch<T, WT>(const LevelArgs<T, WT>&, int, int, cudaStream_t);          \
+    extern template void levels_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int,         \
+                                                    unsigned, unsigned, size_t, cudaStream_t);                \
+    extern template void points_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int,        \
+                                                    unsigned, cudaStream_t);                                  \
+    extern template void levels_convert_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, int, int*,        \
                                                       cudaStream_t);                                           \
+    extern template void level_table_launch<T, WT>(const WT*, code_t<T>*, int, int, int, int, int, int, T,      \
+                                                   const LatentGrid<T>*, cudaStream_t);                       \
+    extern template void wmax_launch<T, WT>(const WT*, size_t, LatentGrid<T>*, T, cudaStream_t);                             \
+    extern template cudaError_t levels_set_smem<T, WT>(int, int);                                             \
+    extern template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, bool, dim3, unsigned,     \
+                                                  size_t, cudaStream_t);                                       \
+    extern template void latent_tma_batch_launch<T, WT>(const LatentArgs<T, WT>*, const Segment*, int, int, int, \
+                                                        bool, bool, unsigned, unsigned, size_t, cudaStream_t); \
+    extern template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, \
+                                                  T, int, const LatentGrid<T>*, int, bool, dim3, unsigned, size_t,         \
+                                                  cudaStream_t);                                               \
+    extern template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned,      \
+                                                      size_t, cudaStream_t);                                           \
     extern template cudaError_t latent_set_smem<T, WT>(int, int);                                             \
     extern template cudaError_t latent_batch_set_smem<T, WT>(int, int);                                       \
     extern template void latent_bwd_tma_launch<T, WT>(const LatentBwdArgs<T, WT>&, int, dim3, unsigned, size_t, \
@@ -120,6 +166,7 @@ cudaError_t latent_bwd_set_smem(int K, int bytes);
     extern template cudaError_t latent_bwd_set_smem<T, WT>(int, int);
 
 #define FUSE_LAUNCH_EXTERN_T(T)                                                                             \
+    extern template void points_launch<T>(const T*, LevelPoint<T>*, size_t, const LatentGrid<T>*, int, cudaStream_t); \
     extern template void pixel_launch<T>(const PixelArgs<T>&, unsigned, unsigned, size_t, cudaStream_t);     \
     extern template void pixel_batch_launch<T>(const PixelArgs<T>*, const Segment*, int, int, unsigned, size_t, \
                                                cudaStream_t);                                                 \

@@ -8,8 +8,8 @@
 namespace fuse {
 
 template <typename T, typename WT>
-void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, dim3 grid, unsigned threads,
-                       size_t smem, cudaStream_t s) {
+void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, bool on_grid, dim3 grid,
+                       unsigned threads, size_t smem, cudaStream_t s) {
     constexpr int TVEC = 32 / sizeof(T);
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
@@ -19,13 +19,19 @@ void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, dim3
                 return;
             }
         }
+        if constexpr (latent_grid_k(KK)) {
+            if (on_grid) {
+                latent_tma_kernel<T, WT, KK, TVEC, T, true><<<grid, threads, smem, s>>>(a);
+                return;
+            }
+        }
         latent_tma_kernel<T, WT, KK, TVEC><<<grid, threads, smem, s>>>(a);
     });
 }
 
 template <typename T, typename WT>
 void latent_tma_batch_launch(const LatentArgs<T, WT>* args, const Segment* seg, int nseg, int zero_in, int K,
-                             bool int16_state, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s) {
+                             bool int16_state, bool on_grid, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s) {
     constexpr int TVEC = 32 / sizeof(T);
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
@@ -35,24 +41,48 @@ void latent_tma_batch_launch(const LatentArgs<T, WT>* args, const Segment* seg, 
                 return;
             }
         }
+        if constexpr (latent_grid_k(KK)) {
+            if (on_grid) {
+                latent_tma_batch_kernel<T, WT, KK, TVEC, T, true><<<blocks, threads, smem, s>>>(args, seg, nseg, zero_in);
+                return;
+            }
+        }
         latent_tma_batch_kernel<T, WT, KK, TVEC><<<blocks, threads, smem, s>>>(args, seg, nseg, zero_in);
     });
 }
 
 template <typename T, typename WT>
-void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, dim3 grid, unsigned threads, size_t smem,
+void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, bool on_grid, dim3 grid, unsigned threads, size_t smem,
                            cudaStream_t s) {
     constexpr int TVEC = 32 / sizeof(T);
-    with_k(K, [&](auto k) { latent_tma_monitor_kernel<T, WT, decltype(k)::value, TVEC><<<grid, threads, smem, s>>>(a); });
+    with_k(K, [&](auto k) {
+        constexpr int KK = decltype(k)::value;
+        if constexpr (latent_grid_k(KK)) {
+            if (on_grid) {
+                latent_tma_monitor_kernel<T, WT, KK, TVEC, true><<<grid, threads, smem, s>>>(a);
+                return;
+            }
+        }
+        latent_tma_monitor_kernel<T, WT, KK, TVEC, false><<<grid, threads, smem, s>>>(a);
+    });
 }
 
 template <typename T, typename WT>
 void latent_reg_launch(const T* X, const WT* omega, const T* Sig, T* Sout, T* planes, int H, int W, int Ls, int S,
-                       int Ty, T coef, int half, int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s) {
+                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, int K, bool on_grid, dim3 grid, unsigned threads,
+                       size_t smem, cudaStream_t s) {
     constexpr int VEC = 16 / sizeof(T);
     with_k(K, [&](auto k) {
-        latent_kernel<T, WT, decltype(k)::value, VEC><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W,
-                                                                                   Ls, S, Ty, coef, half);
+        constexpr int KK = decltype(k)::value;
+        if constexpr (latent_grid_k(KK)) {
+            if (on_grid) {
+                latent_kernel<T, WT, KK, VEC, true><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W, Ls,
+                                                                                S, Ty, coef, half, grid_d);
+                return;
+            }
+        }
+        latent_kernel<T, WT, KK, VEC, false><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W, Ls, S, Ty,
+                                                                         coef, half, grid_d);
     });
 }
 
@@ -63,9 +93,14 @@ cudaError_t latent_set_smem(int K, int bytes) {
     cudaError_t e = cudaSuccess;
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        e = cudaFuncSetAttribute(latent_kernel<T, WT, KK, VEC>, A, bytes);
+        e = cudaFuncSetAttribute(latent_kernel<T, WT, KK, VEC, false>, A, bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_kernel<T, WT, KK, TVEC>, A, bytes);
-        if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_monitor_kernel<T, WT, KK, TVEC>, A, bytes);
+        if constexpr (latent_grid_k(KK)) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_kernel<T, WT, KK, VEC, true>, A, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_kernel<T, WT, KK, TVEC, T, true>, A, bytes);
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_monitor_kernel<T, WT, KK, TVEC, true>, A, bytes);
+        }
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_monitor_kernel<T, WT, KK, TVEC, false>, A, bytes);
         if constexpr (sizeof(T) == 4) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_kernel<T, WT, KK, TVEC, int16_t>, A, bytes);
         }
@@ -81,6 +116,9 @@ cudaError_t latent_batch_set_smem(int K, int bytes) {
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
         e = cudaFuncSetAttribute(latent_tma_batch_kernel<T, WT, KK, TVEC>, A, bytes);
+        if constexpr (latent_grid_k(KK)) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_batch_kernel<T, WT, KK, TVEC, T, true>, A, bytes);
+        }
         if constexpr (sizeof(T) == 4) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_batch_kernel<T, WT, KK, TVEC, int16_t>, A, bytes);
         }
@@ -89,14 +127,14 @@ cudaError_t latent_batch_set_smem(int K, int bytes) {
 }
 
 #define FUSE_LATENT_INST(T, WT)                                                                               \
-    template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned, size_t,          \
+    template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, bool, dim3, unsigned, size_t,    \
                                            cudaStream_t);                                                      \
     template void latent_tma_batch_launch<T, WT>(const LatentArgs<T, WT>*, const Segment*, int, int, int, bool,  \
-                                                 unsigned, unsigned, size_t, cudaStream_t);                    \
-    template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, dim3, unsigned, size_t,            \
+                                                 bool, unsigned, unsigned, size_t, cudaStream_t);                    \
+    template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned, size_t,      \
                                                cudaStream_t);                                                  \
     template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, T,    \
-                                           int, int, dim3, unsigned, size_t, cudaStream_t);                    \
+                                           int, const LatentGrid<T>*, int, bool, dim3, unsigned, size_t, cudaStream_t);    \
     template cudaError_t latent_set_smem<T, WT>(int, int);                                                      \
     template cudaError_t latent_batch_set_smem<T, WT>(int, int);
 
