@@ -505,38 +505,41 @@ void levels_free(fuse_ctx* c) {
     }
 }
 
-// Launch shape of the latent pass on the compact state: `threads` per block, rows for about as many
-// pixels, and as many bands as the event lists and `room` bytes of shared memory allow.
+// Launch shape of the latent pass on the compact state: kLevelThreads per block, rows for about as many
+// pixels, and as many bands as the event lists and kLevelRoom allow, evenly split.  The room lets seven
+// blocks share the 164 KB that the pass takes of an SM (launch_levels.cu).  Measured with 15, 19, 22.5
+// and 27 KB a block: 24 tiles of 96 to 384 (40 iterations) 2.85, 2.76, 2.67, 2.77 ms per pass; HS+MS
+// 256 x 256 (iteration 64) 303, 304, 250, 249 us; FP64 HS+MS 128 x 128 (first 16) 263, 246, 246, 284 us.
+// 200 x 180, 11 bands, 5 x 5 windows: 133 us with the split 5 + 5 + 1 of the bands, 62 us with 4 + 4 + 3.
+constexpr int kLevelThreads = 128;
+constexpr size_t kLevelRoom = 164 * 1024 / 7 - 1024;
 struct LevelShape {
     int Ty = 1, nb = 0;         // nb 0: the pass does not fit
     size_t smem = 0;
 };
-LevelShape level_shape(const fuse_ctx* c, int threads, size_t room) {
+// Shared memory of a block with b bands.
+size_t level_smem(const fuse_ctx* c, int b, int Ty) {
+    const int steps = b * (2 * c->S + 1), tile = Ty * c->W;
+    return c->esz == 8 ? levels_smem<double>(steps, tile) : levels_smem<float>(steps, tile);
+}
+LevelShape level_shape(const fuse_ctx* c) {
     LevelShape z;
     const int nt2 = 2 * c->S + 1;
-    z.Ty = std::max(1, std::min(threads / c->W, c->H));
+    z.Ty = std::max(1, std::min(kLevelThreads / c->W, c->H));
     const int tile = z.Ty * c->W;
     if (!latent_grid_k(c->K) || nt2 > kLevelSteps || tile > kLevelTile) return z;
-    auto smem = [&](int b) { return c->esz == 8 ? levels_smem<double>(b * nt2, tile) : levels_smem<float>(b * nt2, tile); };
     z.nb = std::min(c->Ls, kLevelSteps / nt2);
-    while (z.nb > 1 && smem(z.nb) > room) --z.nb;
-    z.smem = smem(z.nb);
+    while (z.nb > 1 && level_smem(c, z.nb, z.Ty) > kLevelRoom) --z.nb;
+    const int gz = (c->Ls + z.nb - 1) / z.nb;
+    z.nb = (c->Ls + gz - 1) / gz;
+    z.smem = level_smem(c, z.nb, z.Ty);
     if (z.smem > (size_t)kMaxSmem) z.nb = 0;
     return z;
 }
-// Threads an SM holds at the kernel's registers (64 in FP32, 80 in FP64) and the shared memory that
-// lets it hold them in blocks of kLevelThreads.  Measured at HS+MS 256 x 256 (iteration 64): 262 us with
-// 128 threads and 28 KB a block, 272 us with 256 threads and 56 KB, 319 us with 128 threads and 20 KB;
-// 24 tiles of 96 to 384: 2.5 ms with 128 threads and 20 KB, 2.7 ms with 32 KB.
-constexpr int kLevelThreads = 128;
-int level_sm_threads(size_t esz) { return esz == 8 ? 768 : 1024; }
-size_t level_room(size_t esz) { return (size_t)227 * 1024 / (level_sm_threads(esz) / kLevelThreads) - 1024; }
 
-// A problem alone: fewer bands per block until the pass has about three blocks per SM; blocks of half
-// the threads where those all fit the device at once and the larger ones do not (FP64 pansharpening
-// at 128 x 128: 35 us against 45).
+// A problem alone: fewer bands per block until the pass has about six blocks per SM.
 void levels_shape(fuse_ctx* c) {
-    const LevelShape z = level_shape(c, kLevelThreads, level_room(c->esz));
+    const LevelShape z = level_shape(c);
     c->lv_threads = 0;
     if (z.nb == 0) return;
     const long long rows = (long long)((c->H + z.Ty - 1) / z.Ty) * (c->half ? c->S + 1 : 2 * c->S + 1);
@@ -544,10 +547,8 @@ void levels_shape(fuse_ctx* c) {
     c->lv_Ty = z.Ty;
     c->lv_nb = z.nb;
     while (c->lv_nb > 1 && blocks(c->lv_nb) < 6ll * c->nsm) --c->lv_nb;
-    c->lv_smem = z.smem / z.nb * c->lv_nb;
+    c->lv_smem = level_smem(c, c->lv_nb, c->lv_Ty);
     c->lv_threads = kLevelThreads;
-    const long long slots = (long long)c->nsm * level_sm_threads(c->esz) / kLevelThreads;
-    if (blocks(c->lv_nb) > slots && blocks(c->lv_nb) <= 2 * slots) c->lv_threads = kLevelThreads / 2;
 }
 
 // The latent state lives on the grid (latent_grid.cuh), whichever form and kernel a solve uses.
@@ -565,13 +566,13 @@ bool levels_alloc(fuse_ctx* c) {
         return false;
     }
     const size_t nk = c->half ? c->nW / 2 : c->nW;
-    const size_t img = c->n * c->Ls * c->esz;
+    const size_t pts = (size_t)c->Ls * c->H * (c->W + 2 * c->S) * 4 * c->esz;
     void** p[] = {&c->hdr, &c->tab, &c->pt, &c->omega_was};
-    const size_t bytes[] = {header_bytes(c->K, nk, c->Ls, c->n, c->esz), nk * c->nP * c->n * c->esz, 4 * img,
+    const size_t bytes[] = {header_bytes(c->K, nk, c->Ls, c->n, c->esz), nk * c->nP * c->n * c->esz, pts,
                             (size_t)c->nW * c->n * c->wsz};
     bool ok = true;
     for (int i = 0; i < 4 && ok; ++i) ok = *p[i] || cudaMalloc(p[i], bytes[i]) == cudaSuccess;
-    ok = ok && cudaMemsetAsync(c->pt, 0, 4 * img, c->stream) == cudaSuccess;
+    ok = ok && cudaMemsetAsync(c->pt, 0, pts, c->stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
         levels_free(c);
@@ -714,9 +715,8 @@ struct Impl {
         const bool taped = c->lat_in || c->lat_out;
         if (c->form == 1 && !taped) {
             dim3 grid((unsigned)((c->H + c->lv_Ty - 1) / c->lv_Ty), (unsigned)((c->Ls + c->lv_nb - 1) / c->lv_nb), rowsW);
-            points_launch<T>((const T*)c->X, (LevelPoint<T>*)c->pt, c->n * c->Ls, (const LatentGrid<T>*)c->grid, zero_in,
-                             s);
             const LevelArgs<T, WT> a = lv_args<WT>(c);
+            points_launch<T, WT>(a, zero_in, s);
             if (zero_in) levels_init_launch<T, WT>(a, c->K, c->half ? c->nW / 2 : c->nW, s);
             // X of a cold first iteration is zero with the paper's splitting, and so are the planes
             if (!zero_in || c->xmode == 1)
@@ -1351,8 +1351,7 @@ struct fuse_batch {
     int fr_rpb = 4, fc_cw = 8;
     // device tables: [args of every problem] and segments per kernel
     void* d_lat = nullptr; Segment* d_lat_seg = nullptr; int lat_nseg = 0, lat_blocks = 0;
-    // latent pass on the compact state (levels: every problem allows it): its arguments, blocks of the
-    // pass and of the points
+    // latent pass on the compact state (levels: every problem allows it) and its points
     bool levels = false;
     void* d_lv = nullptr; Segment* d_lv_seg = nullptr; Segment* d_pt_seg = nullptr;
     int lv_nseg = 0, lv_blocks = 0, pt_nseg = 0, pt_blocks = 0;
@@ -1471,11 +1470,11 @@ struct BatchImpl {
                 fuse_ctx* c = b->ctx[i];
                 // the launch fills the device whatever one problem's size: as many bands per block as fit
                 lv[i] = Impl<T>::template lv_args<WT>(c);
-                const LevelShape z = level_shape(c, kLevelThreads, level_room(esz));
+                const LevelShape z = level_shape(c);
                 lv[i].Ty = z.Ty;
                 lv[i].nb = z.nb;
                 b->lv_smem = std::max(b->lv_smem, z.smem);
-                add_segment(sp, i, (int)((c->n * c->Ls + 1023) / 1024), 1, 1, 0, &np);
+                add_segment(sp, i, (c->H * c->Ls + 7) / 8, 1, 1, 0, &np);
             }
             for (int heavy = 1; heavy >= 0; --heavy)       // tau1 != 0 rows of every problem first
                 for (int i = 0; i < n; ++i)

@@ -96,7 +96,7 @@ latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Si
             for (int j = 0; j < VEC; ++j) {
                 const T xs = Xc[(size_t)ys * W + wrap1(x0 + j - t2, W)];
                 delta[j] = Xm[j] - xs;
-                if constexpr (GRID) { dc[j] = delta_code<T>(Xm[j], xs, gr.ig); acc[j] = 0; }
+                if constexpr (GRID) { dc[j] = delta_code<T>(Xm[j], xs, gr); acc[j] = 0; }
             }
             const WT* om = omega + (size_t)tm.w_index(t1, t2) * n;
             const size_t soff = ((size_t)tm.s_index(t1, t2) * NP * Ls + c) * n + (size_t)y * W + x0;
@@ -398,7 +398,7 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
                 const T xm = delta[j], xs = active ? Xs[(size_t)r * W + ishift<VEC>(tcol, j - t2, tpr)] : T(0);
                 delta[j] = active ? xm - xs : T(0);
                 if constexpr (GRID) {
-                    dc[j] = active ? delta_code<T>(xm, xs, gr.ig) : code_t<T>(0);
+                    dc[j] = active ? delta_code<T>(xm, xs, gr) : code_t<T>(0);
                     acc[j] = 0;
                     if constexpr (MON) accm[j] = 0;
                 }

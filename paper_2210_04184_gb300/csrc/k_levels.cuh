@@ -3,8 +3,8 @@
 // NP entries of a (tau, c, m) kept as levels.  Layouts: records [|W|][L_s][H][W] (|W| the kept
 // offsets) and, for 25 entries, the level masks in the same order; level values [|W|][NP][L_s][H][W]
 // (plane p of a (tau, c, m) in use for its level of height p); prefix sums of the sorted threshold
-// codes of every patch window [|W|][H][W][NP], formed once per weights; points [L_s][H][W]: X with the
-// running sum of its codes after this X update and before it, so w = sum(m - tau) - sum(m).
+// codes of every patch window [|W|][H][W][NP], formed once per weights; points (X with its running sums,
+// written by the X update's last pass), so w = after(m - tau) - after(m).
 //
 // One block owns rows [y0, y0 + Ty) of one tau1 row and nb bands.  Per band and tau2 (a step) a thread
 // reads its pixel's record and the shifted point; with its own point these give delta, w and the
@@ -20,13 +20,6 @@
 #include "latent_grid.cuh"
 
 namespace fuse {
-
-// X and the running sum of its codes, after the current X update and before it.
-template <typename T>
-struct alignas(4 * sizeof(T)) LevelPoint {
-    T x;
-    ucode_t<T> after, before;
-};
 
 template <typename T, typename WT>
 struct LevelArgs {
@@ -77,53 +70,21 @@ __device__ __forceinline__ void store_record(LevelRecord<C>* p, const LevelRecor
     }
 }
 
+// The points of one row of the new X (a warp); first: the sums start at zero.
 template <typename T>
-__device__ __forceinline__ LevelPoint<T> load_point(const LevelPoint<T>* p) {
-    LevelPoint<T> r;
-    if constexpr (sizeof(T) == 4) {
-        const int4 v = __ldg(reinterpret_cast<const int4*>(p));
-        r.x = __int_as_float(v.x);
-        r.after = (uint32_t)v.y;
-        r.before = (uint32_t)v.z;
-    } else {
-        const longlong2 a = __ldg(reinterpret_cast<const longlong2*>(p));
-        r.x = __longlong_as_double(a.x);
-        r.after = (uint64_t)a.y;
-        r.before = (uint64_t)__ldg(reinterpret_cast<const long long*>(p) + 2);
-    }
-    return r;
+__device__ __forceinline__ void points_row(const T* __restrict__ X, LevelPoint<T>* __restrict__ pt, int W, int S,
+                                           const LatentGrid<T>* grid, int first, size_t row, int lane) {
+    const T ig = grid->ig;
+    for (int x = lane; x < W; x += 32)
+        update_point<T>(pt + row * (W + 2 * S), x, W, S, X[row * W + x], ig, first);
 }
-template <typename T>
-__device__ __forceinline__ void store_point(LevelPoint<T>* p, T x, ucode_t<T> after, ucode_t<T> before) {
-    if constexpr (sizeof(T) == 4) {
-        *reinterpret_cast<int4*>(p) = make_int4(__float_as_int(x), (int)after, (int)before, 0);
-    } else {
-        longlong2 a, b;
-        a.x = __double_as_longlong(x);
-        a.y = (long long)after;
-        b.x = (long long)before;
-        b.y = 0;
-        reinterpret_cast<longlong2*>(p)[0] = a;
-        reinterpret_cast<longlong2*>(p)[1] = b;
-    }
-}
-
-// The points of the current X; first: the sums start at zero.  Elements i0, i0 + step, ... below n.
-template <typename T>
-__device__ __forceinline__ void points_body(const T* __restrict__ X, LevelPoint<T>* __restrict__ pt, size_t n,
-                                            const LatentGrid<T>* grid, int first, size_t i0, size_t step) {
-    using U = ucode_t<T>;
-    const LatentGrid<T> gr = *grid;
-    for (size_t i = i0; i < n; i += step) {
-        const T x = X[i];
-        const U was = first ? U(0) : pt[i].after;
-        store_point<T>(pt + i, x, was + (U)x_code(x, gr.ig), was);
-    }
-}
+// Eight rows per block.
 template <typename T>
 __global__ void __launch_bounds__(256)
-points_kernel(const T* __restrict__ X, LevelPoint<T>* __restrict__ pt, size_t n, const LatentGrid<T>* grid, int first) {
-    points_body<T>(X, pt, n, grid, first, (size_t)blockIdx.x * 256 + threadIdx.x, (size_t)gridDim.x * 256);
+points_kernel(const T* __restrict__ X, LevelPoint<T>* __restrict__ pt, int rows, int W, int S,
+              const LatentGrid<T>* grid, int first) {
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (row < rows) points_row<T>(X, pt, W, S, grid, first, row, threadIdx.x & 31);
 }
 
 template <typename C>
@@ -216,7 +177,8 @@ levels_init_kernel(LevelRecord<ucode_t<T>>* __restrict__ rec, uint2* __restrict_
     const size_t p = (size_t)blockIdx.x * 128 + threadIdx.x;
     if (p >= n) return;
     const size_t si = blockIdx.y, kst = (size_t)Ls * n;
-    const LevelRecord<U> q{0, 0, (U)tab[(si * n + p) * NP], levels_meta<NP>(Levels{1u << (NP - 1), 0u, 0, true, true})};
+    LevelRecord<U> q{0, 0, 0, levels_meta<NP>(Levels{1u << (NP - 1), 0u, 0, true, true})};
+    level_free_range<U>(q, 0, (U)tab[(si * n + p) * NP]);
     for (int c = 0; c < Ls; ++c) {
         const size_t o = si * kst + (size_t)c * n + p;
         store_record(rec + o, q);
@@ -225,10 +187,10 @@ levels_init_kernel(LevelRecord<ucode_t<T>>* __restrict__ rec, uint2* __restrict_
     }
 }
 
-// Shared memory: H [steps][tile], the first event list [steps tile] and the second [steps tile / 4].
+// Shared memory: H [steps][tile], the first event list [steps tile] and the second [steps tile / 16].
 template <typename T>
 __host__ __device__ constexpr size_t levels_smem(int steps, int tile) {
-    return (size_t)steps * tile * sizeof(T) + ((size_t)steps * tile + (size_t)steps * tile / 4) * sizeof(uint16_t);
+    return (size_t)steps * tile * sizeof(T) + ((size_t)steps * tile + (size_t)steps * tile / 16) * sizeof(uint16_t);
 }
 
 template <typename T, typename WT, int K>
@@ -253,7 +215,8 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
     const uint32_t n = (uint32_t)H * W;
     const int side = 2 * S + 1;
     const LatentGrid<T> gr = *a.grid;
-    const LevelPoint<T>* pt = a.pt + (size_t)c0 * n;
+    const int Wp = W + 2 * S;
+    const LevelPoint<T>* pt = a.pt + (size_t)c0 * H * Wp;
     const size_t kst = (size_t)Ls * n;                                // records of one offset
     const size_t s0i = (size_t)tm.s_index(t1, tm.t2_of(t1, 0));       // kept offsets of a row are consecutive
     LevelRecord<U>* rec = a.rec + s0i * kst + (size_t)c0 * n;
@@ -267,16 +230,16 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
         uint32_t ev = 0;                                              // steps with an event
         if (p < npix) {
             const int r = a.Ty == 1 ? 0 : p / W, x = p - r * W, y = y0 + r;
-            const uint32_t pix = (uint32_t)y * W + x, prow = (uint32_t)wrap1(y - t1, H) * W;
+            const uint32_t pix = (uint32_t)y * W + x;
+            const LevelPoint<T>* pu = pt + ((size_t)y * Wp + S + x);
+            const LevelPoint<T>* pr = pt + ((size_t)wrap1(y - t1, H) * Wp + S + x - t2first);
             T* Hp = Hs + p;
             uint32_t bit = 1u;
-            for (int b = 0; b < nb; ++b) {
-                const LevelPoint<T> u = load_point(pt + (size_t)b * n + pix);
-                const LevelPoint<T>* ptb = pt + (size_t)b * n;
+            for (int b = 0; b < nb; ++b, pu += (size_t)H * Wp, pr += (size_t)H * Wp) {
+                const LevelPoint<T> u = load_point(pu);
                 for (int part = 0; part < nt2; part += gap) {         // one part but for that skip
-                    const int end = part + gap < nt2 ? part + gap : nt2;
-                    uint32_t xs = prow + wrap1(x - t2first - part - (part ? 1 : 0), W);
-                    const LevelRecord<U>* rb = rec + (size_t)part * kst + (size_t)b * n;
+                    const LevelPoint<T>* pv = pr - part - (part ? 1 : 0);
+                    const LevelRecord<U>* rb = rec + (size_t)part * kst + (size_t)b * n + pix;
                     // D steps whose records are loaded together
                     auto batch = [&](auto dd) {
                         constexpr int D = decltype(dd)::value;
@@ -284,28 +247,24 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
                         LevelPoint<T> v[D];
 #pragma unroll
                         for (int i = 0; i < D; ++i) {
-                            q[i] = load_record(rb + pix);
+                            q[i] = load_record(rb);
                             rb += kst;
                         }
 #pragma unroll
-                        for (int i = 0; i < D; ++i) {
-                            v[i] = load_point(ptb + xs);
-                            xs = xs == prow ? xs + (W - 1) : xs - 1;
-                        }
+                        for (int i = 0; i < D; ++i) v[i] = load_point(pv - i);
+                        pv -= D;
 #pragma unroll
                         for (int i = 0; i < D; ++i) {
                             const T delta = u.x - v[i].x;
                             const U w1 = v[i].after - u.after, w0 = v[i].before - u.before;
-                            const bool due = level_due<U>(q[i], w1, delta < T(0), delta > T(0),
-                                                          big_move<T>(delta, gr.ig));
-                            const U t = q[i].alpha + (q[i].meta & 31u) * (2 * w1 - w0);
+                            if (level_due<U>(q[i], w0, w1, delta < T(0), delta > T(0), big_move(delta, gr.g))) ev |= bit;
+                            const U t = q[i].alpha + (q[i].meta & 31u) * (v[i].z - u.z);
                             *Hp = latent_h<NP>(delta, signed_of(t), gr.g);
-                            if (due) ev |= bit;
                             Hp += tile;
                             bit <<= 1;
                         }
                     };
-                    int left = end - part;
+                    int left = part + gap < nt2 ? gap : nt2 - part;
                     for (; left >= 4; left -= 4) batch(std::integral_constant<int, 4>{});
                     if (left == 3) batch(std::integral_constant<int, 3>{});
                     else if (left == 2) batch(std::integral_constant<int, 2>{});
@@ -329,23 +288,26 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
     int todo = cnt[0];
     if (todo > 0) {
         const uint16_t* src = list1;
+        const int per_nt2 = 65536 / nt2 + 1, per_w = 65536 / W + 1;
         // one (pixel, step) pair: the event, then its H_tau
         auto pair = [&](int item, bool grow) {
-            const int p = item & (kLevelTile - 1), step = item >> 11, b = step / nt2, jt = step - b * nt2;
-            const int r = a.Ty == 1 ? 0 : p / W, x = p - r * W, y = y0 + r;
+            // quotients by multiplication: steps < 32, and more than one row only of less than 128 pixels
+            const int p = item & (kLevelTile - 1), step = item >> 11, b = (step * per_nt2) >> 16, jt = step - b * nt2;
+            const int r = a.Ty == 1 ? 0 : (p * per_w) >> 16, x = p - r * W, y = y0 + r;
             const uint32_t pix = (uint32_t)y * W + x;
-            const uint32_t pxs = (uint32_t)wrap1(y - t1, H) * W + wrap1(x - tm.t2_of(t1, jt), W);
             const size_t o = (size_t)b * n + pix;
             uint2* mp = NP == 9 ? nullptr : a.masks + (s0i + jt) * kst + (size_t)c0 * n + o;
             LevelRecord<U>* rp = rec + jt * kst + o;
             LevelRecord<U> q = load_record(rp);
             const uint2 mk = NP == 9 ? make_uint2(0u, 0u) : *mp;
-            const LevelPoint<T> u = load_point(pt + o), v = load_point(pt + ((size_t)b * n + pxs));
+            const LevelPoint<T>* pb = pt + (size_t)b * H * Wp + S + x;
+            const LevelPoint<T> u = load_point(pb + (size_t)y * Wp);
+            const LevelPoint<T> v = load_point(pb + ((ptrdiff_t)wrap1(y - t1, H) * Wp - tm.t2_of(t1, jt)));
             const T delta = u.x - v.x;
             const U w1 = v.after - u.after, w0 = v.before - u.before;
             const U s0 = q.alpha + (q.meta & 31u) * w0;
             Levels l = levels_of<NP>(q.meta, mk);
-            const bool big = big_move<T>(delta, gr.ig);
+            const bool big = big_move(delta, gr.g);
             const code_t<T>* Pc = a.tab + ((s0i + jt) * n + pix) * NP - 1;
             auto P = [&](int k) { return k == 0 ? U(0) : (U)__ldg(Pc + k); };
             if (grow) {
@@ -362,7 +324,7 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
             Hs[step * tile + p] = latent_h<NP>(delta, signed_of(2 * s1 - s0), gr.g);
             return true;
         };
-        if (todo <= cap / 4) {
+        if (todo <= cap / 16) {
             for (int i0 = tid - lane; i0 < todo; i0 += nt) {
                 const bool has = i0 + lane < todo;
                 const int item = has ? src[i0 + lane] : 0;
@@ -436,12 +398,13 @@ __global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT>
     window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
                           gr.ig, key);
     const size_t kst = (size_t)a.Ls * n;
-    const size_t ps = (size_t)wrap1((int)(p / a.W) - t1, a.H) * a.W + wrap1((int)(p % a.W) - t2, a.W);
+    const size_t Wp = a.W + 2 * a.S, img = a.H * Wp, y = p / a.W, x = p % a.W;
+    const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
     for (int c = 0; c < a.Ls; ++c) {
         const size_t o = ((size_t)si * a.Ls + c) * n + p;
         const Levels l = levels_of<NP>(load_record(a.rec + o).meta, NP == 9 ? make_uint2(0u, 0u) : a.masks[o]);
         U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
-        const U w = a.pt[(size_t)c * n + ps].after - a.pt[(size_t)c * n + p].after;
+        const U w = a.pt[c * img + ps].after - a.pt[c * img + po].after;
         C s[NP];
         int height = bits_set(l.E);
         C d = 0, sg = 0;
@@ -481,7 +444,8 @@ __global__ void __launch_bounds__(128) entries_to_levels_kernel(LevelArgs<T, WT>
     window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
                           gr.ig, key);
     const size_t kst = (size_t)a.Ls * n;
-    const size_t ps = (size_t)wrap1((int)(p / a.W) - t1, a.H) * a.W + wrap1((int)(p % a.W) - t2, a.W);
+    const size_t Wp = a.W + 2 * a.S, img = a.H * Wp, y = p / a.W, x = p % a.W;
+    const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
     for (int c = 0; c < a.Ls; ++c) {
         U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
         const T* eb = reinterpret_cast<const T*>(ob);
@@ -503,68 +467,16 @@ __global__ void __launch_bounds__(128) entries_to_levels_kernel(LevelArgs<T, WT>
             if (!ok) atomicOr(bad, 1);
             continue;
         }
-        // From the largest threshold down: a level is extended while one of its forms s = d,
-        // s = mu + d, s = -mu + d still fits (d = w - e).  alpha accumulates the closed levels.
-        const U w = a.pt[(size_t)c * n + ps].after - a.pt[(size_t)c * n + p].after;
-        Levels l = {0u, 0u, 0, false, false};
-        bool f0 = true, fp = true, fm = true;
-        C d0 = 0, dp = 0, dm = 0;
-        int height = 0, end = NP - 1;
-        U alpha = 0, trig = 0, half = 0;
-        U run = 0;                                    // sum of the open level's thresholds
-        U le = 0, lmu = 0;                            // last closed level: e, its smallest threshold
-        bool lplus = false, lfree = false;
-        auto close = [&](C mu_low) {
-            lfree = f0;
-            lplus = !f0 && fp;
-            le = w - (U)(f0 ? d0 : (fp ? dp : dm));
-            lmu = (U)mu_low;
-            ob[(size_t)height * kst] = le;
-            ++height;
-        };
+        U su[NP], mu[NP];
 #pragma unroll
-        for (int r = NP - 1; r >= 0; --r) {
-            const C mu = (C)(key[r] >> 5);
-            if (r < NP - 1) {
-                const bool k0 = f0 && s[r] == d0, kp = fp && s[r] - mu == dp, km = fm && s[r] + mu == dm;
-                if (k0 || kp || km) {
-                    f0 = k0;
-                    fp = kp;
-                    fm = km;
-                    run += (U)mu;
-                    continue;
-                }
-                close((C)(key[r + 1] >> 5));
-                l.E |= 1u << end;
-                if (lfree) l.free = true;
-                if (lplus) l.G |= 1u << end;
-                alpha += (lfree ? U(0) : (lplus ? run : U(0) - run)) - (U)(end - r) * le;
-                end = r;
-            }
-            run = (U)mu;
-            f0 = r == NP - 1;                         // sigma = 0: the highest level only
-            fp = fm = true;
-            d0 = s[r];
-            dp = s[r] - mu;
-            dm = s[r] + mu;
+        for (int r = 0; r < NP; ++r) {
+            su[r] = (U)s[r];
+            mu[r] = key[r] >> 5;
         }
-        l.E |= 1u << end;
-        if ((fp && dp == 0) || (fm && dm == 0)) {     // saturated
-            l.up = fp && dp == 0;
-            l.q = end + 1;
-            if (l.up) l.G |= 1u << end;
-            alpha += l.up ? run : U(0) - run;
-            const U a2 = lfree ? lmu : (lplus == l.up ? U(0) : 2 * lmu);
-            if (l.q < NP) trig = l.up ? le + a2 : le - a2 + 1;
-        } else {
-            close((C)(key[0] >> 5));
-            if (lfree) l.free = true;
-            if (lplus) l.G |= 1u << end;
-            alpha += (lfree ? U(0) : (lplus ? run : U(0) - run)) - (U)(end + 1) * le;
-            half = lmu;
-            trig = lfree ? le : (lplus ? le - lmu : le + lmu);
-        }
-        const LevelRecord<U> q{alpha, trig, half, levels_meta<NP>(l)};
+        const U w = a.pt[c * img + ps].after - a.pt[c * img + po].after;
+        Levels l;
+        LevelRecord<U> q;
+        levels_from_entries<NP, U>(su, mu, w, l, q, [&](int pl, U e) { ob[(size_t)pl * kst] = e; });
         const size_t o = ((size_t)si * a.Ls + c) * n + p;
         store_record(a.rec + o, q);
         if constexpr (NP != 9) a.masks[o] = make_uint2(l.E, l.G);
@@ -597,17 +509,16 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 8 : 6) latent_levels_ker
     latent_levels_body<T, WT, K>(a, blockIdx.x, blockIdx.y, blockIdx.z, smem_levels);
 }
 
-// Batched forms over the segment table (see latent_tma_batch_kernel): the points (blocks of 1024
-// elements of one problem) and the latent pass.
+// Batched forms over the segment table (see latent_tma_batch_kernel): the points, the latent pass.
 template <typename T, typename WT>
 __global__ void __launch_bounds__(256)
 points_batch_kernel(const LevelArgs<T, WT>* __restrict__ args, const Segment* __restrict__ seg, int nseg, int first) {
     int prob, bx, by, bz;
     segment_of_block(seg, nseg, blockIdx.x, &prob, &bx, &by, &bz);
     const LevelArgs<T, WT>& a = args[prob];
-    const size_t n = (size_t)a.H * a.W * a.Ls, end = (size_t)(bx + 1) * 1024;
-    points_body<T>(a.X, const_cast<LevelPoint<T>*>(a.pt), n < end ? n : end, a.grid, first,
-                   (size_t)bx * 1024 + threadIdx.x, 256);
+    const int row = bx * 8 + (threadIdx.x >> 5);
+    if (row < a.H * a.Ls)
+        points_row<T>(a.X, const_cast<LevelPoint<T>*>(a.pt), a.W, a.S, a.grid, first, row, threadIdx.x & 31);
 }
 
 template <typename T, typename WT, int K>

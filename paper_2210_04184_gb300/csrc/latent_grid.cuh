@@ -22,6 +22,8 @@
 // (25 entries): 1.4 levels on average after 50 iterations; events in 5% of the records per
 // iteration from the 20th on.
 #pragma once
+#include <type_traits>
+
 #include "common.cuh"
 
 // The level arithmetic is also compiled for the host, to be checked there against the entry-by-entry
@@ -103,21 +105,16 @@ __device__ __forceinline__ int64_t x_code(double x, double ig) {
 }
 // A move of at least this many steps saturates every entry whatever its state (thresholds are at
 // most 2^B steps).  Not-a-number counts as such a move.
-template <typename T> __device__ __forceinline__ bool big_move(T delta, T ig);
-template <> __device__ __forceinline__ bool big_move<float>(float delta, float ig) {
-    return !(fabsf(delta) * ig < 67108864.0f);                  // 2^26
-}
-template <> __device__ __forceinline__ bool big_move<double>(double delta, double ig) {
-    return !(fabs(delta) * ig < 36028797018963968.0);           // 2^55
-}
+__device__ __forceinline__ bool big_move(float delta, float g) { return !(fabsf(delta) < 67108864.0f * g); }
+__device__ __forceinline__ bool big_move(double delta, double g) { return !(fabs(delta) < 36028797018963968.0 * g); }
 // Code of delta = a - b for the entry-by-entry update.
 template <typename T>
-__device__ __forceinline__ code_t<T> delta_code(T a, T b, T ig) {
+__device__ __forceinline__ code_t<T> delta_code(T a, T b, const LatentGrid<T>& gr) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     const T d = a - b;
-    if (big_move<T>(d, ig)) return d < T(0) ? -(C(4) << grid_code<T>::B) : (C(4) << grid_code<T>::B);
-    return (C)((U)x_code(a, ig) - (U)x_code(b, ig));
+    if (big_move(d, gr.g)) return d < T(0) ? -(C(4) << grid_code<T>::B) : (C(4) << grid_code<T>::B);
+    return (C)((U)x_code(a, gr.ig) - (U)x_code(b, gr.ig));
 }
 __device__ __forceinline__ int32_t to_code(float v) { return __float2int_rn(v); }
 __device__ __forceinline__ int64_t to_code(double v) { return __double2ll_rn(v); }
@@ -143,10 +140,10 @@ struct Levels {
     bool up, free;
 };
 // Record: S(w) = alpha + beta w.  With q > 0 the stretch ends when w turns or reaches the next
-// rank's threshold, at w >= trig going up and w < trig going down; with q = 0 when |w - trig| reaches
-// half.  meta: beta (bits 0-4), free (5), q > 0 (30), not up (31), and with 9 ranks E (bits 6-14) and
-// G (bits 15-23); with 25 ranks E and G have their own words.
-constexpr uint32_t kRecordSat = 1u << 30, kRecordDown = 1u << 31;
+// rank's threshold value t (trig = -t going up, t + 1 going down, see level_due); with q = 0 when w
+// leaves [trig, trig + half].  meta: beta (bits 0-4), free (5), q > 0 (30), q > 0 and up (31), and with
+// 9 ranks E (bits 6-14) and G (bits 15-23); with 25 ranks E and G have their own words.
+constexpr uint32_t kRecordSat = 1u << 30, kRecordUp = 1u << 31;
 template <typename C>
 struct alignas(4 * sizeof(C)) LevelRecord {
     C alpha, trig, half;
@@ -155,7 +152,7 @@ struct alignas(4 * sizeof(C)) LevelRecord {
 
 template <int NP>
 FUSE_LEVEL_FN uint32_t levels_meta(const Levels& l) {
-    uint32_t m = (uint32_t)(NP - l.q) | (l.free ? 32u : 0u) | (l.q > 0 ? kRecordSat : 0u) | (l.up ? 0u : kRecordDown);
+    uint32_t m = (uint32_t)(NP - l.q) | (l.free ? 32u : 0u) | (l.q > 0 ? kRecordSat | (l.up ? kRecordUp : 0u) : 0u);
     if constexpr (NP == 9) m |= l.E << 6 | l.G << 15;
     return m;
 }
@@ -163,7 +160,7 @@ template <int NP>
 FUSE_LEVEL_FN Levels levels_of(uint32_t meta, uint2 masks) {
     Levels l;
     l.q = NP - (int)(meta & 31u);
-    l.up = !(meta & kRecordDown);
+    l.up = meta & kRecordUp;
     l.free = meta & 32u;
     if constexpr (NP == 9) {
         l.E = (meta >> 6) & 0x1ffu;
@@ -188,6 +185,13 @@ FUSE_LEVEL_FN int lowest_bit(uint32_t v) {      // 1-based, v != 0
 #else
     return __builtin_ffs((int)v);
 #endif
+}
+
+// The range of w without an event when no rank is saturated: |w - centre| < mu (w = centre for mu = 0).
+template <typename C>
+FUSE_LEVEL_FN void level_free_range(LevelRecord<C>& rec, C centre, C mu) {
+    rec.trig = mu > 0 ? centre - mu + 1 : centre;
+    rec.half = mu > 0 ? 2 * mu - 2 : C(0);
 }
 
 // An event: the levels and the record after the move from w0 to w1 (all: a big move, which saturates
@@ -249,10 +253,11 @@ FUSE_LEVEL_FN void level_event(Levels& l, LevelRecord<C>& rec, C w0, C w1, bool 
         alpha += up ? Pq : C(0) - Pq;
         if (q > 0) {
             const C a = fr ? mu : (plus == up ? C(0) : 2 * mu);
-            trig = up ? e + a : e - a + 1;
+            trig = up ? C(0) - (e + a) : e - a + 1;
         } else {
-            trig = fr ? e : (plus ? e - mu : e + mu);
-            half = mu;
+            level_free_range<C>(rec, fr ? e : (plus ? e - mu : e + mu), mu);
+            trig = rec.trig;
+            half = rec.half;
         }
     } else {
         q = NP;
@@ -289,7 +294,7 @@ FUSE_LEVEL_FN bool level_grow(Levels& l, LevelRecord<C>& rec, C w0, C w1, bool b
     const bool fr = l.free && (Er & (Er - 1)) == 0;
     if (!fr && (((l.G >> (hi - 1)) & 1u) != 0) == l.up) return false;
     int q = l.q;
-    C alpha = rec.alpha, trig = l.up ? rec.trig : rec.trig - 1;
+    C alpha = rec.alpha, trig = l.up ? C(0) - rec.trig : rec.trig - 1;
     if (signed_of(l.up ? w1 - trig : trig - w1) < 0) return false;
     C P1 = P(q + 1), mu = P1 - P(q);
     for (int i = 0; i < kGrowRanks; ++i) {
@@ -305,7 +310,7 @@ FUSE_LEVEL_FN bool level_grow(Levels& l, LevelRecord<C>& rec, C w0, C w1, bool b
             l.G = (l.G & ~((1u << q) - 1u)) | (l.up ? 1u << (q - 1) : 0u);
             l.q = q;
             rec.alpha = alpha;
-            rec.trig = l.up ? trig : trig + 1;
+            rec.trig = l.up ? C(0) - trig : trig + 1;
             rec.meta = levels_meta<NP>(l);
             return true;
         }
@@ -313,14 +318,137 @@ FUSE_LEVEL_FN bool level_grow(Levels& l, LevelRecord<C>& rec, C w0, C w1, bool b
     return false;
 }
 
-// Whether the linear stretch of a record ends with the move to w1 = w0 - delta: up = delta < 0,
-// down = delta > 0, big = big_move.  With every rank saturated (beta = 0) only a turn ends it.
+// The levels and the record of given entries s (ascending thresholds mu, |s| <= mu, 1-Lipschitz in mu)
+// at w; st(p, e) as above.  The saturated prefix first, as long as it goes, so that w lies strictly
+// inside the stretch; then from the largest threshold down: a level is extended while one of its
+// forms s = d, s = mu + d, s = -mu + d still fits (d = w - e).
+template <int NP, typename C, typename FS>
+FUSE_LEVEL_FN void levels_from_entries(const C (&s)[NP], const C (&mu)[NP], C w, Levels& l, LevelRecord<C>& rec, FS st) {
+    int qu = 0, qd = 0;
+    C P = 0;
+    for (int r = 0; r < NP; ++r) {
+        if (qu == r && s[r] == mu[r]) ++qu;
+        if (qd == r && s[r] == C(0) - mu[r]) ++qd;
+    }
+    l = Levels{0u, 0u, qu >= qd ? qu : qd, qu >= qd, false};
+    C alpha = 0, run = 0, low = 0, d0 = 0, dp = 0, dm = 0, le = 0;
+    bool f0 = false, fp = false, fm = false, plus = false;
+    int height = 0, end = NP - 1;
+    auto close = [&](int first) {                     // ranks [first, end]
+        const bool fr = f0;
+        plus = !fr && fp;
+        le = w - (fr ? d0 : (fp ? dp : dm));
+        st(height++, le);
+        l.E |= 1u << end;
+        if (plus) l.G |= 1u << end;
+        if (fr) l.free = true;
+        alpha += (fr ? C(0) : (plus ? run : C(0) - run)) - (C)(end + 1 - first) * le;
+    };
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+    for (int r = NP - 1; r >= 0; --r) {
+        if (r < l.q) {
+            P += mu[r];
+            continue;
+        }
+        const bool k0 = f0 && s[r] == d0, kp = fp && s[r] - mu[r] == dp, km = fm && s[r] + mu[r] == dm;
+        if (k0 || kp || km) {
+            f0 = k0;
+            fp = kp;
+            fm = km;
+            run += mu[r];
+        } else {
+            if (r < NP - 1) close(r + 1);
+            end = r;
+            run = mu[r];
+            f0 = r == NP - 1;                         // sigma = 0: the highest level only
+            fp = fm = true;
+            d0 = s[r];
+            dp = s[r] - mu[r];
+            dm = s[r] + mu[r];
+        }
+        low = mu[r];
+    }
+    rec.trig = rec.half = 0;
+    if (l.q < NP) {
+        close(l.q);
+        const bool fr = f0;
+        const C a = fr ? low : (plus == l.up ? C(0) : 2 * low);
+        if (l.q > 0) rec.trig = l.up ? C(0) - (le + a) : le - a + 1;
+        else level_free_range<C>(rec, fr ? le : (plus ? le - low : le + low), low);
+    }
+    if (l.q > 0) {
+        l.E |= 1u << (l.q - 1);
+        if (l.up) l.G |= 1u << (l.q - 1);
+        alpha += l.up ? P : C(0) - P;
+    }
+    rec.alpha = alpha;
+    rec.meta = levels_meta<NP>(l);
+}
+
+// Whether the linear stretch of a record ends with the move from w0 to w1 = w0 - delta: up = delta < 0,
+// down = delta > 0, big = big_move.  With every rank saturated (beta = 0) only a turn ends it; else, with
+// m = -1 for ranks saturated upwards, the stretch is (w1 ^ m) - trig <= (w0 ^ m) - trig as unsigned
+// integers: w1 in [w0, t) or (t, w0].
 template <typename C>
-FUSE_LEVEL_FN bool level_due(const LevelRecord<C>& r, C w1, bool up, bool down, bool big) {
-    const bool dn = (r.meta & kRecordDown) != 0, sat = (r.meta & kRecordSat) != 0;
-    const auto c = signed_of(w1 - r.trig);
-    const auto v = sat ? (dn ? ~c : c) : (c < 0 ? -c : c) - signed_of(r.half);
-    return (sat && (dn ? up : down)) || ((r.meta & 31u) != 0 && (v >= 0 || big));
+FUSE_LEVEL_FN bool level_due(const LevelRecord<C>& r, C w0, C w1, bool up, bool down, bool big) {
+    const C m = (C)(typename std::make_signed<C>::type)((int32_t)r.meta >> 31);
+    const C a = (w1 ^ m) - r.trig, b = (r.meta & kRecordSat) ? (w0 ^ m) - r.trig : r.half;
+    return (r.meta & 31u) ? (a > b || big) : ((r.meta & kRecordUp) ? down : up);
+}
+
+// A point: X and the running sum of its codes after the current X update and before it, and z = 2
+// after - before.  Points [L_s][H][W + 2S]: each row with S points of its other end on either side,
+// so the pass reads m - tau without a wrap.
+template <typename T>
+struct alignas(4 * sizeof(T)) LevelPoint {
+    T x;
+    ucode_t<T> after, before, z;
+};
+template <typename T>
+__device__ __forceinline__ LevelPoint<T> load_point(const LevelPoint<T>* p) {
+    LevelPoint<T> r;
+    if constexpr (sizeof(T) == 4) {
+        const int4 v = __ldg(reinterpret_cast<const int4*>(p));
+        r.x = __int_as_float(v.x);
+        r.after = (uint32_t)v.y;
+        r.before = (uint32_t)v.z;
+        r.z = (uint32_t)v.w;
+    } else {
+        const longlong2 a = __ldg(reinterpret_cast<const longlong2*>(p)), b = __ldg(reinterpret_cast<const longlong2*>(p) + 1);
+        r.x = __longlong_as_double(a.x);
+        r.after = (uint64_t)a.y;
+        r.before = (uint64_t)b.x;
+        r.z = (uint64_t)b.y;
+    }
+    return r;
+}
+template <typename T>
+__device__ __forceinline__ void store_point(LevelPoint<T>* p, T x, ucode_t<T> after, ucode_t<T> before) {
+    const ucode_t<T> z = 2 * after - before;
+    if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<int4*>(p) = make_int4(__float_as_int(x), (int)after, (int)before, (int)z);
+    } else {
+        longlong2 a, b;
+        a.x = __double_as_longlong(x);
+        a.y = (long long)after;
+        b.x = (long long)before;
+        b.y = (long long)z;
+        reinterpret_cast<longlong2*>(p)[0] = a;
+        reinterpret_cast<longlong2*>(p)[1] = b;
+    }
+}
+// The point of column x of a row (row: its first point, the halo's) from the new X; first: the sums
+// start at zero.
+template <typename T>
+__device__ __forceinline__ void update_point(LevelPoint<T>* row, int x, int W, int S, T v, T ig, int first) {
+    LevelPoint<T>* p = row + S + x;
+    const ucode_t<T> was = first ? ucode_t<T>(0) : p->after;
+    const ucode_t<T> now = was + (ucode_t<T>)x_code(v, ig);
+    store_point<T>(p, v, now, was);
+    if (x < S) store_point<T>(p + W, v, now, was);
+    if (x >= W - S) store_point<T>(p - W, v, now, was);
 }
 
 }  // namespace fuse

@@ -49,7 +49,7 @@ void levels_launch(const LevelArgs<T, WT>& a, int K, dim3 grid, unsigned threads
 // The zero state of `kept` offsets (in place of the pass of an iteration whose X is zero).
 template <typename T, typename WT>
 void levels_init_launch(const LevelArgs<T, WT>& a, int K, int kept, cudaStream_t s);
-// Batched forms over segment tables.
+// Batched form over a segment table.
 template <typename T, typename WT>
 void levels_batch_launch(const LevelArgs<T, WT>* args, const Segment* seg, int nseg, int K, unsigned blocks,
                          unsigned threads, size_t smem, cudaStream_t s);
@@ -57,8 +57,8 @@ template <typename T, typename WT>
 void points_batch_launch(const LevelArgs<T, WT>* args, const Segment* seg, int nseg, int first, unsigned blocks,
                          cudaStream_t s);
 // The points of the current X (one launch per iteration, before the latent pass).
-template <typename T>
-void points_launch(const T* X, LevelPoint<T>* pt, size_t n, const LatentGrid<T>* grid, int first, cudaStream_t s);
+template <typename T, typename WT>
+void points_launch(const LevelArgs<T, WT>& a, int first, cudaStream_t s);
 // The sorted threshold codes of the current weights, as prefix sums.
 template <typename T, typename WT>
 void level_table_launch(const WT* omega, code_t<T>* tab, int H, int W, int K, int S, int half, int kept, T coef,
@@ -139,6 +139,7 @@ cudaError_t latent_bwd_set_smem(int K, int bytes);
                                                     unsigned, unsigned, size_t, cudaStream_t);                \
     extern template void points_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int,        \
                                                     unsigned, cudaStream_t);                                  \
+    extern template void points_launch<T, WT>(const LevelArgs<T, WT>&, int, cudaStream_t);                    \
     extern template void levels_convert_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, int, int*,        \
                                                       cudaStream_t);                                           \
     extern template void level_table_launch<T, WT>(const WT*, code_t<T>*, int, int, int, int, int, int, T,      \
@@ -166,7 +167,6 @@ cudaError_t latent_bwd_set_smem(int K, int bytes);
     extern template cudaError_t latent_bwd_set_smem<T, WT>(int, int);
 
 #define FUSE_LAUNCH_EXTERN_T(T)                                                                             \
-    extern template void points_launch<T>(const T*, LevelPoint<T>*, size_t, const LatentGrid<T>*, int, cudaStream_t); \
     extern template void pixel_launch<T>(const PixelArgs<T>&, unsigned, unsigned, size_t, cudaStream_t);     \
     extern template void pixel_batch_launch<T>(const PixelArgs<T>*, const Segment*, int, int, unsigned, size_t, \
                                                cudaStream_t);                                                 \

@@ -40,6 +40,13 @@ void points_batch_launch(const LevelArgs<T, WT>* args, const Segment* seg, int n
 }
 
 template <typename T, typename WT>
+void points_launch(const LevelArgs<T, WT>& a, int first, cudaStream_t s) {
+    const int rows = a.H * a.Ls;
+    points_kernel<T><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(a.X, const_cast<LevelPoint<T>*>(a.pt), rows, a.W, a.S,
+                                                               a.grid, first);
+}
+
+template <typename T, typename WT>
 void levels_convert_launch(const LevelArgs<T, WT>& a, int K, int kept, int to_levels, int check, int* bad,
                            cudaStream_t s) {
     const dim3 grid((unsigned)(((size_t)a.H * a.W + 127) / 128), (unsigned)kept);
@@ -48,12 +55,6 @@ void levels_convert_launch(const LevelArgs<T, WT>& a, int K, int kept, int to_le
         if (to_levels) entries_to_levels_kernel<T, WT, KK><<<grid, 128, 0, s>>>(a, check, bad);
         else levels_to_entries_kernel<T, WT, KK><<<grid, 128, 0, s>>>(a);
     });
-}
-
-template <typename T>
-void points_launch(const T* X, LevelPoint<T>* pt, size_t n, const LatentGrid<T>* grid, int first, cudaStream_t s) {
-    const unsigned blocks = (unsigned)((n + 255) / 256 < 2432 ? (n + 255) / 256 : 2432);
-    points_kernel<T><<<blocks, 256, 0, s>>>(X, pt, n, grid, first);
 }
 
 template <typename T, typename WT>
@@ -79,6 +80,12 @@ cudaError_t levels_set_smem(int K, int bytes) {
         const auto A = cudaFuncAttributeMaxDynamicSharedMemorySize;
         e = cudaFuncSetAttribute(latent_levels_kernel<T, WT, KK>, A, bytes);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_levels_batch_kernel<T, WT, KK>, A, bytes);
+        // 164 KB of shared memory per SM (72%), the rest L1: the events' scattered reads of the table and
+        // the points gain more from L1 than the pass from two more blocks (24 tiles of 96 to 384, 40
+        // iterations: 2.75 ms per pass, 2.91 with 196 or 228 KB, 4.0 with 132 KB)
+        const auto P = cudaFuncAttributePreferredSharedMemoryCarveout;
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_levels_kernel<T, WT, KK>, P, 72);
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_levels_batch_kernel<T, WT, KK>, P, 72);
     });
     return e;
 }
@@ -90,15 +97,13 @@ cudaError_t levels_set_smem(int K, int bytes) {
     template void levels_init_launch<T, WT>(const LevelArgs<T, WT>&, int, int, cudaStream_t);                   \
     template void points_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int, unsigned,        \
                                              cudaStream_t);                                                    \
+    template void points_launch<T, WT>(const LevelArgs<T, WT>&, int, cudaStream_t);                             \
     template void levels_convert_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, int, int*, cudaStream_t); \
     template void level_table_launch<T, WT>(const WT*, code_t<T>*, int, int, int, int, int, int, T,              \
                                             const LatentGrid<T>*, cudaStream_t);                               \
     template void wmax_launch<T, WT>(const WT*, size_t, LatentGrid<T>*, T, cudaStream_t);                                       \
     template cudaError_t levels_set_smem<T, WT>(int, int);
 
-template void points_launch<float>(const float*, LevelPoint<float>*, size_t, const LatentGrid<float>*, int, cudaStream_t);
-template void points_launch<double>(const double*, LevelPoint<double>*, size_t, const LatentGrid<double>*, int,
-                                    cudaStream_t);
 FUSE_LEVELS_INST(float, float)
 FUSE_LEVELS_INST(float, __nv_bfloat16)
 FUSE_LEVELS_INST(double, double)

@@ -34,10 +34,10 @@ int walk(int seed) {
         std::vector<uint32_t> planes(NP, 0x55555555u);
         planes[0] = 0;
         Levels l{1u << (NP - 1), 0u, 0, true, true};
-        LevelRecord<uint32_t> rec{0, 0, (uint32_t)mu[0], levels_meta<NP>(l)};
+        LevelRecord<uint32_t> rec{0, 0, 0, levels_meta<NP>(l)};
         uint32_t w = r();                             // the running sums start anywhere modulo 2^32
         planes[0] = w;
-        rec.trig = w;
+        level_free_range<uint32_t>(rec, w, (uint32_t)mu[0]);
         rec.alpha = 0u - (uint32_t)NP * w;
         double scale = std::pow(2.0, r() % 27);
         const double decay = 0.5 + (r() % 100) / 150.0;
@@ -66,7 +66,7 @@ int walk(int seed) {
                 s1 += s[i];
             }
             REQUIRE(signed_of(rec.alpha + (rec.meta & 31u) * w0) == s0);
-            if (level_due<uint32_t>(rec, w1, up, down, big)) {
+            if (level_due<uint32_t>(rec, w0, w1, up, down, big)) {
                 ++events;
                 bool in_range = true;
                 auto pre = [&](int q) { in_range = in_range && q >= 0 && q <= NP; return (uint32_t)P[in_range ? q : 0]; };
@@ -85,6 +85,16 @@ int walk(int seed) {
                 }
             }
             w = w1;
+            if (r() % 8 == 0) {                       // the same state formed anew from its entries
+                uint32_t su[NP], mm[NP];
+                for (int i = 0; i < NP; ++i) { su[i] = (uint32_t)s[i]; mm[i] = (uint32_t)mu[i]; }
+                bool fits = true;
+                levels_from_entries<NP, uint32_t>(su, mm, w, l, rec, [&](int p, uint32_t e) {
+                    fits = fits && p >= 0 && p < NP;
+                    if (fits) planes[p] = e;
+                });
+                REQUIRE(fits);
+            }
             REQUIRE(signed_of(rec.alpha + (rec.meta & 31u) * w1) == s1);
             // every entry from the levels
             int lo = 0, height = bits_set(l.E) - 1;
