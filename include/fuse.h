@@ -80,7 +80,8 @@ enum {
                                     register-staged loads.  By default (3 x 3 and 5 x 5 patches, state
                                     in the iterate type, S <= 15) solves keep the entries of a (tau,
                                     pixel, band) as a few levels and update those; the same results
-                                    bit for bit.  Where the levels do not apply (other patches, the
+                                    bit for bit.  Where the levels do not apply (other patches,
+                                    FP32 with 3 x 3 patches and a 3 x 3 search, the
                                     16-bit state, a state or weights set while a solve is continued,
                                     no memory for them) the entries stream through a bulk-copy ring,
                                     which the next three options shape. */
