@@ -48,7 +48,8 @@ LATENT_TRAFFIC = {
     # latent_tma_batch_kernel, the batch workload's first 8 problems (K = 1, S = 3, L_s = 8)
     "batch": {"bytes_per_pixel": (4.697702656e9 + 4.726860800e9) / 667648, "sources": "bd69776d19227011"},
 }
-LATENT_SOURCES = ("k_latent.cuh", "tma.cuh", "common.cuh", "launch_latent.cu")
+LATENT_SOURCES = ("k_levels.cuh", "latent_grid.cuh", "launch_levels.cu", "k_latent.cuh", "tma.cuh", "common.cuh",
+                  "launch_latent.cu")
 UNIT = "Mpx*band*iter/s"
 
 
@@ -191,6 +192,18 @@ def latent_bytes(p, esz, wsz, half=True, ssz=None):
     ssz = ssz or esz
     return (2 * nK * nP * p.L_s * n * ssz + nK * n * wsz + p.L_s * n * esz
             + 2 * rows * p.L_s * n * esz)
+
+
+def level_bytes(p, esz, half=True):
+    """Algorithmic bytes of one latent-pass launch on levels (3 x 3 and 5 x 5 windows, state in the iterate
+    type): the record of four words of every kept offset, band and pixel, read once, the point of four
+    words of every band and pixel, and the adjoint planes.  What the events of an iteration read and
+    write comes on top: it depends on the data."""
+    n = p.H * p.W
+    nW = (2 * p.S + 1) ** 2 - 1
+    nK = nW // 2 if half else nW
+    rows = p.S + 1 if half else 2 * p.S + 1
+    return (4 * nK + 4 + 2 * rows) * p.L_s * n * esz
 
 
 def _sources_digest():
@@ -563,7 +576,7 @@ def run_batch(a, rank, world, local_rank):
     peak_src = "measured" if hbm else "fallback"
     hbm = hbm or 6800.0
     per_launch_ms = lat_ms / max(lat_n, 1)
-    lb = sum(latent_bytes(p, 4, 2) for p in ps)
+    lb = sum(level_bytes(p, 4) for p in ps)
     achieved = lb / (per_launch_ms / 1e3) / 1e9
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
@@ -571,7 +584,7 @@ def run_batch(a, rank, world, local_rank):
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": dict(batch_config(ps, iters, world), latent_shape=shape),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                     "traffic": latent_traffic("batch", px), "kernel": "latent_tma_batch_kernel",
+                     "traffic": latent_traffic("batch", px), "kernel": "latent_levels_batch_kernel",
                      "algorithmic_bytes_per_launch": lb, "avg_launch_ms": per_launch_ms, "launches": lat_n,
                      "timing": "CUDA events around each latent launch in a separate profiled step",
                      "peak_source": peak_src, "nominal_peak": NOMINAL_HBM_GBS},
@@ -768,7 +781,8 @@ def single_problem(a, name, rank, dist, keep=False):
     hbm = hbm or 6800.0
     per_launch_ms = lat_ms / max(lat_n, 1)
     fixed = keep and a.fixed_state
-    lb = latent_bytes(p, esz, wsz, ssz=2 if fixed else None)
+    levels = p.K in (1, 2) and not fixed and not (p.K == 1 and p.S == 1 and esz == 4)
+    lb = level_bytes(p, esz) if levels else latent_bytes(p, esz, wsz, ssz=2 if fixed else None)
     traffic = None
     if name.startswith("hsms") and meta["wdtype"] == "bf16" and not fixed:
         traffic = latent_traffic("hsms", p.H * p.W)
@@ -777,7 +791,7 @@ def single_problem(a, name, rank, dist, keep=False):
            "dtype": meta["dtype"], "config": dict(_config(p, meta, name, world), launch_shapes=tuned),
            "iters_per_s": p.iters * a.steps * world / (ms / 1e3),
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
-                        "frac": achieved / hbm, "traffic": traffic, "kernel": "latent_tma_kernel",
+                        "frac": achieved / hbm, "traffic": traffic, "kernel": "latent_levels_kernel" if levels else "latent_tma_kernel",
                         "algorithmic_bytes_per_launch": lb, "avg_launch_ms": per_launch_ms, "launches": lat_n,
                         "timing": "CUDA events around each latent launch in a separate profiled step",
                         "peak_source": peak_src, "nominal_peak": NOMINAL_HBM_GBS},
