@@ -395,9 +395,11 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
             for (int j = 0; j < VEC; ++j) {
                 Hacc[j] = T(0);
                 if constexpr (MON) Macc[j] = T(0);
-                const T xm = delta[j], xs = active ? Xs[(size_t)r * W + ishift<VEC>(tcol, j - t2, tpr)] : T(0);
-                delta[j] = active ? xm - xs : T(0);
-                if constexpr (GRID) {
+                if constexpr (!GRID) {
+                    delta[j] = active ? delta[j] - Xs[(size_t)r * W + ishift<VEC>(tcol, j - t2, tpr)] : T(0);
+                } else {
+                    const T xm = delta[j], xs = active ? Xs[(size_t)r * W + ishift<VEC>(tcol, j - t2, tpr)] : T(0);
+                    delta[j] = active ? xm - xs : T(0);
                     dc[j] = active ? delta_code<T>(xm, xs, gr) : code_t<T>(0);
                     acc[j] = 0;
                     if constexpr (MON) accm[j] = 0;
