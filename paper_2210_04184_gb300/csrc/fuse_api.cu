@@ -1109,9 +1109,12 @@ fuse_status monitored_iteration(fuse_ctx* c, bool zero_in) {
     if (c->lt_smem + 2 * (size_t)c->lt_Ty * c->W * c->esz > (size_t)kMaxSmem)
         return fail(c, FUSE_EUNSUPPORTED, "the monitoring latent pass does not fit shared memory");
     fuse_status st = FUSE_OK;
-    if (zero_in) c->form = 0;                  // the pass reads no state and writes entries
-    else if ((st = need_entries(c)) != FUSE_OK) return st;
-    c->entries_ok = true;
+    if (zero_in) {                             // the pass reads no state and writes the entries of a run
+        c->form = 0;
+        c->entries_ok = true;
+    } else if ((st = need_entries(c)) != FUSE_OK) {
+        return st;                             // other entries stay what they were before it
+    }
     const size_t img = c->n * c->Ls * c->esz;
     cudaStream_t s = c->stream;
     CK(c, cudaMemcpyAsync(c->mL1, c->Lam1, img, cudaMemcpyDeviceToDevice, s));
