@@ -6,9 +6,13 @@
 //
 // Grid.  X (in the update of s), mu_k and therefore s_k are kept on a grid g Z, g a power of two
 // with mu_max <= 2^B g (B = 24 in FP32, 53 in FP64; mu_max = lambda2/rho times the largest weight):
-// X is rounded to the grid and mu_k rounded down to it.  Every s_k is then a multiple of g of at
+// X and mu_k are rounded to the grid, to nearest.  Every s_k is then a multiple of g of at
 // most 2^B g, an exact value of the iterate type, the update is exact, and so is the sum over k in
-// any order.  The grid is as fine as the iterate type's own spacing below mu_max.
+// any order.  In the topmost binade below mu_max the grid is the iterate type's own spacing; smaller
+// values keep the same absolute step.  Error of X from this, all else in FP64 (relative, 40 iterations,
+// three 32 x 32 scenes, lambda2/rho = 0.1, 0.2, 0.5, with 2^B g = 0.26, 0.52, 2.1 of the data's rms, 25
+// entries): 1.44e-7, 1.50e-7, 1.47e-7, against 1.48e-7, 1.52e-7, 1.40e-7 with entries in FP32; with
+// mu_k rounded down, all in one direction, 1.72e-7, 2.71e-7, 6.8e-7.
 //
 // Compact form.  With w = -sum_t delta_t (in units of g) s is, as a function of its threshold mu, the
 // state of a stop operator driven by w.  In ascending order of mu it consists of levels: a run of
@@ -76,16 +80,16 @@ inline __host__ __device__ LatentGrid<double> latent_grid(double coef, double wm
     return {ldexp(1.0, e - grid_code<double>::B), ldexp(1.0, grid_code<double>::B - e), wmax};
 }
 
-// Code of a threshold: rounded down; a weight that is not a number or infinite acts as the largest.
+// Code of a threshold: rounded to nearest; a weight that is not a number or infinite acts as the largest.
 __device__ __forceinline__ int32_t mu_code(float mu, float ig) {
     const float cap = 16777216.0f;                              // 2^B
     const float c = fabsf(mu) * ig;
-    return __float2int_rz(c <= cap ? c : cap);
+    return __float2int_rn(c <= cap ? c : cap);
 }
 __device__ __forceinline__ int64_t mu_code(double mu, double ig) {
     const double cap = 9007199254740992.0;                      // 2^B
     const double c = fabs(mu) * ig;
-    return __double2ll_rz(c <= cap ? c : cap);
+    return __double2ll_rn(c <= cap ? c : cap);
 }
 // Code of an X value: rounded to nearest, modulo 2^32 (FP64: 2^64).  Differences of codes are taken
 // modulo as well; they are used only where |delta| < kBigMove g.

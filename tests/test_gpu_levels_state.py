@@ -1,6 +1,8 @@
 """The latent state between its forms over sequences of calls: which arithmetic and form a solve runs
 after changes of weights, states and data.  References are the same calls with every entry kept
 (FUSE_OPT_LATENT_IMPL = 0), bit for bit, and the FP64 oracle."""
+import math
+
 import pytest
 
 from paper_2210_04184_gb300 import synth
@@ -54,3 +56,26 @@ def test_monitored_solve_of_a_foreign_state(K, foreign):
         f.close()
     for a, b in zip(*runs):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("K", [1, 2])
+def test_thresholds_are_rounded_to_nearest(K):
+    # thresholds far below the moves of X saturate nearly every entry: |s| is the threshold on the
+    # grid, half a step at most from lambda2/rho times the weight
+    p = small(K=K, lam2=1e-7)
+    f = Fusion.from_problem(p, dtype="f32", wdtype="f32")
+    yl, yh = dev(p.Yl), dev(p.Yh)
+    f.weights(yh)
+    f.solve(yl, yh, 6)
+    n, nk, nP, Ls = p.H * p.W, f.nW // 2, (2 * K + 1) ** 2, p.L_s
+    mu = (torch.tensor(p.lam2 / p.rho, dtype=torch.float32, device="cuda") * f.get_weights().reshape(f.nW, n)).double()
+    s = f.get_state().view(torch.float32)[5 * Ls * n:][:nk * nP * Ls * n].reshape(nk, nP, Ls, n)
+    # the centre of the patch (k = 0) has the threshold of its own pixel; the kept offsets are the
+    # second half of the window
+    s, mu = s[:, nP // 2].abs().double(), mu[nk:, None]
+    g = 2.0 ** (math.frexp(p.lam2 / p.rho)[1] - 24)
+    off = (s - mu).abs()
+    at = off <= g
+    assert at.double().mean() > 0.9
+    assert (off[at] <= g / 2 * (1 + 1e-9)).all()
+    f.close()
