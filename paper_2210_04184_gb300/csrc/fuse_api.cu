@@ -59,7 +59,7 @@ constexpr int kGraphIters = 256;
 // remainder of a long solve), the least recently used one is replaced.
 struct LoopGraph {
     cudaGraphExec_t exec = nullptr;
-    int len = 0, cold = 0, form = 0;        // form: that of the latent state (fuse_ctx::form)
+    int len = 0, cold = 0, path = 0;        // path: kernels of the latent pass (fuse_ctx::path)
     long long launches = 0;
     unsigned long long used = 0;
 };
@@ -67,9 +67,9 @@ struct LoopGraph {
 struct LoopCache {
     LoopGraph g[2];
     unsigned long long tick = 0;
-    LoopGraph* find(int len, int cold, int form) {
+    LoopGraph* find(int len, int cold, int path) {
         for (LoopGraph& x : g)
-            if (x.exec && x.len == len && x.cold == cold && x.form == form) { x.used = ++tick; return &x; }
+            if (x.exec && x.len == len && x.cold == cold && x.path == path) { x.used = ++tick; return &x; }
         return nullptr;
     }
     LoopGraph* victim() { return g[0].used <= g[1].used ? &g[0] : &g[1]; }
@@ -88,21 +88,27 @@ struct GradWork;
 // Second capture stream of a captured iteration loop: B X and the pixel updates of an iteration
 // need only X, like the latent pass, so in a captured loop they run on this stream beside the
 // latent pass (fork after the inverse DFT); the next iteration's right-hand side, which reads
-// their U1 and U2, waits for them (join).
+// their U1 and U2, waits for them (join).  The entry kernel that stands beside the pass on the compact
+// state has a stream of its own (e, joined the same way): it runs, or returns at once, beside both.
 struct SideBranch {
-    cudaStream_t s = nullptr;
-    cudaEvent_t fork = nullptr, join = nullptr;
+    cudaStream_t s = nullptr, e = nullptr;
+    cudaEvent_t fork = nullptr, join = nullptr, join_e = nullptr;
     bool create() {
         return cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess &&
+               cudaStreamCreateWithFlags(&e, cudaStreamNonBlocking) == cudaSuccess &&
                cudaEventCreateWithFlags(&fork, cudaEventDisableTiming) == cudaSuccess &&
-               cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess;
+               cudaEventCreateWithFlags(&join, cudaEventDisableTiming) == cudaSuccess &&
+               cudaEventCreateWithFlags(&join_e, cudaEventDisableTiming) == cudaSuccess;
     }
     void destroy() {
-        if (fork) cudaEventDestroy(fork);
-        if (join) cudaEventDestroy(join);
-        if (s) cudaStreamDestroy(s);
-        s = nullptr;
-        fork = join = nullptr;
+        for (cudaEvent_t* v : {&fork, &join, &join_e}) {
+            if (*v) cudaEventDestroy(*v);
+            *v = nullptr;
+        }
+        for (cudaStream_t* v : {&s, &e}) {
+            if (*v) cudaStreamDestroy(*v);
+            *v = nullptr;
+        }
     }
 };
 
@@ -168,14 +174,17 @@ struct fuse_ctx {
     int sfmt = 0;
     // Compact latent state (k_levels.cuh; patch half-sizes 1 and 2, state in the iterate type):
     // records and level masks in hdr, level values in Sig, sorted thresholds of the current weights in
-    // tab (formed by the first solve that needs them), X with its code sums in pt.  form: what the state is kept as, 0 = entries in Sig, 1 = levels.
-    // grid [3]: the state's grid, that for omega_was, and that for weights up to 1 (fuse_weights).
-    // entries_ok: the entries are known to be those of a run on the current weights, so they convert to
-    // levels.  was: the weights changed since the levels were formed; omega_was holds the old ones.
+    // tab, X with its code sums in pt.  grid [3]: the state's grid, that for omega_was (the weights that
+    // levels were formed with, once those have changed), and that for weights up to 1 (fuse_weights).
+    // What the state holds is known on the device only (ctl, LatentCtl).  path: kernels of the
+    // iterations' latent pass, 1 = those of k_levels.cuh, which follow ctl, 0 = the entry kernels.
+    // settled: the last solve's `want` (see settle) while nothing has touched the state since, else -1;
+    // captured: a call was captured by the caller, whose replays the host does not see.
     // reg_chosen: the caller selected the register-staged pass.
     void *hdr = nullptr, *tab = nullptr, *pt = nullptr, *grid = nullptr, *omega_was = nullptr;
-    int form = 0;
-    bool entries_ok = false, was = false, grid_set = false, reg_chosen = false, tab_ok = false, lv_refused = false;
+    LatentCtl* ctl = nullptr;
+    int path = 0, settled = -1;
+    bool captured = false, reg_chosen = false, lv_refused = false;
     int lv_Ty = 1, lv_threads = 0, lv_nb = 1;
     size_t lv_smem = 0;
     // sampling mask [H][W] (uint8, ratio 1) replacing the regular lattice; NULL = lattice.
@@ -560,21 +569,26 @@ void levels_shape(fuse_ctx* c) {
 // bits in a batch of any size.  The next state up, a 5 x 5 search: 64 x 64, 14 bands 835, 810; 96 x 320, 14
 // bands 2263, 2157; 256 x 256, 8 bands 2358, 2398 (60 iterations: 5734, 5325); 512 x 512, 18 bands 20221,
 // 15989; five by five patches with a 3 x 3 search: 96 x 320, 14 bands 2094, 1960; FP64: 9594, 5734 at 256 x 256.
-bool on_grid(const fuse_ctx* c) {
-    return c->lv_threads > 0 && c->sfmt == 0 && !(c->esz == 4 && c->K == 1 && c->S == 1);
+bool grid_options(const fuse_ctx* c) { return c->lv_threads > 0 && !(c->esz == 4 && c->K == 1 && c->S == 1); }
+bool on_grid(const fuse_ctx* c) { return c->sfmt == 0 && grid_options(c); }
+
+// The caller captures the stream.  Its replays change the state behind the host's back: from then on
+// every call leaves it to the device what there is to do.
+bool capturing(fuse_ctx* c) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool yes = cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (yes) cudaGetLastError();
+    c->captured = c->captured || yes;
+    return yes;
 }
 
-// The buffers of the compact state, allocated by the first solve that would use them (not while its
-// stream is captured) and kept.  Without the memory for them solves keep the state as entries, with the
-// same results.
+// The buffers of the compact state, allocated by the first solve that would use them and kept.  A context
+// whose weights or solves were captured before that goes without: the captured calls know of no levels.
+// Without the buffers solves keep the state as entries, in the arithmetic of the iterate type.
 bool levels_alloc(fuse_ctx* c) {
     if (c->hdr) return true;
     if (c->lv_refused || c->fault_alloc >= 0) return false;
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-        cudaGetLastError();
-        return false;
-    }
+    if (capturing(c) || c->captured) return false;
     const size_t nk = c->half ? c->nW / 2 : c->nW;
     const size_t pts = (size_t)c->Ls * c->H * (c->W + 2 * c->S) * 4 * c->esz;
     void** p[] = {&c->hdr, &c->tab, &c->pt, &c->omega_was};
@@ -591,7 +605,7 @@ bool levels_alloc(fuse_ctx* c) {
     return ok;
 }
 
-// Solves keep the latent state as levels.
+// Solves run the latent pass on the compact state.
 bool uses_levels(fuse_ctx* c) { return on_grid(c) && !c->reg_chosen && levels_alloc(c); }
 
 // Dynamic shared-memory cap of the monitoring latent kernels of this context's types.
@@ -633,6 +647,8 @@ struct Impl {
                             c->Ls, c->S, Ty, ncons, D, (T)(c->lam2 / c->rho), c->d_err, c->wait_limit,
                             c->half, bpb, zero_in};
         a.grid = (const LatentGrid<T>*)c->grid;
+        // NULL where the state is never anything but entries of the iterate type's arithmetic
+        a.ctl = on_grid(c) && c->path == 1 && !c->lat_in && !c->lat_out ? c->ctl : nullptr;
         return a;
     }
     // old: the weights (and their bound) from before the last change
@@ -644,7 +660,7 @@ struct Impl {
         return LevelArgs<T, WT>{(const T*)c->X, (const WT*)(old ? c->omega_was : c->omega), rec,
                                 (uint2*)(rec + nk * c->Ls * c->n), (C*)c->Sig,
                                 (const code_t<T>*)c->tab, (const LevelPoint<T>*)c->pt, (T*)c->planes, c->H, c->W, c->Ls, c->S, c->lv_Ty, c->lv_nb,
-                                (T)(c->lam2 / c->rho), (const LatentGrid<T>*)c->grid + (old ? 1 : 0), c->half};
+                                (T)(c->lam2 / c->rho), (const LatentGrid<T>*)c->grid + (old ? 1 : 0), c->half, c->ctl};
     }
 
     static fuse_status set_attrs(fuse_ctx* c) {
@@ -719,52 +735,64 @@ struct Impl {
 
     // zero_in: the state entering this pass is zero (the first iteration of a cold solve); the
     // bulk-copy pass then reads none of it.  The register-staged pass always reads it.
+    // se: stream of the entry kernel beside the pass on the compact state (s itself, or a branch).
     template <typename WT>
-    static void latent(fuse_ctx* c, cudaStream_t s, bool zero_in) {
+    static void latent(fuse_ctx* c, cudaStream_t s, cudaStream_t se, bool zero_in) {
         const unsigned rowsW = (unsigned)(c->half ? c->S + 1 : 2 * c->S + 1);
-        const bool taped = c->lat_in || c->lat_out;
-        if (c->form == 1 && !taped) {
+        const bool taped = c->lat_in || c->lat_out, beside = c->path == 1 && !taped;
+        if (beside) {
             dim3 grid((unsigned)((c->H + c->lv_Ty - 1) / c->lv_Ty), (unsigned)((c->Ls + c->lv_nb - 1) / c->lv_nb), rowsW);
             const LevelArgs<T, WT> a = lv_args<WT>(c);
             points_launch<T, WT>(a, zero_in, s);
-            if (zero_in) levels_init_launch<T, WT>(a, c->K, c->half ? c->nW / 2 : c->nW, s);
+            if (zero_in) {
+                levels_init_launch<T, WT>(a, c->K, kept(c), c->lat_impl == 0, s);
+                if (c->lat_impl == 0) se = s;                 // reads the zero entries
+            }
             // X of a cold first iteration is zero with the paper's splitting, and so are the planes
             if (!zero_in || c->xmode == 1)
                 levels_launch<T, WT>(a, c->K, grid, (unsigned)c->lv_threads, c->lv_smem, s);
-            return;
+        } else {
+            se = s;
         }
         if (c->lat_impl == 1) {
             dim3 grid((unsigned)((c->H + c->lt_Ty - 1) / c->lt_Ty), (unsigned)((c->Ls + c->lat_bpb - 1) / c->lat_bpb),
                       rowsW);
             const LatentArgs<T, WT> a = lat_args<WT>(c, c->lt_Ty, c->lt_ncons, c->lat_stages, c->lat_bpb, zero_in);
-            latent_tma_launch<T, WT>(a, c->K, c->sfmt == 1, on_grid(c) && !taped, grid, (unsigned)(c->lt_ncons + 32), c->lt_smem, s);
+            latent_tma_launch<T, WT>(a, c->K, c->sfmt == 1, grid, (unsigned)(c->lt_ncons + 32), c->lt_smem, se);
             return;
         }
         dim3 grid((unsigned)((c->H + c->lat_Ty - 1) / c->lat_Ty), (unsigned)c->Ls, rowsW);
+        const bool both = on_grid(c) && !taped;
         latent_reg_launch<T, WT>((const T*)c->X, (const WT*)c->omega, (const T*)lat_src(c), (T*)lat_dst(c),
                                  (T*)c->planes, c->H, c->W, c->Ls, c->S, c->lat_Ty, (T)(c->lam2 / c->rho), c->half,
-                                 (const LatentGrid<T>*)c->grid, c->K, on_grid(c) && !taped, grid, (unsigned)c->lat_threads, c->lat_smem, s);
+                                 (const LatentGrid<T>*)c->grid, both ? c->ctl : nullptr, both && !beside, c->K, grid,
+                                 (unsigned)c->lat_threads, c->lat_smem, se);
     }
 
-    // The state between its two forms, in place (see levels_convert_launch).
+    // The conversions of the latent state, in place, each run by the device where it is due.
     template <typename WT>
-    static void convert(fuse_ctx* c, bool to_levels, bool check, int* bad) {
-        const int kept = c->half ? c->nW / 2 : c->nW;
-        levels_convert_launch<T, WT>(lv_args<WT>(c, !to_levels && c->was), c->K, kept, to_levels, check, bad, c->stream);
+    static void to_entries(fuse_ctx* c, int want) {
+        levels_to_entries_launch<T, WT>(lv_args<WT>(c), lv_args<WT>(c, true), c->K, kept(c), c->nsm, want, c->stream);
     }
-    static void convert_any(fuse_ctx* c, bool to_levels, bool check, int* bad);
+    template <typename WT>
+    static void check_entries(fuse_ctx* c) {
+        entries_check_launch<T, WT>(lv_args<WT>(c), c->K, kept(c), c->nsm, c->stream);
+    }
+    template <typename WT>
+    static void to_levels(fuse_ctx* c) {
+        entries_to_levels_launch<T, WT>(lv_args<WT>(c), c->K, kept(c), c->nsm, c->stream);
+    }
     template <typename WT>
     static void table(fuse_ctx* c) {
-        level_table_launch<T, WT>((const WT*)c->omega, (code_t<T>*)c->tab, c->H, c->W, c->K, c->S, c->half,
-                                  c->half ? c->nW / 2 : c->nW, (T)(c->lam2 / c->rho), (const LatentGrid<T>*)c->grid, c->stream);
+        level_table_launch<T, WT>(lv_args<WT>(c), c->K, kept(c), c->nsm, c->stream);
     }
-    static void table_any(fuse_ctx* c);
+    static int kept(const fuse_ctx* c) { return c->half ? c->nW / 2 : c->nW; }
     template <typename WT>
     static void weights_bound(fuse_ctx* c) {
         wmax_launch<T, WT>((const WT*)c->omega, (size_t)c->nW * c->n, (LatentGrid<T>*)c->grid, (T)(c->lam2 / c->rho), c->stream);
     }
 
-    static void latent_any(fuse_ctx* c, cudaStream_t s, bool zero_in);
+    static void latent_any(fuse_ctx* c, cudaStream_t s, cudaStream_t se, bool zero_in);
 
     // The monitoring latent pass (bulk-copy kernel, state in the iterate type) and the residual
     // sums of the iteration that ran it (k_monitor.cuh).
@@ -774,11 +802,12 @@ struct Impl {
         dim3 grid((unsigned)((c->H + c->lt_Ty - 1) / c->lt_Ty), (unsigned)((c->Ls + c->lat_bpb - 1) / c->lat_bpb),
                   rowsW);
         LatentArgs<T, WT> a = lat_args<WT>(c, c->lt_Ty, c->lt_ncons, c->lat_stages, c->lat_bpb, zero_in);
+        a.ctl = on_grid(c) ? c->ctl : nullptr;
         a.mplanes = (T*)c->mPm;
         a.mpart = c->mon_part;
         c->mon_lat = (size_t)grid.x * grid.y * grid.z;
         const size_t smem = c->lt_smem + 2 * (size_t)c->lt_Ty * c->W * sizeof(T);     // two more tiles
-        latent_monitor_launch<T, WT>(a, c->K, on_grid(c), grid, (unsigned)(c->lt_ncons + 32), smem, s);
+        latent_monitor_launch<T, WT>(a, c->K, grid, (unsigned)(c->lt_ncons + 32), smem, s);
     }
 
     static fuse_status monitor_sums(fuse_ctx* c, cudaStream_t s) {
@@ -808,7 +837,9 @@ struct Impl {
     // join_prev: wait for the previous iteration's side branch before the right-hand side.
     static fuse_status iterate(fuse_ctx* c, cudaStream_t s, bool timed, bool zero_in = false, bool monitor = false,
                                bool side = false, bool join_prev = false) {
+        const bool branch = side && c->path == 1;       // an entry kernel beside the pass on the compact state
         if (side && join_prev) CK(c, cudaStreamWaitEvent(s, c->side.join, 0));
+        if (branch && join_prev) CK(c, cudaStreamWaitEvent(s, c->side.join_e, 0));
         if (c->xmode == 1) {
             dim3 grid((unsigned)((c->W + ST_TX - 1) / ST_TX), (unsigned)((c->H + ST_TY - 1) / ST_TY), (unsigned)c->Ls);
             rhs_sum_kernel<T><<<grid, dim3(ST_TX, ST_BY), 0, s>>>(st_args(c, c->U1, c->C, nullptr));
@@ -838,6 +869,7 @@ struct Impl {
         if (side) {
             CK(c, cudaEventRecord(c->side.fork, s));
             CK(c, cudaStreamWaitEvent(c->side.s, c->side.fork, 0));
+            if (branch) CK(c, cudaStreamWaitEvent(c->side.e, c->side.fork, 0));
             sp = c->side.s;
         }
         if (c->xmode != 1) {
@@ -856,7 +888,7 @@ struct Impl {
             }
             Event2& e = c->ev[c->ev_used++];
             CK(c, cudaEventRecord(e.a, s));
-            latent_any(c, s, zero_in);
+            latent_any(c, s, s, zero_in);
             CK(c, cudaEventRecord(e.b, s));
         } else if (monitor) {
             if constexpr (sizeof(T) == 8) {
@@ -866,9 +898,10 @@ struct Impl {
                 else latent_monitor<float>(c, s, zero_in);
             }
         } else {
-            latent_any(c, s, zero_in);
+            latent_any(c, s, branch ? c->side.e : s, zero_in);
         }
         CKL(c, "latent kernel");
+        if (branch) CK(c, cudaEventRecord(c->side.join_e, c->side.e));
         if (monitor) return monitor_sums(c, s);
         return FUSE_OK;
     }
@@ -912,32 +945,12 @@ struct Impl {
 };
 
 template <typename T>
-void Impl<T>::latent_any(fuse_ctx* c, cudaStream_t s, bool zero_in) {
+void Impl<T>::latent_any(fuse_ctx* c, cudaStream_t s, cudaStream_t se, bool zero_in) {
     if constexpr (sizeof(T) == 8) {
-        latent<double>(c, s, zero_in);
+        latent<double>(c, s, se, zero_in);
     } else {
-        if (c->wdtype == FUSE_BF16) latent<__nv_bfloat16>(c, s, zero_in);
-        else latent<float>(c, s, zero_in);
-    }
-}
-
-template <typename T>
-void Impl<T>::convert_any(fuse_ctx* c, bool to_levels, bool check, int* bad) {
-    if constexpr (sizeof(T) == 8) {
-        convert<double>(c, to_levels, check, bad);
-    } else {
-        if (c->wdtype == FUSE_BF16) convert<__nv_bfloat16>(c, to_levels, check, bad);
-        else convert<float>(c, to_levels, check, bad);
-    }
-}
-
-template <typename T>
-void Impl<T>::table_any(fuse_ctx* c) {
-    if constexpr (sizeof(T) == 8) {
-        table<double>(c);
-    } else {
-        if (c->wdtype == FUSE_BF16) table<__nv_bfloat16>(c);
-        else table<float>(c);
+        if (c->wdtype == FUSE_BF16) latent<__nv_bfloat16>(c, s, se, zero_in);
+        else latent<float>(c, s, se, zero_in);
     }
 }
 
@@ -988,55 +1001,72 @@ fuse_status guard(fuse_ctx* c) {
     return FUSE_OK;
 }
 
-fuse_status convert_state(fuse_ctx* c, bool to_levels, bool check = false, int* bad = nullptr) {
-    if (c->dtype == FUSE_F64) Impl<double>::convert_any(c, to_levels, check, bad);
-    else Impl<float>::convert_any(c, to_levels, check, bad);
+// Calls f with Impl<T> and a value of the weight type, for the context's types.
+template <typename F>
+void with_types(const fuse_ctx* c, F&& f) {
+    if (c->dtype == FUSE_F64) f(Impl<double>{}, double{});
+    else if (c->wdtype == FUSE_BF16) f(Impl<float>{}, __nv_bfloat16{});
+    else f(Impl<float>{}, float{});
+}
+
+// The state as entries, for a reader or a pass of them.  want: as in settle.
+fuse_status need_entries(fuse_ctx* c, int want = kStateGrid) {
+    if (!c->hdr || !grid_options(c)) return FUSE_OK;        // never levels
+    with_types(c, [&](auto im, auto w) { im.template to_entries<decltype(w)>(c, want); });
     c->launches_all++;
-    CKL(c, "latent state conversion");
+    CKL(c, "levels_to_entries_kernel");
+    c->settled = -1;
     return FUSE_OK;
 }
 
-// The state as entries.  Levels formed with weights that have changed since give entries that need
-// not be those of a run on the current ones.
-fuse_status need_entries(fuse_ctx* c) {
-    if (c->form == 0) return FUSE_OK;
-    const fuse_status st = convert_state(c, false);
-    if (st != FUSE_OK) return st;
-    c->form = 0;
-    c->entries_ok = !c->was;
-    c->was = false;
-    return FUSE_OK;
-}
-
-// The sorted thresholds of the current weights, which the iterations on levels read.
-fuse_status need_table(fuse_ctx* c) {
-    if (c->form != 1 || c->tab_ok) return FUSE_OK;
-    if (c->dtype == FUSE_F64) Impl<double>::table_any(c);
-    else Impl<float>::table_any(c);
-    c->launches_all++;
-    CKL(c, "level_table_kernel");
-    c->tab_ok = true;
-    return FUSE_OK;
-}
-
-// The form in which the iterations of a warm solve continue: levels where the state allows it.
-fuse_status warm_form(fuse_ctx* c) {
-    if (c->form == 1 && (c->was || !uses_levels(c))) return need_entries(c);
-    if (c->form == 0 && c->entries_ok && uses_levels(c)) {
-        const fuse_status st = convert_state(c, true);
-        if (st != FUSE_OK) return st;
-        c->form = 1;
+// Brings the latent state into the form in which the iterations of a solve continue or start, `want`:
+//   kStateLevels   levels (path 1), or entries where the state is not that of a run on the current weights
+//   kStateGrid     entries, on the grid where they are those of such a run
+//   kStateEntries  entries in the arithmetic of the iterate type
+// A context whose state nothing touched since a solve with the same `want` has nothing to do.
+fuse_status settle(fuse_ctx* c, bool cold, int want) {
+    if (!on_grid(c)) return FUSE_OK;
+    const bool touched = capturing(c) || c->captured || c->settled != want;
+    if (cold || touched) {
+        latent_begin_launch(c->ctl, cold, want, c->stream);
+        c->launches_all++;
+        CKL(c, "latent_begin_kernel");
     }
+    if (!cold && touched) {
+        const fuse_status st = need_entries(c, want);
+        if (st != FUSE_OK) return st;
+        if (want != kStateEntries) {
+            with_types(c, [&](auto im, auto w) { im.template check_entries<decltype(w)>(c); });
+            c->launches_all++;
+            CKL(c, "entries_check_kernel");
+        }
+        if (want == kStateLevels) {
+            with_types(c, [&](auto im, auto w) { im.template to_levels<decltype(w)>(c); });
+            c->launches_all++;
+            CKL(c, "entries_to_levels_kernel");
+        }
+    }
+    if (want == kStateLevels && (cold || touched)) {        // the thresholds that the levels are read with
+        with_types(c, [&](auto im, auto w) { im.template table<decltype(w)>(c); });
+        c->launches_all++;
+        CKL(c, "level_table_kernel");
+    }
+    c->settled = want;
     return FUSE_OK;
 }
 
-// Before the weights change: levels stay readable through the weights they were formed with.
+// Before the weights change.
 fuse_status weights_change(fuse_ctx* c) {
-    c->entries_ok = c->tab_ok = false;
-    if (c->form != 1 || !c->have_state || c->was) return FUSE_OK;
-    CK(c, cudaMemcpyAsync(c->omega_was, c->omega, (size_t)c->nW * c->n * c->wsz, cudaMemcpyDeviceToDevice, c->stream));
-    CK(c, cudaMemcpyAsync((char*)c->grid + 3 * c->esz, c->grid, 3 * c->esz, cudaMemcpyDeviceToDevice, c->stream));
-    c->was = true;
+    if (!grid_options(c)) return FUSE_OK;
+    capturing(c);
+    c->settled = -1;
+    const size_t bytes = (size_t)c->nW * c->n * c->wsz;
+    if (c->dtype == FUSE_F64)
+        weights_change_launch<double>(c->omega, c->omega_was, bytes, (LatentGrid<double>*)c->grid, c->ctl, c->nsm, c->stream);
+    else
+        weights_change_launch<float>(c->omega, c->omega_was, bytes, (LatentGrid<float>*)c->grid, c->ctl, c->nsm, c->stream);
+    c->launches_all++;
+    CKL(c, "weights_change_kernel");
     return FUSE_OK;
 }
 
@@ -1055,12 +1085,12 @@ fuse_status zero_state(fuse_ctx* c, cudaStream_t s, bool clear_sigma = true) {
 }
 
 // kernels launched by one iteration (Impl::iterate)
-int iteration_launches(const fuse_ctx* c) { return (c->xmode == 1 ? 6 : 7) + (c->form == 1 ? 1 : 0); }
+int iteration_launches(const fuse_ctx* c) { return (c->xmode == 1 ? 6 : 7) + (c->path == 1 ? 2 : 0); }
 
 // Replays `len` iterations from one captured graph (captured on first use; `cold`: the first
 // iteration's latent pass reads no state).
 fuse_status launch_loop(fuse_ctx* c, int len, bool cold) {
-    LoopGraph* lg = c->loops.find(len, cold, c->form);
+    LoopGraph* lg = c->loops.find(len, cold, c->path);
     if (!lg) {
         const bool f64 = c->dtype == FUSE_F64;
         CK(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -1069,8 +1099,10 @@ fuse_status launch_loop(fuse_ctx* c, int len, bool cold) {
         for (int t = 0; t < len && st == FUSE_OK; ++t, ++forked)
             st = f64 ? Impl<double>::iterate(c, c->cap_stream, false, cold && t == 0, false, true, t > 0)
                      : Impl<float>::iterate(c, c->cap_stream, false, cold && t == 0, false, true, t > 0);
-        // the side branch of the last iteration joins the loop's stream before the capture ends
-        if (forked && cudaStreamWaitEvent(c->cap_stream, c->side.join, 0) != cudaSuccess && st == FUSE_OK)
+        // the branches of the last iteration join the loop's stream before the capture ends
+        if (forked &&
+            (cudaStreamWaitEvent(c->cap_stream, c->side.join, 0) != cudaSuccess ||
+             (c->path == 1 && cudaStreamWaitEvent(c->cap_stream, c->side.join_e, 0) != cudaSuccess)) && st == FUSE_OK)
             st = fail(c, FUSE_ECUDA, "cudaStreamWaitEvent");
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
@@ -1084,7 +1116,7 @@ fuse_status launch_loop(fuse_ctx* c, int len, bool cold) {
         if (e != cudaSuccess) { lg->exec = nullptr; return fail_cuda(c, "cudaGraphInstantiate", e); }
         lg->len = len;
         lg->cold = cold;
-        lg->form = c->form;
+        lg->path = c->path;
         lg->launches = (long long)len * iteration_launches(c);
         lg->used = ++c->loops.tick;
     }
@@ -1109,12 +1141,7 @@ fuse_status monitored_iteration(fuse_ctx* c, bool zero_in) {
     if (c->lt_smem + 2 * (size_t)c->lt_Ty * c->W * c->esz > (size_t)kMaxSmem)
         return fail(c, FUSE_EUNSUPPORTED, "the monitoring latent pass does not fit shared memory");
     fuse_status st = FUSE_OK;
-    if (zero_in) {                             // the pass reads no state and writes the entries of a run
-        c->form = 0;
-        c->entries_ok = true;
-    } else if ((st = need_entries(c)) != FUSE_OK) {
-        return st;                             // other entries stay what they were before it
-    }
+    if (!zero_in && (st = need_entries(c)) != FUSE_OK) return st;
     const size_t img = c->n * c->Ls * c->esz;
     cudaStream_t s = c->stream;
     CK(c, cudaMemcpyAsync(c->mL1, c->Lam1, img, cudaMemcpyDeviceToDevice, s));
@@ -1159,7 +1186,9 @@ fuse_status run_iterations_plain(fuse_ctx* c, int iters, bool cold) {
     return FUSE_OK;
 }
 
-fuse_status solve_impl(fuse_ctx* c, const void* Yl, const void* Yh, int iters, int warm, void* Xo, void* Zo) {
+// taped: the taped iterations follow, whose state is entries in the arithmetic of the iterate type.
+fuse_status solve_impl(fuse_ctx* c, const void* Yl, const void* Yh, int iters, int warm, void* Xo, void* Zo,
+                       bool taped = false) {
     const bool f64 = c->dtype == FUSE_F64;
     fuse_status st;
     ++c->epoch;
@@ -1170,21 +1199,19 @@ fuse_status solve_impl(fuse_ctx* c, const void* Yl, const void* Yh, int iters, i
     st = f64 ? Impl<double>::band_mix(c, c->stream, Yh, c->D9b, c->Mh, c->n, c->Lh, c->Ls)
              : Impl<float>::band_mix(c, c->stream, Yh, c->D9b, c->Mh, c->n, c->Lh, c->Ls);
     if (st != FUSE_OK) return st;
-    // A cold start with at least one iteration leaves the latent state uncleared: the first
-    // latent pass of the bulk-copy kernel takes it as zero and overwrites every entry.
-    bool cold = false;
-    if (!warm || !c->have_state) {
-        cold = iters > 0 && (c->lat_impl == 1 || uses_levels(c));
+    // A cold start with at least one iteration leaves the latent state uncleared: the first latent pass
+    // of the bulk-copy kernel, or that on the compact state, takes it as zero and overwrites it.
+    c->path = !taped && uses_levels(c) ? 1 : 0;
+    const bool start = !warm || !c->have_state, cold = start && iters > 0 && (c->lat_impl == 1 || c->path == 1);
+    int want = c->path == 1 ? kStateLevels : c->lat_impl == 0 && !taped ? kStateGrid : kStateEntries;
+    if (start) {
         st = zero_state(c, c->stream, !cold);
         if (st != FUSE_OK) return st;
         c->have_state = true;
-        c->form = cold && uses_levels(c) ? 1 : 0;
-        c->entries_ok = true;                  // zeros are the entries of a run on any weights
-        c->was = false;
-    } else if ((st = warm_form(c)) != FUSE_OK) {
-        return st;
+        // cleared entries, or entries that a monitored first iteration writes
+        if (!cold || (c->monitor && iters == 1)) want = std::min<int>(want, kStateGrid);
     }
-    if ((st = need_table(c)) != FUSE_OK) return st;
+    if ((st = settle(c, start, want)) != FUSE_OK) return st;
     if (c->xmode == 1) {
         // the fixed data term of the variant: U1 = G = B^T S^T Y_l E^T / rho (B X as scratch)
         st = f64 ? Impl<double>::sb_data_term(c, c->stream) : Impl<float>::sb_data_term(c, c->stream);
@@ -1208,10 +1235,6 @@ fuse_status weights_impl(fuse_ctx* c, const void* G) {
     fuse_status st;
     ++c->epoch;
     if ((st = weights_change(c)) != FUSE_OK) return st;
-    if (c->grid_set) {
-        CK(c, cudaMemcpyAsync(c->grid, (char*)c->grid + 6 * c->esz, 3 * c->esz, cudaMemcpyDeviceToDevice, c->stream));
-        c->grid_set = false;
-    }
     if (c->dtype == FUSE_F64) st = Impl<double>::weights<double>(c, G);
     else if (c->wdtype == FUSE_BF16) st = Impl<float>::weights<__nv_bfloat16>(c, G);
     else st = Impl<float>::weights<float>(c, G);
@@ -1236,8 +1259,8 @@ fuse_status realloc_state(fuse_ctx* c, int h, int f) {
     c->sig_bytes = bytes;
     c->half = h;
     c->sfmt = f;
-    c->form = 0;
-    c->entries_ok = c->was = c->tab_ok = false;
+    c->path = 0;
+    c->settled = -1;
     latent_tma_shape(c);
     levels_shape(c);
     ++c->epoch;
@@ -1448,9 +1471,12 @@ struct BatchImpl {
             if (nc > b->lat_ncons) b->lat_ncons = nc;
         }
         b->lat_smem = 0;
+        b->levels = true;
+        for (fuse_ctx* c : b->ctx) b->levels = b->levels && on_grid(c) && levels_alloc(c);
         for (int i = 0; i < n; ++i) {
             fuse_ctx* c = b->ctx[i];
             la[i] = Impl<T>::template lat_args<WT>(c, Ty[i], b->lat_ncons, b->lat_stages, b->lat_bpb);
+            la[i].ctl = b->levels ? c->ctl : nullptr;
             const size_t ssz = b->sfmt ? 2 : esz;
             const size_t sm = (size_t)b->lat_stages * Ty[i] * c->W * ssz + 5 * (size_t)Ty[i] * c->W * esz +
                               2 * (size_t)b->lat_stages * 8;
@@ -1470,8 +1496,6 @@ struct BatchImpl {
         if ((st = bupload(b, &b->d_lat, la)) != FUSE_OK) return st;
         if ((st = bupload(b, (void**)&b->d_lat_seg, seg)) != FUSE_OK) return st;
 
-        b->levels = true;
-        for (fuse_ctx* c : b->ctx) b->levels = b->levels && on_grid(c) && levels_alloc(c);
         if (b->levels) {
             std::vector<LevelArgs<T, WT>> lv(n);
             std::vector<Segment> sp;
@@ -1593,7 +1617,9 @@ struct BatchImpl {
     // captured loops).
     static fuse_status iterate(fuse_batch* b, cudaStream_t s, bool timed, bool zero_in = false, bool side = false,
                                bool join_prev = false) {
+        const bool branch = side && b->levels;          // the entry kernel beside the pass on the compact state
         if (side && join_prev) BCK(b, cudaStreamWaitEvent(s, b->side.join, 0));
+        if (branch && join_prev) BCK(b, cudaStreamWaitEvent(s, b->side.join_e, 0));
         // square blurs shared by every problem: taps in the argument space (from problem 0)
         const fuse_ctx* c0 = b->ctx[0];
         const bool sq = b->bh == b->bw && b->same_taps;
@@ -1609,6 +1635,7 @@ struct BatchImpl {
         if (side) {
             BCK(b, cudaEventRecord(b->side.fork, s));
             BCK(b, cudaStreamWaitEvent(b->side.s, b->side.fork, 0));
+            if (branch) BCK(b, cudaStreamWaitEvent(b->side.e, b->side.fork, 0));
             sp = b->side.s;
         }
         stencil_batch_launch<T, 0>((const StencilArgs<T>*)b->d_st0, sep ? b->d_sep0_seg : b->d_st_seg,
@@ -1636,15 +1663,16 @@ struct BatchImpl {
             points_batch_launch<T, WT>(lv, b->d_pt_seg, b->pt_nseg, zero_in ? 1 : 0, (unsigned)b->pt_blocks, s);
             if (zero_in) {              // X of a cold first iteration is zero, and so are the planes
                 for (fuse_ctx* c : b->ctx)
-                    levels_init_launch<T, WT>(Impl<T>::template lv_args<WT>(c), c->K, c->half ? c->nW / 2 : c->nW, s);
+                    levels_init_launch<T, WT>(Impl<T>::template lv_args<WT>(c), c->K, Impl<T>::kept(c), 0, s);
             } else {
                 levels_batch_launch<T, WT>(lv, b->d_lv_seg, b->lv_nseg, b->K, (unsigned)b->lv_blocks, kLevelThreads,
                                            b->lv_smem, s);
             }
-        } else
+        }
         latent_tma_batch_launch<T, WT>((const LatentArgs<T, WT>*)b->d_lat, b->d_lat_seg, b->lat_nseg, zero_in ? 1 : 0,
-                                       b->K, b->sfmt != 0, on_grid(b->ctx[0]), (unsigned)b->lat_blocks, (unsigned)(b->lat_ncons + 32),
-                                       b->lat_smem, s);
+                                       b->K, b->sfmt != 0, (unsigned)b->lat_blocks, (unsigned)(b->lat_ncons + 32),
+                                       b->lat_smem, branch ? b->side.e : s);
+        if (branch) BCK(b, cudaEventRecord(b->side.join_e, b->side.e));
         if (timed) BCK(b, cudaEventRecord(e1, s));
         BCK(b, cudaGetLastError());
         return FUSE_OK;
@@ -1701,8 +1729,10 @@ fuse_status batch_launch_loop(fuse_batch* b, int len, bool cold) {
         int forked = 0;
         for (int t = 0; t < len && st == FUSE_OK; ++t, ++forked)
             st = batch_iterate(b, b->cap_stream, false, cold && t == 0, true, t > 0);
-        // the side branch of the last iteration joins the loop's stream before the capture ends
-        if (forked && cudaStreamWaitEvent(b->cap_stream, b->side.join, 0) != cudaSuccess && st == FUSE_OK)
+        // the branches of the last iteration join the loop's stream before the capture ends
+        if (forked &&
+            (cudaStreamWaitEvent(b->cap_stream, b->side.join, 0) != cudaSuccess ||
+             (b->levels && cudaStreamWaitEvent(b->cap_stream, b->side.join_e, 0) != cudaSuccess)) && st == FUSE_OK)
             st = bfail(b, FUSE_ECUDA, "cudaStreamWaitEvent");
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(b->cap_stream, &g);
@@ -1716,7 +1746,7 @@ fuse_status batch_launch_loop(fuse_batch* b, int len, bool cold) {
         if (e != cudaSuccess) { lg->exec = nullptr; BCK(b, e); }
         lg->len = len;
         lg->cold = cold;
-        lg->launches = (b->levels ? 8LL : 7LL) * len;
+        lg->launches = (b->levels ? 9LL : 7LL) * len;
         lg->used = ++b->loops.tick;
     }
     BCK(b, cudaGraphLaunch(lg->exec, b->stream));
@@ -1733,7 +1763,7 @@ fuse_status batch_run(fuse_batch* b, int iters, bool cold = false) {
         for (int t = 0; t < iters; ++t) {
             fuse_status st = batch_iterate(b, b->stream, b->profile, cold && t == 0);
             if (st != FUSE_OK) return st;
-            b->launches_all += b->levels ? 8 : 7;
+            b->launches_all += b->levels ? 9 : 7;
             b->launches_latent += 1;
         }
         return FUSE_OK;
@@ -1989,6 +2019,8 @@ fuse_status fuse_init(fuse_ctx** out, const fuse_geometry* g, const double* blur
             }
         }
         if ((st = upload_any(c, &c->grid, gv)) != FUSE_OK) return bail(st);
+        if ((st = dalloc(c, (void**)&c->ctl, sizeof(LatentCtl))) != FUSE_OK) return bail(st);
+        if (cudaMemset(c->ctl, 0, sizeof(LatentCtl)) != cudaSuccess) { cudaGetLastError(); return bail(FUSE_ECUDA); }
     }
     if ((st = upload_any(c, &c->tapsT, tT)) != FUSE_OK) return bail(st);
     if ((st = upload_any(c, &c->tapsB, tB)) != FUSE_OK) return bail(st);
@@ -2072,14 +2104,13 @@ fuse_status fuse_set_weights(fuse_ctx* c, const void* w) {
     if (!w) return fail(c, FUSE_EINVAL, "weights pointer is NULL");
     if ((st = weights_change(c)) != FUSE_OK) return st;
     CK(c, cudaMemcpyAsync(c->omega, w, (size_t)c->nW * c->n * c->wsz, cudaMemcpyDefault, c->stream));
-    if (latent_grid_k(c->K)) {
+    if (grid_options(c)) {
         // the grid of the latent state is set by the largest weight
         CK(c, cudaMemsetAsync(c->grid, 0, 3 * c->esz, c->stream));
         if (c->dtype == FUSE_F64) Impl<double>::weights_bound<double>(c);
         else if (c->wdtype == FUSE_BF16) Impl<float>::weights_bound<__nv_bfloat16>(c);
         else Impl<float>::weights_bound<float>(c);
         c->launches_all += 2;
-        c->grid_set = true;
         CKL(c, "wmax_kernel");
     }
     c->have_weights = true;
@@ -2202,17 +2233,11 @@ fuse_status fuse_set_state(fuse_ctx* c, const void* src) {
     CK(c, cudaMemcpyAsync(c->Sig, p, c->sig_bytes, cudaMemcpyDefault, c->stream));
     p += c->sig_bytes;
     CK(c, cudaMemcpyAsync(c->planes, p, c->plane_bytes, cudaMemcpyDefault, c->stream));
-    c->form = 0;
-    c->entries_ok = c->was = false;
-    if (c->have_weights && uses_levels(c)) {
-        // a state saved from a run on these weights continues as levels, any other as entries
-        int* bad = (int*)c->partial;
-        int flag = 0;
-        CK(c, cudaMemsetAsync(bad, 0, sizeof(int), c->stream));
-        if ((st = convert_state(c, true, true, bad)) != FUSE_OK) return st;
-        CK(c, cudaMemcpyAsync(&flag, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-        CK(c, cudaStreamSynchronize(c->stream));
-        c->entries_ok = flag == 0;
+    if (on_grid(c)) {
+        latent_begin_launch(c->ctl, 1, kStateGiven, c->stream);
+        c->launches_all++;
+        CKL(c, "latent_begin_kernel");
+        c->settled = -1;
     }
     CK(c, cudaStreamSynchronize(c->stream));
     c->have_state = true;
@@ -2420,10 +2445,11 @@ fuse_status fuse_autotune(fuse_ctx* c, const void* Yl, const void* Yh, int iters
     // inputs and a zero state (the timed iterations run on it; the next solve starts over)
     st = solve_impl(c, Yl, Yh, 0, 0, nullptr, nullptr);
     if (st != FUSE_OK) return st;
-    if ((st = warm_form(c)) != FUSE_OK || (st = need_table(c)) != FUSE_OK) return st;
+    if ((st = settle(c, false, c->path == 1 ? kStateLevels : c->lat_impl == 0 ? kStateGrid : kStateEntries)) != FUSE_OK)
+        return st;
     double best = 1e30, t = 0;
     // 1. latent pass: ring shape and bands per block (the pass on the compact state has one shape)
-    if (c->lat_impl == 1 && c->form == 0) {
+    if (c->lat_impl == 1 && c->path == 0) {
         const int bt = c->lat_target, bs = c->lat_stages, bb = c->lat_bpb;
         int best_t = bt, best_s = bs, best_b = bb;
         const int threads[] = {128, 192, 256}, stages[] = {4, 6, 8, 12, 16, 24}, bands[] = {1, 2};
@@ -2597,10 +2623,8 @@ fuse_status fuse_batch_solve(fuse_batch* b, const void* const* Yl, const void* c
         if (st == FUSE_OK) st = zero_state(c, b->stream, iters == 0);
         if (st != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
         c->have_state = true;
-        c->form = b->levels && iters > 0 ? 1 : 0;
-        c->entries_ok = iters == 0;
-        c->was = false;
-        if ((st = need_table(c)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
+        c->path = b->levels ? 1 : 0;
+        if ((st = settle(c, true, b->levels ? (iters > 0 ? kStateLevels : kStateGiven) : kStateEntries)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
     }
     fuse_status st = batch_run(b, iters, iters > 0);
     if (st != FUSE_OK) return st;

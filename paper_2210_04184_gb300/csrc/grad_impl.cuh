@@ -459,7 +459,7 @@ fuse_status grad_forward_impl(fuse_ctx* c, const void* Yl, const void* Yh, int i
     fuse_status st = grad_prepare(c, iters);
     if (st != FUSE_OK) return st;
     // D9a, D9b and zero state, as a cold solve
-    st = solve_impl(c, Yl, Yh, 0, 0, nullptr, nullptr);
+    st = solve_impl(c, Yl, Yh, 0, 0, nullptr, nullptr, true);
     if (st != FUSE_OK) return st;
     GradWork* g = c->gw;
     if (iters > 0) {
@@ -471,7 +471,6 @@ fuse_status grad_forward_impl(fuse_ctx* c, const void* Yl, const void* Yh, int i
             return FUSE_OK;
         });
         if (st != FUSE_OK) return st;
-        c->entries_ok = false;                  // entries rounded to the iterate type, not on the grid
     }
     c->have_x = true;
     const size_t img = c->n * c->Ls * c->esz;

@@ -30,33 +30,22 @@
 // Layouts: X [L_s][H][W]; omega [|W|][H][W]; Sig' [|W| or |W|/2][|P|][L_s][H][W];
 // planes [L_s][2(2S+1)][H][W].  Threads: (W/VEC) x Ty, each owning VEC consecutive pixels.
 //
-// GRID (K = 1, 2, every pass but the taped forward's): the update on the grid of latent_grid.cuh,
-// where each entry and the sums over k are exact, so these kernels and the pass on the compact state
-// (k_levels.cuh) give the same bits; without it the entries are rounded to the iterate type.
+// GRID (K = 1, 2): the update on the grid of latent_grid.cuh, where each entry and the sums over k are
+// exact, so these kernels and the pass on the compact state (k_levels.cuh) give the same bits; without
+// it the entries are rounded to the iterate type.  Where a context's state can be levels or on the grid,
+// the kernels are launched with `ctl` and those that the state does not call for return at once.
 #pragma once
 #include "common.cuh"
 #include "latent_grid.cuh"
 
 namespace fuse {
 
-// The threshold of one weight column: in the iterate type, or as a code on the grid.
-template <typename T, bool GRID>
-struct latent_bound {
-    SymBound<T> b;
-    __device__ __forceinline__ static latent_bound of(T mu, T) { return {SymBound<T>::of(mu)}; }
-    __device__ __forceinline__ T clamp(T u) const { return b.clamp(u); }
-};
-template <typename T>
-struct latent_bound<T, true> {
-    code_t<T> m;
-    __device__ __forceinline__ static latent_bound of(T mu, T ig) { return {mu_code(mu, ig)}; }
-    __device__ __forceinline__ code_t<T> clamp(code_t<T> u) const { return u > m ? m : (u < -m ? -m : u); }
-};
-
 template <typename T, typename WT, int K, int VEC, bool GRID>
 __global__ void __launch_bounds__(256)
 latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Sig, T* Sout,
-              T* __restrict__ planes, int H, int W, int Ls, int S, int Ty, T coef, int half, const LatentGrid<T>* grid) {
+              T* __restrict__ planes, int H, int W, int Ls, int S, int Ty, T coef, int half, const LatentGrid<T>* grid,
+              const LatentCtl* ctl) {
+    if (!entries_due(ctl, GRID)) return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* Hs = reinterpret_cast<T*>(smem_raw);           // [(2S+1)][Ty][W]
     constexpr int PS = 2 * K + 1;
@@ -212,7 +201,8 @@ struct LatentArgs {
     // layout as `planes`) and one FP64 sum of (Sigma' - Sigma)^2 per block
     T* mplanes;
     double* mpart;
-    const LatentGrid<T>* grid;  // GRID only
+    const LatentGrid<T>* grid;  // monitoring instance only
+    const LatentCtl* ctl;       // see entries_due
 };
 
 __device__ __forceinline__ void consumer_barrier(int ncons) {
@@ -594,16 +584,18 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
 template <typename ST>
 constexpr int latent_max_regs() { return sizeof(ST) == 2 ? 96 : 112; }
 
-template <typename T, typename WT, int K, int VEC, typename ST = T, bool GRID = false>
+template <typename T, typename WT, int K, int VEC, typename ST = T>
 __global__ void __maxnreg__(latent_max_regs<ST>()) latent_tma_kernel(LatentArgs<T, WT> args) {
+    if (!entries_due(args.ctl, false)) return;
     extern __shared__ __align__(128) unsigned char smem_tma[];
-    latent_tma_body<T, WT, K, VEC, ST, GRID>(args, blockIdx.x, blockIdx.y, blockIdx.z, smem_tma);
+    latent_tma_body<T, WT, K, VEC, ST, false>(args, blockIdx.x, blockIdx.y, blockIdx.z, smem_tma);
 }
 
 // The monitoring instance (state in the iterate type): the same update, plus the latent parts of
 // the ADMM residuals (see latent_tma_body); needs (2S+1) Ty W more elements of shared memory.
 template <typename T, typename WT, int K, int VEC, bool GRID>
 __global__ void __launch_bounds__(288, 1) latent_tma_monitor_kernel(LatentArgs<T, WT> args) {
+    if (!entries_due(args.ctl, GRID)) return;
     extern __shared__ __align__(128) unsigned char smem_tma[];
     latent_tma_body<T, WT, K, VEC, T, GRID, true>(args, blockIdx.x, blockIdx.y, blockIdx.z, smem_tma);
 }
@@ -611,7 +603,7 @@ __global__ void __launch_bounds__(288, 1) latent_tma_monitor_kernel(LatentArgs<T
 // One launch over many problems (batched uneven sizes): blocks are mapped to (problem, block)
 // by the segment table; every problem's launch shape fits the common block size and shared
 // memory size of the launch.  zero_in applies to every problem (see LatentArgs).
-template <typename T, typename WT, int K, int VEC, typename ST = T, bool GRID = false>
+template <typename T, typename WT, int K, int VEC, typename ST = T>
 __global__ void __maxnreg__(latent_max_regs<ST>())
 latent_tma_batch_kernel(const LatentArgs<T, WT>* __restrict__ args, const Segment* __restrict__ seg, int nseg,
                         int zero_in) {
@@ -619,8 +611,9 @@ latent_tma_batch_kernel(const LatentArgs<T, WT>* __restrict__ args, const Segmen
     int prob, bx, by, bz;
     segment_of_block(seg, nseg, blockIdx.x, &prob, &bx, &by, &bz);
     LatentArgs<T, WT> a = args[prob];
+    if (!entries_due(a.ctl, false)) return;
     a.zero_in = zero_in;
-    latent_tma_body<T, WT, K, VEC, ST, GRID>(a, bx, by, bz, smem_tma);
+    latent_tma_body<T, WT, K, VEC, ST, false>(a, bx, by, bz, smem_tma);
 }
 
 }  // namespace fuse

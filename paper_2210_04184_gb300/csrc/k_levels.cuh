@@ -14,6 +14,9 @@
 // rare paths run with full warps, evenly spread.  Every H_tau of the block is kept in shared memory, and
 // A(m) = sum H_tau(m), V(m) = sum H_tau(m + (0, tau2)) are formed at the end in the order of tau2,
 // whatever the order of the lists.
+//
+// A state that is not kept as levels (LatentCtl) runs the entry kernels instead: an iteration launches
+// both, side by side in a captured loop, and the one whose turn it is not returns at once.
 #pragma once
 #include <type_traits>
 
@@ -35,7 +38,23 @@ struct LevelArgs {
     T coef;
     const LatentGrid<T>* grid;  // device
     int half;
+    LatentCtl* ctl;             // device
 };
+
+// Whether this is the last block of a launch to finish; true for all of its threads or none.  What the
+// other blocks wrote before is visible to it, and no block reads the state's mode after that.
+__device__ __forceinline__ bool last_block(LatentCtl* ctl) {
+    __shared__ int last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicAdd(&ctl->done, 1u) == gridDim.x * gridDim.y - 1;
+        if (last) ctl->done = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    return last;
+}
 
 template <typename C>
 __device__ __forceinline__ LevelRecord<C> load_record(const LevelRecord<C>* p) {
@@ -82,7 +101,8 @@ __device__ __forceinline__ void points_row(const T* __restrict__ X, LevelPoint<T
 template <typename T>
 __global__ void __launch_bounds__(256)
 points_kernel(const T* __restrict__ X, LevelPoint<T>* __restrict__ pt, int rows, int W, int S,
-              const LatentGrid<T>* grid, int first) {
+              const LatentGrid<T>* grid, int first, const LatentCtl* ctl) {
+    if (ctl->mode != kStateLevels) return;
     const int row = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (row < rows) points_row<T>(X, pt, W, S, grid, first, row, threadIdx.x & 31);
 }
@@ -130,53 +150,67 @@ __device__ __forceinline__ void window_codes(const WT* __restrict__ om, int y, i
     }
 }
 
-// Prefix sums of the sorted threshold codes of every window; grid (ceil(n / 128), kept offsets).
+// Prefix sums of the sorted threshold codes of every window, unless they are those of the current weights
+// already; `work` runs of 128 pixels of one kept offset, shared out over the blocks.
 template <typename T, typename WT, int K>
 __global__ void __launch_bounds__(128)
 level_table_kernel(const WT* __restrict__ omega, code_t<T>* __restrict__ tab, int H, int W, int S, int half, T coef,
-                   const LatentGrid<T>* grid) {
+                   const LatentGrid<T>* grid, int work, LatentCtl* ctl) {
     using C = code_t<T>;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     __shared__ C sm[128 * NP];                        // NP is odd: conflict-free
+    if (ctl->table) return;
     const size_t n = (size_t)H * W;
-    const size_t p0 = (size_t)blockIdx.x * 128, p = p0 + threadIdx.x;
-    const int si = blockIdx.y;
+    const int runs = (int)((n + 127) / 128);
     const TauMap tm{S, half};
-    int t1, t2;
-    tau_of_state_index(si, S, half, &t1, &t2);
-    if (p < n) {
-        const LatentGrid<T> gr = *grid;
-        C v[NP];
-        window_codes<T, WT, K>(omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / W), (int)(p % W), H, W, coef, gr.ig, v);
-        sort_network<NP>(v);
-        C sum = 0;
+    const LatentGrid<T> gr = *grid;
+    for (int job = blockIdx.x; job < work; job += gridDim.x) {
+        const int si = job / runs;
+        const size_t p0 = (size_t)(job - si * runs) * 128, p = p0 + threadIdx.x;
+        int t1, t2;
+        tau_of_state_index(si, S, half, &t1, &t2);
+        if (p < n) {
+            C v[NP];
+            window_codes<T, WT, K>(omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / W), (int)(p % W), H, W, coef, gr.ig,
+                                   v);
+            sort_network<NP>(v);
+            C sum = 0;
 #pragma unroll
-        for (int q = 0; q < NP; ++q) {
-            sum += v[q];
-            sm[threadIdx.x * NP + q] = sum;
+            for (int q = 0; q < NP; ++q) {
+                sum += v[q];
+                sm[threadIdx.x * NP + q] = sum;
+            }
         }
+        __syncthreads();
+        const int cnt = (int)(n - p0 < 128 ? n - p0 : 128) * NP;
+        C* out = tab + ((size_t)si * n + p0) * NP;
+        for (int i = threadIdx.x; i < cnt; i += 128) out[i] = sm[i];
+        __syncthreads();
     }
-    __syncthreads();
-    const int cnt = (int)(n - p0 < 128 ? n - p0 : 128) * NP;
-    C* out = tab + ((size_t)si * n + p0) * NP;
-    for (int i = threadIdx.x; i < cnt; i += 128) out[i] = sm[i];
+    if (last_block(ctl) && threadIdx.x == 0) ctl->table = 1;
 }
 
 // Steps (bands x offsets) of a block: one bit each in a thread's event mask, five in a list entry.
 constexpr int kLevelSteps = 32;
 constexpr int kLevelTile = 2048;                      // pixels of a block: eleven bits in a list entry
 
-// The zero state: no rank has reached its threshold, e = 0, and the first event is |w| reaching the
-// smallest threshold.  Grid (ceil(n / 128), kept offsets).
+// The zero state.  As levels: no rank has reached its threshold, e = 0, and the first event is |w|
+// reaching the smallest threshold.  Else zero entries, with `clear`.  Grid (ceil(n / 128), kept offsets).
 template <typename T, int K>
 __global__ void __launch_bounds__(128)
 levels_init_kernel(LevelRecord<ucode_t<T>>* __restrict__ rec, uint2* __restrict__ masks, ucode_t<T>* __restrict__ e,
-                   const code_t<T>* __restrict__ tab, size_t n, int Ls) {
+                   const code_t<T>* __restrict__ tab, size_t n, int Ls, int clear,
+                   const LatentCtl* ctl) {
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     using U = ucode_t<T>;
     const size_t p = (size_t)blockIdx.x * 128 + threadIdx.x;
     if (p >= n) return;
     const size_t si = blockIdx.y, kst = (size_t)Ls * n;
+    if (ctl->mode != kStateLevels) {
+        U* eb = e + si * NP * kst + p;
+        for (int i = 0; clear && i < NP * Ls; ++i) eb[(size_t)i * n] = 0;
+        return;
+    }
     LevelRecord<U> q{0, 0, 0, levels_meta<NP>(Levels{1u << (NP - 1), 0u, 0, true, true})};
     level_free_range<U>(q, 0, (U)tab[(si * n + p) * NP]);
     for (int c = 0; c < Ls; ++c) {
@@ -198,6 +232,7 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
                                                    unsigned char* smem_raw) {
     using U = ucode_t<T>;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    if (a.ctl->mode != kStateLevels) return;
     const int H = a.H, W = a.W, Ls = a.Ls, S = a.S;
     const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31;
     const TauMap tm{S, a.half};
@@ -363,9 +398,12 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
     }
 }
 
-// ---- the two forms of the state ---------------------------------------------------------------
-// Both conversions are exact and in place: the thread of a (tau, pixel) reads every word of one
-// (tau, c, m) before it writes any, and no other thread touches those words.
+// ---- the forms of the state -------------------------------------------------------------------
+// The conversions are exact and in place: the thread of a (tau, pixel) reads every word of one
+// (tau, c, m) before it writes any, and no other thread touches those words.  Each launch looks at the
+// state on the device and does nothing where that does not call for it; `work` runs of 128 pixels of
+// one kept offset are shared out over the blocks, a few per SM, so that such a launch costs a few
+// microseconds whatever the problem's size.
 
 // Threshold codes of a window, ascending, each with its patch index in the low 5 bits.
 template <typename T, typename WT, int K>
@@ -380,106 +418,169 @@ __device__ __forceinline__ void window_keys(const WT* __restrict__ om, int y, in
     sort_network<NP>(key);
 }
 
-// Levels -> entries s_k (in the iterate type).
-template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT> a) {
-    using C = code_t<T>;
-    using U = typename grid_code<T>::utype;
+// The pixels of a conversion: f(kept offset, pixel, tau, keys of its window).
+template <typename T, typename WT, int K, typename F>
+__device__ __forceinline__ void each_window(const LevelArgs<T, WT>& a, int work, F f) {
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     const size_t n = (size_t)a.H * a.W;
-    const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int si = blockIdx.y;
+    const int runs = (int)((n + 127) / 128);
     const TauMap tm{a.S, a.half};
-    int t1, t2;
-    tau_of_state_index(si, a.S, a.half, &t1, &t2);
-    const LatentGrid<T> gr = *a.grid;
-    U key[NP];
-    window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
-                          gr.ig, key);
-    const size_t kst = (size_t)a.Ls * n;
-    const size_t Wp = a.W + 2 * a.S, img = a.H * Wp, y = p / a.W, x = p % a.W;
-    const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
-    for (int c = 0; c < a.Ls; ++c) {
-        const size_t o = ((size_t)si * a.Ls + c) * n + p;
-        const Levels l = levels_of<NP>(load_record(a.rec + o).meta, NP == 9 ? make_uint2(0u, 0u) : a.masks[o]);
-        U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
-        const U w = a.pt[c * img + ps].after - a.pt[c * img + po].after;
-        C s[NP];
-        int height = bits_set(l.E);
-        C d = 0, sg = 0;
-#pragma unroll
-        for (int r = 0; r < NP; ++r) {
-            if (r == 0 || ((l.E >> (r == 0 ? 0 : r - 1)) & 1u)) {
-                --height;
-                const int end = r + lowest_bit(l.E >> r) - 1;
-                sg = l.free && height == 0 ? 0 : (((l.G >> end) & 1u) ? 1 : -1);
-                d = r == 0 && l.q > 0 ? C(0) : (C)(w - ob[(size_t)height * kst]);
-            }
-            s[r] = sg * (C)(key[r] >> 5) + d;
-        }
-        T* eb = reinterpret_cast<T*>(ob);
-#pragma unroll
-        for (int r = 0; r < NP; ++r) eb[(size_t)(key[r] & 31u) * kst] = (T)s[r] * gr.g;
+    const T ig = a.grid->ig;
+    for (int job = blockIdx.x; job < work; job += gridDim.x) {
+        const int si = job / runs;
+        const size_t p = (size_t)(job - si * runs) * 128 + threadIdx.x;
+        if (p >= n) continue;
+        int t1, t2;
+        tau_of_state_index(si, a.S, a.half, &t1, &t2);
+        ucode_t<T> key[NP];
+        window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
+                              ig, key);
+        f(si, p, t1, t2, key);
     }
 }
 
-// Entries -> levels.  check: nothing is written; *bad is set when some entry is off the grid or
-// the entries of some (tau, c, m) are not the state of a stop operator (|s| <= mu, 1-Lipschitz in
-// mu), which the level update needs.
+// Levels -> entries s_k (in the iterate type), where the coming calls want entries (want below
+// kStateLevels) or the weights have changed since the levels were formed (old: the arguments from
+// before).  The entries are then those of a run on the current weights, or to be looked at; with
+// want = kStateEntries they go on in the iterate type's arithmetic.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128) entries_to_levels_kernel(LevelArgs<T, WT> a, int check, int* bad) {
+__global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, int want) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
-    const size_t n = (size_t)a.H * a.W;
-    const size_t p = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const int si = blockIdx.y;
-    const TauMap tm{a.S, a.half};
-    int t1, t2;
-    tau_of_state_index(si, a.S, a.half, &t1, &t2);
-    const LatentGrid<T> gr = *a.grid;
-    U key[NP];
-    window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
-                          gr.ig, key);
-    const size_t kst = (size_t)a.Ls * n;
-    const size_t Wp = a.W + 2 * a.S, img = a.H * Wp, y = p / a.W, x = p % a.W;
-    const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
-    for (int c = 0; c < a.Ls; ++c) {
-        U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
-        const T* eb = reinterpret_cast<const T*>(ob);
-        C s[NP];
-        bool ok = true;
+    if (now.ctl->mode != kStateLevels || !(now.ctl->was || want < kStateLevels)) return;
+    const LevelArgs<T, WT> a = now.ctl->was ? old : now;
+    const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
+    const T g = a.grid->g;
+    each_window<T, WT, K>(a, work, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
+        const size_t y = p / a.W, x = p % a.W;
+        const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
+        for (int c = 0; c < a.Ls; ++c) {
+            const size_t o = ((size_t)si * a.Ls + c) * n + p;
+            const Levels l = levels_of<NP>(load_record(a.rec + o).meta, NP == 9 ? make_uint2(0u, 0u) : a.masks[o]);
+            U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
+            const U w = a.pt[c * img + ps].after - a.pt[c * img + po].after;
+            C s[NP];
+            int height = bits_set(l.E);
+            C d = 0, sg = 0;
 #pragma unroll
-        for (int r = 0; r < NP; ++r) {
-            const T v = eb[(size_t)(key[r] & 31u) * kst] * gr.ig;
-            const T lim = (T)(key[r] >> 5);
-            ok = ok && v >= -lim && v <= lim && v == trunc(v);
-            s[r] = to_code(v);
+            for (int r = 0; r < NP; ++r) {
+                if (r == 0 || ((l.E >> (r == 0 ? 0 : r - 1)) & 1u)) {
+                    --height;
+                    const int end = r + lowest_bit(l.E >> r) - 1;
+                    sg = l.free && height == 0 ? 0 : (((l.G >> end) & 1u) ? 1 : -1);
+                    d = r == 0 && l.q > 0 ? C(0) : (C)(w - ob[(size_t)height * kst]);
+                }
+                s[r] = sg * (C)(key[r] >> 5) + d;
+            }
+            T* eb = reinterpret_cast<T*>(ob);
+#pragma unroll
+            for (int r = 0; r < NP; ++r) eb[(size_t)(key[r] & 31u) * kst] = (T)s[r] * g;
         }
-        if (check) {
+    });
+    if (last_block(now.ctl) && threadIdx.x == 0) {
+        now.ctl->mode = want == kStateEntries ? kStateEntries : now.ctl->was ? kStateGiven : kStateGrid;
+        now.ctl->was = 0;
+    }
+}
+
+// The codes of the NP entries at ob, in the order of the keys; false if one is off the grid or above its
+// threshold.
+template <typename T, int NP>
+__device__ __forceinline__ bool entry_codes(const T* eb, size_t kst, T ig, const ucode_t<T> (&key)[NP], code_t<T> (&s)[NP]) {
+    bool ok = true;
+#pragma unroll
+    for (int r = 0; r < NP; ++r) {
+        const T v = eb[(size_t)(key[r] & 31u) * kst] * ig, lim = (T)(key[r] >> 5);
+        ok = ok && v >= -lim && v <= lim && v == trunc(v);
+        s[r] = to_code(v);
+    }
+    return ok;
+}
+
+// Whether given entries are those of a run on the current weights, which the update on the grid and the
+// levels need: on the grid, |s| <= mu, and 1-Lipschitz in mu, the state of a stop operator.
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128) entries_check_kernel(LevelArgs<T, WT> a, int work) {
+    using C = code_t<T>;
+    using U = typename grid_code<T>::utype;
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    if (a.ctl->mode != kStateGiven) return;
+    const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n;
+    const T ig = a.grid->ig;
+    volatile int* off = &a.ctl->off;
+    each_window<T, WT, K>(a, work, [&](int si, size_t p, int, int, const U (&key)[NP]) {
+        for (int c = 0; c < a.Ls && !*off; ++c) {
+            C s[NP];
+            bool ok = entry_codes<T, NP>(reinterpret_cast<const T*>(a.e + (size_t)si * NP * kst + (size_t)c * n + p), kst, ig,
+                                         key, s);
 #pragma unroll
             for (int r = 1; r < NP; ++r) {
                 const C dm = (C)(key[r] >> 5) - (C)(key[r - 1] >> 5), ds = s[r] - s[r - 1];
                 ok = ok && ds <= dm && -ds <= dm;
             }
-            if (!ok) atomicOr(bad, 1);
-            continue;
+            if (!ok) *off = 1;
         }
-        U su[NP], mu[NP];
+    });
+    if (last_block(a.ctl) && threadIdx.x == 0) {
+        a.ctl->mode = *off ? kStateEntries : kStateGrid;
+        *off = 0;
+    }
+}
+
+// Entries of a run on the current weights -> levels.
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128) entries_to_levels_kernel(LevelArgs<T, WT> a, int work) {
+    using C = code_t<T>;
+    using U = typename grid_code<T>::utype;
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    if (a.ctl->mode != kStateGrid) return;
+    const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
+    const T ig = a.grid->ig;
+    each_window<T, WT, K>(a, work, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
+        const size_t y = p / a.W, x = p % a.W;
+        const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
+        for (int c = 0; c < a.Ls; ++c) {
+            U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
+            C s[NP];
+            entry_codes<T, NP>(reinterpret_cast<const T*>(ob), kst, ig, key, s);
+            U su[NP], mu[NP];
 #pragma unroll
-        for (int r = 0; r < NP; ++r) {
-            su[r] = (U)s[r];
-            mu[r] = key[r] >> 5;
+            for (int r = 0; r < NP; ++r) {
+                su[r] = (U)s[r];
+                mu[r] = key[r] >> 5;
+            }
+            const U w = a.pt[c * img + ps].after - a.pt[c * img + po].after;
+            Levels l;
+            LevelRecord<U> q;
+            levels_from_entries<NP, U>(su, mu, w, l, q, [&](int pl, U e) { ob[(size_t)pl * kst] = e; });
+            const size_t o = ((size_t)si * a.Ls + c) * n + p;
+            store_record(a.rec + o, q);
+            if constexpr (NP != 9) a.masks[o] = make_uint2(l.E, l.G);
         }
-        const U w = a.pt[c * img + ps].after - a.pt[c * img + po].after;
-        Levels l;
-        LevelRecord<U> q;
-        levels_from_entries<NP, U>(su, mu, w, l, q, [&](int pl, U e) { ob[(size_t)pl * kst] = e; });
-        const size_t o = ((size_t)si * a.Ls + c) * n + p;
-        store_record(a.rec + o, q);
-        if constexpr (NP != 9) a.masks[o] = make_uint2(l.E, l.G);
+    });
+    if (last_block(a.ctl) && threadIdx.x == 0) a.ctl->mode = kStateLevels;
+}
+
+// Before the weights change (words: those of the weights, 16 bytes each): levels stay readable through
+// the weights and the grid that they were formed with, kept in `was`; entries have to be looked at again.  The grid is then
+// that for weights up to 1, which fuse_weights gives; given weights set their own.
+template <typename T>
+__global__ void __launch_bounds__(256)
+weights_change_kernel(const uint4* __restrict__ omega, uint4* __restrict__ was, size_t words, LatentGrid<T>* grid,
+                      LatentCtl* ctl) {
+    const bool keep = ctl->mode == kStateLevels && !ctl->was;
+    if (keep)
+        for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (size_t)gridDim.x * blockDim.x)
+            was[i] = omega[i];
+    if (last_block(ctl) && threadIdx.x == 0) {
+        if (keep) {
+            grid[1] = grid[0];
+            ctl->was = 1;
+        }
+        if (ctl->mode == kStateGrid) ctl->mode = kStateGiven;
+        ctl->table = 0;
+        grid[0] = grid[2];
     }
 }
 
@@ -517,7 +618,7 @@ points_batch_kernel(const LevelArgs<T, WT>* __restrict__ args, const Segment* __
     segment_of_block(seg, nseg, blockIdx.x, &prob, &bx, &by, &bz);
     const LevelArgs<T, WT>& a = args[prob];
     const int row = bx * 8 + (threadIdx.x >> 5);
-    if (row < a.H * a.Ls)
+    if (row < a.H * a.Ls && a.ctl->mode == kStateLevels)
         points_row<T>(a.X, const_cast<LevelPoint<T>*>(a.pt), a.W, a.S, a.grid, first, row, threadIdx.x & 31);
 }
 

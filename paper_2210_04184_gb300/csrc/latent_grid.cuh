@@ -64,6 +64,29 @@ template <typename T> struct LatentGrid {
     T wmax;                     // the largest weight it was made for
 };
 
+// What the latent state of a context holds, kept on the device: the calls that change it and the
+// kernels that depend on it are ordered by the stream, and a captured call that is replayed later finds
+// the state as it is then.
+//   kStateEntries  entries of the iterate type, updated in its arithmetic
+//   kStateGrid     entries on the grid, those of a run on the current weights
+//   kStateLevels   levels, formed with the current weights or, with `was`, with the ones before them
+//   kStateGiven    entries not looked at yet: set by the caller, or left by other weights
+enum : int { kStateEntries = 0, kStateGrid = 1, kStateLevels = 2, kStateGiven = 3 };
+struct LatentCtl {
+    int mode;
+    int was;                    // omega_was and grid[1] describe the levels
+    int table;                  // the threshold table is that of the current weights
+    int off;                    // some entry is not that of a run on the current weights
+    unsigned done;              // blocks of the running kernel that have finished
+};
+// Whether an entry kernel is to run: ctl NULL, always; else where the state is entries, on the grid or not
+// as the kernel's arithmetic.
+__device__ __forceinline__ bool entries_due(const LatentCtl* ctl, bool grid) {
+    if (!ctl) return true;
+    const int mode = ctl->mode;
+    return grid ? mode == kStateGrid : mode == kStateEntries || mode == kStateGiven;
+}
+
 // The grid of thresholds coef w, 0 <= w <= wmax: 2^e >= coef wmax, g = 2^(e - B).
 inline __host__ __device__ LatentGrid<float> latent_grid(float coef, float wmax) {
     int e = 0;
@@ -91,6 +114,20 @@ __device__ __forceinline__ int64_t mu_code(double mu, double ig) {
     const double c = fabs(mu) * ig;
     return __double2ll_rn(c <= cap ? c : cap);
 }
+// The threshold of one weight column: in the iterate type, or as a code on the grid.
+template <typename T, bool GRID>
+struct latent_bound {
+    SymBound<T> b;
+    __device__ __forceinline__ static latent_bound of(T mu, T) { return {SymBound<T>::of(mu)}; }
+    __device__ __forceinline__ T clamp(T u) const { return b.clamp(u); }
+};
+template <typename T>
+struct latent_bound<T, true> {
+    code_t<T> m;
+    __device__ __forceinline__ static latent_bound of(T mu, T ig) { return {mu_code(mu, ig)}; }
+    __device__ __forceinline__ code_t<T> clamp(code_t<T> u) const { return u > m ? m : (u < -m ? -m : u); }
+};
+
 // Code of an X value: rounded to nearest, modulo 2^32 (FP64: 2^64).  Differences of codes are taken
 // modulo as well; they are used only where |delta| < kBigMove g.
 __device__ __forceinline__ int32_t x_code(float x, float ig) {

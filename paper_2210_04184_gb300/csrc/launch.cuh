@@ -20,22 +20,23 @@ namespace fuse {
 
 // ---- latent pass (k_latent.cuh) ----
 // Bulk-copy latent pass of one problem; K = patch half-size; int16_state: 16-bit fixed-point
-// state (T = float only); on_grid: the arithmetic of latent_grid.cuh (K = 1, 2; ignored otherwise).
+// state (T = float only).
 template <typename T, typename WT>
-void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, bool on_grid, dim3 grid,
-                       unsigned threads, size_t smem, cudaStream_t s);
+void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, dim3 grid, unsigned threads,
+                       size_t smem, cudaStream_t s);
 // Batched bulk-copy latent pass over the segment table.
 template <typename T, typename WT>
 void latent_tma_batch_launch(const LatentArgs<T, WT>* args, const Segment* seg, int nseg, int zero_in, int K,
-                             bool int16_state, bool on_grid, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s);
-// Register-staged latent pass.
+                             bool int16_state, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s);
+// Register-staged latent pass; ctl: run where the state is entries, with `on_grid` also those on the
+// grid (NULL: run, in the iterate type's arithmetic).
 template <typename T, typename WT>
 void latent_reg_launch(const T* X, const WT* omega, const T* Sig, T* Sout, T* planes, int H, int W, int Ls, int S,
-                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, int K, bool on_grid, dim3 grid, unsigned threads,
-                       size_t smem, cudaStream_t s);
-// Monitoring latent pass (state in the iterate type): also the latent parts of the residuals.
+                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, const LatentCtl* ctl, bool on_grid,
+                       int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s);
+// Monitoring latent pass (state as entries of the iterate type): also the latent parts of the residuals.
 template <typename T, typename WT>
-void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, bool on_grid, dim3 grid, unsigned threads, size_t smem,
+void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, dim3 grid, unsigned threads, size_t smem,
                            cudaStream_t s);
 // Dynamic shared-memory cap of the single-problem and batched latent kernels for patch size K.
 template <typename T, typename WT>
@@ -46,9 +47,10 @@ cudaError_t latent_batch_set_smem(int K, int bytes);
 // ---- latent pass on the compact state (k_levels.cuh; K = 1, 2) ----
 template <typename T, typename WT>
 void levels_launch(const LevelArgs<T, WT>& a, int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s);
-// The zero state of `kept` offsets (in place of the pass of an iteration whose X is zero).
+// The zero state of `kept` offsets (in place of the pass of an iteration whose X is zero); clear: also
+// where it is entries.
 template <typename T, typename WT>
-void levels_init_launch(const LevelArgs<T, WT>& a, int K, int kept, cudaStream_t s);
+void levels_init_launch(const LevelArgs<T, WT>& a, int K, int kept, int clear, cudaStream_t s);
 // Batched form over a segment table.
 template <typename T, typename WT>
 void levels_batch_launch(const LevelArgs<T, WT>* args, const Segment* seg, int nseg, int K, unsigned blocks,
@@ -59,15 +61,23 @@ void points_batch_launch(const LevelArgs<T, WT>* args, const Segment* seg, int n
 // The points of the current X (one launch per iteration, before the latent pass).
 template <typename T, typename WT>
 void points_launch(const LevelArgs<T, WT>& a, int first, cudaStream_t s);
-// The sorted threshold codes of the current weights, as prefix sums.
+// Conversions between the forms of the state, and the table of sorted thresholds, of `kept` offsets: each
+// looks on the device at whether it has to run (k_levels.cuh); nsm: SMs of the device.
 template <typename T, typename WT>
-void level_table_launch(const WT* omega, code_t<T>* tab, int H, int W, int K, int S, int half, int kept, T coef,
-                        const LatentGrid<T>* grid, cudaStream_t s);
-// In-place conversion of the state of `kept` offsets (to_levels: entries to levels, check only
-// validates and sets *bad; else levels to entries).
+void levels_to_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, int K, int kept, int nsm, int want,
+                              cudaStream_t s);
 template <typename T, typename WT>
-void levels_convert_launch(const LevelArgs<T, WT>& a, int K, int kept, int to_levels, int check, int* bad,
+void entries_check_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s);
+template <typename T, typename WT>
+void entries_to_levels_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s);
+template <typename T, typename WT>
+void level_table_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s);
+// Before the weights change (bytes of them at omega; was: where those of levels are kept, or NULL).
+template <typename T>
+void weights_change_launch(const void* omega, void* was, size_t bytes, LatentGrid<T>* grid, LatentCtl* ctl, int nsm,
                            cudaStream_t s);
+// The state that a solve starts with: from zero as `want` (kState...), or a continued one.
+void latent_begin_launch(LatentCtl* ctl, int cold, int want, cudaStream_t s);
 // The grid of n weights from the largest finite one (grid zeroed by the caller); two launches.
 template <typename T, typename WT>
 void wmax_launch(const WT* w, size_t n, LatentGrid<T>* grid, T coef, cudaStream_t s);
@@ -134,27 +144,28 @@ cudaError_t latent_bwd_set_smem(int K, int bytes);
 
 #define FUSE_LAUNCH_EXTERN_T_WT(T, WT)                                                                      \
     extern template void levels_launch<T, WT>(const LevelArgs<T, WT>&, int, dim3, unsigned, size_t, cudaStream_t); \
-    extern template void levels_init_launch<T, WT>(const LevelArgs<T, WT>&, int, int, cudaStream_t);          \
+    extern template void levels_init_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);     \
     extern template void levels_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int,         \
                                                     unsigned, unsigned, size_t, cudaStream_t);                \
     extern template void points_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int,        \
                                                     unsigned, cudaStream_t);                                  \
     extern template void points_launch<T, WT>(const LevelArgs<T, WT>&, int, cudaStream_t);                    \
-    extern template void levels_convert_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, int, int*,        \
-                                                      cudaStream_t);                                           \
-    extern template void level_table_launch<T, WT>(const WT*, code_t<T>*, int, int, int, int, int, int, T,      \
-                                                   const LatentGrid<T>*, cudaStream_t);                       \
+    extern template void levels_to_entries_launch<T, WT>(const LevelArgs<T, WT>&, const LevelArgs<T, WT>&, int, \
+                                                         int, int, int, cudaStream_t);                        \
+    extern template void entries_check_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);    \
+    extern template void entries_to_levels_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t); \
+    extern template void level_table_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);      \
     extern template void wmax_launch<T, WT>(const WT*, size_t, LatentGrid<T>*, T, cudaStream_t);                             \
     extern template cudaError_t levels_set_smem<T, WT>(int, int);                                             \
-    extern template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, bool, dim3, unsigned,     \
-                                                  size_t, cudaStream_t);                                       \
-    extern template void latent_tma_batch_launch<T, WT>(const LatentArgs<T, WT>*, const Segment*, int, int, int, \
-                                                        bool, bool, unsigned, unsigned, size_t, cudaStream_t); \
-    extern template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, \
-                                                  T, int, const LatentGrid<T>*, int, bool, dim3, unsigned, size_t,         \
+    extern template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned, size_t,    \
                                                   cudaStream_t);                                               \
-    extern template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned,      \
-                                                      size_t, cudaStream_t);                                           \
+    extern template void latent_tma_batch_launch<T, WT>(const LatentArgs<T, WT>*, const Segment*, int, int, int, \
+                                                        bool, unsigned, unsigned, size_t, cudaStream_t);       \
+    extern template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, \
+                                                  T, int, const LatentGrid<T>*, const LatentCtl*, bool, int, dim3, unsigned, \
+                                                  size_t, cudaStream_t);                                       \
+    extern template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, dim3, unsigned, size_t,    \
+                                                      cudaStream_t);                                           \
     extern template cudaError_t latent_set_smem<T, WT>(int, int);                                             \
     extern template cudaError_t latent_batch_set_smem<T, WT>(int, int);                                       \
     extern template void latent_bwd_tma_launch<T, WT>(const LatentBwdArgs<T, WT>&, int, dim3, unsigned, size_t, \

@@ -8,8 +8,8 @@
 namespace fuse {
 
 template <typename T, typename WT>
-void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, bool on_grid, dim3 grid,
-                       unsigned threads, size_t smem, cudaStream_t s) {
+void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, dim3 grid, unsigned threads,
+                       size_t smem, cudaStream_t s) {
     constexpr int TVEC = 32 / sizeof(T);
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
@@ -19,19 +19,13 @@ void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, bool
                 return;
             }
         }
-        if constexpr (latent_grid_k(KK)) {
-            if (on_grid) {
-                latent_tma_kernel<T, WT, KK, TVEC, T, true><<<grid, threads, smem, s>>>(a);
-                return;
-            }
-        }
         latent_tma_kernel<T, WT, KK, TVEC><<<grid, threads, smem, s>>>(a);
     });
 }
 
 template <typename T, typename WT>
 void latent_tma_batch_launch(const LatentArgs<T, WT>* args, const Segment* seg, int nseg, int zero_in, int K,
-                             bool int16_state, bool on_grid, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s) {
+                             bool int16_state, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s) {
     constexpr int TVEC = 32 / sizeof(T);
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
@@ -41,27 +35,18 @@ void latent_tma_batch_launch(const LatentArgs<T, WT>* args, const Segment* seg, 
                 return;
             }
         }
-        if constexpr (latent_grid_k(KK)) {
-            if (on_grid) {
-                latent_tma_batch_kernel<T, WT, KK, TVEC, T, true><<<blocks, threads, smem, s>>>(args, seg, nseg, zero_in);
-                return;
-            }
-        }
         latent_tma_batch_kernel<T, WT, KK, TVEC><<<blocks, threads, smem, s>>>(args, seg, nseg, zero_in);
     });
 }
 
 template <typename T, typename WT>
-void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, bool on_grid, dim3 grid, unsigned threads, size_t smem,
+void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, dim3 grid, unsigned threads, size_t smem,
                            cudaStream_t s) {
     constexpr int TVEC = 32 / sizeof(T);
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
         if constexpr (latent_grid_k(KK)) {
-            if (on_grid) {
-                latent_tma_monitor_kernel<T, WT, KK, TVEC, true><<<grid, threads, smem, s>>>(a);
-                return;
-            }
+            if (a.ctl) latent_tma_monitor_kernel<T, WT, KK, TVEC, true><<<grid, threads, smem, s>>>(a);
         }
         latent_tma_monitor_kernel<T, WT, KK, TVEC, false><<<grid, threads, smem, s>>>(a);
     });
@@ -69,20 +54,18 @@ void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, bool on_grid, dim3
 
 template <typename T, typename WT>
 void latent_reg_launch(const T* X, const WT* omega, const T* Sig, T* Sout, T* planes, int H, int W, int Ls, int S,
-                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, int K, bool on_grid, dim3 grid, unsigned threads,
-                       size_t smem, cudaStream_t s) {
+                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, const LatentCtl* ctl, bool on_grid,
+                       int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s) {
     constexpr int VEC = 16 / sizeof(T);
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
         if constexpr (latent_grid_k(KK)) {
-            if (on_grid) {
+            if (on_grid)
                 latent_kernel<T, WT, KK, VEC, true><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W, Ls,
-                                                                                S, Ty, coef, half, grid_d);
-                return;
-            }
+                                                                                S, Ty, coef, half, grid_d, ctl);
         }
         latent_kernel<T, WT, KK, VEC, false><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W, Ls, S, Ty,
-                                                                         coef, half, grid_d);
+                                                                         coef, half, grid_d, ctl);
     });
 }
 
@@ -97,7 +80,6 @@ cudaError_t latent_set_smem(int K, int bytes) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_kernel<T, WT, KK, TVEC>, A, bytes);
         if constexpr (latent_grid_k(KK)) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_kernel<T, WT, KK, VEC, true>, A, bytes);
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_kernel<T, WT, KK, TVEC, T, true>, A, bytes);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_monitor_kernel<T, WT, KK, TVEC, true>, A, bytes);
         }
         if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_monitor_kernel<T, WT, KK, TVEC, false>, A, bytes);
@@ -116,9 +98,6 @@ cudaError_t latent_batch_set_smem(int K, int bytes) {
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
         e = cudaFuncSetAttribute(latent_tma_batch_kernel<T, WT, KK, TVEC>, A, bytes);
-        if constexpr (latent_grid_k(KK)) {
-            if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_batch_kernel<T, WT, KK, TVEC, T, true>, A, bytes);
-        }
         if constexpr (sizeof(T) == 4) {
             if (e == cudaSuccess) e = cudaFuncSetAttribute(latent_tma_batch_kernel<T, WT, KK, TVEC, int16_t>, A, bytes);
         }
@@ -127,14 +106,15 @@ cudaError_t latent_batch_set_smem(int K, int bytes) {
 }
 
 #define FUSE_LATENT_INST(T, WT)                                                                               \
-    template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, bool, dim3, unsigned, size_t,    \
+    template void latent_tma_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned, size_t,          \
                                            cudaStream_t);                                                      \
     template void latent_tma_batch_launch<T, WT>(const LatentArgs<T, WT>*, const Segment*, int, int, int, bool,  \
-                                                 bool, unsigned, unsigned, size_t, cudaStream_t);                    \
-    template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, bool, dim3, unsigned, size_t,      \
+                                                 unsigned, unsigned, size_t, cudaStream_t);                    \
+    template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, dim3, unsigned, size_t,            \
                                                cudaStream_t);                                                  \
     template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, T,    \
-                                           int, const LatentGrid<T>*, int, bool, dim3, unsigned, size_t, cudaStream_t);    \
+                                           int, const LatentGrid<T>*, const LatentCtl*, bool, int, dim3, unsigned,       \
+                                           size_t, cudaStream_t);                                              \
     template cudaError_t latent_set_smem<T, WT>(int, int);                                                      \
     template cudaError_t latent_batch_set_smem<T, WT>(int, int);
 

@@ -17,11 +17,12 @@ void levels_launch(const LevelArgs<T, WT>& a, int K, dim3 grid, unsigned threads
 }
 
 template <typename T, typename WT>
-void levels_init_launch(const LevelArgs<T, WT>& a, int K, int kept, cudaStream_t s) {
+void levels_init_launch(const LevelArgs<T, WT>& a, int K, int kept, int clear, cudaStream_t s) {
     const size_t n = (size_t)a.H * a.W;
     const dim3 grid((unsigned)((n + 127) / 128), (unsigned)kept);
     with_grid_k(K, [&](auto k) {
-        levels_init_kernel<T, decltype(k)::value><<<grid, 128, 0, s>>>(a.rec, a.masks, a.e, a.tab, n, a.Ls);
+        levels_init_kernel<T, decltype(k)::value><<<grid, 128, 0, s>>>(a.rec, a.masks, a.e, a.tab, n, a.Ls, clear,
+                                                                        a.ctl);
     });
 }
 
@@ -43,27 +44,70 @@ template <typename T, typename WT>
 void points_launch(const LevelArgs<T, WT>& a, int first, cudaStream_t s) {
     const int rows = a.H * a.Ls;
     points_kernel<T><<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(a.X, const_cast<LevelPoint<T>*>(a.pt), rows, a.W, a.S,
-                                                               a.grid, first);
+                                                               a.grid, first, a.ctl);
+}
+
+// Runs of 128 pixels over the kept offsets, and blocks of a launch over them: as many as fit a device at
+// once (16 of 128 threads per SM), so that a launch that finds nothing to do ends in microseconds.
+template <typename T, typename WT>
+static int window_runs(const LevelArgs<T, WT>& a, int kept) {
+    return kept * (int)(((size_t)a.H * a.W + 127) / 128);
+}
+static unsigned window_blocks(int runs, int nsm) { return (unsigned)(runs < 16 * nsm ? runs : 16 * nsm); }
+
+template <typename T, typename WT>
+void levels_to_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, int K, int kept, int nsm, int want,
+                              cudaStream_t s) {
+    const int runs = window_runs(now, kept);
+    with_grid_k(K, [&](auto k) {
+        levels_to_entries_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(now, old, runs, want);
+    });
 }
 
 template <typename T, typename WT>
-void levels_convert_launch(const LevelArgs<T, WT>& a, int K, int kept, int to_levels, int check, int* bad,
+void entries_check_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
+    const int runs = window_runs(a, kept);
+    with_grid_k(K, [&](auto k) {
+        entries_check_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(a, runs);
+    });
+}
+
+template <typename T, typename WT>
+void entries_to_levels_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
+    const int runs = window_runs(a, kept);
+    with_grid_k(K, [&](auto k) {
+        entries_to_levels_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(a, runs);
+    });
+}
+
+template <typename T, typename WT>
+void level_table_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
+    const int runs = window_runs(a, kept);
+    with_grid_k(K, [&](auto k) {
+        level_table_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(
+            a.omega, const_cast<code_t<T>*>(a.tab), a.H, a.W, a.S, a.half, a.coef, a.grid, runs, a.ctl);
+    });
+}
+
+template <typename T>
+void weights_change_launch(const void* omega, void* was, size_t bytes, LatentGrid<T>* grid, LatentCtl* ctl, int nsm,
                            cudaStream_t s) {
-    const dim3 grid((unsigned)(((size_t)a.H * a.W + 127) / 128), (unsigned)kept);
-    with_grid_k(K, [&](auto k) {
-        constexpr int KK = decltype(k)::value;
-        if (to_levels) entries_to_levels_kernel<T, WT, KK><<<grid, 128, 0, s>>>(a, check, bad);
-        else levels_to_entries_kernel<T, WT, KK><<<grid, 128, 0, s>>>(a);
-    });
+    const size_t words = was ? bytes / 16 : 0, need = (words + 1023) / 1024;
+    const unsigned blocks = (unsigned)(need < 1 ? 1 : need < (size_t)4 * nsm ? need : (size_t)4 * nsm);
+    weights_change_kernel<T><<<blocks, 256, 0, s>>>((const uint4*)omega, (uint4*)was, words, grid, ctl);
 }
 
-template <typename T, typename WT>
-void level_table_launch(const WT* omega, code_t<T>* tab, int H, int W, int K, int S, int half, int kept, T coef,
-                        const LatentGrid<T>* grid, cudaStream_t s) {
-    const dim3 blocks((unsigned)(((size_t)H * W + 127) / 128), (unsigned)kept);
-    with_grid_k(K, [&](auto k) {
-        level_table_kernel<T, WT, decltype(k)::value><<<blocks, 128, 0, s>>>(omega, tab, H, W, S, half, coef, grid);
-    });
+// The state that a solve starts with.
+static __global__ void latent_begin_kernel(LatentCtl* ctl, int cold, int want) {
+    if (cold) {
+        ctl->mode = want;
+        ctl->was = 0;
+    } else if (want == kStateEntries && ctl->mode != kStateLevels) {
+        ctl->mode = kStateEntries;
+    }
+}
+void latent_begin_launch(LatentCtl* ctl, int cold, int want, cudaStream_t s) {
+    latent_begin_kernel<<<1, 1, 0, s>>>(ctl, cold, want);
 }
 
 template <typename T, typename WT>
@@ -94,18 +138,22 @@ cudaError_t levels_set_smem(int K, int bytes) {
     template void levels_launch<T, WT>(const LevelArgs<T, WT>&, int, dim3, unsigned, size_t, cudaStream_t);      \
     template void levels_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int, unsigned,        \
                                              unsigned, size_t, cudaStream_t);                                  \
-    template void levels_init_launch<T, WT>(const LevelArgs<T, WT>&, int, int, cudaStream_t);                   \
+    template void levels_init_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);              \
     template void points_batch_launch<T, WT>(const LevelArgs<T, WT>*, const Segment*, int, int, unsigned,        \
                                              cudaStream_t);                                                    \
     template void points_launch<T, WT>(const LevelArgs<T, WT>&, int, cudaStream_t);                             \
-    template void levels_convert_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, int, int*, cudaStream_t); \
-    template void level_table_launch<T, WT>(const WT*, code_t<T>*, int, int, int, int, int, int, T,              \
-                                            const LatentGrid<T>*, cudaStream_t);                               \
+    template void levels_to_entries_launch<T, WT>(const LevelArgs<T, WT>&, const LevelArgs<T, WT>&, int, int, int, \
+                                                  int, cudaStream_t);                                          \
+    template void entries_check_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);            \
+    template void entries_to_levels_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);        \
+    template void level_table_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);              \
     template void wmax_launch<T, WT>(const WT*, size_t, LatentGrid<T>*, T, cudaStream_t);                                       \
     template cudaError_t levels_set_smem<T, WT>(int, int);
 
 FUSE_LEVELS_INST(float, float)
 FUSE_LEVELS_INST(float, __nv_bfloat16)
 FUSE_LEVELS_INST(double, double)
+template void weights_change_launch<float>(const void*, void*, size_t, LatentGrid<float>*, LatentCtl*, int, cudaStream_t);
+template void weights_change_launch<double>(const void*, void*, size_t, LatentGrid<double>*, LatentCtl*, int, cudaStream_t);
 
 }  // namespace fuse

@@ -3,6 +3,7 @@ after changes of weights, states and data.  References are the same calls with e
 (FUSE_OPT_LATENT_IMPL = 0), bit for bit, and the FP64 oracle."""
 import math
 
+import numpy as np
 import pytest
 
 from paper_2210_04184_gb300 import synth
@@ -10,8 +11,10 @@ from paper_2210_04184_gb300 import synth
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
+from oracle import nlpr  # noqa: E402
 from paper_2210_04184_gb300 import build as _build  # noqa: E402
-from paper_2210_04184_gb300.fuse import Fusion, FUSE_OPT_LATENT_IMPL, FUSE_OPT_RESIDUALS  # noqa: E402
+from paper_2210_04184_gb300.fuse import (Fusion, FUSE_OPT_GRAPH, FUSE_OPT_LATENT_IMPL,  # noqa: E402
+                                         FUSE_OPT_RESIDUALS)
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -79,3 +82,136 @@ def test_thresholds_are_rounded_to_nearest(K):
     assert at.double().mean() > 0.9
     assert (off[at] <= g / 2 * (1 + 1e-9)).all()
     f.close()
+
+
+def oracle_runs(p, steps):
+    """X of the FP64 oracle after each (weights, iterations) of `steps`, continued from one to the next."""
+    st, out = None, []
+    for om, iters in steps:
+        X, st, _ = nlpr.admm(nlpr.to_hwl(p.Yl), nlpr.to_hwl(p.Yh), p.blur, p.d, p.R, p.E, p.K, p.S, p.lam1, p.lam2,
+                             p.rho, om, iters, state=st, fast=True)
+        out.append(nlpr.to_lhw(X))
+    return out
+
+
+def rel(a, b):
+    a = a.double().cpu().numpy()
+    return np.linalg.norm(a - b) / np.linalg.norm(b)
+
+
+# FP32 iterates against the FP64 oracle: the bound of the parity tests
+FP32_BOUND = 1e-5
+
+
+@pytest.mark.parametrize("K", [1, 2])
+@pytest.mark.parametrize("scale", [1.0, 1 / 8, 1 / 64, 1 / 4096, 8.0, 64.0])
+@pytest.mark.parametrize("impl", [1, 0])
+def test_weights_scaled_under_a_state(K, scale, impl):
+    # the entering entries reach far beyond the new thresholds, or not near them
+    p = small(K=K)
+    om = nlpr.weights(nlpr.to_hwl(p.Yh), p.K, p.S, p.h).astype(np.float32).astype(np.float64)
+    f = Fusion.from_problem(p, dtype="f32", wdtype="f32")
+    f.set_option(FUSE_OPT_LATENT_IMPL, impl)
+    yl, yh = dev(p.Yl), dev(p.Yh)
+    steps = [(om, 8), (om * scale, 1), (om * scale, 5), (om, 4)]
+    ref = oracle_runs(p, steps)
+    for i, (w, iters) in enumerate(steps):
+        f.set_weights(dev(w))
+        X, _ = f.solve(yl, yh, iters, warm=i > 0)
+        assert rel(X, ref[i]) <= FP32_BOUND
+    f.close()
+
+
+@pytest.mark.parametrize("K", [1, 2])
+@pytest.mark.parametrize("factor", [1 / 64, 64.0])
+def test_state_of_another_lambda2(K, factor):
+    # parameter continuation: the state of a run with lambda2 starts one with lambda2 times the factor
+    p = small(K=K)
+    q = small(K=K, lam2=p.lam2 * factor)
+    om = nlpr.weights(nlpr.to_hwl(p.Yh), p.K, p.S, p.h)
+    _, st, _ = nlpr.admm(nlpr.to_hwl(p.Yl), nlpr.to_hwl(p.Yh), p.blur, p.d, p.R, p.E, p.K, p.S, p.lam1, p.lam2, p.rho, om,
+                         8, fast=True)
+    X1, _, _ = nlpr.admm(nlpr.to_hwl(p.Yl), nlpr.to_hwl(p.Yh), p.blur, p.d, p.R, p.E, p.K, p.S, p.lam1, q.lam2, p.rho, om,
+                         6, state=st, fast=True)
+    a, b = (Fusion.from_problem(x, dtype="f32", wdtype="f32") for x in (p, q))
+    yl, yh = dev(p.Yl), dev(p.Yh)
+    a.weights(yh)
+    b.weights(yh)
+    a.solve(yl, yh, 8)
+    b.set_state(a.get_state())
+    X, _ = b.solve(yl, yh, 6, warm=True)
+    assert rel(X, nlpr.to_lhw(X1)) <= FP32_BOUND
+    a.close()
+    b.close()
+
+
+@pytest.mark.parametrize("K", [1, 2])
+def test_state_set_before_the_weights(K):
+    # a saved state continues bit for bit also where the weights are set after it, or set again
+    p = small(K=K)
+    a, b = (Fusion.from_problem(p, dtype="f32", wdtype="f32") for _ in range(2))
+    yl, yh = dev(p.Yl), dev(p.Yh)
+    a.weights(yh)
+    a.solve(yl, yh, 5)
+    st = a.get_state()
+    a.weights(yh)
+    Xa, _ = a.solve(yl, yh, 7, warm=True)
+    b.set_state(st)
+    b.weights(yh)
+    Xb, _ = b.solve(yl, yh, 7, warm=True)
+    X, _ = b.solve(yl, yh, 12)
+    assert torch.equal(Xa, X) and torch.equal(Xb, X)
+    a.close()
+    b.close()
+
+
+def test_captured_solves():
+    # a solve captured by the caller (direct launches) and replayed after other calls: the thresholds, the
+    # state and its form are those of the replay's time
+    p, q = small(K=2, seed=5), small(K=2, seed=6)
+    yl, yh, g2 = dev(p.Yl), dev(p.Yh), dev(q.Yh)
+
+    def context():
+        f = Fusion.from_problem(p, dtype="f32", wdtype="f32")
+        f.set_option(FUSE_OPT_GRAPH, 0)
+        return f
+
+    ref = context()
+    f, guide = context(), yh.clone()
+    for warm in (False, True):                            # every buffer and loop of the calls to come
+        f.weights(guide)
+        f.solve(yl, yh, 5, warm=warm)
+    f.sync()
+    cold, warm, both = (torch.cuda.CUDAGraph() for _ in range(3))
+    with torch.cuda.graph(cold):
+        Xc, _ = f.solve(yl, yh, 5)
+    with torch.cuda.graph(warm):
+        Xw, _ = f.solve(yl, yh, 5, warm=True)
+    with torch.cuda.graph(both):
+        f.weights(guide)
+        Xb, _ = f.solve(yl, yh, 5)
+    torch.cuda.synchronize()
+
+    def equal(x, y):
+        torch.cuda.synchronize()
+        assert torch.equal(x, y)
+
+    for g in (yh, g2):
+        f.weights(g)                                      # direct, then replays of solves captured before it
+        ref.weights(g)
+        cold.replay()
+        equal(Xc, ref.solve(yl, yh, 5)[0])
+        warm.replay()
+        warm.replay()
+        equal(Xw, ref.solve(yl, yh, 10, warm=True)[0])
+        assert torch.equal(f.get_state(), ref.get_state())  # direct, after the replays
+        warm.replay()
+        equal(Xw, ref.solve(yl, yh, 5, warm=True)[0])
+        equal(f.solve(yl, yh, 3, warm=True)[0], ref.solve(yl, yh, 3, warm=True)[0])
+        guide.copy_(g2 if g is yh else yh)                # weights within the replay
+        both.replay()
+        ref.weights(guide)
+        equal(Xb, ref.solve(yl, yh, 5)[0])
+        equal(f.solve(yl, yh, 4, warm=True)[0], ref.solve(yl, yh, 4, warm=True)[0])
+    f.close()
+    ref.close()
