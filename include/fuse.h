@@ -76,15 +76,20 @@ enum {
                                     solves replay it and one graph for the remainder), captured
                                     on first use and kept while the launch configuration holds;
                                     0: direct launches */
-    FUSE_OPT_LATENT_IMPL = 3,    /* latent pass: 1 (default) or 0: keep the state entry by entry, with
-                                    register-staged loads.  By default (3 x 3 and 5 x 5 patches, state
-                                    in the iterate type, S <= 15) solves keep the entries of a (tau,
-                                    pixel, band) as a few levels and update those; the same results
-                                    bit for bit.  Where the levels do not apply (other patches,
-                                    FP32 with 3 x 3 patches and a 3 x 3 search, the
-                                    16-bit state, a state or weights set while a solve is continued,
-                                    no memory for them) the entries stream through a bulk-copy ring,
-                                    which the next three options shape. */
+    FUSE_OPT_LATENT_IMPL = 3,    /* latent pass.  1 (default): with 3 x 3 and 5 x 5 patches, the state
+                                    in the iterate type and S <= 15 (not FP32 with 3 x 3 patches and
+                                    a 3 x 3 search) solves keep the entries of a (tau, pixel, band) as
+                                    a few levels, on a power-of-two grid below the largest
+                                    threshold, and update those.  Every other state is kept entry by
+                                    entry in the arithmetic of the iterate type and streamed
+                                    through a bulk-copy ring, which the next three options shape:
+                                    other patches, the 16-bit state, no memory for the levels, a
+                                    state that is not that of a run on the current weights (set by
+                                    the caller, or after new weights, until the next solve from
+                                    zero), a context whose first solve the caller captured.
+                                    2: always entries through the ring.
+                                    0: entries with register-staged loads, in the arithmetic (grid
+                                    or not) that the default would use, and with its bits. */
     FUSE_OPT_LATENT_THREADS = 4, /* consumer threads per latent block, 32..256 (default 128;
                                     256 in batches) */
     FUSE_OPT_LATENT_STAGES = 5,  /* ring slots of the bulk-copy latent pass, 2..32 (default 6) */
@@ -137,7 +142,7 @@ enum {
                                     B^2; the same operator up to rounding; W % 4 == 0, else the
                                     2D stencil); 0: always the 2D stencil.  A batch follows its
                                     first context. */
-    FUSE_OPT_FFT_IMPL = 17       /* DFT solve of the X system: 1 = register-resident passes (one
+    FUSE_OPT_FFT_IMPL = 17,      /* DFT solve of the X system: 1 = register-resident passes (one
                                     warp per line, exchanges by warp shuffles; default when H and
                                     W are 32 P with P in {1, 2, 3, 4, 5, 6, 8, 10, 12, 16});
                                     0 = shared-memory Stockham passes (any H, W factoring into 2,
@@ -146,6 +151,10 @@ enum {
                                     FUSE_EUNSUPPORTED.  The variant FUSE_OPT_X_UPDATE = 1 always
                                     uses the Stockham passes.  In a batch every problem keeps the
                                     form its context had when the batch was created. */
+    FUSE_OPT_LATENT_FORM = 18    /* read only (fuse_get_option, synchronises the stream): how the
+                                    latent state of the last call is kept: 2 levels, 1 entries on
+                                    the levels' grid, 0 entries in the arithmetic of the iterate
+                                    type.  FUSE_ESTATE without a state. */
 };
 
 /* Kernel groups for fuse_profile. */
@@ -157,8 +166,9 @@ enum {
 /* Bytes of device memory fuse_init would allocate for this problem (state in the default
  * half-window mode, weights, FFT buffers and constants).  The first solve (fuse_batch_create for a
  * batch) also allocates the records of the compact state where that applies: 16 bytes (FP64: 32) per
- * kept offset, band and pixel, 8 more with 5 x 5 patches, and one value per kept offset, patch entry
- * and pixel; without the memory for them solves run on the entries alone.  No device work.  Errors: FUSE_EINVAL, FUSE_EUNSUPPORTED. */
+ * kept offset, band and pixel, 8 more with 5 x 5 patches, one value per kept offset, patch entry
+ * and pixel, 16 bytes (FP64: 32) per band and pixel, and a copy of the weights; without the memory for
+ * them, or with FUSE_OPT_LATENT_IMPL 0 or 2, solves run on the entries alone.  No device work.  Errors: FUSE_EINVAL, FUSE_EUNSUPPORTED. */
 fuse_status fuse_workspace_bytes(const fuse_geometry* g, int K, int S, int ratio,
                                  fuse_dtype dtype, fuse_dtype wdtype, size_t* bytes);
 

@@ -180,11 +180,12 @@ struct fuse_ctx {
     // iterations' latent pass, 1 = those of k_levels.cuh, which follow ctl, 0 = the entry kernels.
     // settled: the last solve's `want` (see settle) while nothing has touched the state since, else -1;
     // captured: a call was captured by the caller, whose replays the host does not see.
-    // reg_chosen: the caller selected the register-staged pass.
+    // lat_choice: FUSE_OPT_LATENT_IMPL as the caller chose it, 1 = levels where they apply.
     void *hdr = nullptr, *tab = nullptr, *pt = nullptr, *grid = nullptr, *omega_was = nullptr;
     LatentCtl* ctl = nullptr;
     int path = 0, settled = -1;
-    bool captured = false, reg_chosen = false, lv_refused = false;
+    int lat_choice = 1;
+    bool captured = false, lv_refused = false;
     int lv_Ty = 1, lv_threads = 0, lv_nb = 1;
     size_t lv_smem = 0;
     // sampling mask [H][W] (uint8, ratio 1) replacing the regular lattice; NULL = lattice.
@@ -606,7 +607,7 @@ bool levels_alloc(fuse_ctx* c) {
 }
 
 // Solves run the latent pass on the compact state.
-bool uses_levels(fuse_ctx* c) { return on_grid(c) && !c->reg_chosen && levels_alloc(c); }
+bool uses_levels(fuse_ctx* c) { return on_grid(c) && c->lat_choice == 1 && levels_alloc(c); }
 
 // Dynamic shared-memory cap of the monitoring latent kernels of this context's types.
 bool set_monitor_smem(fuse_ctx* c) {
@@ -1472,7 +1473,7 @@ struct BatchImpl {
         }
         b->lat_smem = 0;
         b->levels = true;
-        for (fuse_ctx* c : b->ctx) b->levels = b->levels && on_grid(c) && levels_alloc(c);
+        for (fuse_ctx* c : b->ctx) b->levels = b->levels && on_grid(c) && c->lat_choice != 2 && levels_alloc(c);
         for (int i = 0; i < n; ++i) {
             fuse_ctx* c = b->ctx[i];
             la[i] = Impl<T>::template lat_args<WT>(c, Ty[i], b->lat_ncons, b->lat_stages, b->lat_bpb);
@@ -2268,16 +2269,24 @@ fuse_status fuse_set_option(fuse_ctx* c, int option, long long value) {
             if (option == FUSE_OPT_LATENT_IMPL && !value && c->sfmt)
                 return fail(c, FUSE_EUNSUPPORTED, "the fixed-point state needs the bulk-copy latent pass");
             const int old_impl = c->lat_impl, old_t = c->lat_target, old_d = c->lat_stages;
-            if (option == FUSE_OPT_LATENT_IMPL) c->lat_impl = value ? 1 : 0;
+            const bool impl = option == FUSE_OPT_LATENT_IMPL;
+            if (impl) c->lat_impl = value ? 1 : 0;
             if (option == FUSE_OPT_LATENT_THREADS) c->lat_target = (int)value;
             if (option == FUSE_OPT_LATENT_STAGES) c->lat_stages = (int)value;
             if (c->lat_target < 32 || c->lat_target > 256 || c->lat_stages < 2 || c->lat_stages > 32 ||
                 (c->lat_impl == 1 && !latent_tma_shape(c))) {
+                if (impl && value && value != 2 && on_grid(c)) {
+                    // the default form needs no ring: register-staged loads for what is not levels
+                    c->lat_impl = 0;
+                    c->lat_choice = 1;
+                    drop_graphs(c);
+                    return FUSE_OK;
+                }
                 c->lat_impl = old_impl; c->lat_target = old_t; c->lat_stages = old_d;
                 latent_tma_shape(c);
                 return fail(c, FUSE_EINVAL, "latent launch option out of range");
             }
-            if (option == FUSE_OPT_LATENT_IMPL) c->reg_chosen = !value;
+            if (impl) c->lat_choice = value == 0 ? 0 : value == 2 ? 2 : 1;
             drop_graphs(c);
             return FUSE_OK;
         }
@@ -2323,6 +2332,7 @@ fuse_status fuse_set_option(fuse_ctx* c, int option, long long value) {
                     return fail(c, FUSE_EUNSUPPORTED, "fixed-point state needs the bulk-copy latent pass (W % 8 == 0)");
                 }
                 c->sfmt = 0;
+                if (c->lat_choice == 0) c->lat_choice = 1;
             }
             return realloc_state(c, c->half, f);
         }
@@ -2500,7 +2510,19 @@ fuse_status fuse_get_option(fuse_ctx* c, int option, long long* value) {
     switch (option) {
         case FUSE_OPT_PROFILE: *value = c->profile; return FUSE_OK;
         case FUSE_OPT_GRAPH: *value = c->use_graph; return FUSE_OK;
-        case FUSE_OPT_LATENT_IMPL: *value = c->lat_impl; return FUSE_OK;
+        case FUSE_OPT_LATENT_IMPL: *value = c->lat_choice == 2 ? 2 : c->lat_impl; return FUSE_OK;
+        case FUSE_OPT_LATENT_FORM: {
+            fuse_status st = guard(c);
+            if (st != FUSE_OK) return st;
+            if (!c->have_state) return FUSE_ESTATE;
+            int mode = kStateEntries;
+            if (on_grid(c)) {
+                CK(c, cudaMemcpyAsync(&mode, &c->ctl->mode, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+                CK(c, cudaStreamSynchronize(c->stream));
+            }
+            *value = mode == kStateLevels ? 2 : mode == kStateGrid ? 1 : 0;
+            return FUSE_OK;
+        }
         case FUSE_OPT_LATENT_THREADS: *value = c->lat_target; return FUSE_OK;
         case FUSE_OPT_LATENT_STAGES: *value = c->lat_stages; return FUSE_OK;
         case FUSE_OPT_WAIT_LIMIT: *value = c->wait_limit; return FUSE_OK;

@@ -25,6 +25,7 @@ FUSE_OPT_LATENT_IMPL, FUSE_OPT_LATENT_THREADS, FUSE_OPT_LATENT_STAGES, FUSE_OPT_
 FUSE_OPT_HALF_WINDOW, FUSE_OPT_LATENT_BANDS, FUSE_OPT_FFT_ROWS, FUSE_OPT_FFT_COLS = 7, 8, 9, 10
 FUSE_OPT_GRAD_SEGMENT, FUSE_OPT_GRAD_WEIGHTS, FUSE_OPT_STATE_FORMAT = 11, 12, 13
 FUSE_OPT_X_UPDATE, FUSE_OPT_RESIDUALS, FUSE_OPT_SEPARABLE_BLUR, FUSE_OPT_FFT_IMPL = 14, 15, 16, 17
+FUSE_OPT_LATENT_FORM = 18
 FUSE_K_ALL, FUSE_K_LATENT = 0, 1
 
 DTYPES = {"f32": FUSE_F32, "f64": FUSE_F64, "bf16": FUSE_BF16}
