@@ -728,7 +728,8 @@ struct Impl {
     static fuse_status weights(fuse_ctx* c, const void* G) {
         dim3 grid((unsigned)((c->H + c->w_Ty - 1) / c->w_Ty), (unsigned)c->nW);
         weights_kernel<T, WT><<<grid, 256, c->w_smem, c->stream>>>(
-            (const T*)G, (WT*)c->omega, c->H, c->W, c->Lg, c->K, c->S, c->w_Ty, (T)(1.0 / (c->h * c->h)));
+            (const T*)G, (WT*)c->omega, c->H, c->W, c->Lg, c->K, c->S, c->w_Ty, (T)(1.0 / (c->h * c->h)),
+            grid_options(c) ? &((LatentGrid<T>*)c->grid)->wmax : nullptr);
         c->launches_all++;
         CKL(c, "weights_kernel");
         return FUSE_OK;
@@ -1020,22 +1021,40 @@ fuse_status need_entries(fuse_ctx* c, int want = kStateGrid) {
     return FUSE_OK;
 }
 
+// The state that a solve of the inputs Yl (NULL: of none yet) starts with.
+void begin_state(fuse_ctx* c, const void* Yl, bool cold, int want) {
+    const size_t count = Yl && want != kStateEntries && want != kStateGiven ? (size_t)c->Ll * c->nl : 0;
+    // X = Z E^T / eps where E E^T = eps I, and |B| <= sum |b|
+    double taps = 0.0;
+    for (double t : c->htapsB) taps += std::fabs(t);
+    const double gain = taps * std::sqrt(c->eet_eps), coef = c->lam2 / c->rho;
+    if (c->dtype == FUSE_F64)
+        latent_begin_launch<double>((const double*)Yl, count, (const uint8_t*)c->mask, c->n, gain, coef,
+                                    (const LatentGrid<double>*)c->grid, c->ctl, cold, want, c->stream);
+    else
+        latent_begin_launch<float>((const float*)Yl, count, (const uint8_t*)c->mask, c->n, gain, coef,
+                                   (const LatentGrid<float>*)c->grid, c->ctl, cold, want, c->stream);
+    c->launches_all++;
+}
+
 // Brings the latent state into the form in which the iterations of a solve continue or start, `want`:
 //   kStateLevels   levels (path 1), or entries where the state is not that of a run on the current weights
 //   kStateGrid     entries, on the grid where they are those of such a run
 //   kStateEntries  entries in the arithmetic of the iterate type
-// A context whose state nothing touched since a solve with the same `want` has nothing to do.
-fuse_status settle(fuse_ctx* c, bool cold, int want) {
+// off the grid where it does not carry the inputs Yl.  Where nothing touched the state since a solve with
+// the same `want`, those are all that can have changed.
+fuse_status settle(fuse_ctx* c, const void* Yl, bool cold, int want) {
     if (!on_grid(c)) return FUSE_OK;
     const bool touched = capturing(c) || c->captured || c->settled != want;
-    if (cold || touched) {
-        latent_begin_launch(c->ctl, cold, want, c->stream);
-        c->launches_all++;
+    if (cold || touched || want != kStateEntries) {
+        begin_state(c, Yl, cold, want);
         CKL(c, "latent_begin_kernel");
     }
-    if (!cold && touched) {
+    if (!cold && (touched || want != kStateEntries)) {
         const fuse_status st = need_entries(c, want);
         if (st != FUSE_OK) return st;
+    }
+    if (!cold && touched) {
         if (want != kStateEntries) {
             with_types(c, [&](auto im, auto w) { im.template check_entries<decltype(w)>(c); });
             c->launches_all++;
@@ -1212,7 +1231,7 @@ fuse_status solve_impl(fuse_ctx* c, const void* Yl, const void* Yh, int iters, i
         // cleared entries, or entries that a monitored first iteration writes
         if (!cold || (c->monitor && iters == 1)) want = std::min<int>(want, kStateGrid);
     }
-    if ((st = settle(c, start, want)) != FUSE_OK) return st;
+    if ((st = settle(c, Yl, start, want)) != FUSE_OK) return st;
     if (c->xmode == 1) {
         // the fixed data term of the variant: U1 = G = B^T S^T Y_l E^T / rho (B X as scratch)
         st = f64 ? Impl<double>::sb_data_term(c, c->stream) : Impl<float>::sb_data_term(c, c->stream);
@@ -2235,8 +2254,7 @@ fuse_status fuse_set_state(fuse_ctx* c, const void* src) {
     p += c->sig_bytes;
     CK(c, cudaMemcpyAsync(c->planes, p, c->plane_bytes, cudaMemcpyDefault, c->stream));
     if (on_grid(c)) {
-        latent_begin_launch(c->ctl, 1, kStateGiven, c->stream);
-        c->launches_all++;
+        begin_state(c, nullptr, true, kStateGiven);
         CKL(c, "latent_begin_kernel");
         c->settled = -1;
     }
@@ -2455,7 +2473,7 @@ fuse_status fuse_autotune(fuse_ctx* c, const void* Yl, const void* Yh, int iters
     // inputs and a zero state (the timed iterations run on it; the next solve starts over)
     st = solve_impl(c, Yl, Yh, 0, 0, nullptr, nullptr);
     if (st != FUSE_OK) return st;
-    if ((st = settle(c, false, c->path == 1 ? kStateLevels : c->lat_impl == 0 ? kStateGrid : kStateEntries)) != FUSE_OK)
+    if ((st = settle(c, Yl, false, c->path == 1 ? kStateLevels : c->lat_impl == 0 ? kStateGrid : kStateEntries)) != FUSE_OK)
         return st;
     double best = 1e30, t = 0;
     // 1. latent pass: ring shape and bands per block (the pass on the compact state has one shape)
@@ -2646,7 +2664,7 @@ fuse_status fuse_batch_solve(fuse_batch* b, const void* const* Yl, const void* c
         if (st != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
         c->have_state = true;
         c->path = b->levels ? 1 : 0;
-        if ((st = settle(c, true, b->levels ? (iters > 0 ? kStateLevels : kStateGiven) : kStateEntries)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
+        if ((st = settle(c, Yl[i], true, b->levels ? (iters > 0 ? kStateLevels : kStateGiven) : kStateEntries)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
     }
     fuse_status st = batch_run(b, iters, iters > 0);
     if (st != FUSE_OK) return st;

@@ -440,15 +440,15 @@ __device__ __forceinline__ void each_window(const LevelArgs<T, WT>& a, int work,
 }
 
 // Levels -> entries s_k (in the iterate type), where the coming calls want entries (want below
-// kStateLevels) or the weights have changed since the levels were formed (old: the arguments from
-// before).  The entries are then those of a run on the current weights, or to be looked at; with
-// want = kStateEntries they go on in the iterate type's arithmetic.
+// kStateLevels), the grid does not carry their inputs, or the weights have changed since the levels were
+// formed (old: the arguments from before).  The entries are then those of a run on the current weights,
+// or to be looked at; with want = kStateEntries or off the grid they go on in the iterate type's arithmetic.
 template <typename T, typename WT, int K>
 __global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, int want) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
-    if (now.ctl->mode != kStateLevels || !(now.ctl->was || want < kStateLevels)) return;
+    if (now.ctl->mode != kStateLevels || !(now.ctl->was || want < kStateLevels || !now.ctl->fit)) return;
     const LevelArgs<T, WT> a = now.ctl->was ? old : now;
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
     const T g = a.grid->g;
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT>
         }
     });
     if (last_block(now.ctl) && threadIdx.x == 0) {
-        now.ctl->mode = want == kStateEntries ? kStateEntries : now.ctl->was ? kStateGiven : kStateGrid;
+        now.ctl->mode = want == kStateEntries || !now.ctl->fit ? kStateEntries : now.ctl->was ? kStateGiven : kStateGrid;
         now.ctl->was = 0;
     }
 }
@@ -584,15 +584,78 @@ weights_change_kernel(const uint4* __restrict__ omega, uint4* __restrict__ was, 
     }
 }
 
-// grid->wmax = the largest finite |w| of n weights (zeroed before; the order of non-negative
-// floating-point values is that of their bit patterns); then the grid from it.
+// The state that a solve starts with, and whether the grid carries its inputs: their size is the rms of
+// the `count` samples of Y_l that S keeps (mask, over n pixels, or all), divided by `gain`, the most that B and E
+// can have raised that of X.  Sums in FP64, in the same order on every device; latency-bound, about
+// 5 us for 131 thousand samples.
+template <typename T>
+__global__ void __launch_bounds__(256)
+latent_begin_kernel(const T* __restrict__ Y, size_t count, const uint8_t* __restrict__ mask, size_t n, double gain,
+                    double coef, const LatentGrid<T>* grid, LatentCtl* ctl, int cold, int want) {
+    __shared__ double red[2][8];
+    double sq = 0.0, seen = 0.0;
+    // the block's sums, in thread 0
+    auto reduce = [&]() {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            sq += __shfl_down_sync(0xffffffffu, sq, o);
+            seen += __shfl_down_sync(0xffffffffu, seen, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            red[0][threadIdx.x >> 5] = sq;
+            red[1][threadIdx.x >> 5] = seen;
+        }
+        __syncthreads();
+        for (int w = 1; threadIdx.x == 0 && w < 8; ++w) {
+            sq += red[0][w];
+            seen += red[1][w];
+        }
+    };
+    const size_t step = (size_t)gridDim.x * 256, first = (size_t)blockIdx.x * 256 + threadIdx.x;
+    size_t p = first % n;                             // the sample's pixel (with a mask)
+#pragma unroll 4
+    for (size_t i = first; i < count; i += step) {
+        if (!mask || mask[p]) {
+            const double v = (double)Y[i];
+            sq += v * v;
+            seen += 1.0;
+        }
+        if (mask) p = (p + step) % n;
+    }
+    reduce();
+    if (threadIdx.x == 0) {
+        ctl->part[blockIdx.x] = sq;
+        ctl->seen[blockIdx.x] = seen;
+    }
+    if (!last_block(ctl)) return;
+    sq = seen = 0.0;
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += 256) {
+        sq += __ldcg(&ctl->part[b]);
+        seen += __ldcg(&ctl->seen[b]);
+    }
+    reduce();
+    if (threadIdx.x != 0) return;
+    const double top = ldexp((double)grid->g, grid_code<T>::B), wmax = (double)grid->wmax;
+    // thresholds that are all zero leave the entries zero, on the grid of anything
+    const bool fit = wmax <= 1e308 && (coef * wmax == 0.0 || top * gain <= sqrt(sq / seen));
+    ctl->fit = fit;
+    if (cold) {
+        ctl->mode = fit || want == kStateGiven ? want : kStateEntries;
+        ctl->was = 0;
+    } else if (ctl->mode != kStateLevels && (want == kStateEntries || !fit)) {
+        ctl->mode = kStateEntries;
+    }
+}
+
+// grid->wmax = the largest of n weights, infinite if one is not a finite number >= 0 (zeroed before; the
+// order of non-negative floating-point values is that of their bit patterns); then the grid from it.
 template <typename T, typename WT>
 __global__ void __launch_bounds__(256) wmax_kernel(const WT* __restrict__ w, size_t n, LatentGrid<T>* grid) {
     T m = T(0);
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
         const T v = (T)wload(w + i);
-        const T av = v < T(0) ? -v : v;
-        if (av > m && av <= (sizeof(T) == 4 ? (T)3.0e38 : (T)1.0e308)) m = av;
+        if (v > m) m = v;
+        if (!(v >= T(0))) m = (T)INFINITY;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = tmax(m, __shfl_xor_sync(0xffffffffu, m, o));

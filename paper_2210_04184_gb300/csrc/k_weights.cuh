@@ -4,7 +4,8 @@
 // difference e_tau(j) = sum_c (G_c(j) - G_c(j - tau))^2, i.e. a (2K+1)^2 box sum of e_tau.
 // One block owns Ty output rows (full width) of one offset tau: it forms e_tau on the rows
 // [y0-K, y0+Ty+K) in shared memory, box-sums along x, then along y, and stores
-// exp(-s/h^2) in the weight type (bf16 rounding is round-to-nearest-even).
+// exp(-s/h^2) in the weight type (bf16 rounding is round-to-nearest-even).  Weights that are not a
+// number (a guide that is not finite) raise *wmax, where given, to infinity: see LatentGrid.
 #pragma once
 #include "common.cuh"
 
@@ -13,7 +14,7 @@ namespace fuse {
 template <typename T, typename WT>
 __global__ void __launch_bounds__(256)
 weights_kernel(const T* __restrict__ G, WT* __restrict__ omega, int H, int W, int Lg, int K, int S,
-               int Ty, T inv_h2) {
+               int Ty, T inv_h2, T* __restrict__ wmax) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int rows = Ty + 2 * K;
     T* e = reinterpret_cast<T*>(smem_raw);          // [rows][W]
@@ -50,7 +51,9 @@ weights_kernel(const T* __restrict__ G, WT* __restrict__ omega, int H, int W, in
         if (y >= H) continue;
         T s = T(0);
         for (int k1 = -K; k1 <= K; ++k1) s += hs[(r + K - k1) * W + x];
-        wstore(omega + (size_t)tidx * n + (size_t)y * W + x, texp(-s * inv_h2));
+        const T w = texp(-s * inv_h2);
+        wstore(omega + (size_t)tidx * n + (size_t)y * W + x, w);
+        if (wmax && !(w <= T(1))) *wmax = (T)INFINITY;
     }
 }
 

@@ -9,10 +9,18 @@
 // X and mu_k are rounded to the grid, to nearest.  Every s_k is then a multiple of g of at
 // most 2^B g, an exact value of the iterate type, the update is exact, and so is the sum over k in
 // any order.  In the topmost binade below mu_max the grid is the iterate type's own spacing; smaller
-// values keep the same absolute step.  Error of X from this, all else in FP64 (relative, 40 iterations,
-// three 32 x 32 scenes, lambda2/rho = 0.1, 0.2, 0.5, with 2^B g = 0.26, 0.52, 2.1 of the data's rms, 25
-// entries): 1.44e-7, 1.50e-7, 1.47e-7, against 1.48e-7, 1.52e-7, 1.40e-7 with entries in FP32; with
-// mu_k rounded down, all in one direction, 1.72e-7, 2.71e-7, 6.8e-7.
+// values keep the same absolute step.
+//
+// Where it is used.  The iterate type keeps small values to more bits than the grid does, so a solve is
+// on the grid only while its range 2^B g (mu_max to the next power of two) is at most the size of X,
+// taken from the rms of the Y_l samples (latent_begin_kernel); else, and with weights that are not finite or negative, it runs
+// the arithmetic of the iterate type.  Error of X from the latent update alone, all else in FP64
+// (relative, 40 iterations, means over three 32 x 32 scenes, 25 entries), by range / rms:
+//   0.26  grid 1.44e-7, FP32 entries 1.48e-7        4.1  grid 1.86e-7, FP32 entries 1.39e-7
+//   0.52  grid 1.50e-7, FP32 entries 1.52e-7       16.5  grid 4.54e-7, FP32 entries 1.30e-7
+//   0.86  grid 1.38e-7, FP32 entries 1.38e-7        132  grid 2.62e-6, FP32 entries 1.05e-7
+//   2.1   grid 1.47e-7, FP32 entries 1.40e-7
+// (mu_k rounded down, all in one direction, gave 1.7e-7, 2.7e-7 and 3.2e-7 in the first three rows.)
 //
 // Compact form.  With w = -sum_t delta_t (in units of g) s is, as a function of its threshold mu, the
 // state of a stop operator driven by w.  In ascending order of mu it consists of levels: a run of
@@ -61,7 +69,8 @@ __host__ __device__ constexpr bool latent_grid_k(int K) { return K == 1 || K == 
 
 template <typename T> struct LatentGrid {
     T g, ig;                    // grid step and its reciprocal (powers of two)
-    T wmax;                     // the largest weight it was made for
+    T wmax;                     // the largest weight it was made for; infinite if one is not a finite
+                                // number >= 0
 };
 
 // What the latent state of a context holds, kept on the device: the calls that change it and the
@@ -71,13 +80,16 @@ template <typename T> struct LatentGrid {
 //   kStateGrid     entries on the grid, those of a run on the current weights
 //   kStateLevels   levels, formed with the current weights or, with `was`, with the ones before them
 //   kStateGiven    entries not looked at yet: set by the caller, or left by other weights
+constexpr int kBeginBlocks = 512;       // most blocks of latent_begin_kernel
 enum : int { kStateEntries = 0, kStateGrid = 1, kStateLevels = 2, kStateGiven = 3 };
 struct LatentCtl {
     int mode;
     int was;                    // omega_was and grid[1] describe the levels
     int table;                  // the threshold table is that of the current weights
     int off;                    // some entry is not that of a run on the current weights
+    int fit;                    // the grid carries the thresholds and X of the last solve's inputs
     unsigned done;              // blocks of the running kernel that have finished
+    double part[kBeginBlocks], seen[kBeginBlocks];
 };
 // Whether an entry kernel is to run: ctl NULL, always; else where the state is entries, on the grid or not
 // as the kernel's arithmetic.
@@ -103,7 +115,7 @@ inline __host__ __device__ LatentGrid<double> latent_grid(double coef, double wm
     return {ldexp(1.0, e - grid_code<double>::B), ldexp(1.0, grid_code<double>::B - e), wmax};
 }
 
-// Code of a threshold: rounded to nearest; a weight that is not a number or infinite acts as the largest.
+// Code of a threshold: rounded to nearest.
 __device__ __forceinline__ int32_t mu_code(float mu, float ig) {
     const float cap = 16777216.0f;                              // 2^B
     const float c = fabsf(mu) * ig;

@@ -97,17 +97,12 @@ void weights_change_launch(const void* omega, void* was, size_t bytes, LatentGri
     weights_change_kernel<T><<<blocks, 256, 0, s>>>((const uint4*)omega, (uint4*)was, words, grid, ctl);
 }
 
-// The state that a solve starts with.
-static __global__ void latent_begin_kernel(LatentCtl* ctl, int cold, int want) {
-    if (cold) {
-        ctl->mode = want;
-        ctl->was = 0;
-    } else if (want == kStateEntries && ctl->mode != kStateLevels) {
-        ctl->mode = kStateEntries;
-    }
-}
-void latent_begin_launch(LatentCtl* ctl, int cold, int want, cudaStream_t s) {
-    latent_begin_kernel<<<1, 1, 0, s>>>(ctl, cold, want);
+template <typename T>
+void latent_begin_launch(const T* Y, size_t count, const uint8_t* mask, size_t n, double gain, double coef,
+                         const LatentGrid<T>* grid, LatentCtl* ctl, int cold, int want, cudaStream_t s) {
+    const size_t need = (count + 2047) / 2048;
+    const unsigned blocks = (unsigned)(need < 1 ? 1 : need < (size_t)kBeginBlocks ? need : (size_t)kBeginBlocks);
+    latent_begin_kernel<T><<<blocks, 256, 0, s>>>(Y, count, mask, n, gain, coef, grid, ctl, cold, want);
 }
 
 template <typename T, typename WT>
@@ -154,6 +149,10 @@ FUSE_LEVELS_INST(float, float)
 FUSE_LEVELS_INST(float, __nv_bfloat16)
 FUSE_LEVELS_INST(double, double)
 template void weights_change_launch<float>(const void*, void*, size_t, LatentGrid<float>*, LatentCtl*, int, cudaStream_t);
+template void latent_begin_launch<float>(const float*, size_t, const uint8_t*, size_t, double, double,
+                                         const LatentGrid<float>*, LatentCtl*, int, int, cudaStream_t);
+template void latent_begin_launch<double>(const double*, size_t, const uint8_t*, size_t, double, double,
+                                          const LatentGrid<double>*, LatentCtl*, int, int, cudaStream_t);
 template void weights_change_launch<double>(const void*, void*, size_t, LatentGrid<double>*, LatentCtl*, int, cudaStream_t);
 
 }  // namespace fuse

@@ -13,8 +13,8 @@ torch = pytest.importorskip("torch")
 
 from oracle import nlpr  # noqa: E402
 from paper_2210_04184_gb300 import build as _build  # noqa: E402
-from paper_2210_04184_gb300.fuse import (Fusion, FUSE_OPT_GRAPH, FUSE_OPT_LATENT_IMPL,  # noqa: E402
-                                         FUSE_OPT_RESIDUALS)
+from paper_2210_04184_gb300.fuse import (Fusion, FusionBatch, FUSE_OPT_GRAPH, FUSE_OPT_LATENT_FORM,  # noqa: E402
+                                         FUSE_OPT_LATENT_IMPL, FUSE_OPT_RESIDUALS)
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -215,3 +215,155 @@ def test_captured_solves():
         equal(f.solve(yl, yh, 4, warm=True)[0], ref.solve(yl, yh, 4, warm=True)[0])
     f.close()
     ref.close()
+
+
+def _given(nW, H, W, value):
+    """Symmetric weights in (0, 1], one pair of them `value`."""
+    g = torch.Generator().manual_seed(3)
+    w = torch.rand(nW, H, W, generator=g) * 0.9 + 0.1
+    S = (math.isqrt(nW + 1) - 1) // 2
+    offs = [(a, b) for a in range(-S, S + 1) for b in range(-S, S + 1) if (a, b) != (0, 0)]
+    for i, t in enumerate(offs[:nW // 2]):                # omega_{i,-tau} = omega_{i+tau,tau}
+        w[i] = torch.roll(w[nW - 1 - i], (t[0], t[1]), (0, 1))
+    w[nW - 1, 7, 9] = value
+    a, b = offs[0]
+    w[0, (7 + a) % H, (9 + b) % W] = value
+    return w
+
+
+# (problem, scale of the data, one weight, whether the grid carries them): FP32_BOUND is what the former
+# arithmetic is held to at every one of them
+RANGES = [
+    (dict(), 1.0, 0.5, True),
+    (dict(lam2=1.0, rho=5e-2), 1.0, 0.5, False),          # lambda2/rho = 20
+    (dict(lam2=2.0, rho=5e-2), 1.0, 0.5, False),          # 40
+    (dict(lam2=2.0, rho=5e-2), 1e3, 0.5, True),
+    (dict(), 1e-2, 0.5, False),
+    (dict(), 1e-4, 0.5, False),
+    (dict(), 1e4, 0.5, True),
+    (dict(), 1.0, 1e2, False),
+    (dict(), 1.0, 1e4, False),
+    (dict(), 1.0, 1e8, False),
+    (dict(lam2=0.0), 1e-4, 0.5, True),                    # thresholds of zero
+]
+
+
+@pytest.mark.parametrize("K", [1, 2])
+@pytest.mark.parametrize("dtype,bound", [("f32", FP32_BOUND), ("f64", 1e-11)])
+@pytest.mark.parametrize("kw,scale,weight,grid", RANGES)
+def test_grid_only_where_it_carries_the_inputs(K, dtype, bound, kw, scale, weight, grid):
+    p = small(K=K, **kw)
+    p.Yl, p.Yh = p.Yl * scale, p.Yh * scale
+    td = torch.float64 if dtype == "f64" else torch.float32
+    w = _given((2 * p.S + 1) ** 2 - 1, p.H, p.W, weight).to(td)
+    Xo = oracle_runs(p, [(w.double().numpy(), 30)])[0]
+    got = {}
+    for impl in (1, 0, 2):
+        f = Fusion.from_problem(p, dtype=dtype, wdtype=dtype)
+        f.set_option(FUSE_OPT_LATENT_IMPL, impl)
+        f.set_weights(w.cuda())
+        X, _ = f.solve(dev(p.Yl, td), dev(p.Yh, td), 30)
+        assert f.get_option(FUSE_OPT_LATENT_FORM) == ({1: 2, 0: 1, 2: 0}[impl] if grid else 0)
+        assert rel(X, Xo) <= bound
+        got[impl] = (X.clone(), f.get_state())
+        f.close()
+    assert torch.equal(got[1][0], got[0][0]) and torch.equal(got[1][1], got[0][1])
+    if not grid:                                          # the former arithmetic, bit for bit
+        assert torch.equal(got[1][0], got[2][0]) and torch.equal(got[1][1], got[2][1])
+
+
+@pytest.mark.parametrize("bad", ["inf", "nan", "negative", "guide"])
+def test_weights_that_are_no_thresholds(bad):
+    # infinite or not a number: no threshold, as entries have it; FP32 and FP64 alike
+    p = small(K=2)
+    for dtype in ("f32", "f64"):
+        td = torch.float64 if dtype == "f64" else torch.float32
+        out = []
+        for impl in (1, 2):
+            f = Fusion.from_problem(p, dtype=dtype, wdtype=dtype)
+            f.set_option(FUSE_OPT_LATENT_IMPL, impl)
+            if bad == "guide":
+                g = dev(p.Yh, td)
+                g[0, 3, 4] = float("nan")
+                f.weights(g)
+            else:
+                v = {"inf": float("inf"), "nan": float("nan"), "negative": -0.5}[bad]
+                f.set_weights(_given(f.nW, p.H, p.W, v).to(td).cuda())
+            out.append(f.solve(dev(p.Yl, td), dev(p.Yh, td), 12)[0].clone())
+            assert f.get_option(FUSE_OPT_LATENT_FORM) == 0 and torch.isfinite(out[-1]).all()
+            f.weights(dev(p.Yh, td))                      # ordinary ones again
+            f.solve(dev(p.Yl, td), dev(p.Yh, td), 2)
+            assert f.get_option(FUSE_OPT_LATENT_FORM) == (2 if impl == 1 else 0)
+            f.close()
+        assert torch.equal(*out)
+
+
+def test_size_of_the_data():
+    # X is what counts: E scaled up makes it smaller than Y_l; samples off a mask do not count
+    p = small(K=2)
+    for kw, s, form in ((dict(), 1e3, 0), (dict(lam2=2.0), 1e-3, 2), (dict(lam2=2.0), 1.0, 0)):
+        q = small(K=2, **kw)
+        q.E = q.E * s
+        f = Fusion.from_problem(q, dtype="f32", wdtype="f32")
+        f.weights(dev(q.Yh))
+        f.solve(dev(q.Yl), dev(q.Yh), 3)
+        assert f.get_option(FUSE_OPT_LATENT_FORM) == form
+        f.close()
+    q = small(K=2, d=1, blur_size=1)
+    mask = torch.zeros(q.H, q.W, dtype=torch.bool, device="cuda")
+    mask[::2, ::3] = True
+    xs = []
+    for fill in (0.0, float("nan"), 1e9):
+        f = Fusion.from_problem(q, dtype="f32", wdtype="f32")
+        f.set_mask(mask)
+        yl = torch.where(mask, dev(q.Yl), fill)
+        f.weights(dev(q.Yh))
+        xs.append(f.solve(yl, dev(q.Yh), 5)[0].clone())
+        assert f.get_option(FUSE_OPT_LATENT_FORM) == 2
+        f.close()
+    assert torch.equal(xs[0], xs[1]) and torch.equal(xs[0], xs[2])
+
+
+def test_continued_with_other_data():
+    # frames of a scene that goes dark: the state leaves the grid, and stays off it until a new start
+    p = small(K=2)
+    om = nlpr.weights(nlpr.to_hwl(p.Yh), p.K, p.S, p.h).astype(np.float32)
+    f = Fusion.from_problem(p, dtype="f32", wdtype="f32")
+    f.set_weights(dev(om))
+    st = None
+    for i, (scale, form) in enumerate([(1.0, 2), (0.8, 2), (1e-3, 0), (1.0, 0)]):
+        Yl, Yh = p.Yl * scale, p.Yh * scale
+        X, _ = f.solve(dev(Yl), dev(Yh), 5, warm=i > 0)
+        assert f.get_option(FUSE_OPT_LATENT_FORM) == form
+        Xo, st, _ = nlpr.admm(nlpr.to_hwl(Yl), nlpr.to_hwl(Yh), p.blur, p.d, p.R, p.E, p.K, p.S, p.lam1, p.lam2, p.rho,
+                              om.astype(np.float64), 5, state=st, fast=True)
+        assert rel(X, nlpr.to_lhw(Xo)) <= FP32_BOUND
+    f.solve(dev(p.Yl), dev(p.Yh), 5)
+    assert f.get_option(FUSE_OPT_LATENT_FORM) == 2
+    f.close()
+
+
+def test_batch_of_both_kinds():
+    # problems on the grid and off it in one batch: each as alone
+    ps = [small(K=1, S=3, H=h, W=w, L_s=5, seed=30 + i) for i, (h, w) in enumerate([(24, 40), (40, 160), (64, 24)])]
+    ps[1].Yl, ps[1].Yh = ps[1].Yl * 1e-3, ps[1].Yh * 1e-3
+    ctx = [Fusion.from_problem(p, dtype="f32", wdtype="bf16") for p in ps]
+    yl, yh = [dev(p.Yl) for p in ps], [dev(p.Yh) for p in ps]
+    ref = []
+    for f, a, b in zip(ctx, yl, yh):
+        f.weights(b)
+        ref.append(f.solve(a, b, 9)[0].clone())
+    forms = [f.get_option(FUSE_OPT_LATENT_FORM) for f in ctx]
+    assert forms == [2, 0, 2]
+    batch = FusionBatch(ctx)
+    for _ in range(2):
+        Xs, _ = batch.solve(yl, yh, 9)
+        batch.sync()
+        assert [f.get_option(FUSE_OPT_LATENT_FORM) for f in ctx] == forms
+        for x, y in zip(Xs, ref):
+            assert torch.equal(x, y)
+    batch.close()
+    for f, a, b, r in zip(ctx, yl, yh, ref):              # and continue alone
+        x = f.solve(a, b, 3, warm=True)[0].clone()
+        assert torch.equal(x, f.solve(a, b, 12)[0])
+        f.close()
