@@ -1407,8 +1407,11 @@ struct fuse_batch {
     int fr_rpb = 4, fc_cw = 8;
     // device tables: [args of every problem] and segments per kernel
     void* d_lat = nullptr; Segment* d_lat_seg = nullptr; int lat_nseg = 0, lat_blocks = 0;
-    // latent pass on the compact state (levels: every problem allows it) and its points
+    // latent pass on the compact state and its points, of the problems that allow it (on_levels; levels:
+    // there are some); the others are entries whatever stands beside them in the batch
+    std::vector<char> on_levels;
     bool levels = false;
+    bool bands_set = false;     // the caller or the tuner chose lat_bpb
     void* d_lv = nullptr; Segment* d_lv_seg = nullptr; Segment* d_pt_seg = nullptr;
     int lv_nseg = 0, lv_blocks = 0, pt_nseg = 0, pt_blocks = 0;
     size_t lv_smem = 0;
@@ -1491,12 +1494,28 @@ struct BatchImpl {
             if (nc > b->lat_ncons) b->lat_ncons = nc;
         }
         b->lat_smem = 0;
-        b->levels = true;
-        for (fuse_ctx* c : b->ctx) b->levels = b->levels && on_grid(c) && c->lat_choice != 2 && levels_alloc(c);
+        b->on_levels.assign(n, 0);
+        b->levels = false;
         for (int i = 0; i < n; ++i) {
             fuse_ctx* c = b->ctx[i];
-            la[i] = Impl<T>::template lat_args<WT>(c, Ty[i], b->lat_ncons, b->lat_stages, b->lat_bpb);
-            la[i].ctl = b->levels ? c->ctl : nullptr;
+            b->on_levels[i] = on_grid(c) && c->lat_choice != 2 && levels_alloc(c);
+            b->levels = b->levels || b->on_levels[i];
+        }
+        // Bands per block of the ring.  Where it stands beside levels most of its blocks return at once, and a
+        // launch costs by their number: as many bands as leave eight blocks per SM (24 tiles of 96 to 384, 40
+        // iterations on levels: 124.6 ms with 8 bands, 126.5 with 2; data off the grid 194.2 and 198.9).
+        auto ring_blocks = [&](int bands) {
+            long long t = 0;
+            for (int i = 0; i < n; ++i) t += (long long)((b->ctx[i]->H + Ty[i] - 1) / Ty[i]) * ((b->Ls + bands - 1) / bands) * rows;
+            return t;
+        };
+        int bpb = b->lat_bpb;
+        if (b->levels && !b->bands_set)
+            while (bpb < b->Ls && ring_blocks(std::min(2 * bpb, b->Ls)) >= 8ll * b->ctx[0]->nsm) bpb = std::min(2 * bpb, b->Ls);
+        for (int i = 0; i < n; ++i) {
+            fuse_ctx* c = b->ctx[i];
+            la[i] = Impl<T>::template lat_args<WT>(c, Ty[i], b->lat_ncons, b->lat_stages, bpb);
+            la[i].ctl = b->on_levels[i] ? c->ctl : nullptr;
             const size_t ssz = b->sfmt ? 2 : esz;
             const size_t sm = (size_t)b->lat_stages * Ty[i] * c->W * ssz + 5 * (size_t)Ty[i] * c->W * esz +
                               2 * (size_t)b->lat_stages * 8;
@@ -1505,7 +1524,7 @@ struct BatchImpl {
         if (b->lat_smem > (size_t)kMaxSmem) return bfail(b, FUSE_EUNSUPPORTED, "batched latent ring exceeds shared memory");
         std::vector<Segment> seg;
         int next = 0;
-        const int groups = (b->Ls + b->lat_bpb - 1) / b->lat_bpb;
+        const int groups = (b->Ls + bpb - 1) / bpb;
         for (int i = 0; i < n; ++i)          // heavy block rows (tau1 != 0) of every problem first
             add_segment(seg, i, (b->ctx[i]->H + Ty[i] - 1) / Ty[i], groups, rows - 1, 0, &next);
         for (int i = 0; i < n; ++i)          // then the lighter tau1 = 0 rows
@@ -1524,6 +1543,7 @@ struct BatchImpl {
             next = 0;
             b->lv_smem = 0;
             for (int i = 0; i < n; ++i) {
+                if (!b->on_levels[i]) continue;
                 fuse_ctx* c = b->ctx[i];
                 // the launch fills the device whatever one problem's size: as many bands per block as fit
                 lv[i] = Impl<T>::template lv_args<WT>(c);
@@ -1535,7 +1555,7 @@ struct BatchImpl {
             }
             for (int heavy = 1; heavy >= 0; --heavy)       // tau1 != 0 rows of every problem first
                 for (int i = 0; i < n; ++i)
-                    add_segment(seg, i, (b->ctx[i]->H + lv[i].Ty - 1) / lv[i].Ty, (b->Ls + lv[i].nb - 1) / lv[i].nb,
+                    if (b->on_levels[i]) add_segment(seg, i, (b->ctx[i]->H + lv[i].Ty - 1) / lv[i].Ty, (b->Ls + lv[i].nb - 1) / lv[i].nb,
                                 heavy ? rows - 1 : 1, heavy ? 0 : rows - 1, &next);
             b->lv_nseg = (int)seg.size();
             b->lv_blocks = next;
@@ -1682,8 +1702,10 @@ struct BatchImpl {
             const LevelArgs<T, WT>* lv = (const LevelArgs<T, WT>*)b->d_lv;
             points_batch_launch<T, WT>(lv, b->d_pt_seg, b->pt_nseg, zero_in ? 1 : 0, (unsigned)b->pt_blocks, s);
             if (zero_in) {              // X of a cold first iteration is zero, and so are the planes
-                for (fuse_ctx* c : b->ctx)
-                    levels_init_launch<T, WT>(Impl<T>::template lv_args<WT>(c), c->K, Impl<T>::kept(c), 0, s);
+                for (size_t i = 0; i < b->ctx.size(); ++i) {
+                    fuse_ctx* c = b->ctx[i];
+                    if (b->on_levels[i]) levels_init_launch<T, WT>(Impl<T>::template lv_args<WT>(c), c->K, Impl<T>::kept(c), 0, s);
+                }
             } else {
                 levels_batch_launch<T, WT>(lv, b->d_lv_seg, b->lv_nseg, b->K, (unsigned)b->lv_blocks, kLevelThreads,
                                            b->lv_smem, s);
@@ -2663,8 +2685,8 @@ fuse_status fuse_batch_solve(fuse_batch* b, const void* const* Yl, const void* c
         if (st == FUSE_OK) st = zero_state(c, b->stream, iters == 0);
         if (st != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
         c->have_state = true;
-        c->path = b->levels ? 1 : 0;
-        if ((st = settle(c, Yl[i], true, b->levels ? (iters > 0 ? kStateLevels : kStateGiven) : kStateEntries)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
+        c->path = b->on_levels[i] ? 1 : 0;
+        if ((st = settle(c, Yl[i], true, b->on_levels[i] ? (iters > 0 ? kStateLevels : kStateGiven) : kStateEntries)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
     }
     fuse_status st = batch_run(b, iters, iters > 0);
     if (st != FUSE_OK) return st;
@@ -2740,8 +2762,13 @@ fuse_status fuse_batch_set_option(fuse_batch* b, int option, long long value) {
             return batch_set_shape(b, (int)value, b->lat_stages, b->lat_bpb);
         case FUSE_OPT_LATENT_STAGES:
             return batch_set_shape(b, b->lat_target, (int)value, b->lat_bpb);
-        case FUSE_OPT_LATENT_BANDS:
-            return batch_set_shape(b, b->lat_target, b->lat_stages, (int)value);
+        case FUSE_OPT_LATENT_BANDS: {
+            const bool was = b->bands_set;
+            b->bands_set = true;
+            const fuse_status st = batch_set_shape(b, b->lat_target, b->lat_stages, (int)value);
+            if (st != FUSE_OK) b->bands_set = was;
+            return st;
+        }
         default: return bfail(b, FUSE_EINVAL, "unknown batch option");
     }
 }
@@ -2761,10 +2788,13 @@ fuse_status fuse_batch_get_option(fuse_batch* b, int option, long long* value) {
 fuse_status fuse_batch_autotune(fuse_batch* b, const void* const* Yl, const void* const* Yh, int iters) {
     if (!b || !Yl || !Yh || iters < 1) return FUSE_EINVAL;
     if (b->sticky != FUSE_OK) return FUSE_ESTATE;
-    if (b->levels) return fuse_batch_solve(b, Yl, Yh, 0, nullptr, nullptr);   // the pass has one shape
+    // the pass on the compact state has one shape
+    if (std::all_of(b->on_levels.begin(), b->on_levels.end(), [](char v) { return v != 0; }))
+        return fuse_batch_solve(b, Yl, Yh, 0, nullptr, nullptr);
     const bool g = b->use_graph, pr = b->profile;
     b->use_graph = false;
     b->profile = false;
+    b->bands_set = true;
     fuse_status st = fuse_batch_solve(b, Yl, Yh, 0, nullptr, nullptr);   // inputs and zero state
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (st == FUSE_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess))

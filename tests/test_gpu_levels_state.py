@@ -367,3 +367,31 @@ def test_batch_of_both_kinds():
         x = f.solve(a, b, 3, warm=True)[0].clone()
         assert torch.equal(x, f.solve(a, b, 12)[0])
         f.close()
+
+
+@pytest.mark.parametrize("entries", [(0,), (1, 2), (0, 1, 2, 3)])
+def test_batch_of_levels_and_entries(entries):
+    # problems that are not on levels (by choice here, or for want of memory) beside others that are: the
+    # bits of each are those it has alone
+    ps = [small(K=2, S=2, L_s=5, H=h, W=w, seed=40 + h) for h, w in ((32, 64), (40, 40), (48, 160), (24, 24))]
+    ctx = [Fusion.from_problem(p, dtype="f32", wdtype="bf16") for p in ps]
+    yl, yh = [dev(p.Yl) for p in ps], [dev(p.Yh) for p in ps]
+    ref = []
+    for i, (f, a, b) in enumerate(zip(ctx, yl, yh)):
+        if i in entries:
+            f.set_option(FUSE_OPT_LATENT_IMPL, 2)
+        f.weights(b)
+        ref.append(f.solve(a, b, 6)[0].clone())
+    forms = [f.get_option(FUSE_OPT_LATENT_FORM) for f in ctx]
+    assert forms == [0 if i in entries else 2 for i in range(4)]
+    batch = FusionBatch(ctx)
+    for step in range(3):
+        if step == 2:
+            batch.autotune(yl, yh, 1)
+        batch.set_option(FUSE_OPT_GRAPH, int(step != 1))
+        Xs, _ = batch.solve(yl, yh, 6)
+        batch.sync()
+        assert [f.get_option(FUSE_OPT_LATENT_FORM) for f in ctx] == forms
+        for x, y in zip(Xs, ref):
+            assert torch.equal(x, y)
+    batch.close()
