@@ -508,11 +508,12 @@ bool latent_tma_shape(fuse_ctx* c) {
     return true;
 }
 
+// Device memory that the compact state does not take the last of.
+constexpr size_t kLevelsLeave = (size_t)256 << 20;
+
 void levels_free(fuse_ctx* c) {
-    for (void** p : {&c->hdr, &c->tab, &c->pt, &c->omega_was}) {
-        if (*p) cudaFree(*p);
-        *p = nullptr;
-    }
+    if (c->hdr) cudaFree(c->hdr);                           // one allocation
+    c->hdr = c->tab = c->pt = c->omega_was = nullptr;
 }
 
 // Launch shape of the latent pass on the compact state: kLevelThreads per block, rows for about as many
@@ -595,8 +596,18 @@ bool levels_alloc(fuse_ctx* c) {
     void** p[] = {&c->hdr, &c->tab, &c->pt, &c->omega_was};
     const size_t bytes[] = {header_bytes(c->K, nk, c->Ls, c->n, c->esz), nk * c->nP * c->n * c->esz, pts,
                             (size_t)c->nW * c->n * c->wsz};
-    bool ok = true;
-    for (int i = 0; i < 4 && ok; ++i) ok = *p[i] || cudaMalloc(p[i], bytes[i]) == cudaSuccess;
+    size_t total = 0, room = 0, all = 0;
+    for (size_t b : bytes) total += (b + 255) / 256 * 256;
+    // one allocation, hdr; some memory is left for what else a program allocates
+    bool ok = cudaMemGetInfo(&room, &all) == cudaSuccess && room >= total + kLevelsLeave &&
+              cudaMalloc(&c->hdr, total) == cudaSuccess;
+    if (ok) {
+        char* q = (char*)c->hdr;
+        for (int i = 0; i < 4; ++i) {
+            *p[i] = q;
+            q += (bytes[i] + 255) / 256 * 256;
+        }
+    }
     ok = ok && cudaMemsetAsync(c->pt, 0, pts, c->stream) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
