@@ -403,7 +403,14 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
 // (tau, c, m) before it writes any, and no other thread touches those words.  Each launch looks at the
 // state on the device and does nothing where that does not call for it; `work` runs of 128 pixels of
 // one kept offset are shared out over the blocks, a few per SM, so that such a launch costs a few
-// microseconds whatever the problem's size.
+// microseconds whatever the problem's size.  The ranks of a thread lie in planes of their own, so a
+// thread takes its entries through a column of shared memory, and the planes are read and written in
+// whole rows.
+
+// Blocks of a conversion per SM.  Bound by the latency of its scattered reads: the caps trade registers
+// (unbounded 227 for 25 entries in FP32, two blocks) for blocks.
+template <typename T, int K>
+constexpr int window_resident() { return sizeof(T) == 8 ? (K == 1 ? 4 : 2) : (K == 1 ? 6 : 4); }
 
 // Threshold codes of a window, ascending, each with its patch index in the low 5 bits.
 template <typename T, typename WT, int K>
@@ -444,7 +451,7 @@ __device__ __forceinline__ void each_window(const LevelArgs<T, WT>& a, int work,
 // formed (old: the arguments from before).  The entries are then those of a run on the current weights,
 // or to be looked at; with want = kStateEntries or off the grid they go on in the iterate type's arithmetic.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, int want) {
+__global__ void __launch_bounds__(128, window_resident<T, K>()) levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, int want) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
@@ -452,6 +459,8 @@ __global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT>
     const LevelArgs<T, WT> a = now.ctl->was ? old : now;
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
     const T g = a.grid->g;
+    __shared__ T stage[NP * 128];
+    T* col = stage + threadIdx.x;
     each_window<T, WT, K>(a, work, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
         const size_t y = p / a.W, x = p % a.W;
         const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
@@ -475,7 +484,9 @@ __global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT>
             }
             T* eb = reinterpret_cast<T*>(ob);
 #pragma unroll
-            for (int r = 0; r < NP; ++r) eb[(size_t)(key[r] & 31u) * kst] = (T)s[r] * g;
+            for (int r = 0; r < NP; ++r) col[(key[r] & 31u) * 128] = (T)s[r] * g;
+#pragma unroll
+            for (int k = 0; k < NP; ++k) eb[(size_t)k * kst] = col[k * 128];
         }
     });
     if (last_block(now.ctl) && threadIdx.x == 0) {
@@ -484,14 +495,17 @@ __global__ void __launch_bounds__(128) levels_to_entries_kernel(LevelArgs<T, WT>
     }
 }
 
-// The codes of the NP entries at ob, in the order of the keys; false if one is off the grid or above its
-// threshold.
+// The codes of the NP entries at eb, in the order of the keys (col: the thread's column of shared memory);
+// false if one is off the grid or above its threshold.
 template <typename T, int NP>
-__device__ __forceinline__ bool entry_codes(const T* eb, size_t kst, T ig, const ucode_t<T> (&key)[NP], code_t<T> (&s)[NP]) {
+__device__ __forceinline__ bool entry_codes(const T* eb, size_t kst, T ig, const ucode_t<T> (&key)[NP], T* col,
+                                            code_t<T> (&s)[NP]) {
     bool ok = true;
 #pragma unroll
+    for (int k = 0; k < NP; ++k) col[k * 128] = eb[(size_t)k * kst];
+#pragma unroll
     for (int r = 0; r < NP; ++r) {
-        const T v = eb[(size_t)(key[r] & 31u) * kst] * ig, lim = (T)(key[r] >> 5);
+        const T v = col[(key[r] & 31u) * 128] * ig, lim = (T)(key[r] >> 5);
         ok = ok && v >= -lim && v <= lim && v == trunc(v);
         s[r] = to_code(v);
     }
@@ -501,7 +515,7 @@ __device__ __forceinline__ bool entry_codes(const T* eb, size_t kst, T ig, const
 // Whether given entries are those of a run on the current weights, which the update on the grid and the
 // levels need: on the grid, |s| <= mu, and 1-Lipschitz in mu, the state of a stop operator.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128) entries_check_kernel(LevelArgs<T, WT> a, int work) {
+__global__ void __launch_bounds__(128, window_resident<T, K>()) entries_check_kernel(LevelArgs<T, WT> a, int work) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
@@ -509,11 +523,13 @@ __global__ void __launch_bounds__(128) entries_check_kernel(LevelArgs<T, WT> a, 
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n;
     const T ig = a.grid->ig;
     volatile int* off = &a.ctl->off;
+    __shared__ T stage[NP * 128];
+    T* col = stage + threadIdx.x;
     each_window<T, WT, K>(a, work, [&](int si, size_t p, int, int, const U (&key)[NP]) {
         for (int c = 0; c < a.Ls && !*off; ++c) {
             C s[NP];
             bool ok = entry_codes<T, NP>(reinterpret_cast<const T*>(a.e + (size_t)si * NP * kst + (size_t)c * n + p), kst, ig,
-                                         key, s);
+                                         key, col, s);
 #pragma unroll
             for (int r = 1; r < NP; ++r) {
                 const C dm = (C)(key[r] >> 5) - (C)(key[r - 1] >> 5), ds = s[r] - s[r - 1];
@@ -530,20 +546,22 @@ __global__ void __launch_bounds__(128) entries_check_kernel(LevelArgs<T, WT> a, 
 
 // Entries of a run on the current weights -> levels.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128) entries_to_levels_kernel(LevelArgs<T, WT> a, int work) {
+__global__ void __launch_bounds__(128, window_resident<T, K>()) entries_to_levels_kernel(LevelArgs<T, WT> a, int work) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     if (a.ctl->mode != kStateGrid) return;
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
     const T ig = a.grid->ig;
+    __shared__ T stage[NP * 128];
+    T* col = stage + threadIdx.x;
     each_window<T, WT, K>(a, work, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
         const size_t y = p / a.W, x = p % a.W;
         const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
         for (int c = 0; c < a.Ls; ++c) {
             U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
             C s[NP];
-            entry_codes<T, NP>(reinterpret_cast<const T*>(ob), kst, ig, key, s);
+            entry_codes<T, NP>(reinterpret_cast<const T*>(ob), kst, ig, key, col, s);
             U su[NP], mu[NP];
 #pragma unroll
             for (int r = 0; r < NP; ++r) {
@@ -612,6 +630,7 @@ latent_begin_kernel(const T* __restrict__ Y, size_t count, const uint8_t* __rest
         }
     };
     const size_t step = (size_t)gridDim.x * 256, first = (size_t)blockIdx.x * 256 + threadIdx.x;
+    const size_t pstep = step % n;
     size_t p = first % n;                             // the sample's pixel (with a mask)
 #pragma unroll 4
     for (size_t i = first; i < count; i += step) {
@@ -620,7 +639,8 @@ latent_begin_kernel(const T* __restrict__ Y, size_t count, const uint8_t* __rest
             sq += v * v;
             seen += 1.0;
         }
-        if (mask) p = (p + step) % n;
+        p += pstep;
+        if (p >= n) p -= n;
     }
     reduce();
     if (threadIdx.x == 0) {

@@ -47,20 +47,23 @@ void points_launch(const LevelArgs<T, WT>& a, int first, cudaStream_t s) {
                                                                a.grid, first, a.ctl);
 }
 
-// Runs of 128 pixels over the kept offsets, and blocks of a launch over them: as many as fit a device at
-// once (16 of 128 threads per SM), so that a launch that finds nothing to do ends in microseconds.
+// Runs of 128 pixels over the kept offsets, and blocks of a launch over them: as many as fit the device at
+// once, `resident` per SM, so that a launch that finds nothing to do ends in microseconds.
 template <typename T, typename WT>
 static int window_runs(const LevelArgs<T, WT>& a, int kept) {
     return kept * (int)(((size_t)a.H * a.W + 127) / 128);
 }
-static unsigned window_blocks(int runs, int nsm) { return (unsigned)(runs < 16 * nsm ? runs : 16 * nsm); }
+static unsigned window_blocks(int runs, int nsm, int resident) {
+    return (unsigned)(runs < resident * nsm ? runs : resident * nsm);
+}
 
 template <typename T, typename WT>
 void levels_to_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, int K, int kept, int nsm, int want,
                               cudaStream_t s) {
     const int runs = window_runs(now, kept);
     with_grid_k(K, [&](auto k) {
-        levels_to_entries_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(now, old, runs, want);
+        constexpr int KK = decltype(k)::value;
+        levels_to_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(now, old, runs, want);
     });
 }
 
@@ -68,7 +71,8 @@ template <typename T, typename WT>
 void entries_check_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
     const int runs = window_runs(a, kept);
     with_grid_k(K, [&](auto k) {
-        entries_check_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(a, runs);
+        constexpr int KK = decltype(k)::value;
+        entries_check_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(a, runs);
     });
 }
 
@@ -76,7 +80,8 @@ template <typename T, typename WT>
 void entries_to_levels_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
     const int runs = window_runs(a, kept);
     with_grid_k(K, [&](auto k) {
-        entries_to_levels_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(a, runs);
+        constexpr int KK = decltype(k)::value;
+        entries_to_levels_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(a, runs);
     });
 }
 
@@ -84,7 +89,7 @@ template <typename T, typename WT>
 void level_table_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
     const int runs = window_runs(a, kept);
     with_grid_k(K, [&](auto k) {
-        level_table_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm), 128, 0, s>>>(
+        level_table_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm, 16), 128, 0, s>>>(
             a.omega, const_cast<code_t<T>*>(a.tab), a.H, a.W, a.S, a.half, a.coef, a.grid, runs, a.ctl);
     });
 }
