@@ -788,6 +788,10 @@ struct Impl {
         levels_to_entries_launch<T, WT>(lv_args<WT>(c), lv_args<WT>(c, true), c->K, kept(c), c->nsm, want, c->stream);
     }
     template <typename WT>
+    static void save_entries(fuse_ctx* c, void* out) {
+        save_entries_launch<T, WT>(lv_args<WT>(c), lv_args<WT>(c, true), (T*)out, c->K, kept(c), c->nsm, c->stream);
+    }
+    template <typename WT>
     static void check_entries(fuse_ctx* c) {
         entries_check_launch<T, WT>(lv_args<WT>(c), c->K, kept(c), c->nsm, c->stream);
     }
@@ -1020,6 +1024,11 @@ void with_types(const fuse_ctx* c, F&& f) {
     if (c->dtype == FUSE_F64) f(Impl<double>{}, double{});
     else if (c->wdtype == FUSE_BF16) f(Impl<float>{}, __nv_bfloat16{});
     else f(Impl<float>{}, float{});
+}
+
+// The state is known to be entries.
+bool is_entries(const fuse_ctx* c) {
+    return !c->hdr || !grid_options(c) || (!c->captured && (c->settled == kStateEntries || c->settled == kStateGrid));
 }
 
 // The state as entries, for a reader or a pass of them.  want: as in settle.
@@ -2263,12 +2272,24 @@ fuse_status fuse_get_state(fuse_ctx* c, void* dst) {
     if (st != FUSE_OK) return st;
     if (!dst) return fail(c, FUSE_EINVAL, "NULL state buffer");
     if (!c->have_state) return FUSE_ESTATE;
-    if ((st = need_entries(c)) != FUSE_OK) return st;
     const size_t img = c->n * c->Ls * c->esz;
     char* p = (char*)dst;
     void* bufs[] = {c->Lam1, c->U1, c->Lam2, c->U2, c->X};
     for (void* b : bufs) { CK(c, cudaMemcpyAsync(p, b, img, cudaMemcpyDefault, c->stream)); p += img; }
-    CK(c, cudaMemcpyAsync(p, c->Sig, c->sig_bytes, cudaMemcpyDefault, c->stream));
+    // levels go as entries straight to a buffer of this device and stay levels; for any other buffer they
+    // become entries first
+    cudaPointerAttributes at{};
+    const bool here = !is_entries(c) && (uintptr_t)p % c->esz == 0 && cudaPointerGetAttributes(&at, p) == cudaSuccess &&
+                      at.type == cudaMemoryTypeDevice && at.device == c->device;
+    cudaGetLastError();
+    if (here) {
+        with_types(c, [&](auto im, auto w) { im.template save_entries<decltype(w)>(c, p); });
+        c->launches_all++;
+        CKL(c, "save_entries_kernel");
+    } else {
+        if (!is_entries(c) && (st = need_entries(c)) != FUSE_OK) return st;
+        CK(c, cudaMemcpyAsync(p, c->Sig, c->sig_bytes, cudaMemcpyDefault, c->stream));
+    }
     p += c->sig_bytes;
     CK(c, cudaMemcpyAsync(p, c->planes, c->plane_bytes, cudaMemcpyDefault, c->stream));
     CK(c, cudaStreamSynchronize(c->stream));

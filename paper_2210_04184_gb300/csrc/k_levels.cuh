@@ -446,28 +446,21 @@ __device__ __forceinline__ void each_window(const LevelArgs<T, WT>& a, int work,
     }
 }
 
-// Levels -> entries s_k (in the iterate type), where the coming calls want entries (want below
-// kStateLevels), the grid does not carry their inputs, or the weights have changed since the levels were
-// formed (old: the arguments from before).  The entries are then those of a run on the current weights,
-// or to be looked at; with want = kStateEntries or off the grid they go on in the iterate type's arithmetic.
+// Entries s_k of levels, in the iterate type; a: the arguments that the levels were formed with.  out: the
+// entries' planes, which may be those of the levels' values.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128, window_resident<T, K>()) levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, int want) {
+__device__ __forceinline__ void write_entries(const LevelArgs<T, WT>& a, T* out, int work, T* col) {
     using C = code_t<T>;
-    using U = typename grid_code<T>::utype;
+    using U = ucode_t<T>;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
-    if (now.ctl->mode != kStateLevels || !(now.ctl->was || want < kStateLevels || !now.ctl->fit)) return;
-    const LevelArgs<T, WT> a = now.ctl->was ? old : now;
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
     const T g = a.grid->g;
-    __shared__ T stage[NP * 128];
-    T* col = stage + threadIdx.x;
     each_window<T, WT, K>(a, work, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
         const size_t y = p / a.W, x = p % a.W;
         const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
         for (int c = 0; c < a.Ls; ++c) {
-            const size_t o = ((size_t)si * a.Ls + c) * n + p;
+            const size_t o = ((size_t)si * a.Ls + c) * n + p, e0 = (size_t)si * NP * kst + (size_t)c * n + p;
             const Levels l = levels_of<NP>(load_record(a.rec + o).meta, NP == 9 ? make_uint2(0u, 0u) : a.masks[o]);
-            U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
             const U w = a.pt[c * img + ps].after - a.pt[c * img + po].after;
             C s[NP];
             int height = bits_set(l.E);
@@ -478,21 +471,50 @@ __global__ void __launch_bounds__(128, window_resident<T, K>()) levels_to_entrie
                     --height;
                     const int end = r + lowest_bit(l.E >> r) - 1;
                     sg = l.free && height == 0 ? 0 : (((l.G >> end) & 1u) ? 1 : -1);
-                    d = r == 0 && l.q > 0 ? C(0) : (C)(w - ob[(size_t)height * kst]);
+                    d = r == 0 && l.q > 0 ? C(0) : (C)(w - a.e[e0 + (size_t)height * kst]);
                 }
                 s[r] = sg * (C)(key[r] >> 5) + d;
             }
-            T* eb = reinterpret_cast<T*>(ob);
 #pragma unroll
             for (int r = 0; r < NP; ++r) col[(key[r] & 31u) * 128] = (T)s[r] * g;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) eb[(size_t)k * kst] = col[k * 128];
+            for (int k = 0; k < NP; ++k) out[e0 + (size_t)k * kst] = col[k * 128];
         }
     });
+}
+
+// Levels -> entries in place, where the coming calls want entries (want below kStateLevels), the grid does
+// not carry their inputs, or the weights have changed since the levels were formed (old: the arguments
+// from before).  The entries are then those of a run on the current weights, or to be looked at; with
+// want = kStateEntries or off the grid they go on in the iterate type's arithmetic.
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128, window_resident<T, K>())
+levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, int want) {
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    __shared__ T stage[NP * 128];
+    if (now.ctl->mode != kStateLevels || !(now.ctl->was || want < kStateLevels || !now.ctl->fit)) return;
+    const LevelArgs<T, WT> a = now.ctl->was ? old : now;
+    write_entries<T, WT, K>(a, reinterpret_cast<T*>(a.e), work, stage + threadIdx.x);
     if (last_block(now.ctl) && threadIdx.x == 0) {
         now.ctl->mode = want == kStateEntries || !now.ctl->fit ? kStateEntries : now.ctl->was ? kStateGiven : kStateGrid;
         now.ctl->was = 0;
     }
+}
+
+// The state's entries to another buffer, whichever form it is in; it stays what it is.  words: entries.
+template <typename T, typename WT, int K>
+__global__ void __launch_bounds__(128, window_resident<T, K>())
+save_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, T* out, size_t words, int work) {
+    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    __shared__ T stage[NP * 128];
+    if (now.ctl->mode == kStateLevels) {
+        const LevelArgs<T, WT> a = now.ctl->was ? old : now;
+        write_entries<T, WT, K>(a, out, work, stage + threadIdx.x);
+        return;
+    }
+    const T* e = reinterpret_cast<const T*>(now.e);
+#pragma unroll 8
+    for (size_t i = (size_t)blockIdx.x * 128 + threadIdx.x; i < words; i += (size_t)gridDim.x * 128) out[i] = e[i];
 }
 
 // The codes of the NP entries at eb, in the order of the keys (col: the thread's column of shared memory);

@@ -67,6 +67,9 @@ template <typename T, typename WT>
 void levels_to_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, int K, int kept, int nsm, int want,
                               cudaStream_t s);
 template <typename T, typename WT>
+void save_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, T* out, int K, int kept, int nsm,
+                         cudaStream_t s);
+template <typename T, typename WT>
 void entries_check_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s);
 template <typename T, typename WT>
 void entries_to_levels_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s);
@@ -156,6 +159,8 @@ cudaError_t latent_bwd_set_smem(int K, int bytes);
     extern template void points_launch<T, WT>(const LevelArgs<T, WT>&, int, cudaStream_t);                    \
     extern template void levels_to_entries_launch<T, WT>(const LevelArgs<T, WT>&, const LevelArgs<T, WT>&, int, \
                                                          int, int, int, cudaStream_t);                        \
+    extern template void save_entries_launch<T, WT>(const LevelArgs<T, WT>&, const LevelArgs<T, WT>&, T*, int, int, \
+                                                    int, cudaStream_t);                                       \
     extern template void entries_check_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);    \
     extern template void entries_to_levels_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t); \
     extern template void level_table_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);      \

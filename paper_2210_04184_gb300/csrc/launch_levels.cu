@@ -68,6 +68,18 @@ void levels_to_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT
 }
 
 template <typename T, typename WT>
+void save_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, T* out, int K, int kept, int nsm,
+                         cudaStream_t s) {
+    const int runs = window_runs(now, kept);
+    with_grid_k(K, [&](auto k) {
+        constexpr int KK = decltype(k)::value;
+        const size_t words = (size_t)kept * (2 * KK + 1) * (2 * KK + 1) * now.Ls * now.H * now.W;
+        save_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(now, old, out,
+                                                                                                        words, runs);
+    });
+}
+
+template <typename T, typename WT>
 void entries_check_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
     const int runs = window_runs(a, kept);
     with_grid_k(K, [&](auto k) {
@@ -144,6 +156,8 @@ cudaError_t levels_set_smem(int K, int bytes) {
     template void points_launch<T, WT>(const LevelArgs<T, WT>&, int, cudaStream_t);                             \
     template void levels_to_entries_launch<T, WT>(const LevelArgs<T, WT>&, const LevelArgs<T, WT>&, int, int, int, \
                                                   int, cudaStream_t);                                          \
+    template void save_entries_launch<T, WT>(const LevelArgs<T, WT>&, const LevelArgs<T, WT>&, T*, int, int, int, \
+                                             cudaStream_t);                                                    \
     template void entries_check_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);            \
     template void entries_to_levels_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);        \
     template void level_table_launch<T, WT>(const LevelArgs<T, WT>&, int, int, int, cudaStream_t);              \

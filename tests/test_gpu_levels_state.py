@@ -13,6 +13,7 @@ torch = pytest.importorskip("torch")
 
 from oracle import nlpr  # noqa: E402
 from paper_2210_04184_gb300 import build as _build  # noqa: E402
+from paper_2210_04184_gb300 import fuse  # noqa: E402
 from paper_2210_04184_gb300.fuse import (Fusion, FusionBatch, FUSE_OPT_GRAPH, FUSE_OPT_LATENT_FORM,  # noqa: E402
                                          FUSE_OPT_LATENT_IMPL, FUSE_OPT_RESIDUALS)
 
@@ -395,3 +396,33 @@ def test_batch_of_levels_and_entries(entries):
         for x, y in zip(Xs, ref):
             assert torch.equal(x, y)
     batch.close()
+
+
+@pytest.mark.parametrize("K,dtype", [(1, "f32"), (2, "f32"), (2, "f64")])
+def test_saved_states(K, dtype):
+    # a state saved to device memory, or through host memory, or at an odd offset, is the same, and what
+    # it was saved from goes on as if it had not been
+    p = small(K=K)
+    td = torch.float64 if dtype == "f64" else torch.float32
+    f = Fusion.from_problem(p, dtype=dtype, wdtype=dtype)
+    yl, yh = dev(p.Yl, td), dev(p.Yh, td)
+    f.weights(yh)
+    whole = f.solve(yl, yh, 13)[0].clone()
+    f.solve(yl, yh, 6)
+    a = f.get_state()
+    assert f.get_option(FUSE_OPT_LATENT_FORM) == 2        # still levels
+    f.solve(yl, yh, 3, warm=True)
+    odd = torch.empty(a.numel() + 1, dtype=torch.uint8, device="cuda")[1:]
+    host = torch.empty(a.numel(), dtype=torch.uint8)
+    b = f.get_state()
+    f.weights(dev(small(K=K, seed=3).Yh, td))             # saved under other weights: the entries of the run
+    assert torch.equal(f.get_state(), b)
+    f.weights(yh)
+    fuse.fuse_get_state(f.ctx, odd.data_ptr())
+    fuse.fuse_get_state(f.ctx, host.data_ptr())
+    assert torch.equal(odd, b) and torch.equal(host.cuda(), b)
+    assert torch.equal(f.solve(yl, yh, 4, warm=True)[0], whole)
+    f.set_state(a)
+    assert torch.equal(f.get_state(), a)                  # of a state not looked at yet
+    assert torch.equal(f.solve(yl, yh, 7, warm=True)[0], whole)
+    f.close()
