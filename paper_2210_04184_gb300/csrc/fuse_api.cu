@@ -177,7 +177,8 @@ struct fuse_ctx {
     // tab, X with its code sums in pt.  grid [3]: the state's grid, that for omega_was (the weights that
     // levels were formed with, once those have changed), and that for weights up to 1 (fuse_weights).
     // What the state holds is known on the device only (ctl, LatentCtl).  path: kernels of the
-    // iterations' latent pass, 1 = those of k_levels.cuh, which follow ctl, 0 = the entry kernels.
+    // iterations' latent pass, 0 = an entry kernel; and kernels of which ctl picks one: 1 = the pass on
+    // levels and an entry kernel, 2 = the entry kernels of either arithmetic.
     // settled: the last solve's `want` (see settle) while nothing has touched the state since, else -1;
     // captured: a call was captured by the caller, whose replays the host does not see.
     // lat_choice: FUSE_OPT_LATENT_IMPL as the caller chose it, 1 = levels where they apply.
@@ -660,7 +661,7 @@ struct Impl {
                             c->half, bpb, zero_in};
         a.grid = (const LatentGrid<T>*)c->grid;
         // NULL where the state is never anything but entries of the iterate type's arithmetic
-        a.ctl = on_grid(c) && c->path == 1 && !c->lat_in && !c->lat_out ? c->ctl : nullptr;
+        a.ctl = on_grid(c) && c->path != 0 && !c->lat_in && !c->lat_out ? c->ctl : nullptr;
         return a;
     }
     // old: the weights (and their bound) from before the last change
@@ -752,33 +753,36 @@ struct Impl {
     template <typename WT>
     static void latent(fuse_ctx* c, cudaStream_t s, cudaStream_t se, bool zero_in) {
         const unsigned rowsW = (unsigned)(c->half ? c->S + 1 : 2 * c->S + 1);
-        const bool taped = c->lat_in || c->lat_out, beside = c->path == 1 && !taped;
-        if (beside) {
+        const bool taped = c->lat_in || c->lat_out, beside = c->path != 0 && !taped, reg = c->lat_impl == 0;
+        if (beside && c->path == 1) {
             dim3 grid((unsigned)((c->H + c->lv_Ty - 1) / c->lv_Ty), (unsigned)((c->Ls + c->lv_nb - 1) / c->lv_nb), rowsW);
             const LevelArgs<T, WT> a = lv_args<WT>(c);
             points_launch<T, WT>(a, zero_in, s);
             if (zero_in) {
-                levels_init_launch<T, WT>(a, c->K, kept(c), c->lat_impl == 0, s);
-                if (c->lat_impl == 0) se = s;                 // reads the zero entries
+                levels_init_launch<T, WT>(a, c->K, kept(c), reg, s);
+                if (reg) se = s;                              // reads the zero entries
             }
             // X of a cold first iteration is zero with the paper's splitting, and so are the planes
             if (!zero_in || c->xmode == 1)
                 levels_launch<T, WT>(a, c->K, grid, (unsigned)c->lv_threads, c->lv_smem, s);
-        } else {
+        } else if (!beside) {
             se = s;
         }
-        if (c->lat_impl == 1) {
+        if (!reg) {
             dim3 grid((unsigned)((c->H + c->lt_Ty - 1) / c->lt_Ty), (unsigned)((c->Ls + c->lat_bpb - 1) / c->lat_bpb),
                       rowsW);
             const LatentArgs<T, WT> a = lat_args<WT>(c, c->lt_Ty, c->lt_ncons, c->lat_stages, c->lat_bpb, zero_in);
             latent_tma_launch<T, WT>(a, c->K, c->sfmt == 1, grid, (unsigned)(c->lt_ncons + 32), c->lt_smem, se);
-            return;
+            if (!beside || c->path == 1) return;
+            se = s;
         }
+        // the arithmetics that are left to it: on the grid, where the state may be entries on the grid
+        const bool any = on_grid(c) && !taped;
+        const int which = (reg ? 1 : 0) | (any && c->path != 1 ? 2 : 0);
         dim3 grid((unsigned)((c->H + c->lat_Ty - 1) / c->lat_Ty), (unsigned)c->Ls, rowsW);
-        const bool both = on_grid(c) && !taped;
         latent_reg_launch<T, WT>((const T*)c->X, (const WT*)c->omega, (const T*)lat_src(c), (T*)lat_dst(c),
                                  (T*)c->planes, c->H, c->W, c->Ls, c->S, c->lat_Ty, (T)(c->lam2 / c->rho), c->half,
-                                 (const LatentGrid<T>*)c->grid, both ? c->ctl : nullptr, both && !beside, c->K, grid,
+                                 (const LatentGrid<T>*)c->grid, any ? c->ctl : nullptr, which, c->K, grid,
                                  (unsigned)c->lat_threads, c->lat_smem, se);
     }
 
@@ -854,7 +858,7 @@ struct Impl {
     // join_prev: wait for the previous iteration's side branch before the right-hand side.
     static fuse_status iterate(fuse_ctx* c, cudaStream_t s, bool timed, bool zero_in = false, bool monitor = false,
                                bool side = false, bool join_prev = false) {
-        const bool branch = side && c->path == 1;       // an entry kernel beside the pass on the compact state
+        const bool branch = side && c->path != 0;       // a second latent kernel, see fuse_ctx::path
         if (side && join_prev) CK(c, cudaStreamWaitEvent(s, c->side.join, 0));
         if (branch && join_prev) CK(c, cudaStreamWaitEvent(s, c->side.join_e, 0));
         if (c->xmode == 1) {
@@ -1070,7 +1074,7 @@ fuse_status settle(fuse_ctx* c, const void* Yl, bool cold, int want) {
         begin_state(c, Yl, cold, want);
         CKL(c, "latent_begin_kernel");
     }
-    if (!cold && (touched || want != kStateEntries)) {
+    if (!cold && (touched || want == kStateLevels)) {
         const fuse_status st = need_entries(c, want);
         if (st != FUSE_OK) return st;
     }
@@ -1125,7 +1129,7 @@ fuse_status zero_state(fuse_ctx* c, cudaStream_t s, bool clear_sigma = true) {
 }
 
 // kernels launched by one iteration (Impl::iterate)
-int iteration_launches(const fuse_ctx* c) { return (c->xmode == 1 ? 6 : 7) + (c->path == 1 ? 2 : 0); }
+int iteration_launches(const fuse_ctx* c) { return (c->xmode == 1 ? 6 : 7) + (c->path == 0 ? 0 : c->path == 1 ? 2 : 1); }
 
 // Replays `len` iterations from one captured graph (captured on first use; `cold`: the first
 // iteration's latent pass reads no state).
@@ -1142,7 +1146,7 @@ fuse_status launch_loop(fuse_ctx* c, int len, bool cold) {
         // the branches of the last iteration join the loop's stream before the capture ends
         if (forked &&
             (cudaStreamWaitEvent(c->cap_stream, c->side.join, 0) != cudaSuccess ||
-             (c->path == 1 && cudaStreamWaitEvent(c->cap_stream, c->side.join_e, 0) != cudaSuccess)) && st == FUSE_OK)
+             (c->path != 0 && cudaStreamWaitEvent(c->cap_stream, c->side.join_e, 0) != cudaSuccess)) && st == FUSE_OK)
             st = fail(c, FUSE_ECUDA, "cudaStreamWaitEvent");
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
@@ -1181,7 +1185,7 @@ fuse_status monitored_iteration(fuse_ctx* c, bool zero_in) {
     if (c->lt_smem + 2 * (size_t)c->lt_Ty * c->W * c->esz > (size_t)kMaxSmem)
         return fail(c, FUSE_EUNSUPPORTED, "the monitoring latent pass does not fit shared memory");
     fuse_status st = FUSE_OK;
-    if (!zero_in && (st = need_entries(c)) != FUSE_OK) return st;
+    if (!zero_in && !is_entries(c) && (st = need_entries(c)) != FUSE_OK) return st;
     const size_t img = c->n * c->Ls * c->esz;
     cudaStream_t s = c->stream;
     CK(c, cudaMemcpyAsync(c->mL1, c->Lam1, img, cudaMemcpyDeviceToDevice, s));
@@ -1243,7 +1247,12 @@ fuse_status solve_impl(fuse_ctx* c, const void* Yl, const void* Yh, int iters, i
     // of the bulk-copy kernel, or that on the compact state, takes it as zero and overwrites it.
     c->path = !taped && uses_levels(c) ? 1 : 0;
     const bool start = !warm || !c->have_state, cold = start && iters > 0 && (c->lat_impl == 1 || c->path == 1);
-    int want = c->path == 1 ? kStateLevels : c->lat_impl == 0 && !taped ? kStateGrid : kStateEntries;
+    // A monitored iteration needs entries.  Levels pay for their forming and unforming in a continued solve
+    // from so many iterations on.  Calls of 4 and 8 iterations, 25 entries (HS+MS 256): 5.7 and 11.1 ms with
+    // entries on the grid, 6.3 and 7.3 with levels; 9 entries (inpainting 256): 1.05 and 1.85, 1.36 and 1.74.
+    const int plain = iters - (c->monitor && iters > 0 ? 1 : 0), worth = c->K == 1 ? 6 : 4;
+    if (c->path == 1 && c->monitor && !start && plain < worth) c->path = 2;
+    int want = c->path == 1 ? kStateLevels : c->path == 2 || (c->lat_impl == 0 && !taped) ? kStateGrid : kStateEntries;
     if (start) {
         st = zero_state(c, c->stream, !cold);
         if (st != FUSE_OK) return st;

@@ -379,6 +379,7 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
             const int t2 = tm.t2_of(t1, jt);
             T Hacc[VEC], delta[VEC];
             T Macc[MON ? VEC : 1];
+            unsigned long long isq = 0;                  // GRID and MON in FP32: at most 25 VEC terms
             code_t<T> dc[GRID ? VEC : 1], acc[GRID ? VEC : 1], accm[GRID && MON ? VEC : 1];
             if (active) vload<T, VEC>(xo, delta);
 #pragma unroll
@@ -431,8 +432,15 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
                                     acc[j] += 2 * s2 - sc;
                                     if constexpr (MON) {
                                         accm[j] += s2;                      // Q' + Sigma = delta + Sigma'
-                                        const double dd = (double)(s2 - sc) * (double)gr.g;
-                                        dsq += dd * dd;
+                                        // in units of g^2: exact integers in FP32 (at most 2^50 each), one
+                                        // FP64 product per entry less than in units of X
+                                        if constexpr (sizeof(T) == 4) {
+                                            const long long dd = s2 - sc;
+                                            isq += (unsigned long long)(dd * dd);
+                                        } else {
+                                            const double dd = (double)(s2 - sc);
+                                            dsq += dd * dd;
+                                        }
                                     }
                                     sv[j] = (T)s2 * gr.g;
                                 } else {
@@ -519,6 +527,7 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
                     Hacc[j] = active ? latent_h<NP>(delta[j], acc[j], gr.g) : T(0);
                     if constexpr (MON) Macc[j] = active ? latent_h<NP>(delta[j], accm[j], gr.g) : T(0);
                 }
+                if constexpr (MON && sizeof(T) == 4) dsq += (double)isq;
             }
             // A += H_tau; publish H_tau so the row can form V(m) += H_tau(m + (0, tau2))
             T* ht = Hb + (size_t)hb * tile + (size_t)r * W;
@@ -562,6 +571,7 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
         // Xs is rewritten by the next band only after every thread has crossed the last tau2's
         // barrier, that is after every read of it (Xo and Vs are read by their owner only)
     }
+    if constexpr (MON && GRID) dsq *= (double)gr.g * (double)gr.g;
     if constexpr (MON) {
         // the block's sum of (Sigma' - Sigma)^2 over its consumers, in a fixed order
         __shared__ double s_red[8];

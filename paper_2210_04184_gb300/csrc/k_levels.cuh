@@ -150,8 +150,8 @@ __device__ __forceinline__ void window_codes(const WT* __restrict__ om, int y, i
     }
 }
 
-// Prefix sums of the sorted threshold codes of every window, unless they are those of the current weights
-// already; `work` runs of 128 pixels of one kept offset, shared out over the blocks.
+// Prefix sums of the sorted threshold codes of every window, where levels need them and they are not those
+// of the current weights already; `work` runs of 128 pixels of one kept offset, shared out over the blocks.
 template <typename T, typename WT, int K>
 __global__ void __launch_bounds__(128)
 level_table_kernel(const WT* __restrict__ omega, code_t<T>* __restrict__ tab, int H, int W, int S, int half, T coef,
@@ -159,7 +159,7 @@ level_table_kernel(const WT* __restrict__ omega, code_t<T>* __restrict__ tab, in
     using C = code_t<T>;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     __shared__ C sm[128 * NP];                        // NP is odd: conflict-free
-    if (ctl->table) return;
+    if (ctl->table || ctl->mode != kStateLevels) return;
     const size_t n = (size_t)H * W;
     const int runs = (int)((n + 127) / 128);
     const TauMap tm{S, half};

@@ -28,11 +28,11 @@ void latent_tma_launch(const LatentArgs<T, WT>& a, int K, bool int16_state, dim3
 template <typename T, typename WT>
 void latent_tma_batch_launch(const LatentArgs<T, WT>* args, const Segment* seg, int nseg, int zero_in, int K,
                              bool int16_state, unsigned blocks, unsigned threads, size_t smem, cudaStream_t s);
-// Register-staged latent pass; ctl: run where the state is entries, with `on_grid` also those on the
-// grid (NULL: run, in the iterate type's arithmetic).
+// Register-staged latent pass: which & 1 in the iterate type's arithmetic, which & 2 on the grid; ctl: each
+// where the state calls for it (NULL: anyway).
 template <typename T, typename WT>
 void latent_reg_launch(const T* X, const WT* omega, const T* Sig, T* Sout, T* planes, int H, int W, int Ls, int S,
-                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, const LatentCtl* ctl, bool on_grid,
+                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, const LatentCtl* ctl, int which,
                        int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s);
 // Monitoring latent pass (state as entries of the iterate type): also the latent parts of the residuals.
 template <typename T, typename WT>
@@ -171,7 +171,7 @@ cudaError_t latent_bwd_set_smem(int K, int bytes);
     extern template void latent_tma_batch_launch<T, WT>(const LatentArgs<T, WT>*, const Segment*, int, int, int, \
                                                         bool, unsigned, unsigned, size_t, cudaStream_t);       \
     extern template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, \
-                                                  T, int, const LatentGrid<T>*, const LatentCtl*, bool, int, dim3, unsigned, \
+                                                  T, int, const LatentGrid<T>*, const LatentCtl*, int, int, dim3, unsigned, \
                                                   size_t, cudaStream_t);                                       \
     extern template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, dim3, unsigned, size_t,    \
                                                       cudaStream_t);                                           \

@@ -54,17 +54,18 @@ void latent_monitor_launch(const LatentArgs<T, WT>& a, int K, dim3 grid, unsigne
 
 template <typename T, typename WT>
 void latent_reg_launch(const T* X, const WT* omega, const T* Sig, T* Sout, T* planes, int H, int W, int Ls, int S,
-                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, const LatentCtl* ctl, bool on_grid,
+                       int Ty, T coef, int half, const LatentGrid<T>* grid_d, const LatentCtl* ctl, int which,
                        int K, dim3 grid, unsigned threads, size_t smem, cudaStream_t s) {
     constexpr int VEC = 16 / sizeof(T);
     with_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
         if constexpr (latent_grid_k(KK)) {
-            if (on_grid)
+            if (which & 2)
                 latent_kernel<T, WT, KK, VEC, true><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W, Ls,
                                                                                 S, Ty, coef, half, grid_d, ctl);
         }
-        latent_kernel<T, WT, KK, VEC, false><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W, Ls, S, Ty,
+        if (which & 1)
+            latent_kernel<T, WT, KK, VEC, false><<<grid, threads, smem, s>>>(X, omega, Sig, Sout, planes, H, W, Ls, S, Ty,
                                                                          coef, half, grid_d, ctl);
     });
 }
@@ -113,7 +114,7 @@ cudaError_t latent_batch_set_smem(int K, int bytes) {
     template void latent_monitor_launch<T, WT>(const LatentArgs<T, WT>&, int, dim3, unsigned, size_t,            \
                                                cudaStream_t);                                                  \
     template void latent_reg_launch<T, WT>(const T*, const WT*, const T*, T*, T*, int, int, int, int, int, T,    \
-                                           int, const LatentGrid<T>*, const LatentCtl*, bool, int, dim3, unsigned,       \
+                                           int, const LatentGrid<T>*, const LatentCtl*, int, int, dim3, unsigned,       \
                                            size_t, cudaStream_t);                                              \
     template cudaError_t latent_set_smem<T, WT>(int, int);                                                      \
     template cudaError_t latent_batch_set_smem<T, WT>(int, int);

@@ -426,3 +426,27 @@ def test_saved_states(K, dtype):
     assert torch.equal(f.get_state(), a)                  # of a state not looked at yet
     assert torch.equal(f.solve(yl, yh, 7, warm=True)[0], whole)
     f.close()
+
+
+@pytest.mark.parametrize("K", [1, 2])
+def test_monitored_calls_of_every_length(K):
+    # calls of few iterations stay entries between their monitored ones, long ones form levels: the
+    # same bits as without the monitor, and the monitor's own results
+    p = small(K=K)
+    f, g = (Fusion.from_problem(p, dtype="f32", wdtype="f32") for _ in range(2))
+    e = Fusion.from_problem(p, dtype="f32", wdtype="f32")
+    f.set_option(FUSE_OPT_RESIDUALS, 1)
+    e.set_option(FUSE_OPT_RESIDUALS, 1)
+    yl, yh = dev(p.Yl), dev(p.Yh)
+    for c in (f, g, e):
+        c.weights(yh)
+    done = 0
+    for i, it in enumerate((1, 1, 2, 3, 20, 1, 9, 25, 4)):
+        X = f.solve(yl, yh, it, warm=i > 0)[0].clone()
+        assert torch.equal(X, g.solve(yl, yh, it, warm=i > 0)[0])
+        done += it
+        e.solve(yl, yh, done)
+        assert f.residuals() == e.residuals()
+    assert torch.equal(f.get_state(), g.get_state())
+    for c in (f, g, e):
+        c.close()
