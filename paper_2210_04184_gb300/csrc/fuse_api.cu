@@ -599,9 +599,13 @@ bool levels_alloc(fuse_ctx* c) {
                             (size_t)c->nW * c->n * c->wsz};
     size_t total = 0, room = 0, all = 0;
     for (size_t b : bytes) total += (b + 255) / 256 * 256;
-    // one allocation, hdr; some memory is left for what else a program allocates
+    // one allocation, hdr; some memory is left for what else a program allocates.  A stream that another
+    // thread captures meanwhile, in whichever mode, is not disturbed by it.
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     bool ok = cudaMemGetInfo(&room, &all) == cudaSuccess && room >= total + kLevelsLeave &&
               cudaMalloc(&c->hdr, total) == cudaSuccess;
+    cudaThreadExchangeStreamCaptureMode(&mode);
     if (ok) {
         char* q = (char*)c->hdr;
         for (int i = 0; i < 4; ++i) {

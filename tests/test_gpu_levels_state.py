@@ -450,3 +450,69 @@ def test_monitored_calls_of_every_length(K):
     assert torch.equal(f.get_state(), g.get_state())
     for c in (f, g, e):
         c.close()
+
+
+def test_first_solve_while_another_thread_captures():
+    # the first solve of a context allocates the levels' buffers: a capture that another thread has under
+    # way, in the mode that forbids allocations everywhere, goes on, and the solve is on levels
+    import threading
+    p = small(K=2)
+    yl, yh = dev(p.Yl), dev(p.Yh)
+    ref, f = (Fusion.from_problem(p, dtype="f32", wdtype="f32") for _ in range(2))
+    ref.weights(yh)
+    want = ref.solve(yl, yh, 5)[0].clone()
+    X, mine, a, errors = torch.empty_like(want), torch.cuda.Stream(), torch.ones(64, device="cuda"), []
+    f.weights(yh)
+    fuse.fuse_set_option(f.ctx, FUSE_OPT_GRAPH, 0)
+    torch.cuda.synchronize()
+
+    def run():
+        try:
+            fuse.fuse_set_stream(f.ctx, mine.cuda_stream)
+            fuse.fuse_solve(f.ctx, yl.data_ptr(), yh.data_ptr(), 5, 0, X.data_ptr(), None)
+        except Exception as e:                            # noqa: BLE001
+            errors.append(e)
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="global"):
+        b = a * 2.0
+        t = threading.Thread(target=run)
+        t.start()
+        t.join()
+        b = b + 1.0
+    g.replay()
+    torch.cuda.synchronize()
+    assert not errors and torch.equal(X, want) and (b == 3.0).all()
+    assert f.get_option(FUSE_OPT_LATENT_FORM) == 2
+    f.close()
+    ref.close()
+
+
+def test_captured_batch():
+    # a batch solve captured by the caller: thresholds and forms are those of the replay's time
+    ps = [small(K=2, H=32, W=64, seed=5), small(K=2, H=40, W=40, seed=6)]
+    ctx = [Fusion.from_problem(p, dtype="f32", wdtype="bf16") for p in ps]
+    yl, yh = [dev(p.Yl) for p in ps], [dev(p.Yh) for p in ps]
+    guides = [[dev(small(H=p.H, W=p.W, seed=s).Yh) for p in ps] for s in (7, 8)]
+    batch = FusionBatch(ctx)
+    batch.set_option(FUSE_OPT_GRAPH, 0)
+    for f, b in zip(ctx, yh):
+        f.weights(b)
+    batch.solve(yl, yh, 5)
+    batch.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        Xs, _ = batch.solve(yl, yh, 5)
+    for scale, form in ((1.0, 2), (1e-3, 0), (1.0, 2)):   # the data too
+        for gs in guides:
+            for f, w in zip(ctx, gs):
+                f.weights(w)
+            for a, p in zip(yl, ps):
+                a.copy_(dev(p.Yl) * scale)
+            g.replay()
+            torch.cuda.synchronize()
+            got = [x.clone() for x in Xs]
+            for f, a, b, x in zip(ctx, yl, yh, got):
+                assert f.get_option(FUSE_OPT_LATENT_FORM) == form
+                assert torch.equal(x, f.solve(a, b, 5)[0])
+    batch.close()
