@@ -515,6 +515,8 @@ def run_batch(a, rank, world, local_rank):
     lat_ms, lat_n = batch.profile(FUSE_K_LATENT, reset=True)
     batch.set_option(FUSE_OPT_PROFILE, 0)
     batch.sync()
+    from paper_2210_04184_gb300.fuse import FUSE_OPT_LATENT_FORM
+    on_levels = [f.get_option(FUSE_OPT_LATENT_FORM) == 2 for f in fs]
 
     # end to end through the host-buffer batch entry point: pinned inputs copied in, weights,
     # batched solve, Z of every problem read back, every step
@@ -576,7 +578,7 @@ def run_batch(a, rank, world, local_rank):
     peak_src = "measured" if hbm else "fallback"
     hbm = hbm or 6800.0
     per_launch_ms = lat_ms / max(lat_n, 1)
-    lb = sum(level_bytes(p, 4) for p in ps)
+    lb = sum(level_bytes(p, 4) if lv else latent_bytes(p, 4, 2) for p, lv in zip(ps, on_levels))
     achieved = lb / (per_launch_ms / 1e3) / 1e9
     out = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": a.steps,
@@ -584,7 +586,7 @@ def run_batch(a, rank, world, local_rank):
         "vs_baseline": None, "dtype": "f32", "data": "synthetic",
         "config": dict(batch_config(ps, iters, world), latent_shape=shape),
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
-                     "traffic": latent_traffic("batch", px), "kernel": "latent_levels_batch_kernel",
+                     "traffic": latent_traffic("batch", px), "kernel": "latent_levels_batch_kernel" if any(on_levels) else "latent_tma_batch_kernel",
                      "algorithmic_bytes_per_launch": lb, "avg_launch_ms": per_launch_ms, "launches": lat_n,
                      "timing": "CUDA events around each latent launch in a separate profiled step",
                      "peak_source": peak_src, "nominal_peak": NOMINAL_HBM_GBS},
@@ -755,6 +757,8 @@ def single_problem(a, name, rank, dist, keep=False):
     lat_ms, lat_n = f.profile(FUSE_K_LATENT, reset=True)
     f.set_option(FUSE_OPT_PROFILE, 0)
     f.sync()
+    from paper_2210_04184_gb300.fuse import FUSE_OPT_LATENT_FORM
+    on_levels = f.get_option(FUSE_OPT_LATENT_FORM) == 2
 
     # end to end through the host-buffer entry point (pinned inputs, Z read back each step)
     e2e = None
@@ -781,7 +785,7 @@ def single_problem(a, name, rank, dist, keep=False):
     hbm = hbm or 6800.0
     per_launch_ms = lat_ms / max(lat_n, 1)
     fixed = keep and a.fixed_state
-    levels = p.K in (1, 2) and not fixed and not (p.K == 1 and p.S == 1 and esz == 4)
+    levels = on_levels
     lb = level_bytes(p, esz) if levels else latent_bytes(p, esz, wsz, ssz=2 if fixed else None)
     traffic = None
     if name.startswith("hsms") and meta["wdtype"] == "bf16" and not fixed:
