@@ -111,7 +111,7 @@ latent_kernel(const T* __restrict__ X, const WT* __restrict__ omega, const T* Si
                         if constexpr (GRID) {
                             const code_t<T> sc = to_code(s[k2].v[j] * gr.ig), s2 = mu[j + k2].clamp(sc - dc[j]);
                             acc[j] += 2 * s2 - sc;
-                            s[k2].v[j] = (T)s2 * gr.g;
+                            s[k2].v[j] = mu[j + k2].entry(s2, gr.g);
                         } else {
                             const T u = s[k2].v[j] - delta[j];     // -v
                             const T s2 = mu[j + k2].clamp(u);      // Sigma' = -clamp(v)
@@ -442,7 +442,7 @@ __device__ __forceinline__ void latent_tma_body(const LatentArgs<T, WT>& args, i
                                             dsq += dd * dd;
                                         }
                                     }
-                                    sv[j] = (T)s2 * gr.g;
+                                    sv[j] = mu[j + k2].entry(s2, gr.g);
                                 } else {
                                     const T u = sv[j] - delta[j];
                                     const T s2 = mu[j + k2].clamp(u);

@@ -134,10 +134,16 @@ __device__ __forceinline__ void sort_network(C (&v)[N]) {
     }
 }
 
-// Threshold codes of the patch window of (y, x): code of coef omega_tau(m + k), k in row-major order.
+// Pixels of a run that a block of the conversions takes at a time, a thread each: two columns of shared
+// memory per thread fit 48 KB.
+template <typename T, int K>
+__host__ __device__ constexpr int window_run() { return sizeof(T) == 8 && K == 2 ? 64 : 128; }
+
+// Threshold codes of the patch window of (y, x): code of coef omega_tau(m + k), k in row-major order; the
+// thresholds themselves to a column of shared memory ([NP][window_run]), where given.
 template <typename T, typename WT, int K>
 __device__ __forceinline__ void window_codes(const WT* __restrict__ om, int y, int x, int H, int W, T coef, T ig,
-                                             code_t<T> (&v)[(2 * K + 1) * (2 * K + 1)]) {
+                                             code_t<T> (&v)[(2 * K + 1) * (2 * K + 1)], T* mus = nullptr) {
     constexpr int PS = 2 * K + 1;
     int col[PS];
 #pragma unroll
@@ -146,7 +152,11 @@ __device__ __forceinline__ void window_codes(const WT* __restrict__ om, int y, i
     for (int i = 0; i < PS; ++i) {
         const WT* row = om + (size_t)wrap1(y + i - K, H) * W;
 #pragma unroll
-        for (int j = 0; j < PS; ++j) v[i * PS + j] = mu_code(coef * (T)wload(row + col[j]), ig);
+        for (int j = 0; j < PS; ++j) {
+            const T mu = coef * (T)wload(row + col[j]);
+            v[i * PS + j] = mu_code(mu, ig);
+            if (mus) mus[(i * PS + j) * window_run<T, K>()] = mu;
+        }
     }
 }
 
@@ -401,8 +411,8 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
 // ---- the forms of the state -------------------------------------------------------------------
 // The conversions are exact and in place: the thread of a (tau, pixel) reads every word of one
 // (tau, c, m) before it writes any, and no other thread touches those words.  Each launch looks at the
-// state on the device and does nothing where that does not call for it; `work` runs of 128 pixels of
-// one kept offset are shared out over the blocks, a few per SM, so that such a launch costs a few
+// state on the device and does nothing where that does not call for it; `work` runs of window_run
+// pixels of one kept offset are shared out over the blocks, a few per SM, so that such a launch costs a few
 // microseconds whatever the problem's size.  The ranks of a thread lie in planes of their own, so a
 // thread takes its entries through a column of shared memory, and the planes are read and written in
 // whole rows.
@@ -410,38 +420,39 @@ __device__ __forceinline__ void latent_levels_body(const LevelArgs<T, WT>& a, in
 // Blocks of a conversion per SM.  Bound by the latency of its scattered reads: the caps trade registers
 // (unbounded 227 for 25 entries in FP32, two blocks) for blocks.
 template <typename T, int K>
-constexpr int window_resident() { return sizeof(T) == 8 ? (K == 1 ? 4 : 2) : (K == 1 ? 6 : 4); }
+__host__ __device__ constexpr int window_resident() { return sizeof(T) == 8 ? 4 : (K == 1 ? 6 : 4); }
 
 // Threshold codes of a window, ascending, each with its patch index in the low 5 bits.
 template <typename T, typename WT, int K>
-__device__ __forceinline__ void window_keys(const WT* __restrict__ om, int y, int x, int H, int W, T coef, T ig,
+__device__ __forceinline__ void window_keys(const WT* __restrict__ om, int y, int x, int H, int W, T coef, T ig, T* mus,
                                             typename grid_code<T>::utype (&key)[(2 * K + 1) * (2 * K + 1)]) {
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     using U = typename grid_code<T>::utype;
     code_t<T> v[NP];
-    window_codes<T, WT, K>(om, y, x, H, W, coef, ig, v);
+    window_codes<T, WT, K>(om, y, x, H, W, coef, ig, v, mus);
 #pragma unroll
     for (int k = 0; k < NP; ++k) key[k] = ((U)v[k] << 5) | (U)k;
     sort_network<NP>(key);
 }
 
-// The pixels of a conversion: f(kept offset, pixel, tau, keys of its window).
+// The pixels of a conversion: f(kept offset, pixel, tau, keys of its window); mus: see window_codes.
 template <typename T, typename WT, int K, typename F>
-__device__ __forceinline__ void each_window(const LevelArgs<T, WT>& a, int work, F f) {
+__device__ __forceinline__ void each_window(const LevelArgs<T, WT>& a, int work, T* mus, F f) {
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     const size_t n = (size_t)a.H * a.W;
-    const int runs = (int)((n + 127) / 128);
+    constexpr int R = window_run<T, K>();
+    const int runs = (int)((n + R - 1) / R);
     const TauMap tm{a.S, a.half};
     const T ig = a.grid->ig;
     for (int job = blockIdx.x; job < work; job += gridDim.x) {
         const int si = job / runs;
-        const size_t p = (size_t)(job - si * runs) * 128 + threadIdx.x;
+        const size_t p = (size_t)(job - si * runs) * R + threadIdx.x;
         if (p >= n) continue;
         int t1, t2;
         tau_of_state_index(si, a.S, a.half, &t1, &t2);
         ucode_t<T> key[NP];
         window_keys<T, WT, K>(a.omega + (size_t)tm.w_index(t1, t2) * n, (int)(p / a.W), (int)(p % a.W), a.H, a.W, a.coef,
-                              ig, key);
+                              ig, mus, key);
         f(si, p, t1, t2, key);
     }
 }
@@ -449,13 +460,13 @@ __device__ __forceinline__ void each_window(const LevelArgs<T, WT>& a, int work,
 // Entries s_k of levels, in the iterate type; a: the arguments that the levels were formed with.  out: the
 // entries' planes, which may be those of the levels' values.
 template <typename T, typename WT, int K>
-__device__ __forceinline__ void write_entries(const LevelArgs<T, WT>& a, T* out, int work, T* col) {
+__device__ __forceinline__ void write_entries(const LevelArgs<T, WT>& a, T* out, int work, T* col, T* mus) {
     using C = code_t<T>;
     using U = ucode_t<T>;
-    constexpr int NP = (2 * K + 1) * (2 * K + 1);
+    constexpr int NP = (2 * K + 1) * (2 * K + 1), R = window_run<T, K>();
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
     const T g = a.grid->g;
-    each_window<T, WT, K>(a, work, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
+    each_window<T, WT, K>(a, work, mus, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
         const size_t y = p / a.W, x = p % a.W;
         const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
         for (int c = 0; c < a.Ls; ++c) {
@@ -476,9 +487,10 @@ __device__ __forceinline__ void write_entries(const LevelArgs<T, WT>& a, T* out,
                 s[r] = sg * (C)(key[r] >> 5) + d;
             }
 #pragma unroll
-            for (int r = 0; r < NP; ++r) col[(key[r] & 31u) * 128] = (T)s[r] * g;
+            for (int r = 0; r < NP; ++r) col[(key[r] & 31u) * R] = (T)s[r] * g;
 #pragma unroll
-            for (int k = 0; k < NP; ++k) out[e0 + (size_t)k * kst] = col[k * 128];
+            for (int k = 0; k < NP; ++k)                  // see latent_bound::entry
+                out[e0 + (size_t)k * kst] = SymBound<T>::of(mus[k * R]).clamp(col[k * R]);
         }
     });
 }
@@ -488,13 +500,14 @@ __device__ __forceinline__ void write_entries(const LevelArgs<T, WT>& a, T* out,
 // from before).  The entries are then those of a run on the current weights, or to be looked at; with
 // want = kStateEntries or off the grid they go on in the iterate type's arithmetic.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128, window_resident<T, K>())
+__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>())
 levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, int want) {
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
-    __shared__ T stage[NP * 128];
+    constexpr int R = window_run<T, K>();
+    __shared__ T stage[2 * NP * R];
     if (now.ctl->mode != kStateLevels || !(now.ctl->was || want < kStateLevels || !now.ctl->fit)) return;
     const LevelArgs<T, WT> a = now.ctl->was ? old : now;
-    write_entries<T, WT, K>(a, reinterpret_cast<T*>(a.e), work, stage + threadIdx.x);
+    write_entries<T, WT, K>(a, reinterpret_cast<T*>(a.e), work, stage + threadIdx.x, stage + NP * R + threadIdx.x);
     if (last_block(now.ctl) && threadIdx.x == 0) {
         now.ctl->mode = want == kStateEntries || !now.ctl->fit ? kStateEntries : now.ctl->was ? kStateGiven : kStateGrid;
         now.ctl->was = 0;
@@ -503,32 +516,33 @@ levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, i
 
 // The state's entries to another buffer, whichever form it is in; it stays what it is.  words: entries.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128, window_resident<T, K>())
+__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>())
 save_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, T* out, size_t words, int work) {
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
-    __shared__ T stage[NP * 128];
+    constexpr int R = window_run<T, K>();
+    __shared__ T stage[2 * NP * R];
     if (now.ctl->mode == kStateLevels) {
         const LevelArgs<T, WT> a = now.ctl->was ? old : now;
-        write_entries<T, WT, K>(a, out, work, stage + threadIdx.x);
+        write_entries<T, WT, K>(a, out, work, stage + threadIdx.x, stage + NP * R + threadIdx.x);
         return;
     }
     const T* e = reinterpret_cast<const T*>(now.e);
 #pragma unroll 8
-    for (size_t i = (size_t)blockIdx.x * 128 + threadIdx.x; i < words; i += (size_t)gridDim.x * 128) out[i] = e[i];
+    for (size_t i = (size_t)blockIdx.x * R + threadIdx.x; i < words; i += (size_t)gridDim.x * R) out[i] = e[i];
 }
 
 // The codes of the NP entries at eb, in the order of the keys (col: the thread's column of shared memory);
-// false if one is off the grid or above its threshold.
-template <typename T, int NP>
+// false if one is above its threshold's code, or neither on the grid nor at its threshold (mus).
+template <typename T, int NP, int R>
 __device__ __forceinline__ bool entry_codes(const T* eb, size_t kst, T ig, const ucode_t<T> (&key)[NP], T* col,
-                                            code_t<T> (&s)[NP]) {
+                                            const T* mus, code_t<T> (&s)[NP]) {
     bool ok = true;
 #pragma unroll
-    for (int k = 0; k < NP; ++k) col[k * 128] = eb[(size_t)k * kst];
+    for (int k = 0; k < NP; ++k) col[k * R] = eb[(size_t)k * kst];
 #pragma unroll
     for (int r = 0; r < NP; ++r) {
-        const T v = col[(key[r] & 31u) * 128] * ig, lim = (T)(key[r] >> 5);
-        ok = ok && v >= -lim && v <= lim && v == trunc(v);
+        const T e = col[(key[r] & 31u) * R], v = e * ig, lim = (T)(key[r] >> 5);
+        ok = ok && v >= -lim && v <= lim && (v == trunc(v) || (e < T(0) ? -e : e) == mus[(key[r] & 31u) * R]);
         s[r] = to_code(v);
     }
     return ok;
@@ -537,7 +551,7 @@ __device__ __forceinline__ bool entry_codes(const T* eb, size_t kst, T ig, const
 // Whether given entries are those of a run on the current weights, which the update on the grid and the
 // levels need: on the grid, |s| <= mu, and 1-Lipschitz in mu, the state of a stop operator.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128, window_resident<T, K>()) entries_check_kernel(LevelArgs<T, WT> a, int work) {
+__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>()) entries_check_kernel(LevelArgs<T, WT> a, int work) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
@@ -545,13 +559,14 @@ __global__ void __launch_bounds__(128, window_resident<T, K>()) entries_check_ke
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n;
     const T ig = a.grid->ig;
     volatile int* off = &a.ctl->off;
-    __shared__ T stage[NP * 128];
-    T* col = stage + threadIdx.x;
-    each_window<T, WT, K>(a, work, [&](int si, size_t p, int, int, const U (&key)[NP]) {
+    constexpr int R = window_run<T, K>();
+    __shared__ T stage[2 * NP * R];
+    T *col = stage + threadIdx.x, *mus = col + NP * R;
+    each_window<T, WT, K>(a, work, mus, [&](int si, size_t p, int, int, const U (&key)[NP]) {
         for (int c = 0; c < a.Ls && !*off; ++c) {
             C s[NP];
-            bool ok = entry_codes<T, NP>(reinterpret_cast<const T*>(a.e + (size_t)si * NP * kst + (size_t)c * n + p), kst, ig,
-                                         key, col, s);
+            bool ok = entry_codes<T, NP, R>(reinterpret_cast<const T*>(a.e + (size_t)si * NP * kst + (size_t)c * n + p), kst, ig,
+                                         key, col, mus, s);
 #pragma unroll
             for (int r = 1; r < NP; ++r) {
                 const C dm = (C)(key[r] >> 5) - (C)(key[r - 1] >> 5), ds = s[r] - s[r - 1];
@@ -568,22 +583,23 @@ __global__ void __launch_bounds__(128, window_resident<T, K>()) entries_check_ke
 
 // Entries of a run on the current weights -> levels.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(128, window_resident<T, K>()) entries_to_levels_kernel(LevelArgs<T, WT> a, int work) {
+__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>()) entries_to_levels_kernel(LevelArgs<T, WT> a, int work) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
     if (a.ctl->mode != kStateGrid) return;
     const size_t n = (size_t)a.H * a.W, kst = (size_t)a.Ls * n, Wp = a.W + 2 * a.S, img = a.H * Wp;
     const T ig = a.grid->ig;
-    __shared__ T stage[NP * 128];
-    T* col = stage + threadIdx.x;
-    each_window<T, WT, K>(a, work, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
+    constexpr int R = window_run<T, K>();
+    __shared__ T stage[2 * NP * R];
+    T *col = stage + threadIdx.x, *mus = col + NP * R;
+    each_window<T, WT, K>(a, work, mus, [&](int si, size_t p, int t1, int t2, const U (&key)[NP]) {
         const size_t y = p / a.W, x = p % a.W;
         const size_t po = y * Wp + a.S + x, ps = (size_t)wrap1((int)y - t1, a.H) * Wp + a.S + x - t2;
         for (int c = 0; c < a.Ls; ++c) {
             U* ob = a.e + (size_t)si * NP * kst + (size_t)c * n + p;
             C s[NP];
-            entry_codes<T, NP>(reinterpret_cast<const T*>(ob), kst, ig, key, col, s);
+            entry_codes<T, NP, R>(reinterpret_cast<const T*>(ob), kst, ig, key, col, mus, s);
             U su[NP], mu[NP];
 #pragma unroll
             for (int r = 0; r < NP; ++r) {

@@ -136,10 +136,13 @@ struct latent_bound {
 template <typename T>
 struct latent_bound<T, true> {
     code_t<T> m;
-    __device__ __forceinline__ static latent_bound of(T mu, T ig) { return {mu_code(mu, ig)}; }
+    SymBound<T> b;
+    __device__ __forceinline__ static latent_bound of(T mu, T ig) { return {mu_code(mu, ig), SymBound<T>::of(mu)}; }
     __device__ __forceinline__ code_t<T> clamp(code_t<T> u) const { return u > m ? m : (u < -m ? -m : u); }
+    // The entry of code s, as it is stored.  An entry at a threshold that was rounded up is stored as the
+    // threshold itself, so |s| <= mu holds for every stored state; its code is that of mu.
+    __device__ __forceinline__ T entry(code_t<T> s, T g) const { return b.clamp((T)s * g); }
 };
-
 // Code of an X value: rounded to nearest, modulo 2^32 (FP64: 2^64).  Differences of codes are taken
 // modulo as well; they are used only where |delta| < kBigMove g.
 __device__ __forceinline__ int32_t x_code(float x, float ig) {

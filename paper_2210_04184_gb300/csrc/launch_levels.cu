@@ -47,11 +47,11 @@ void points_launch(const LevelArgs<T, WT>& a, int first, cudaStream_t s) {
                                                                a.grid, first, a.ctl);
 }
 
-// Runs of 128 pixels over the kept offsets, and blocks of a launch over them: as many as fit the device at
+// Runs of pixels over the kept offsets, and blocks of a launch over them: as many as fit the device at
 // once, `resident` per SM, so that a launch that finds nothing to do ends in microseconds.
 template <typename T, typename WT>
-static int window_runs(const LevelArgs<T, WT>& a, int kept) {
-    return kept * (int)(((size_t)a.H * a.W + 127) / 128);
+static int window_runs(const LevelArgs<T, WT>& a, int kept, int run) {
+    return kept * (int)(((size_t)a.H * a.W + run - 1) / run);
 }
 static unsigned window_blocks(int runs, int nsm, int resident) {
     return (unsigned)(runs < resident * nsm ? runs : resident * nsm);
@@ -60,46 +60,46 @@ static unsigned window_blocks(int runs, int nsm, int resident) {
 template <typename T, typename WT>
 void levels_to_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, int K, int kept, int nsm, int want,
                               cudaStream_t s) {
-    const int runs = window_runs(now, kept);
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        levels_to_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(now, old, runs, want);
+        const int runs = window_runs(now, kept, window_run<T, KK>());
+        levels_to_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(now, old, runs, want);
     });
 }
 
 template <typename T, typename WT>
 void save_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& old, T* out, int K, int kept, int nsm,
                          cudaStream_t s) {
-    const int runs = window_runs(now, kept);
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
+        const int runs = window_runs(now, kept, window_run<T, KK>());
         const size_t words = (size_t)kept * (2 * KK + 1) * (2 * KK + 1) * now.Ls * now.H * now.W;
-        save_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(now, old, out,
+        save_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(now, old, out,
                                                                                                         words, runs);
     });
 }
 
 template <typename T, typename WT>
 void entries_check_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
-    const int runs = window_runs(a, kept);
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        entries_check_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(a, runs);
+        const int runs = window_runs(a, kept, window_run<T, KK>());
+        entries_check_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(a, runs);
     });
 }
 
 template <typename T, typename WT>
 void entries_to_levels_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
-    const int runs = window_runs(a, kept);
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        entries_to_levels_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), 128, 0, s>>>(a, runs);
+        const int runs = window_runs(a, kept, window_run<T, KK>());
+        entries_to_levels_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(a, runs);
     });
 }
 
 template <typename T, typename WT>
 void level_table_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
-    const int runs = window_runs(a, kept);
+    const int runs = window_runs(a, kept, 128);
     with_grid_k(K, [&](auto k) {
         level_table_kernel<T, WT, decltype(k)::value><<<window_blocks(runs, nsm, 16), 128, 0, s>>>(
             a.omega, const_cast<code_t<T>*>(a.tab), a.H, a.W, a.S, a.half, a.coef, a.grid, runs, a.ctl);

@@ -494,14 +494,17 @@ def test_captured_batch():
     ctx = [Fusion.from_problem(p, dtype="f32", wdtype="bf16") for p in ps]
     yl, yh = [dev(p.Yl) for p in ps], [dev(p.Yh) for p in ps]
     guides = [[dev(small(H=p.H, W=p.W, seed=s).Yh) for p in ps] for s in (7, 8)]
-    batch = FusionBatch(ctx)
-    batch.set_option(FUSE_OPT_GRAPH, 0)
+    stream = torch.cuda.Stream()                          # a batch keeps the stream it is created with
     for f, b in zip(ctx, yh):
         f.weights(b)
-    batch.solve(yl, yh, 5)
-    batch.sync()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(stream):
+        batch = FusionBatch(ctx)
+        batch.set_option(FUSE_OPT_GRAPH, 0)
+        batch.solve(yl, yh, 5)
+        batch.sync()
     g = torch.cuda.CUDAGraph()
-    with torch.cuda.graph(g):
+    with torch.cuda.graph(g, stream=stream):
         Xs, _ = batch.solve(yl, yh, 5)
     for scale, form in ((1.0, 2), (1e-3, 0), (1.0, 2)):   # the data too
         for gs in guides:
@@ -509,6 +512,7 @@ def test_captured_batch():
                 f.weights(w)
             for a, p in zip(yl, ps):
                 a.copy_(dev(p.Yl) * scale)
+            torch.cuda.synchronize()
             g.replay()
             torch.cuda.synchronize()
             got = [x.clone() for x in Xs]
@@ -516,3 +520,37 @@ def test_captured_batch():
                 assert f.get_option(FUSE_OPT_LATENT_FORM) == form
                 assert torch.equal(x, f.solve(a, b, 5)[0])
     batch.close()
+
+
+@pytest.mark.parametrize("K,dtype", [(1, "f32"), (2, "f32"), (1, "f64"), (2, "f64")])
+@pytest.mark.parametrize("how", ["levels", "entries", "monitored", "host"])
+def test_stored_entries_stay_within_their_thresholds(K, dtype, how):
+    # a threshold that the grid rounds up: an entry at it is stored as the threshold itself
+    p = small(K=K, lam2=1e-3)
+    td = torch.float64 if dtype == "f64" else torch.float32
+    f = Fusion.from_problem(p, dtype=dtype, wdtype=dtype)
+    if how == "entries":
+        f.set_option(FUSE_OPT_LATENT_IMPL, 0)
+    if how == "monitored":
+        f.set_option(FUSE_OPT_RESIDUALS, 1)
+    yl, yh = dev(p.Yl, td), dev(p.Yh, td)
+    f.weights(yh)
+    f.solve(yl, yh, 6)
+    n, nk, nP, Ls = p.H * p.W, f.nW // 2, (2 * K + 1) ** 2, p.L_s
+    om = torch.tensor(p.lam2 / p.rho, dtype=td, device="cuda") * f.get_weights()
+    if how == "host":                                     # in place, and then to host memory
+        buf = torch.empty(fuse.fuse_state_bytes(f.ctx), dtype=torch.uint8)
+        fuse.fuse_get_state(f.ctx, buf.data_ptr())
+        st = buf.cuda()
+    else:
+        st = f.get_state()
+    s = st.view(td)[5 * Ls * n:][:nk * nP * Ls * n].reshape(nk, nP, Ls, p.H, p.W).abs()
+    hit = 0.0
+    for k, (a, b) in enumerate((a, b) for a in range(-K, K + 1) for b in range(-K, K + 1)):
+        mu = torch.roll(om[nk:], (-a, -b), (1, 2))[:, None]          # omega_tau(m + k)
+        assert (s[:, k] <= mu).all()
+        hit += (s[:, k] == mu).double().mean().item() / nP
+    assert hit > 0.1                                      # the test's point: some are at theirs
+    X = f.solve(yl, yh, 5, warm=True)[0].clone()
+    assert torch.equal(X, f.solve(yl, yh, 11)[0])
+    f.close()
