@@ -1050,19 +1050,26 @@ fuse_status need_entries(fuse_ctx* c, int want = kStateGrid) {
 }
 
 // The state that a solve of the inputs Yl (NULL: of none yet) starts with.
-void begin_state(fuse_ctx* c, const void* Yl, bool cold, int want) {
-    const size_t count = Yl && want != kStateEntries && want != kStateGiven ? (size_t)c->Ll * c->nl : 0;
+template <typename T>
+BeginArgs<T> begin_args(const fuse_ctx* c, const void* Yl, bool cold, int want) {
     // X = Z E^T / eps where E E^T = eps I, and |B| <= sum |b|
     double taps = 0.0;
     for (double t : c->htapsB) taps += std::fabs(t);
-    const double gain = taps * std::sqrt(c->eet_eps), coef = c->lam2 / c->rho;
-    if (c->dtype == FUSE_F64)
-        latent_begin_launch<double>((const double*)Yl, count, (const uint8_t*)c->mask, c->n, gain, coef,
-                                    (const LatentGrid<double>*)c->grid, c->ctl, cold, want, c->stream);
-    else
-        latent_begin_launch<float>((const float*)Yl, count, (const uint8_t*)c->mask, c->n, gain, coef,
-                                   (const LatentGrid<float>*)c->grid, c->ctl, cold, want, c->stream);
-    c->launches_all++;
+    const size_t count = Yl && want != kStateEntries && want != kStateGiven ? (size_t)c->Ll * c->nl : 0;
+    return BeginArgs<T>{(const T*)Yl, (const uint8_t*)c->mask, count, c->n, taps * std::sqrt(c->eet_eps),
+                        c->lam2 / c->rho, (const LatentGrid<T>*)c->grid, c->ctl, cold, want};
+}
+template <typename T>
+void begin_states(fuse_ctx* const* c, const void* const* Yl, const int* want, int n, bool cold, cudaStream_t s) {
+    std::vector<BeginArgs<T>> a;
+    for (int i = 0; i < n; ++i)
+        if (on_grid(c[i])) a.push_back(begin_args<T>(c[i], Yl[i], cold, want[i]));
+    if (!a.empty()) latent_begin_launch<T>(a.data(), (int)a.size(), s);
+    c[0]->launches_all += ((int)a.size() + BeginBatch<T>::kMost - 1) / BeginBatch<T>::kMost;
+}
+void begin_states(fuse_ctx* const* c, const void* const* Yl, const int* want, int n, bool cold, cudaStream_t s) {
+    if (c[0]->dtype == FUSE_F64) begin_states<double>(c, Yl, want, n, cold, s);
+    else begin_states<float>(c, Yl, want, n, cold, s);
 }
 
 // Brings the latent state into the form in which the iterations of a solve continue or start, `want`:
@@ -1071,11 +1078,12 @@ void begin_state(fuse_ctx* c, const void* Yl, bool cold, int want) {
 //   kStateEntries  entries in the arithmetic of the iterate type
 // off the grid where it does not carry the inputs Yl.  Where nothing touched the state since a solve with
 // the same `want`, those are all that can have changed.
-fuse_status settle(fuse_ctx* c, const void* Yl, bool cold, int want) {
+// begun: a launch for several problems has done the first step.
+fuse_status settle(fuse_ctx* c, const void* Yl, bool cold, int want, bool begun = false) {
     if (!on_grid(c)) return FUSE_OK;
     const bool touched = capturing(c) || c->captured || c->settled != want;
-    if (cold || touched || want != kStateEntries) {
-        begin_state(c, Yl, cold, want);
+    if (!begun && (cold || touched || want != kStateEntries)) {
+        begin_states(&c, &Yl, &want, 1, cold, c->stream);
         CKL(c, "latent_begin_kernel");
     }
     if (!cold && (touched || want == kStateLevels)) {
@@ -2321,7 +2329,9 @@ fuse_status fuse_set_state(fuse_ctx* c, const void* src) {
     p += c->sig_bytes;
     CK(c, cudaMemcpyAsync(c->planes, p, c->plane_bytes, cudaMemcpyDefault, c->stream));
     if (on_grid(c)) {
-        begin_state(c, nullptr, true, kStateGiven);
+        const void* none = nullptr;
+        const int given = kStateGiven;
+        begin_states(&c, &none, &given, 1, true, c->stream);
         CKL(c, "latent_begin_kernel");
         c->settled = -1;
     }
@@ -2715,11 +2725,18 @@ fuse_status fuse_batch_solve(fuse_batch* b, const void* const* Yl, const void* c
     if (iters < 0) return bfail(b, FUSE_EINVAL, "iters must be >= 0");
     if (cudaSetDevice(b->device) != cudaSuccess) return bfail(b, FUSE_ECUDA, "cudaSetDevice");
     const int n = (int)b->ctx.size();
+    std::vector<int> want(n);
     for (int i = 0; i < n; ++i) {
         fuse_ctx* c = b->ctx[i];
         if (!Yl[i] || !Yh[i]) return bfail(b, FUSE_EINVAL, "NULL input of a problem");
         if (c->sticky != FUSE_OK || !c->have_weights) return bfail(b, FUSE_ESTATE, "a problem has no weights or holds an error");
         c->stream = b->stream;
+        want[i] = !b->on_levels[i] ? kStateEntries : iters > 0 ? kStateLevels : kStateGiven;
+    }
+    begin_states(b->ctx.data(), Yl, want.data(), n, true, b->stream);
+    BCK(b, cudaGetLastError());
+    for (int i = 0; i < n; ++i) {
+        fuse_ctx* c = b->ctx[i];
         const bool f64 = c->dtype == FUSE_F64;
         fuse_status st = f64 ? Impl<double>::band_mix(c, b->stream, Yl[i], c->D9a, c->Et, c->nl, c->Ll, c->Ls)
                              : Impl<float>::band_mix(c, b->stream, Yl[i], c->D9a, c->Et, c->nl, c->Ll, c->Ls);
@@ -2731,7 +2748,8 @@ fuse_status fuse_batch_solve(fuse_batch* b, const void* const* Yl, const void* c
         if (st != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
         c->have_state = true;
         c->path = b->on_levels[i] ? 1 : 0;
-        if ((st = settle(c, Yl[i], true, b->on_levels[i] ? (iters > 0 ? kStateLevels : kStateGiven) : kStateEntries)) != FUSE_OK) return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
+        if ((st = settle(c, Yl[i], true, want[i], true)) != FUSE_OK)
+            return bfail(b, st, "problem " + std::to_string(i) + ": " + c->err);
     }
     fuse_status st = batch_run(b, iters, iters > 0);
     if (st != FUSE_OK) return st;

@@ -43,12 +43,12 @@ struct LevelArgs {
 
 // Whether this is the last block of a launch to finish; true for all of its threads or none.  What the
 // other blocks wrote before is visible to it, and no block reads the state's mode after that.
-__device__ __forceinline__ bool last_block(LatentCtl* ctl) {
+__device__ __forceinline__ bool last_block(LatentCtl* ctl, unsigned blocks) {
     __shared__ int last;
     __syncthreads();
     if (threadIdx.x == 0) {
         __threadfence();
-        last = atomicAdd(&ctl->done, 1u) == gridDim.x * gridDim.y - 1;
+        last = atomicAdd(&ctl->done, 1u) == blocks - 1;
         if (last) ctl->done = 0;
         __threadfence();
     }
@@ -197,7 +197,7 @@ level_table_kernel(const WT* __restrict__ omega, code_t<T>* __restrict__ tab, in
         for (int i = threadIdx.x; i < cnt; i += 128) out[i] = sm[i];
         __syncthreads();
     }
-    if (last_block(ctl) && threadIdx.x == 0) ctl->table = 1;
+    if (last_block(ctl, gridDim.x) && threadIdx.x == 0) ctl->table = 1;
 }
 
 // Steps (bands x offsets) of a block: one bit each in a thread's event mask, five in a list entry.
@@ -508,7 +508,7 @@ levels_to_entries_kernel(LevelArgs<T, WT> now, LevelArgs<T, WT> old, int work, i
     if (now.ctl->mode != kStateLevels || !(now.ctl->was || want < kStateLevels || !now.ctl->fit)) return;
     const LevelArgs<T, WT> a = now.ctl->was ? old : now;
     write_entries<T, WT, K>(a, reinterpret_cast<T*>(a.e), work, stage + threadIdx.x, stage + NP * R + threadIdx.x);
-    if (last_block(now.ctl) && threadIdx.x == 0) {
+    if (last_block(now.ctl, gridDim.x) && threadIdx.x == 0) {
         now.ctl->mode = want == kStateEntries || !now.ctl->fit ? kStateEntries : now.ctl->was ? kStateGiven : kStateGrid;
         now.ctl->was = 0;
     }
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>()) e
             if (!ok) *off = 1;
         }
     });
-    if (last_block(a.ctl) && threadIdx.x == 0) {
+    if (last_block(a.ctl, gridDim.x) && threadIdx.x == 0) {
         a.ctl->mode = *off ? kStateEntries : kStateGrid;
         *off = 0;
     }
@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>()) e
             if constexpr (NP != 9) a.masks[o] = make_uint2(l.E, l.G);
         }
     });
-    if (last_block(a.ctl) && threadIdx.x == 0) a.ctl->mode = kStateLevels;
+    if (last_block(a.ctl, gridDim.x) && threadIdx.x == 0) a.ctl->mode = kStateLevels;
 }
 
 // Before the weights change (words: those of the weights, 16 bytes each): levels stay readable through
@@ -629,7 +629,7 @@ weights_change_kernel(const uint4* __restrict__ omega, uint4* __restrict__ was, 
     if (keep)
         for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (size_t)gridDim.x * blockDim.x)
             was[i] = omega[i];
-    if (last_block(ctl) && threadIdx.x == 0) {
+    if (last_block(ctl, gridDim.x) && threadIdx.x == 0) {
         if (keep) {
             grid[1] = grid[0];
             ctl->was = 1;
@@ -642,13 +642,38 @@ weights_change_kernel(const uint4* __restrict__ omega, uint4* __restrict__ was, 
 
 // The state that a solve starts with, and whether the grid carries its inputs: their size is the rms of
 // the `count` samples of Y_l that S keeps (mask, over n pixels, or all), divided by `gain`, the most that B and E
-// can have raised that of X.  Sums in FP64, in the same order on every device; latency-bound, about
-// 5 us for 131 thousand samples.
+// can have raised that of X.  Block row y of the launch is problem y.  The sums are formed in the same order
+// on every device.  Latency-bound: a thread has its eight samples in flight at once, a problem of one block
+// (8192 samples) needs no second round, and the problems of a batch share a launch (11 problems of 32
+// to 360: 15 us of a call, 105 with a launch each).
 template <typename T>
-__global__ void __launch_bounds__(256)
-latent_begin_kernel(const T* __restrict__ Y, size_t count, const uint8_t* __restrict__ mask, size_t n, double gain,
-                    double coef, const LatentGrid<T>* grid, LatentCtl* ctl, int cold, int want) {
-    __shared__ double red[2][8];
+struct BeginArgs {
+    const T* Y;
+    const uint8_t* mask;
+    size_t count, n;
+    double gain, coef;
+    const LatentGrid<T>* grid;
+    LatentCtl* ctl;
+    int cold, want;
+};
+template <typename T>
+struct BeginBatch {
+    static constexpr int kMost = 32;                  // problems of a launch: 2.6 KB of arguments
+    BeginArgs<T> a[kMost];
+};
+inline __host__ __device__ int begin_blocks(size_t count) {
+    const size_t need = (count + kBeginSamples - 1) / kBeginSamples;
+    return (int)(need < 1 ? 1 : need < (size_t)kBeginBlocks ? need : (size_t)kBeginBlocks);
+}
+template <typename T>
+__global__ void __launch_bounds__(1024) latent_begin_kernel(const __grid_constant__ BeginBatch<T> batch) {
+    constexpr int R = kBeginSamples / 1024;
+    __shared__ double red[2][32];
+    const BeginArgs<T>& a = batch.a[blockIdx.y];
+    const int blocks = begin_blocks(a.count), tid = threadIdx.x;
+    if ((int)blockIdx.x >= blocks) return;
+    const double g = (double)a.grid->g, wmax = (double)a.grid->wmax;
+    const int mode = a.ctl->mode;
     double sq = 0.0, seen = 0.0;
     // the block's sums, in thread 0
     auto reduce = [&]() {
@@ -657,51 +682,58 @@ latent_begin_kernel(const T* __restrict__ Y, size_t count, const uint8_t* __rest
             sq += __shfl_down_sync(0xffffffffu, sq, o);
             seen += __shfl_down_sync(0xffffffffu, seen, o);
         }
-        if ((threadIdx.x & 31) == 0) {
-            red[0][threadIdx.x >> 5] = sq;
-            red[1][threadIdx.x >> 5] = seen;
+        __syncthreads();
+        if ((tid & 31) == 0) {
+            red[0][tid >> 5] = sq;
+            red[1][tid >> 5] = seen;
         }
         __syncthreads();
-        for (int w = 1; threadIdx.x == 0 && w < 8; ++w) {
-            sq += red[0][w];
-            seen += red[1][w];
+        if (tid < 32) {
+            sq = red[0][tid];
+            seen = red[1][tid];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                sq += __shfl_down_sync(0xffffffffu, sq, o);
+                seen += __shfl_down_sync(0xffffffffu, seen, o);
+            }
         }
     };
-    const size_t step = (size_t)gridDim.x * 256, first = (size_t)blockIdx.x * 256 + threadIdx.x;
-    const size_t pstep = step % n;
-    size_t p = first % n;                             // the sample's pixel (with a mask)
-#pragma unroll 4
-    for (size_t i = first; i < count; i += step) {
-        if (!mask || mask[p]) {
-            const double v = (double)Y[i];
-            sq += v * v;
-            seen += 1.0;
+    for (size_t i0 = (size_t)blockIdx.x * kBeginSamples; i0 < a.count; i0 += (size_t)blocks * kBeginSamples) {
+        T v[R], part = T(0);
+        int kept = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const size_t i = i0 + r * 1024 + tid;
+            const bool keep = i < a.count && (!a.mask || a.mask[i % a.n]);
+            v[r] = keep ? a.Y[i] : T(0);
+            kept += keep;
         }
-        p += pstep;
-        if (p >= n) p -= n;
+#pragma unroll
+        for (int r = 0; r < R; ++r) part += v[r] * v[r];
+        sq += (double)part;
+        seen += (double)kept;
     }
     reduce();
-    if (threadIdx.x == 0) {
-        ctl->part[blockIdx.x] = sq;
-        ctl->seen[blockIdx.x] = seen;
+    if (blocks > 1) {
+        if (tid == 0) {
+            a.ctl->part[blockIdx.x] = sq;
+            a.ctl->seen[blockIdx.x] = seen;
+        }
+        if (!last_block(a.ctl, blocks)) return;
+        sq = tid < blocks ? __ldcg(&a.ctl->part[tid]) : 0.0;
+        seen = tid < blocks ? __ldcg(&a.ctl->seen[tid]) : 0.0;
+        reduce();
     }
-    if (!last_block(ctl)) return;
-    sq = seen = 0.0;
-    for (unsigned b = threadIdx.x; b < gridDim.x; b += 256) {
-        sq += __ldcg(&ctl->part[b]);
-        seen += __ldcg(&ctl->seen[b]);
-    }
-    reduce();
-    if (threadIdx.x != 0) return;
-    const double top = ldexp((double)grid->g, grid_code<T>::B), wmax = (double)grid->wmax;
+    if (tid != 0) return;
+    const double top = ldexp(g, grid_code<T>::B);
     // thresholds that are all zero leave the entries zero, on the grid of anything
-    const bool fit = wmax <= 1e308 && (coef * wmax == 0.0 || top * gain <= sqrt(sq / seen));
-    ctl->fit = fit;
-    if (cold) {
-        ctl->mode = fit || want == kStateGiven ? want : kStateEntries;
-        ctl->was = 0;
-    } else if (ctl->mode != kStateLevels && (want == kStateEntries || !fit)) {
-        ctl->mode = kStateEntries;
+    const bool fit = wmax <= 1e308 && (a.coef * wmax == 0.0 || top * a.gain <= sqrt(sq / seen));
+    a.ctl->fit = fit;
+    if (a.cold) {
+        a.ctl->mode = fit || a.want == kStateGiven ? a.want : kStateEntries;
+        a.ctl->was = 0;
+    } else if (mode != kStateLevels && (a.want == kStateEntries || !fit)) {
+        a.ctl->mode = kStateEntries;
     }
 }
 

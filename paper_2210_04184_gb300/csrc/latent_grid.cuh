@@ -80,7 +80,8 @@ template <typename T> struct LatentGrid {
 //   kStateGrid     entries on the grid, those of a run on the current weights
 //   kStateLevels   levels, formed with the current weights or, with `was`, with the ones before them
 //   kStateGiven    entries not looked at yet: set by the caller, or left by other weights
-constexpr int kBeginBlocks = 512;       // most blocks of latent_begin_kernel
+// latent_begin_kernel: most blocks of a problem, samples of a block at a time
+constexpr int kBeginBlocks = 256, kBeginSamples = 8192;
 enum : int { kStateEntries = 0, kStateGrid = 1, kStateLevels = 2, kStateGiven = 3 };
 struct LatentCtl {
     int mode;

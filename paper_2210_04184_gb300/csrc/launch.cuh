@@ -79,12 +79,11 @@ void level_table_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cud
 template <typename T>
 void weights_change_launch(const void* omega, void* was, size_t bytes, LatentGrid<T>* grid, LatentCtl* ctl, int nsm,
                            cudaStream_t s);
-// The state that a solve starts with, from zero as `want` (kState...) or a continued one, by the size of its
+// The states that n solves start with, from zero as `want` (kState...) or continued ones, by the size of their
 // inputs (latent_begin_kernel); without inputs (count 0) nothing but `want` decides for
 // kStateEntries and kStateGiven.
 template <typename T>
-void latent_begin_launch(const T* Y, size_t count, const uint8_t* mask, size_t n, double gain, double coef,
-                         const LatentGrid<T>* grid, LatentCtl* ctl, int cold, int want, cudaStream_t s);
+void latent_begin_launch(const BeginArgs<T>* a, int n, cudaStream_t s);
 // The grid of n weights from the largest (grid zeroed by the caller); two launches.
 template <typename T, typename WT>
 void wmax_launch(const WT* w, size_t n, LatentGrid<T>* grid, T coef, cudaStream_t s);

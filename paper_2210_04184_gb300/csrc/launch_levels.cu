@@ -115,11 +115,18 @@ void weights_change_launch(const void* omega, void* was, size_t bytes, LatentGri
 }
 
 template <typename T>
-void latent_begin_launch(const T* Y, size_t count, const uint8_t* mask, size_t n, double gain, double coef,
-                         const LatentGrid<T>* grid, LatentCtl* ctl, int cold, int want, cudaStream_t s) {
-    const size_t need = (count + 2047) / 2048;
-    const unsigned blocks = (unsigned)(need < 1 ? 1 : need < (size_t)kBeginBlocks ? need : (size_t)kBeginBlocks);
-    latent_begin_kernel<T><<<blocks, 256, 0, s>>>(Y, count, mask, n, gain, coef, grid, ctl, cold, want);
+void latent_begin_launch(const BeginArgs<T>* a, int n, cudaStream_t s) {
+    for (int i = 0; i < n; i += BeginBatch<T>::kMost) {
+        BeginBatch<T> batch;
+        const int m = n - i < BeginBatch<T>::kMost ? n - i : BeginBatch<T>::kMost;
+        int blocks = 1;
+        for (int j = 0; j < m; ++j) {
+            batch.a[j] = a[i + j];
+            const int k = begin_blocks(a[i + j].count);
+            blocks = k > blocks ? k : blocks;
+        }
+        latent_begin_kernel<T><<<dim3((unsigned)blocks, (unsigned)m), 1024, 0, s>>>(batch);
+    }
 }
 
 template <typename T, typename WT>
@@ -168,10 +175,8 @@ FUSE_LEVELS_INST(float, float)
 FUSE_LEVELS_INST(float, __nv_bfloat16)
 FUSE_LEVELS_INST(double, double)
 template void weights_change_launch<float>(const void*, void*, size_t, LatentGrid<float>*, LatentCtl*, int, cudaStream_t);
-template void latent_begin_launch<float>(const float*, size_t, const uint8_t*, size_t, double, double,
-                                         const LatentGrid<float>*, LatentCtl*, int, int, cudaStream_t);
-template void latent_begin_launch<double>(const double*, size_t, const uint8_t*, size_t, double, double,
-                                          const LatentGrid<double>*, LatentCtl*, int, int, cudaStream_t);
+template void latent_begin_launch<float>(const BeginArgs<float>*, int, cudaStream_t);
+template void latent_begin_launch<double>(const BeginArgs<double>*, int, cudaStream_t);
 template void weights_change_launch<double>(const void*, void*, size_t, LatentGrid<double>*, LatentCtl*, int, cudaStream_t);
 
 }  // namespace fuse
