@@ -86,7 +86,12 @@ enum {
                                     other patches, the 16-bit state, no memory for the levels, a
                                     state that is not that of a run on the current weights (set by
                                     the caller, or after new weights, until the next solve from
-                                    zero), a context whose first solve the caller captured.
+                                    zero), a context whose first solve the caller captured, and
+                                    inputs that the grid does not carry as well: lambda2/rho times
+                                    the largest weight (fuse_weights: 1), up to the next power of
+                                    two, above the rms of the sampled Y_l (for X of its size; sums
+                                    of |blur| and the scale of E are allowed for), or weights that
+                                    are not finite numbers >= 0.  The device decides, per solve.
                                     2: always entries through the ring.
                                     0: entries with register-staged loads, in the arithmetic (grid
                                     or not) that the default would use, and with its bits. */
@@ -210,7 +215,8 @@ fuse_status fuse_set_stream(fuse_ctx* ctx, void* stream);
  * context as [|W|][H][W] of wdtype.  Must precede fuse_solve.  Errors: FUSE_EINVAL, FUSE_ECUDA. */
 fuse_status fuse_weights(fuse_ctx* ctx, const void* guide_dev);
 
-/* Replace the stored weights with w_dev [|W|][H][W] of the context's wdtype (device). */
+/* Replace the stored weights with w_dev [|W|][H][W] of the context's wdtype (device).  Weights are
+ * finite numbers >= 0; one that is infinite or not a number sets no threshold for its entries. */
 fuse_status fuse_set_weights(fuse_ctx* ctx, const void* w_dev);
 
 /* Copy the stored weights into w_dev [|W|][H][W] of the context's wdtype (device). */

@@ -563,15 +563,17 @@ void levels_shape(fuse_ctx* c) {
     c->lv_threads = kLevelThreads;
 }
 
-// The latent state lives on the grid (latent_grid.cuh), whichever form and kernel a solve uses.
+// Contexts whose latent state can be on the grid (latent_grid.cuh), and as levels; whether a solve's is, its
+// inputs decide (latent_begin_kernel).
 // Not FP32 states of 3 x 3 patches and a 3 x 3 search: they have only 36 words per pixel and band, which L2
-// holds for most sizes, and the events of levels cost more than the traffic that they save.  Whole
-// solves of 24 iterations, entries against levels (us): 64 x 64, 14 bands 643, 671; 96 x 320, 14 bands 1316,
-// 1377; 256 x 256, 8 bands 1259, 1627; 512 x 512, 4 bands 2241, 2514; but 64 x 64, 4 bands 600, 516 and
-// 384 x 384, 14 bands 4655, 4346.  The rule looks at the options alone, so that a problem gives the same
-// bits in a batch of any size.  The next state up, a 5 x 5 search: 64 x 64, 14 bands 835, 810; 96 x 320, 14
-// bands 2263, 2157; 256 x 256, 8 bands 2358, 2398 (60 iterations: 5734, 5325); 512 x 512, 18 bands 20221,
-// 15989; five by five patches with a 3 x 3 search: 96 x 320, 14 bands 2094, 1960; FP64: 9594, 5734 at 256 x 256.
+// holds for most sizes, and the events of levels cost more than the traffic that they save at most of
+// them.  Whole solves of 24 iterations, entries against levels (us): 64 x 64, 14 bands 643, 671; 96 x 320, 14
+// bands 1316, 1377; 256 x 256, 8 bands 1259, 1627; 512 x 512, 4 bands 2241, 2514; the other way 64 x 64, 4
+// bands 600, 516 and 384 x 384, 14 bands 4655, 4346.  The rule looks at the options alone, so that a problem
+// gives the same bits in a batch of any size, and is not the best one at every size.  The next state up, a
+// 5 x 5 search: 64 x 64, 14 bands 835, 810; 96 x 320, 14 bands 2263, 2157; 256 x 256, 8 bands 2358, 2398 (60
+// iterations: 5734, 5325); 512 x 512, 18 bands 20221, 15989; five by five patches with a 3 x 3 search: 96 x 320,
+// 14 bands 2094, 1960; FP64: 9594, 5734 at 256 x 256.
 bool grid_options(const fuse_ctx* c) { return c->lv_threads > 0 && !(c->esz == 4 && c->K == 1 && c->S == 1); }
 bool on_grid(const fuse_ctx* c) { return c->sfmt == 0 && grid_options(c); }
 

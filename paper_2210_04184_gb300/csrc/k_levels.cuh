@@ -4,7 +4,7 @@
 // offsets) and, for 25 entries, the level masks in the same order; level values [|W|][NP][L_s][H][W]
 // (plane p of a (tau, c, m) in use for its level of height p); prefix sums of the sorted threshold
 // codes of every patch window [|W|][H][W][NP], formed once per weights; points (X with its running sums,
-// written by the X update's last pass), so w = after(m - tau) - after(m).
+// written by points_kernel from the new X), so w = after(m - tau) - after(m).
 //
 // One block owns rows [y0, y0 + Ty) of one tau1 row and nb bands.  Per band and tau2 (a step) a thread
 // reads its pixel's record and the shifted point; with its own point these give delta, w and the
