@@ -601,11 +601,12 @@ bool levels_alloc(fuse_ctx* c) {
                             (size_t)c->nW * c->n * c->wsz};
     size_t total = 0, room = 0, all = 0;
     for (size_t b : bytes) total += (b + 255) / 256 * 256;
-    // one allocation, hdr; some memory is left for what else a program allocates.  A stream that another
-    // thread captures meanwhile, in whichever mode, is not disturbed by it.
+    // one allocation, hdr; some memory is left for what else a program allocates (asked for large problems
+    // only: the query takes longer than a small allocation).  A stream that another thread captures
+    // meanwhile, in whichever mode, is not disturbed by it.
     cudaStreamCaptureMode mode = cudaStreamCaptureModeThreadLocal;
     cudaThreadExchangeStreamCaptureMode(&mode);
-    bool ok = cudaMemGetInfo(&room, &all) == cudaSuccess && room >= total + kLevelsLeave &&
+    bool ok = (total < kLevelsLeave / 8 || (cudaMemGetInfo(&room, &all) == cudaSuccess && room >= total + kLevelsLeave)) &&
               cudaMalloc(&c->hdr, total) == cudaSuccess;
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (ok) {
@@ -1084,6 +1085,7 @@ void begin_states(fuse_ctx* const* c, const void* const* Yl, const int* want, in
 fuse_status settle(fuse_ctx* c, const void* Yl, bool cold, int want, bool begun = false) {
     if (!on_grid(c)) return FUSE_OK;
     const bool touched = capturing(c) || c->captured || c->settled != want;
+    if (cold || touched) c->settled = -1;                   // until it is done
     if (!begun && (cold || touched || want != kStateEntries)) {
         begin_states(&c, &Yl, &want, 1, cold, c->stream);
         CKL(c, "latent_begin_kernel");
