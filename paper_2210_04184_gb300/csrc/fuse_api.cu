@@ -1551,7 +1551,8 @@ struct BatchImpl {
         // iterations on levels: 124.6 ms with 8 bands, 126.5 with 2; data off the grid 194.2 and 198.9).
         auto ring_blocks = [&](int bands) {
             long long t = 0;
-            for (int i = 0; i < n; ++i) t += (long long)((b->ctx[i]->H + Ty[i] - 1) / Ty[i]) * ((b->Ls + bands - 1) / bands) * rows;
+            for (int i = 0; i < n; ++i)
+                t += (long long)((b->ctx[i]->H + Ty[i] - 1) / Ty[i]) * ((b->Ls + bands - 1) / bands) * rows;
             return t;
         };
         int bpb = b->lat_bpb;
@@ -1600,8 +1601,9 @@ struct BatchImpl {
             }
             for (int heavy = 1; heavy >= 0; --heavy)       // tau1 != 0 rows of every problem first
                 for (int i = 0; i < n; ++i)
-                    if (b->on_levels[i]) add_segment(seg, i, (b->ctx[i]->H + lv[i].Ty - 1) / lv[i].Ty, (b->Ls + lv[i].nb - 1) / lv[i].nb,
-                                heavy ? rows - 1 : 1, heavy ? 0 : rows - 1, &next);
+                    if (b->on_levels[i])
+                        add_segment(seg, i, (b->ctx[i]->H + lv[i].Ty - 1) / lv[i].Ty, (b->Ls + lv[i].nb - 1) / lv[i].nb,
+                                    heavy ? rows - 1 : 1, heavy ? 0 : rows - 1, &next);
             b->lv_nseg = (int)seg.size();
             b->lv_blocks = next;
             b->pt_nseg = (int)sp.size();
@@ -1749,7 +1751,8 @@ struct BatchImpl {
             if (zero_in) {              // X of a cold first iteration is zero, and so are the planes
                 for (size_t i = 0; i < b->ctx.size(); ++i) {
                     fuse_ctx* c = b->ctx[i];
-                    if (b->on_levels[i]) levels_init_launch<T, WT>(Impl<T>::template lv_args<WT>(c), c->K, Impl<T>::kept(c), 0, s);
+                    if (b->on_levels[i])
+                        levels_init_launch<T, WT>(Impl<T>::template lv_args<WT>(c), c->K, Impl<T>::kept(c), 0, s);
                 }
             } else {
                 levels_batch_launch<T, WT>(lv, b->d_lv_seg, b->lv_nseg, b->K, (unsigned)b->lv_blocks, kLevelThreads,

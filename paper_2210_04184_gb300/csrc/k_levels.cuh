@@ -551,7 +551,8 @@ __device__ __forceinline__ bool entry_codes(const T* eb, size_t kst, T ig, const
 // Whether given entries are those of a run on the current weights, which the update on the grid and the
 // levels need: on the grid, |s| <= mu, and 1-Lipschitz in mu, the state of a stop operator.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>()) entries_check_kernel(LevelArgs<T, WT> a, int work) {
+__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>())
+entries_check_kernel(LevelArgs<T, WT> a, int work) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);
@@ -583,7 +584,8 @@ __global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>()) e
 
 // Entries of a run on the current weights -> levels.
 template <typename T, typename WT, int K>
-__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>()) entries_to_levels_kernel(LevelArgs<T, WT> a, int work) {
+__global__ void __launch_bounds__(window_run<T, K>(), window_resident<T, K>())
+entries_to_levels_kernel(LevelArgs<T, WT> a, int work) {
     using C = code_t<T>;
     using U = typename grid_code<T>::utype;
     constexpr int NP = (2 * K + 1) * (2 * K + 1);

@@ -62,8 +62,10 @@ void levels_to_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT
                               cudaStream_t s) {
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        const int runs = window_runs(now, kept, window_run<T, KK>());
-        levels_to_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(now, old, runs, want);
+        constexpr int R = window_run<T, KK>();
+        const int runs = window_runs(now, kept, R);
+        const unsigned blocks = window_blocks(runs, nsm, window_resident<T, KK>());
+        levels_to_entries_kernel<T, WT, KK><<<blocks, R, 0, s>>>(now, old, runs, want);
     });
 }
 
@@ -72,9 +74,11 @@ void save_entries_launch(const LevelArgs<T, WT>& now, const LevelArgs<T, WT>& ol
                          cudaStream_t s) {
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        const int runs = window_runs(now, kept, window_run<T, KK>());
+        constexpr int R = window_run<T, KK>();
+        const int runs = window_runs(now, kept, R);
+        const unsigned blocks = window_blocks(runs, nsm, window_resident<T, KK>());
         const size_t words = (size_t)kept * (2 * KK + 1) * (2 * KK + 1) * now.Ls * now.H * now.W;
-        save_entries_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(now, old, out,
+        save_entries_kernel<T, WT, KK><<<blocks, R, 0, s>>>(now, old, out,
                                                                                                         words, runs);
     });
 }
@@ -83,8 +87,10 @@ template <typename T, typename WT>
 void entries_check_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        const int runs = window_runs(a, kept, window_run<T, KK>());
-        entries_check_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(a, runs);
+        constexpr int R = window_run<T, KK>();
+        const int runs = window_runs(a, kept, R);
+        const unsigned blocks = window_blocks(runs, nsm, window_resident<T, KK>());
+        entries_check_kernel<T, WT, KK><<<blocks, R, 0, s>>>(a, runs);
     });
 }
 
@@ -92,8 +98,10 @@ template <typename T, typename WT>
 void entries_to_levels_launch(const LevelArgs<T, WT>& a, int K, int kept, int nsm, cudaStream_t s) {
     with_grid_k(K, [&](auto k) {
         constexpr int KK = decltype(k)::value;
-        const int runs = window_runs(a, kept, window_run<T, KK>());
-        entries_to_levels_kernel<T, WT, KK><<<window_blocks(runs, nsm, window_resident<T, KK>()), window_run<T, KK>(), 0, s>>>(a, runs);
+        constexpr int R = window_run<T, KK>();
+        const int runs = window_runs(a, kept, R);
+        const unsigned blocks = window_blocks(runs, nsm, window_resident<T, KK>());
+        entries_to_levels_kernel<T, WT, KK><<<blocks, R, 0, s>>>(a, runs);
     });
 }
 
