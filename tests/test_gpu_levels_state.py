@@ -554,3 +554,36 @@ def test_stored_entries_stay_within_their_thresholds(K, dtype, how):
     X = f.solve(yl, yh, 5, warm=True)[0].clone()
     assert torch.equal(X, f.solve(yl, yh, 11)[0])
     f.close()
+
+
+def test_without_memory_for_the_levels(monkeypatch):
+    # a context that gets no buffers for levels (an allocation failure armed and never reached has that
+    # effect) runs entries, alone and beside others in a batch, and takes up a state that was levels
+    p = small(K=2)
+    yl, yh = dev(p.Yl), dev(p.Yh)
+    a = Fusion.from_problem(p, dtype="f32", wdtype="bf16")
+    monkeypatch.setenv("FUSE_FAULT_ALLOC", "1000000")
+    f, g = (Fusion.from_problem(p, dtype="f32", wdtype="bf16") for _ in range(2))
+    monkeypatch.delenv("FUSE_FAULT_ALLOC")
+    g.set_option(FUSE_OPT_LATENT_IMPL, 2)
+    for c in (a, f, g):
+        c.weights(yh)
+    X = f.solve(yl, yh, 9)[0].clone()
+    assert f.get_option(FUSE_OPT_LATENT_FORM) == 0
+    assert torch.equal(X, g.solve(yl, yh, 9)[0])
+    Xa = a.solve(yl, yh, 9)[0].clone()
+    batch = FusionBatch([a, f])
+    Xs, _ = batch.solve([yl, yl], [yh, yh], 9)
+    batch.sync()
+    assert torch.equal(Xs[0], Xa) and torch.equal(Xs[1], X)
+    assert [c.get_option(FUSE_OPT_LATENT_FORM) for c in (a, f)] == [2, 0]
+    f.set_state(a.get_state())
+    om = a.get_weights().double().cpu().numpy()
+    ref = oracle_runs(p, [(om, 15)])[0]
+    assert rel(f.solve(yl, yh, 6, warm=True)[0], ref) <= FP32_BOUND
+    a.set_state(f.get_state())                            # and back: not entries of the grid
+    assert torch.equal(a.solve(yl, yh, 4, warm=True)[0], f.solve(yl, yh, 4, warm=True)[0])
+    assert a.get_option(FUSE_OPT_LATENT_FORM) == 0
+    batch.close()
+    for c in (a, f, g):
+        c.close()
